@@ -5,18 +5,18 @@
 // Each CTA therefore owns a slab of `sw` consecutive 64-bit words of every row
 // (64*sw source columns, 2 <= sw <= 128) and streams the whole level-ordered
 // schedule over it:
-//   * a producer warp copies the schedule, item by item, into a ring of shared
+//   * a producer warp copies the schedule, pack by pack, into a ring of shared
 //     memory stages with bulk asynchronous copies (cp.async.bulk, completion on
 //     an mbarrier), so the ops are read from L2/HBM once per CTA and without
 //     occupying the consumer threads;
 //   * consumer warps (12 when the CTA holds its SM alone, 4 when two CTAs share
-//     an SM) apply an item: a window whose rows fit the shared-memory row
-//     buffer ("local record") is gathered, updated level by level in shared
+//     an SM) apply a pack: a window whose rows fit the shared-memory row
+//     buffer (a record) is gathered, updated level by level in shared
 //     memory and written through at each row's last write; a tile of ops on
-//     rows in HBM ("global tile") runs through a private per-thread ring of
-//     cp.async copies, with hub PULLs as L2 OR-reductions.  The per-item named
+//     rows in HBM (a level of a tile pack) runs through a private per-thread ring of
+//     cp.async copies, with hub PULLs as L2 OR-reductions.  A named
 //     barrier orders one level's stores before the next level's loads.
-// All waits are bounded (TN_ETIMEOUT).  The per-item barrier is a reduction
+// All waits are bounded (TN_ETIMEOUT).  The barrier before a pack is a reduction
 // (bar.red.or) of every consumer's stop condition, so all consumers leave the
 // loop at the same barrier and none can be left waiting on it.
 #include <cuda_runtime.h>
@@ -37,15 +37,15 @@ constexpr int kWarpsAlone = 12;
 constexpr int kWarpsShared = 4;
 constexpr int kMaxThreads = 32 * kWarpsAlone + 32;
 constexpr int kStages = 2;
-constexpr uint32_t kEndItem = 0xFFFFFFFFu;
+constexpr uint32_t kStageShift = 1;
+constexpr size_t kSlabHead = (size_t)kStages * kStageBytes + 64;  // stages, barriers
 constexpr int kMaxPlans = 24;  // networks per launch
 constexpr int kMaxJobs = 2 * kMaxPlans;  // a network spread over a wave has CTAs of two widths
 
 struct Job {
     const uint2 *blob;
-    const uint4 *items;
+    const WinDesc *win;
     const uint32_t *aux;
-    uint64_t nitems;
     uint64_t *S;
     uint64_t ld;    // row stride in words
     uint64_t *tmp;  // saved-row slots of global windows, ld words each
@@ -53,13 +53,13 @@ struct Job {
     uint64_t w_begin;  // first row word of the job's first CTA
     uint32_t sw;    // slab words per CTA (even, 2..kMaxSlabWords)
     uint32_t cpr;   // 16-byte chunks of a row segment = sw / 2
+    uint32_t nwin;  // windows of the schedule
     uint32_t cta_begin;
     uint32_t dcap;  // row slots of the shared-memory row buffer
     // resident-slab form (rw > 0): each CTA keeps rw words of every row in shared memory
     uint32_t rw;     // words of every row per CTA (1, 2 or 4), 0 = column-slab form
     uint32_t rows;   // rows of the matrix (node count of the plan)
     uint32_t ntemp;  // saved-row slots of the plan's tie groups
-    uint64_t blob8;  // schedule length in 8-byte units
 };
 
 struct JobList {
@@ -68,18 +68,82 @@ struct JobList {
     uint32_t smem_bytes;  // dynamic shared memory of the launch
 };
 
-struct StageHdr {
-    uint32_t count;  // ops (global tile) or 8-byte units (local record); kEndItem = stop
-    uint32_t off;    // global tile: index of its first op in the stage (0 or 1)
-    uint32_t local;  // 1 = local record
-    uint32_t pad;
-};
-
 __device__ inline uint32_t find_job(const JobList &jl, uint32_t cta)
 {
     uint32_t j = 0;
     while (j + 1 < jl.count && jl.job[j + 1].cta_begin <= cta) ++j;
     return j;
+}
+
+// The ring of schedule packs: `nst` (a power of two) stages of kStageBytes in
+// shared memory and their full / empty barriers.  Behind the last pack comes a
+// stage whose header says kPackEnd.
+struct PackRing {
+    uint8_t *stage;
+    uint64_t *full, *empty;
+    uint32_t mask, shift;  // of nst
+    __device__ uint8_t *at(uint32_t q) const { return stage + (size_t)(q & mask) * kStageBytes; }
+    __device__ bool wait_full(uint32_t q) const { return mbar_wait_bounded(&full[q & mask], (q >> shift) & 1u); }
+    __device__ bool wait_empty(uint32_t q) const
+    {
+        return q <= mask || mbar_wait_bounded(&empty[q & mask], ((q >> shift) - 1u) & 1u);
+    }
+};
+
+// Producer warp: one bulk copy per pack.  Lane k holds the descriptor of window
+// w0 + k; the next 32 descriptors are loaded one batch ahead.
+__device__ void produce_packs(const Job &J, const PackRing &ring, volatile uint32_t *abort_flag)
+{
+    const uint32_t lane = threadIdx.x & 31u, nwin = J.nwin;
+    const uint4 *win = reinterpret_cast<const uint4 *>(J.win);
+    const uint4 none = make_uint4(0u, 0u, 0u, 0u);
+    uint32_t q = 0;
+    bool ok = true;
+    uint4 na = lane < nwin ? __ldg(win + 2 * lane) : none, nb = lane < nwin ? __ldg(win + 2 * lane + 1) : none;
+    for (uint32_t w0 = 0; w0 < nwin && ok; w0 += 32) {
+        const uint4 da = na, db = nb;
+        const uint32_t ahead = w0 + 32 + lane;
+        if (ahead < nwin) {
+            na = __ldg(win + 2 * (uint64_t)ahead);
+            nb = __ldg(win + 2 * (uint64_t)ahead + 1);
+        }
+        const uint32_t count = nwin - w0 < 32 ? nwin - w0 : 32u;
+        for (uint32_t k = 0; k < count && ok; ++k) {
+            const uint32_t lo = __shfl_sync(0xffffffffu, da.x, k), hi = __shfl_sync(0xffffffffu, da.y, k);
+            const uint32_t np = __shfl_sync(0xffffffffu, da.z, k), tab = __shfl_sync(0xffffffffu, da.w, k);
+            const uint32_t p0 = __shfl_sync(0xffffffffu, db.x, k), p1 = __shfl_sync(0xffffffffu, db.y, k);
+            const uint32_t p2 = __shfl_sync(0xffffffffu, db.z, k), p3 = __shfl_sync(0xffffffffu, db.w, k);
+            const uint2 *src = J.blob + (((uint64_t)hi << 32) | lo);
+            const uint32_t *table = reinterpret_cast<const uint32_t *>(src + tab);
+            if (lane == 0) {
+                for (uint32_t p = 0; p < np; ++p) {
+                    const uint32_t n8 = np > kDescPacks ? __ldg(table + p) : p == 0 ? p0 : p == 1 ? p1 : p == 2 ? p2 : p3;
+                    if (!ring.wait_empty(q)) {
+                        ok = false;
+                        break;
+                    }
+                    uint64_t *bar = &ring.full[q & ring.mask];
+                    mbar_arrive_expect_tx(bar, n8 * 8u);
+                    bulk_g2s(ring.at(q), src, n8 * 8u, bar);
+                    src += n8;
+                    ++q;
+                }
+            }
+            ok = __shfl_sync(0xffffffffu, (int)ok, 0);
+        }
+    }
+    if (lane == 0) {
+        if (ok && ring.wait_empty(q)) {
+            reinterpret_cast<uint32_t *>(ring.at(q))[1] = kPackEnd << 16;
+            mbar_arrive(&ring.full[q & ring.mask]);
+            ++q;
+        } else {
+            record_status(J.status, TN_ETIMEOUT);
+            *abort_flag = 1;
+        }
+        // no bulk copy may still be writing this CTA's shared memory at exit
+        for (uint32_t c = q > ring.mask + 1 ? q - ring.mask - 1 : 0; c < q; ++c) ring.wait_full(c);
+    }
 }
 
 // A consumer thread's place in the slab: `cpr` consecutive threads share one row
@@ -461,19 +525,14 @@ __device__ inline void apply_record(const Job &J, const uint32_t *rec, u64x2 *bu
 // resident slab: for a network small enough that rw words of EVERY row fit in
 // shared memory, the CTA loads its slab of the matrix once, applies the whole
 // schedule there and stores it once; only the schedule streams from L2/HBM.
-// The plan holds global tiles only (node-id ops, one level per tile or more;
-// windows of a resident plan are never local records with ops).  The producer
-// warp copies the schedule blob in fixed chunks of kStageBytes into a ring of
-// `nst` stages with cp.async.bulk; consumers walk the item list, wait for the
-// chunks an item covers, apply its ops (independent inside a level) and meet
-// at a named barrier only where a level ends.  A consumer warp releases a
-// chunk (one arrival on its `empty` barrier) once it has started an item past
-// it, so a stage is refilled only when every warp is done with it.
+// The plan holds tile packs only (node-id ops).  Consumers take one op each of
+// the current segment (its ops are independent), fetch their op of the next
+// segment, and meet at a named barrier; a level costs its barrier and the
+// latency of two dependent shared-memory accesses.
 // Shared memory: barriers | rows[rows] | saved rows[ntemp] | ring.
 // ---------------------------------------------------------------------------
-constexpr uint32_t kChunk8 = kStageBytes / 8;  // 8-byte units per ring stage
 constexpr uint32_t kResidentMaxStages = 8;
-constexpr uint32_t kResidentHead = 2 * kResidentMaxStages * sizeof(uint64_t);  // the ring's barriers
+constexpr uint32_t kResidentHead = 128;  // the ring's barriers
 constexpr uint32_t kResidentMinStages = 2;
 constexpr uint32_t kResidentConsumers = 256;  // consumer threads of a resident CTA (the rest exit)
 
@@ -586,85 +645,47 @@ __device__ inline void resident_op(uint2 op, uint32_t rb, uint32_t tb, const uin
     }
 }
 
-// Lane L of a warp holds item i0 + L of a batch of 32 as (offset, count |
-// flags << 16); the next batch is loaded one batch ahead, so its L2 latency is
-// hidden behind 32 items of work.
-__device__ inline void load_item(const uint4 *items, uint32_t nitems, uint32_t i, uint32_t &off, uint32_t &cf)
-{
-    off = 0;
-    cf = 0;
-    if (i < nitems) {
-        const uint4 it = __ldg(items + i);
-        off = it.x;
-        cf = it.y | (it.z << 16);  // count < 2^16 (at most one stage), flags < 4
-    }
-}
-
 template <bool kMax, int RW>
 __device__ void resident_slab(const Job &J, uint32_t smem_bytes, uint8_t *smem, uint32_t cta)
 {
     __shared__ int32_t r_gate;
+    __shared__ uint32_t r_abort;
     using Row = RRow<RW>;
     // the job's fields in registers (the barriers' memory clobbers would reload them)
-    const uint4 *const items = J.items;
-    const uint32_t nitems = (uint32_t)J.nitems;
     const uint32_t *const aux = J.aux;
-    const uint2 *const blob = J.blob;
-    const uint64_t blob8 = J.blob8;
     int32_t *const status = J.status;
     uint64_t *const S = J.S;
     const uint64_t ld = J.ld;
     const uint32_t rows = J.rows;
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem);
-    uint64_t *empty = full + kResidentMaxStages;
     Row *R = reinterpret_cast<Row *>(smem + kResidentHead);
     const uint32_t rb = smem_addr(R), tb = rb + rows * 8u * RW;  // rows, then saved rows
     const uint32_t ring_off = kResidentHead + (uint32_t)resident_rows_bytes(rows, J.ntemp, RW);
-    uint8_t *ring = smem + ring_off;
     // a power of two of stages (at least kResidentMinStages by the plan's check)
     const uint32_t fit = (smem_bytes - ring_off) / kStageBytes;
     uint32_t nst = kResidentMaxStages;
     while (nst > fit) nst >>= 1;
-    const uint32_t smask = nst - 1, sshift = __ffs(nst) - 1;
+    PackRing ring;
+    ring.full = reinterpret_cast<uint64_t *>(smem);
+    ring.empty = ring.full + kResidentMaxStages;
+    ring.stage = smem + ring_off;
+    ring.mask = nst - 1;
+    ring.shift = __ffs(nst) - 1;
     const uint64_t w0 = J.w_begin + (uint64_t)cta * RW;
-    // Every chunk of the blob holds part of some item: windows' regions and
-    // records are whole 16-byte units, so a window's padding unit (after an odd
-    // number of ops) sits at an odd offset and never begins a chunk.  Every
-    // chunk the producer copies is therefore waited for and released.
-    const uint32_t nchunks = (uint32_t)((blob8 + kChunk8 - 1) / kChunk8);
     const uint32_t C = consumers() < kResidentConsumers ? consumers() : kResidentConsumers;
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
     if (threadIdx.x == 0) {
         r_gate = *(volatile int32_t *)status;  // an earlier error gates this job
+        r_abort = 0;
         for (uint32_t s = 0; s < nst; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], C / 32u);
+            mbar_init(&ring.full[s], 1);
+            mbar_init(&ring.empty[s], C / 32u);
         }
         fence_mbar_init();
     }
     __syncthreads();
-    if (r_gate != 0 || nitems == 0) return;  // no ops: the slab is unchanged
-
+    if (r_gate != 0) return;
     if (warp == 0) {
-        // ---------------- producer: the blob in fixed chunks ----------------
-        if (lane == 0) {
-            uint32_t c = 0;
-            for (; c < nchunks; ++c) {
-                const uint32_t s = c & smask;
-                if (c >= nst && !mbar_wait_bounded(&empty[s], ((c >> sshift) - 1u) & 1u)) {
-                    record_status(status, TN_ETIMEOUT);
-                    break;
-                }
-                const uint64_t b8 = (uint64_t)c * kChunk8;
-                uint32_t n8 = blob8 - b8 < kChunk8 ? (uint32_t)(blob8 - b8) : kChunk8;
-                n8 = (n8 + 1u) & ~1u;  // whole 16-byte units (the blob has two spare units)
-                mbar_arrive_expect_tx(&full[s], n8 * 8u);
-                bulk_g2s(ring + (size_t)s * kStageBytes, blob + b8, n8 * 8u, &full[s]);
-            }
-            // no bulk copy may still be writing this CTA's shared memory at exit
-            for (uint32_t q = c > nst ? c - nst : 0; q < c; ++q)
-                mbar_wait_bounded(&full[q & smask], (q >> sshift) & 1u);
-        }
+        produce_packs(J, ring, &r_abort);
         return;
     }
     // ---------------- consumers ----------------
@@ -681,74 +702,37 @@ __device__ void resident_slab(const Job &J, uint32_t smem_bytes, uint8_t *smem, 
         }
         for (; i < rows; i += C) R[i] = ld_rrow<RW>(S + (uint64_t)i * ld + w0);
     }
-    // op o of the blob, from the stage of its chunk (which has landed)
-    const uint32_t ringa = smem_addr(ring);
-    auto op_at = [&](uint32_t o) -> uint2 {
-        return lds_op(ringa + ((o / kChunk8) & smask) * kStageBytes + (o % kChunk8) * 8u);
-    };
-    bool failed = false;
-    uint32_t waited = 0;    // chunks [0, waited) have landed, as seen by this thread
-    uint32_t released = 0;  // chunks this warp has released
-    uint32_t boff, bcf, noff, ncf;  // this lane's item of the current and of the next batch
-    load_item(items, nitems, lane, boff, bcf);
-    load_item(items, nitems, 32 + lane, noff, ncf);
-    uint32_t off8 = 0, cf = 0;
-    uint2 op0 = make_uint2(0u, 0u);  // this thread's first op of the next item
-    bool have = false;
-    // Prepares item i: releases the chunks before it, waits for the chunks it
-    // covers, and fetches this thread's first op of it.
-    auto prepare = [&](uint32_t i) {
-        const uint32_t k = i & 31u;
-        if (k == 0 && i > 0) {
-            boff = noff;
-            bcf = ncf;
-            load_item(items, nitems, i + 32 + lane, noff, ncf);
+    for (uint32_t q = 0;; ++q) {
+        const bool ready = ring.wait_full(q);
+        if (!ready && ct == 0) record_status(status, TN_ETIMEOUT);
+        const uint32_t *head = reinterpret_cast<const uint32_t *>(ring.at(q));
+        const bool stop = !ready || *(volatile uint32_t *)&r_abort != 0 || ((head[1] >> 16) & kPackEnd);
+        // orders the previous pack's (or the loads') stores before this pack's
+        // loads, and agrees on stopping
+        if (consumers_sync_or(stop, C)) {
+            if (!ready || *(volatile uint32_t *)&r_abort != 0) return;
+            break;
         }
-        off8 = __shfl_sync(0xffffffffu, boff, k);
-        cf = __shfl_sync(0xffffffffu, bcf, k);
-        const uint32_t count = cf & 0xFFFFu;
-        const uint32_t c0 = off8 / kChunk8, c1 = (off8 + count - 1u) / kChunk8;
-        if (released < c0 || waited <= c1) {  // a chunk boundary (one test in the common case)
-            if (released < c0) {  // every lane of the warp is done with these chunks
-                __syncwarp();
-                if (lane == 0)
-                    for (uint32_t q = released; q < c0; ++q) mbar_arrive(&empty[q & smask]);
-                released = c0;
+        const uint16_t *seg = reinterpret_cast<const uint16_t *>(head + 4);
+        const uint32_t nseg = head[1] & 0xFFFFu;
+        const uint32_t opa = smem_addr(head) + kPackHead * 8u;
+        uint32_t b = 0, e = seg[0];
+        uint2 op = lds_op(opa + ct * 8u);  // always inside the stage; used only if ct < e
+        for (uint32_t k = 0;;) {
+            if (b + ct < e) {
+                resident_op<kMax, RW>(op, rb, tb, aux);
+                for (uint32_t o = b + ct + C; o < e; o += C) resident_op<kMax, RW>(lds_op(opa + o * 8u), rb, tb, aux);
             }
-            while (waited <= c1 && !failed) {
-                if (mbar_wait_bounded(&full[waited & smask], (waited >> sshift) & 1u)) {
-                    ++waited;
-                } else {
-                    record_status(status, TN_ETIMEOUT);
-                    failed = true;
-                }
-            }
+            if (++k >= nseg) break;
+            b = e;
+            e = seg[k];
+            const uint32_t o = b + ct;
+            op = lds_op(opa + (o < e ? o : 0u) * 8u);  // the next segment's op loads before the barrier
+            consumers_sync(C);
         }
-        have = !failed && ct < count && !((cf >> 16) & kItemLocal);
-        op0 = op_at(off8 + ct);  // always inside the ring; used only if `have`
-    };
-    consumers_sync(C);
-    prepare(0);
-    uint32_t lev = 0;
-    for (uint32_t i = 0;;) {
-        const uint32_t count = cf & 0xFFFFu, flags = cf >> 16, base8 = off8;
-        if (have) {
-            resident_op<kMax, RW>(op0, rb, tb, aux);
-            for (uint32_t q = ct + C; q < count; q += C) resident_op<kMax, RW>(op_at(base8 + q), rb, tb, aux);
-        }
-        if (++i == nitems) break;
-        prepare(i);  // item info and first op of the next item load before the barrier
-        // the next level reads what this one wrote; every 64th level end also
-        // agrees on stopping (a thread that gave up skips its work until then)
-        if (flags & kItemLevelEnd) {
-            if ((++lev & 63u) == 0) {
-                if (consumers_sync_or(failed, C)) break;
-            } else {
-                consumers_sync(C);
-            }
-        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&ring.empty[q & ring.mask]);
     }
-    if (consumers_sync_or(failed, C)) return;
     for (uint32_t i = ct; i < rows; i += C) st_rrow<RW>(S + (uint64_t)i * ld + w0, R[i]);
 }
 
@@ -756,11 +740,6 @@ template <bool kMax>
 __global__ void __launch_bounds__(kMaxThreads) stream_kernel(const __grid_constant__ JobList jl)
 {
     extern __shared__ __align__(128) uint8_t smem[];
-    uint8_t *stage = smem;  // kStages x kStageBytes
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem + (size_t)kStages * kStageBytes);
-    uint64_t *empty = full + kStages;
-    StageHdr *hdr = reinterpret_cast<StageHdr *>(empty + kStages);
-    u64x2 *rowbuf = reinterpret_cast<u64x2 *>(hdr + kStages);  // 16-byte aligned
     __shared__ uint32_t producer_abort;
     __shared__ int32_t gate;
 
@@ -771,97 +750,58 @@ __global__ void __launch_bounds__(kMaxThreads) stream_kernel(const __grid_consta
         else resident_slab<kMax, 2>(J, jl.smem_bytes, smem, cta);
         return;
     }
+    PackRing ring;  // kStages stages, then the barriers and the row buffer
+    ring.stage = smem;
+    ring.full = reinterpret_cast<uint64_t *>(smem + (size_t)kStages * kStageBytes);
+    ring.empty = ring.full + kStages;
+    ring.mask = kStages - 1;
+    ring.shift = kStageShift;
+    u64x2 *rowbuf = reinterpret_cast<u64x2 *>(smem + kSlabHead);
     const uint64_t w0 = J.w_begin + (uint64_t)(blockIdx.x - J.cta_begin) * J.sw;
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
     if (threadIdx.x == 0) {
         gate = *(volatile int32_t *)J.status;  // an earlier error gates this job
         for (int s = 0; s < kStages; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], consumers() / 32u);
+            mbar_init(&ring.full[s], 1);
+            mbar_init(&ring.empty[s], consumers() / 32u);
         }
         producer_abort = 0;
         fence_mbar_init();
     }
     __syncthreads();
     if (gate != 0) return;
-
     if (warp == 0) {
-        // ---------------- producer: one bulk copy per item ----------------
-        uint64_t slot = 0;  // stage uses so far
-        int ok = 1;
-        for (uint64_t i0 = 0; i0 < J.nitems && ok; i0 += 32) {
-            const uint4 mine = (i0 + lane < J.nitems) ? __ldg(J.items + i0 + lane) : make_uint4(0u, 0u, 0u, 0u);
-            const uint32_t nb = (J.nitems - i0 < 32) ? (uint32_t)(J.nitems - i0) : 32u;
-            for (uint32_t k = 0; k < nb && ok; ++k) {
-                const uint32_t off8 = __shfl_sync(0xffffffffu, mine.x, k);
-                const uint32_t count = __shfl_sync(0xffffffffu, mine.y, k);
-                const uint32_t flags = __shfl_sync(0xffffffffu, mine.z, k);
-                const int s = (int)(slot % kStages);
-                if (lane == 0) {
-                    if (slot >= kStages && !mbar_wait_bounded(&empty[s], (uint32_t)((slot / kStages) - 1) & 1u)) {
-                        record_status(J.status, TN_ETIMEOUT);
-                        producer_abort = 1;
-                        ok = 0;
-                    } else {
-                        uint32_t a0 = off8, n8 = count, off = 0;
-                        if (!(flags & kItemLocal)) {  // global tile: start on a 16-byte boundary
-                            a0 = off8 & ~1u;
-                            off = off8 - a0;
-                            n8 = (count + off + 1u) & ~1u;
-                        }
-                        hdr[s].count = count;
-                        hdr[s].off = off;
-                        hdr[s].local = flags & kItemLocal;
-                        mbar_arrive_expect_tx(&full[s], n8 * 8u);
-                        bulk_g2s(stage + (size_t)s * kStageBytes, J.blob + a0, n8 * 8u, &full[s]);
-                    }
-                }
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                if (ok) ++slot;
+        produce_packs(J, ring, &producer_abort);
+        return;
+    }
+    // ---------------- consumers ----------------
+    const uint32_t ct = threadIdx.x - 32;
+    const Lane L = make_lane(J, ct, w0);
+    for (uint32_t q = 0;; ++q) {
+        const bool ready = ring.wait_full(q);
+        if (!ready && ct == 0) record_status(J.status, TN_ETIMEOUT);
+        const uint32_t *head = reinterpret_cast<const uint32_t *>(ring.at(q));
+        const bool stop = !ready || *(volatile uint32_t *)&producer_abort != 0 || ((head[1] >> 16) & kPackEnd);
+        // level barrier: the previous pack's stores are ordered before this
+        // pack's loads, and all consumers agree on stopping
+        if (consumers_sync_or(stop)) break;
+        const uint32_t meta = head[1];
+        if ((meta >> 16) & kPackLocal) {
+            apply_record<kMax>(J, head + 4, rowbuf, L);
+        } else {
+            const uint16_t *seg = reinterpret_cast<const uint16_t *>(head + 4);
+            const uint2 *ops = reinterpret_cast<const uint2 *>(head) + kPackHead;
+            const uint32_t nseg = meta & 0xFFFFu;
+            for (uint32_t k = 0, b = 0; k < nseg; ++k) {
+                const uint32_t e = seg[k];
+                if (e == b) continue;
+                if (b) consumers_sync();
+                apply_tile<kMax>(J, ops + b, e - b, rowbuf, J.dcap, L);
+                b = e;
             }
         }
-        if (lane == 0) {
-            if (ok) {
-                const int s = (int)(slot % kStages);
-                if (slot >= kStages && !mbar_wait_bounded(&empty[s], (uint32_t)((slot / kStages) - 1) & 1u)) {
-                    record_status(J.status, TN_ETIMEOUT);
-                    producer_abort = 1;
-                } else {
-                    hdr[s].count = kEndItem;
-                    hdr[s].off = 0;
-                    hdr[s].local = 0;
-                    mbar_arrive(&full[s]);
-                    ++slot;
-                }
-            }
-            // no bulk copy may still be writing this CTA's shared memory at exit
-            const uint64_t first = slot > (uint64_t)kStages ? slot - kStages : 0;
-            for (uint64_t q = first; q < slot; ++q)
-                mbar_wait_bounded(&full[q % kStages], (uint32_t)(q / kStages) & 1u);
-        }
-    } else {
-        // ---------------- consumers ----------------
-        const uint32_t ct = threadIdx.x - 32;
-        const Lane L = make_lane(J, ct, w0);
-        for (uint64_t it = 0;; ++it) {
-            const int s = (int)(it % kStages);
-            const uint32_t par = (uint32_t)(it / kStages) & 1u;
-            const bool ready = mbar_wait_bounded(&full[s], par);
-            if (!ready && ct == 0) record_status(J.status, TN_ETIMEOUT);
-            const bool stop = !ready || *(volatile uint32_t *)&producer_abort != 0 ||
-                              (ready && hdr[s].count == kEndItem);
-            // level barrier: the previous item's stores are ordered before this
-            // item's loads, and all consumers agree on stopping
-            if (consumers_sync_or(stop)) break;
-            if (hdr[s].local) {
-                apply_record<kMax>(J, reinterpret_cast<const uint32_t *>(stage + (size_t)s * kStageBytes), rowbuf, L);
-            } else {
-                apply_tile<kMax>(J, reinterpret_cast<const uint2 *>(stage + (size_t)s * kStageBytes) + hdr[s].off,
-                           hdr[s].count, rowbuf, J.dcap, L);
-            }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&empty[s]);
-        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&ring.empty[q & ring.mask]);
     }
 }
 
@@ -1048,7 +988,7 @@ tn_status apply_jobs(const tn_plan *const *plans, uint64_t *const *S, const uint
         // the identity initialisation needs one column per node
         if ((flags & TN_INIT_IDENTITY) && !src[i] && ncols[i] != p->n) return TN_EINVAL;
     }
-    const size_t smem_base = (size_t)kStages * kStageBytes + 2 * kStages * sizeof(uint64_t) + kStages * sizeof(StageHdr);
+    const size_t smem_base = kSlabHead;
     const size_t smem_limit = stream_smem_limit();
     if ((flags & kApplyMax) || !smem_limit)
         for (uint32_t i = 0; i < count; ++i)
@@ -1091,9 +1031,9 @@ tn_status apply_jobs(const tn_plan *const *plans, uint64_t *const *S, const uint
             for (int k = 0; k < parts; ++k) {
                 Job &J = jl.job[jl.count++];
                 J.blob = p->d_blob;
-                J.items = p->d_items;
+                J.win = p->d_win;
                 J.aux = p->d_aux;
-                J.nitems = p->items;
+                J.nwin = (uint32_t)p->windows;
                 J.S = S[i];
                 J.ld = ld;
                 J.tmp = tmps[j];
@@ -1157,9 +1097,9 @@ tn_status apply_jobs(const tn_plan *const *plans, uint64_t *const *S, const uint
             if (need > smem) smem = need;
             Job &J = jl.job[jl.count++];
             J.blob = p->d_blob;
-            J.items = p->d_items;
+            J.win = p->d_win;
             J.aux = p->d_aux;
-            J.nitems = p->items;
+            J.nwin = (uint32_t)p->windows;
             J.S = S[i];
             J.ld = ld;
             J.tmp = nullptr;
@@ -1171,7 +1111,6 @@ tn_status apply_jobs(const tn_plan *const *plans, uint64_t *const *S, const uint
             J.rw = rw;
             J.rows = p->n;
             J.ntemp = (uint32_t)p->temps;
-            J.blob8 = p->blob8;
             J.cta_begin = ctas;
             ctas += (uint32_t)((used + rw - 1) / rw);
         }

@@ -50,24 +50,43 @@ constexpr uint32_t kNoRef = 0xFFFFFFFFu;  // empty slot in a batch of source ref
 
 __host__ __device__ inline uint32_t op_a(uint32_t kind, uint32_t id) { return (kind << kKindShift) | id; }
 
-// Work items of the streaming kernel.  The planner emits one item per window
-// whose rows fit the kernel's shared-memory row buffer (a "local record") and
-// one item per tile of ops for the other windows ("global tiles").  Items are
-// copied whole into one shared-memory staging buffer of kStageBytes.
-//   local record (uint32 words): D, T, nlev, nops | rows[D] (node ids) |
-//     lvl[nlev + 1] (op offsets) | ops[nops] | aux[...] | zero padding to 16 B.
+// Packs of the streaming kernel: what one stage of its shared-memory ring
+// holds, copied whole.  A window of the schedule is a run of consecutive packs
+// (16-byte aligned, sizes in 8-byte units).
+//   tile pack: uint32 ops, uint32 segments | flags << 16, 8 spare bytes,
+//     uint16 end[64] (op offsets where its segments end), then the ops as uint2
+//     (node ids, absolute aux indices).  A segment is a level, or a part of one
+//     when the level does not fit a pack; ops of one segment never conflict.
+//   record pack (kPackLocal; a window whose rows fit the kernel's shared-memory
+//     row buffer): 16 bytes like the above, then uint32 words D, T, nlev, nops |
+//     rows[D] (node ids) | lvl[nlev + 1] (op offsets) | ops[nops] | aux[...] |
+//     zero padding to 16 B.
 //     Rows are named by local slots: 0..D-1 the window's rows, D..D+T-1 saved
 //     copies.  op = kind << 30 | la << 29 | lb << 28 | a << 14 | b  (PULL: b =
 //     aux offset).  la / lb mark the op that writes row a / b for the last time
 //     in the window: its result is also stored to the matrix right away, so the
 //     write-back runs during the levels instead of after them, and rows that
 //     are only read are never written back.
-//   global tile: uint2 ops as above (node ids, absolute aux indices).
-// item = {offset in 8-byte units, count (global: ops; local: 8-byte units), flags, 0}
 constexpr uint32_t kStageBytes = 16384;
-constexpr uint32_t kTileOps = kStageBytes / 8 - 2;
-constexpr uint32_t kItemLocal = 1u;
-constexpr uint32_t kItemLevelEnd = 2u;
+constexpr uint32_t kPackSegs = 64;
+constexpr uint32_t kPackHead = 2 + kPackSegs / 4;          // units
+constexpr uint32_t kPackOps = kStageBytes / 8 - kPackHead;  // 2,030
+constexpr uint32_t kRecordWords = kStageBytes / 4 - 4;
+constexpr uint32_t kPackLocal = 1u;   // a record
+constexpr uint32_t kPackWindow = 2u;  // first pack of its window
+constexpr uint32_t kPackEnd = 4u;     // no pack: the schedule ends here
+// One window of the schedule: `npacks` packs from unit `off` on; their sizes
+// are pack[] while there are at most kDescPacks, else a uint32 table `tab`
+// units behind `off`.
+constexpr uint32_t kDescPacks = 4;
+struct __align__(16) WinDesc {
+    uint64_t off;
+    uint32_t npacks, tab;
+    uint32_t pack[kDescPacks];
+};
+static_assert(sizeof(WinDesc) == 32, "two 16-byte loads");
+struct PlanHead;
+
 constexpr uint32_t kLocalBits = 14;
 constexpr uint32_t kLocalMask = 0x3FFFu;
 constexpr uint32_t kLocalSlotLimit = 0x3FFFu;  // above the 10,240 slots a 160 KB row buffer can hold
@@ -223,7 +242,8 @@ __device__ inline uint32_t block_excl_scan_value(uint32_t x, uint32_t *warp_sums
     return r;
 }
 
-__device__ inline uint32_t block_excl_scan_array(uint32_t *a, uint32_t len, uint32_t *warp_sums, uint32_t *total)
+template <typename I>
+__device__ inline uint32_t block_excl_scan_array(I *a, uint32_t len, uint32_t *warp_sums, uint32_t *total)
 {
     const uint32_t per = (len + blockDim.x - 1u) / blockDim.x;
     const uint32_t b = threadIdx.x * per;
@@ -233,7 +253,7 @@ __device__ inline uint32_t block_excl_scan_array(uint32_t *a, uint32_t len, uint
     uint32_t off = block_excl_scan_value(sum, warp_sums, total);
     for (uint32_t i = b; i < e; ++i) {
         uint32_t x = a[i];
-        a[i] = off;
+        a[i] = (I)off;
         off += x;
     }
     __syncthreads();
@@ -253,12 +273,12 @@ struct tn_plan {
     uint32_t wave_ctas;   // 0, or the number of CTAs one matrix is spread over
     uint32_t dcap;        // row slots of the kernel's shared-memory row buffer
     uint32_t resident;    // 0, or 64-bit words of every row one CTA keeps in shared memory
-    uint2 *d_blob;        // [blob8 + 2]  item payloads (8-byte units)
-    uint4 *d_items;       // [items]      work items in execution order
-    uint32_t *d_aux;      // [aux]        source lists of global PULL ops
-    int64_t *d_tbounds;   // [2]          t_first, t_last
-    int32_t *d_status;    // [1]          first asynchronous error
-    int status_shared;    // d_status belongs to the owner (tn::plan_use_status), not to the plan
+    uint2 *d_blob;        // packs (8-byte units)
+    tn::WinDesc *d_win;   // [windows]    their windows in time order
+    uint32_t *d_aux;      // source lists of PULL ops
+    tn::PlanHead *d_head; // owned: counters, time bounds, status word
+    int64_t *d_tbounds;   // [2]          t_first, t_last (in d_head)
+    int32_t *d_status;    // first asynchronous error (in d_head, or the owner's: tn::plan_use_status)
 };
 
 namespace tn {

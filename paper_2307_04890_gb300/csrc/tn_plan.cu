@@ -1,4 +1,4 @@
-// Scheduling of an event batch for the column-slab streaming kernel.
+// Scheduling of an event batch for the streaming kernel.
 //
 // Algorithm 1 (Section 3.1) is a strict sequence of row updates, but two
 // events that share no node commute, and the columns of the matrix are
@@ -7,9 +7,10 @@
 // row loads at once and only needs a barrier between levels.
 //
 // Equal timestamps (Section 2.1: adjacency needs dt > 0) are applied as one
-// snapshot.  Inside a group G with node counts c(x) (occurrences of x in G):
-//   * an event whose two ends both occur once in G is an ordinary update
-//     (EVENT: r = S[u] | S[v] into both rows);
+// snapshot.  A group whose events share no node is a set of ordinary updates
+// (EVENT: r = S[u] | S[v] into both rows).  Inside any other group G with node
+// counts c(x) (occurrences of x in G):
+//   * an event whose two ends both occur once in G is an ordinary update;
 //   * a node y occurring once, whose partner x occurs several times, gets
 //     ONEWAY: S[y] |= S[x] at level L (x is not written at level L);
 //   * a node x occurring several times gets one PULL at level L+1:
@@ -18,16 +19,22 @@
 //     partner z occurring several times is read from a saved copy of z's old
 //     row (COPY at level L into a temporary slot).
 // This reproduces S_new[x] = S_old[x] | OR_{(x,y) in G} S_old[y] exactly.
+// Directed events x -> y write only y: a lone event is ONEWAY y |= x, a group
+// that shares nodes becomes one PULL per receiver, a sender that also receives
+// in the group being read from its saved old row.
 //
 // The batch is cut into windows of about `window_events` events, never inside
 // a timestamp group.  Each window is scheduled independently by one CTA
 // (levels restart at every window, which acts as one extra barrier):
 //   1. node ids of the window are compacted through a hash table;
-//   2. one thread scans the window's groups in time order and assigns levels
-//      (level of an update = 1 + last level at which any of its rows was
-//      touched), tie-group roles, PULL source lists and COPY slots;
-//   3. the window's updates are counting-sorted by level.
-// A final pass concatenates the windows into one level-ordered op list.
+//   2. groups of up to kPairGroup events are checked for shared nodes, pair by
+//      pair, by all threads;
+//   3. one warp walks the window in time order, 16 events (32 endpoints) at a
+//      time, and assigns levels (level of an update = 1 + last level at which
+//      any of its rows was touched); every group that shares nodes is handed
+//      to the whole CTA;
+//   4. the window's updates are counting-sorted by level into packs that the
+//      streaming kernel copies whole (tn_internal.cuh describes the layout).
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stdlib.h>
@@ -39,36 +46,87 @@
 
 namespace tn {
 
-constexpr int kPlanThreads = 256;
+constexpr int kPlanThreads = 512;
 constexpr uint32_t kDefaultWindow = 640;
 constexpr uint32_t kDefaultSlab = 16;
 constexpr uint32_t kRowBufferBytes = 160 * 1024;  // default shared-memory row buffer, slabs of up to 16 words
 constexpr uint32_t kRowBufferWide = 192 * 1024;   // default (and largest) row buffer for wider slabs
-constexpr uint32_t kWinFields = 8;  // nops, nlev, naux, ntemp, local, blob8, nitems, all ops
 constexpr uint32_t kEmpty = 0xFFFFFFFFu;
-constexpr uint32_t kNone = 0xFFFFFFFFu;
+// Windows of up to this many events may become shared-memory records.
+constexpr uint32_t kRecordEvents = 2048;
+// Groups of at least this many events go to the whole CTA unchecked: comparing
+// their events pair by pair would cost more than the group's own phases.
+constexpr uint32_t kPairGroup = 128;
+// Batches of at least this many events are copied into buffers of their exact
+// size; below it the staging buffers (a few times larger, bounded) are kept.
+constexpr uint64_t kCompactEvents = 1ull << 20;
 
-// event flags stored in the grp array once scheduling is done
-constexpr uint32_t kFlagDir = 1u << 27;   // directed event outside a tie group: one ONEWAY
-constexpr uint32_t kFlagNoop = 1u << 28;
-constexpr uint32_t kFlagIso = 1u << 29;
-constexpr uint32_t kFlagShA = 1u << 30;
-constexpr uint32_t kFlagShB = 1u << 31;
+// event flags of a window
+constexpr uint8_t kFlagStart = 1;   // first event of its timestamp group
+constexpr uint8_t kFlagHard = 2;    // on a group's first event: the group shares nodes
+constexpr uint8_t kFlagDir = 4;     // directed event outside such a group: one ONEWAY
+constexpr uint8_t kFlagNoop = 8;
+constexpr uint8_t kFlagIso = 16;
+constexpr uint8_t kFlagShA = 32;
+constexpr uint8_t kFlagShB = 64;
 
-// arena layout (uint32 words) for a window of E events:
-//   lu[E] lv[E] grp[E] evl[E] run_node[E] run_aux[E] run_lev[E] run_temp[E] rowsg[2E] scratch
-// scratch: hash keys + ids (2*H words, H = hash slots) during id assignment,
-// then node state nlev/ncnt/nrun (3*D words, D <= 2E distinct nodes), then the
-// level histogram (<= 2E + 3 words).
 __host__ __device__ inline uint64_t hash_slots(uint64_t E) { return ((3 * E + 31) / 32) * 32; }
-__host__ __device__ inline uint64_t arena_words(uint64_t E)
+
+// Arena of a window of E events, indices of type I (uint16_t in shared memory,
+// uint32_t for windows scheduled in global memory).  The scratch part holds in
+// turn the hash table (keys, ids), the node state (occurrences, last level,
+// run) and the level bounds, pack table and last writers.
+template <typename I>
+__host__ __device__ inline uint64_t scratch_words(uint64_t E)
 {
     const uint64_t H = hash_slots(E);
-    uint64_t scratch = 2 * H;
-    if (6 * E > scratch) scratch = 6 * E;
-    if (2 * E + 3 > scratch) scratch = 2 * E + 3;
-    return 10 * E + scratch;
+    uint64_t b = H * (4 + sizeof(I));
+    const uint64_t state = 2 * E * (4 + 2 * sizeof(I));
+    if (state > b) b = state;
+    if (b < 16 * E) b = 16 * E;
+    return (b + 3) / 4 + 64;
 }
+
+template <typename I>
+__host__ __device__ inline uint64_t arena_bytes(uint64_t E)
+{
+    return (4 * (scratch_words<I>(E) + 3 * E) + sizeof(I) * 6 * E + 3 * E + 15) & ~15ull;
+}
+
+template <typename I>
+struct Arena {
+    uint32_t *rowsg;    // [2E] global id of every local row id
+    uint32_t *run_lev;  // [E] fill counter, then level, of every PULL
+    uint32_t *scratch;
+    I *lu, *lv, *evl, *run_node, *run_aux, *run_temp;  // [E] each
+    uint8_t *flg;       // [E]
+    uint8_t *claim;     // [2E] a lane of the chunk being checked, per row
+    __device__ Arena(uint8_t *p, uint32_t E)
+    {
+        rowsg = reinterpret_cast<uint32_t *>(p);
+        run_lev = rowsg + 2 * (uint64_t)E;
+        scratch = run_lev + E;
+        lu = reinterpret_cast<I *>(scratch + scratch_words<I>(E));
+        lv = lu + E;
+        evl = lv + E;
+        run_node = evl + E;
+        run_aux = run_node + E;
+        run_temp = run_aux + E;
+        flg = reinterpret_cast<uint8_t *>(run_temp + E);
+        claim = flg + E;
+    }
+};
+
+// Counters of a plan (device, one copy to the host per synchronisation).
+struct PlanCounters {
+    unsigned long long error;       // bit 0: id out of range, bit 1: time order
+    unsigned long long late;        // windows left to the second pass
+    unsigned long long arena;       // arena bytes of those scheduled in global memory
+    unsigned long long big;         // how many of them are
+    unsigned long long blob8, naux, items, ops, levels, local, temps;
+    unsigned long long blob_used, aux_used;  // allocation of the exact buffers
+    long long t_first, t_last;
+};
 
 struct PlanArgs {
     const uint32_t *u, *v;
@@ -79,82 +137,84 @@ struct PlanArgs {
     uint32_t window;     // target events per window
     uint32_t directed;   // 1: events are u -> v (only S[v] is updated)
     uint32_t nw;         // number of windows
+    uint32_t first_max;  // largest window of the first pass (its shared-memory arena)
+    uint32_t smem_max;   // largest window scheduled in shared memory
+    uint32_t dcap;       // row slots of a local window
+    uint32_t unit8;      // staging units (8 bytes) per event
     uint64_t *wstart;    // [nw + 1]
-    uint32_t smem_max_events;
-    uint32_t dcap;          // row slots of a local window
-    uint32_t max_rec_words; // largest local record (words)
-    // per-window results (kWinFields each)
-    uint32_t *wcount;    // [kWinFields * nw]
-    // staging (window w uses the regions starting at 3*s_w / 2*s_w + w / 10*s_w + 8*w)
-    uint2 *ops_stage;    // [3m]
-    uint32_t *aux_stage; // [3m]
-    uint32_t *lvl_stage; // [2m + nw + 1]
-    uint32_t *rec_stage; // [10m + 8nw]
-    // large windows
-    uint32_t *big_list;  // [nw]
-    uint64_t *big_off;   // [nw]
-    uint32_t *big_arena;
-    // global counters: [0] error flags, [1] number of big windows, [2] arena words of
-    // the big windows, [3] largest window scheduled in shared memory
-    unsigned long long *counters;
+    uint32_t *naux_w;    // [nw] source-list entries of every window
+    WinDesc *desc;       // [nw]
+    uint2 *blob;         // window w: units blob_base(w) ...
+    uint32_t *aux;       // window w: words 3 * s_w ...
+    uint32_t *late_list; // [nw] windows of the second pass
+    uint64_t *late_off;  // [nw] their arena offsets (kSmemArena: in shared memory)
+    uint8_t *late_arena;
+    PlanCounters *cnt;
+    int64_t *tbounds;
 };
+constexpr uint64_t kSmemArena = ~0ull;
+
+// Staging region of window w, starting at event s: 4 units per event hold 3 ops
+// and the pack headers (at most one pack of 18 units per 64 levels or 2,030
+// ops, and a window has at most one level per event), 5 units a record (10
+// words per event); an even unit, so packs are 16-byte aligned.
+__host__ __device__ inline uint64_t blob_base(uint64_t s, uint64_t w, uint32_t unit8)
+{
+    return ((unit8 * s + 1) & ~1ull) + 64 * w;
+}
 
 // ---------------------------------------------------------------------------
-// validation (Section 2.1: nodes in [0, n), events time-ordered)
+// validation (Section 2.1: nodes in [0, n), events time-ordered) and windows
 // ---------------------------------------------------------------------------
-__global__ void validate_kernel(PlanArgs a)
+// window w starts at the first timestamp-group start at or after w * window
+__device__ inline uint64_t window_start(const PlanArgs &a, uint64_t w)
 {
+    uint64_t s = w * (uint64_t)a.window;
+    if (w == 0) return 0;
+    if (w >= a.nw || s >= a.m) return a.m;
+    const int64_t key = a.t[s];
+    if (key != a.t[s - 1]) return s;
+    // first index with t > key: gallop, then binary search
+    uint64_t lo = s, step = 1;
+    while (lo + step < a.m && a.t[lo + step] <= key) {
+        lo += step;
+        step *= 2;
+    }
+    uint64_t hi = lo + step < a.m ? lo + step : a.m;  // t[lo] <= key, hi past it or the end
+    while (lo + 1 < hi) {
+        const uint64_t mid = lo + (hi - lo) / 2;
+        if (a.t[mid] > key) hi = mid;
+        else lo = mid;
+    }
+    return hi;
+}
+
+__global__ void inspect_kernel(PlanArgs a)
+{
+    const uint64_t tid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x, nt = (uint64_t)gridDim.x * blockDim.x;
     uint32_t bad = 0;
-    for (uint64_t e = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; e < a.m;
-         e += (uint64_t)gridDim.x * blockDim.x) {
+    for (uint64_t e = tid; e < a.m; e += nt) {
         if (a.u[e] >= a.n || a.v[e] >= a.n) bad |= 1u;
         if (e > 0 && a.t[e] < a.t[e - 1]) bad |= 2u;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0 && a.t_after && a.m > 0 && !(a.t[0] > *a.t_after)) bad |= 2u;
-    if (bad) atomicOr(&a.counters[0], (unsigned long long)bad);
-}
-
-// window w starts at the first timestamp-group start at or after w * window
-__global__ void window_kernel(PlanArgs a)
-{
-    for (uint64_t w = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; w <= a.nw;
-         w += (uint64_t)gridDim.x * blockDim.x) {
-        uint64_t s;
-        if (w == 0) {
-            s = 0;
-        } else if (w == a.nw) {
-            s = a.m;
-        } else {
-            s = w * (uint64_t)a.window;
-            if (s >= a.m) {
-                s = a.m;
-            } else if (a.t[s] == a.t[s - 1]) {
-                // first index with t > t[s] (upper bound) by binary search
-                const int64_t key = a.t[s];
-                uint64_t lo = s, hi = a.m;
-                while (lo < hi) {
-                    uint64_t mid = lo + (hi - lo) / 2;
-                    if (a.t[mid] > key) hi = mid;
-                    else lo = mid + 1;
-                }
-                s = lo;
-            }
-        }
-        a.wstart[w] = s;
+    if (tid == 0) {
+        if (a.t_after && !(a.t[0] > *a.t_after)) bad |= 2u;
+        a.cnt->t_first = a.tbounds[0] = a.t[0];
+        a.cnt->t_last = a.tbounds[1] = a.t[a.m - 1];
+        a.wstart[a.nw] = a.m;
     }
-}
-
-__global__ void big_window_kernel(PlanArgs a)
-{
-    for (uint64_t w = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; w < a.nw;
-         w += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t E = a.wstart[w + 1] - a.wstart[w];
-        if (E <= a.smem_max_events) atomicMax(&a.counters[3], (unsigned long long)E);
-        if (E > a.smem_max_events) {
-            unsigned long long slot = atomicAdd(&a.counters[1], 1ull);
-            unsigned long long off = atomicAdd(&a.counters[2], (unsigned long long)arena_words(E));
-            a.big_list[slot] = (uint32_t)w;
-            a.big_off[slot] = off;
+    if (bad) atomicOr(&a.cnt->error, (unsigned long long)bad);
+    for (uint64_t w = tid; w < a.nw; w += nt) {
+        const uint64_t s = window_start(a, w), e = window_start(a, w + 1);
+        a.wstart[w] = s;
+        if (e <= s || e - s <= a.first_max) continue;  // (e < s only in unordered input, refused as a whole)
+        const uint64_t E = e - s;
+        const unsigned long long slot = atomicAdd(&a.cnt->late, 1ull);
+        a.late_list[slot] = (uint32_t)w;
+        a.late_off[slot] = kSmemArena;
+        if (E > a.smem_max) {
+            atomicAdd(&a.cnt->big, 1ull);
+            a.late_off[slot] = atomicAdd(&a.cnt->arena, (unsigned long long)arena_bytes<uint32_t>(E));
         }
     }
 }
@@ -181,43 +241,51 @@ __device__ inline void hinsert(uint32_t *hkey, uint32_t H, uint32_t key)
     }
 }
 
-__device__ inline uint32_t hlookup(const uint32_t *hkey, const uint32_t *hval, uint32_t H, uint32_t key)
+template <typename I>
+__device__ inline uint32_t hlookup(const uint32_t *hkey, const I *hval, uint32_t H, uint32_t key)
 {
     uint32_t s = hslot(key, H);
     for (uint32_t probe = 0; probe < H && hkey[s] != key; ++probe) s = (s + 1 == H) ? 0 : s + 1;
     return hval[s];
 }
 
-// Timestamp groups of at least this many events are scheduled by the whole CTA.
-constexpr uint32_t kParGroup = 128;
-constexpr uint32_t kClaim = 0xFFFFFFFEu;  // run / temp slot being assigned
+// Appends of a warp to one counter per level: the lanes of one level take
+// consecutive positions with a single shared-memory atomic.  All lanes call it.
+__device__ inline uint32_t level_append(uint32_t *lh, uint32_t level, bool act)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t same = __match_any_sync(0xffffffffu, act ? level : 0xffffffffu);
+    const uint32_t leader = __ffs(same) - 1;
+    uint32_t base = 0;
+    if (act && lane == leader) base = atomicAdd(&lh[level], (uint32_t)__popc(same));
+    return __shfl_sync(0xffffffffu, base, leader) + __popc(same & ((1u << lane) - 1u));
+}
 
-// Scan state shared by the threads of a window's CTA: nruns, naux, ntemp,
-// maxlev, next event, end of the large group at it.
+// Scan state shared by the threads of a window's CTA: runs, source-list words,
+// saved rows, largest level, next event, end of the group handed over.
 enum { kScRuns = 0, kScAux, kScTemp, kScMaxlev, kScNext, kScEnd, kScCount };
 
-// The snapshot rule for one large undirected timestamp group [i, g1), with
-// every thread of the CTA.  It yields the same roles, levels, runs (PULLs),
-// saved-row slots and source lists as the sequential scan; only the numbering
-// of runs and slots and the order of ops inside a level and of sources inside
-// a PULL list may differ, and none of them changes the result.  Nodes that
-// occur once in the group take part in exactly one event, so a lone event
-// (both ends once) touches no other event's rows and gets its level at once;
-// the other events share one level L = 1 + the latest level of their nodes,
-// with the PULLs at L + 1.  Phases are separated by barriers, so a run's
-// and a slot's number are final before anyone reads them.
-__device__ void schedule_group_parallel(uint32_t i, uint32_t g1, const uint32_t *lu, const uint32_t *lv,
-                                        uint32_t *grp, uint32_t *evl, uint32_t *run_node, uint32_t *run_aux,
-                                        uint32_t *run_lev, uint32_t *run_temp, uint32_t *nlev, uint32_t *ncnt,
-                                        uint32_t *nrun, uint32_t *auxw, uint32_t *sc)
+// The snapshot rule for one timestamp group [i, g1) with every thread of the
+// CTA.  The numbering of runs and slots, the order of ops inside a level and
+// of sources inside a PULL list are unspecified; none of them changes the
+// result.  In an undirected group, nodes that occur once take part in exactly
+// one event, so a lone event (both ends once) touches no other event's rows and
+// gets its level at once; the other events share one level L = 1 + the latest
+// level of their nodes, with the PULLs at L + 1.  Phases are separated by
+// barriers, so a run's and a slot's number are final before anyone reads them.
+template <typename I>
+__device__ void schedule_group(uint32_t i, uint32_t g1, bool directed, const Arena<I> &A, uint32_t *ncnt, I *nlev,
+                               I *nrun, uint32_t *auxw, uint32_t *sc)
 {
+    constexpr I kNone = (I)~(I)0, kClaim = (I)(kNone - 1);
     __shared__ uint32_t Lc, any, run0;
     const uint32_t T = blockDim.x, tid = threadIdx.x;
     for (uint32_t j = i + tid; j < g1; j += T) {
-        ncnt[lu[j]] = 0;
-        ncnt[lv[j]] = 0;
-        nrun[lu[j]] = kNone;
-        nrun[lv[j]] = kNone;
+        const uint32_t x = A.lu[j], y = A.lv[j];
+        ncnt[x] = 0;
+        ncnt[y] = 0;
+        nrun[x] = kNone;
+        nrun[y] = kNone;
     }
     if (tid == 0) {
         Lc = 0;
@@ -225,414 +293,349 @@ __device__ void schedule_group_parallel(uint32_t i, uint32_t g1, const uint32_t 
         run0 = sc[kScRuns];
     }
     __syncthreads();
-    for (uint32_t j = i + tid; j < g1; j += T)
-        if (lu[j] != lv[j]) {
-            atomicAdd(&ncnt[lu[j]], 1u);
-            atomicAdd(&ncnt[lv[j]], 1u);
-        }
+    for (uint32_t j = i + tid; j < g1; j += T) {
+        const uint32_t x = A.lu[j], y = A.lv[j];
+        if (x == y) continue;
+        if (!directed) atomicAdd(&ncnt[x], 1u);
+        atomicAdd(&ncnt[y], 1u);
+    }
     __syncthreads();
-    // roles; lone events' levels; one run (PULL) per node occurring several times
+    // roles; lone events' levels; one run (PULL) per node occurring several
+    // times (directed: per receiver)
     auto claim_run = [&](uint32_t x) {
         if (atomicCAS(&nrun[x], kNone, kClaim) != kNone) return;
         const uint32_t r = atomicAdd(&sc[kScRuns], 1u);
         const uint32_t b = atomicAdd(&sc[kScAux], 1u + ncnt[x]);
-        run_node[r] = x;
-        run_aux[r] = b;
-        run_lev[r] = 0;  // fill counter until the level is known
-        run_temp[r] = kNone;
+        A.run_node[r] = (I)x;
+        A.run_aux[r] = (I)b;
+        A.run_lev[r] = 0;  // fill counter until the level is known
+        A.run_temp[r] = kNone;
         auxw[b] = ncnt[x];
-        nrun[x] = r;
+        nrun[x] = (I)r;
     };
     for (uint32_t j = i + tid; j < g1; j += T) {
-        const uint32_t x = lu[j], y = lv[j];
+        const uint32_t x = A.lu[j], y = A.lv[j];
         if (x == y) {
-            grp[j] = kFlagNoop;
+            A.flg[j] = kFlagNoop;
             continue;
         }
-        const bool sx = ncnt[x] > 1, sy = ncnt[y] > 1;
+        const bool sx = directed || ncnt[x] > 1, sy = directed || ncnt[y] > 1;
+        const uint32_t lev = max((uint32_t)nlev[x], (uint32_t)nlev[y]);
         if (!sx && !sy) {
-            const uint32_t L = 1 + max(nlev[x], nlev[y]);
-            nlev[x] = L;
-            nlev[y] = L;
-            evl[j] = L;
-            grp[j] = kFlagIso;
-            atomicMax(&sc[kScMaxlev], L);
+            nlev[x] = (I)(lev + 1);
+            nlev[y] = (I)(lev + 1);
+            A.evl[j] = (I)(lev + 1);
+            A.flg[j] = kFlagIso;
+            atomicMax(&sc[kScMaxlev], lev + 1);
             continue;
         }
-        atomicMax(&Lc, max(nlev[x], nlev[y]));
+        atomicMax(&Lc, lev);
         any = 1;
-        grp[j] = (sx ? kFlagShA : 0u) | (sy ? kFlagShB : 0u);
-        if (sx) claim_run(x);
+        A.flg[j] = (sx ? kFlagShA : 0u) | (sy ? kFlagShB : 0u);
+        if (sx && !directed) claim_run(x);
         if (sy) claim_run(y);
     }
     __syncthreads();
-    // saved rows: a node occurring several times whose partner does too is
-    // read from a copy of its old row
+    // saved rows: a node with a run that another run reads is read from a copy
+    // of its old row
     auto claim_temp = [&](uint32_t r) {
-        if (atomicCAS(&run_temp[r], kNone, kClaim) == kNone) run_temp[r] = atomicAdd(&sc[kScTemp], 1u);
+        if (atomicCAS(&A.run_temp[r], kNone, kClaim) == kNone) A.run_temp[r] = (I)atomicAdd(&sc[kScTemp], 1u);
     };
     for (uint32_t j = i + tid; j < g1; j += T)
-        if (grp[j] == (kFlagShA | kFlagShB)) {
-            claim_temp(nrun[lu[j]]);
-            claim_temp(nrun[lv[j]]);
+        if (A.flg[j] == (kFlagShA | kFlagShB)) {
+            if (nrun[A.lu[j]] != kNone) claim_temp(nrun[A.lu[j]]);
+            if (!directed) claim_temp(nrun[A.lv[j]]);
         }
     __syncthreads();
-    // source lists
+    // source lists (entries: local row ids, or temp references)
+    auto add_source = [&](uint32_t node, uint32_t from) {
+        const uint32_t r = nrun[node];
+        const uint32_t f = nrun[from];
+        const uint32_t ref = f != kNone ? kTempRef | A.run_temp[f] : from;
+        auxw[A.run_aux[r] + 1u + atomicAdd(&A.run_lev[r], 1u)] = ref;
+    };
     for (uint32_t j = i + tid; j < g1; j += T) {
-        const uint32_t f = grp[j];
+        const uint32_t f = A.flg[j];
         if (f & (kFlagNoop | kFlagIso)) continue;
-        const uint32_t x = lu[j], y = lv[j];
-        if (f == (kFlagShA | kFlagShB)) {
-            const uint32_t rx = nrun[x], ry = nrun[y];
-            auxw[run_aux[rx] + 1 + atomicAdd(&run_lev[rx], 1u)] = kTempRef | run_temp[ry];
-            auxw[run_aux[ry] + 1 + atomicAdd(&run_lev[ry], 1u)] = kTempRef | run_temp[rx];
-        } else if (f & kFlagShA) {
-            const uint32_t rx = nrun[x];
-            auxw[run_aux[rx] + 1 + atomicAdd(&run_lev[rx], 1u)] = y;
-        } else {
-            const uint32_t ry = nrun[y];
-            auxw[run_aux[ry] + 1 + atomicAdd(&run_lev[ry], 1u)] = x;
-        }
+        const uint32_t x = A.lu[j], y = A.lv[j];
+        if ((f & kFlagShA) && !directed) add_source(x, y);
+        if (f & kFlagShB) add_source(y, x);
     }
     __syncthreads();
     // levels of the shared part: ONEWAY / COPY at L, PULL at L + 1
     if (any) {
         const uint32_t L = Lc + 1;
         for (uint32_t j = i + tid; j < g1; j += T) {
-            if (grp[j] & (kFlagNoop | kFlagIso)) continue;
-            evl[j] = L;
-            nlev[lu[j]] = L + 1;
-            nlev[lv[j]] = L + 1;
+            if (A.flg[j] & (kFlagNoop | kFlagIso)) continue;
+            A.evl[j] = (I)L;
+            nlev[A.lu[j]] = (I)(L + 1);
+            nlev[A.lv[j]] = (I)(L + 1);
         }
-        for (uint32_t r = run0 + tid; r < sc[kScRuns]; r += T) run_lev[r] = L;
+        for (uint32_t r = run0 + tid; r < sc[kScRuns]; r += T) A.run_lev[r] = L;
         if (tid == 0) atomicMax(&sc[kScMaxlev], L + 1);
     }
     __syncthreads();
 }
 
-__device__ void schedule_window(const PlanArgs &a, uint32_t w, uint32_t *arena)
+// Levels of the events from sc[kScNext] up to the next group that shares
+// nodes, by warp 0: lane 2k + side holds one endpoint of the chunk's event k.
+// Each event's level needs only its two nodes' last levels, so a chunk without
+// repeated nodes takes one round: a shared-memory read, a shuffle, a write.
+// Repeated nodes are found one chunk ahead (every lane writes its number to its
+// node's claim and reads it back), off the chain from level to level; in such a
+// chunk an event waits until the earlier events on its nodes are done.  (The
+// warp's match instruction in every chunk made the walk 7 times as long: 770
+// cycles a chunk.)
+template <typename I>
+__device__ void scan_levels(uint32_t E, bool directed, const Arena<I> &A, I *nlev, uint32_t *sc)
+{
+    const uint32_t lane = threadIdx.x & 31u, side = lane & 1u;
+    const I *mine = side ? A.lv : A.lu;
+    uint32_t i = sc[kScNext], top = 0, end = E;
+    uint32_t x = 0, f = 0, twice = 0;
+    bool run = false, live = false;  // before the group; not a self-loop
+    uint32_t stop = 16u;             // events of the chunk before the group
+    auto fetch = [&](uint32_t at) {
+        const uint32_t e = at + (lane >> 1);
+        x = e < E ? (uint32_t)mine[e] : 0u;
+        f = e < E ? (uint32_t)A.flg[e] : 0u;
+        const uint32_t hard = __ballot_sync(0xffffffffu, f & kFlagHard);
+        stop = hard ? (__ffs(hard) - 1) >> 1 : 16u;
+        run = e < E && (lane >> 1) < stop;
+        const uint32_t other = __shfl_xor_sync(0xffffffffu, x, 1);
+        live = run && x != other;
+        if (live) A.claim[x] = (uint8_t)lane;
+        __syncwarp();
+        const bool lost = live && A.claim[x] != (uint8_t)lane;
+        twice = __ballot_sync(0xffffffffu, lost);
+        __syncwarp();
+    };
+    fetch(i);
+    while (i < E) {
+        const uint32_t node = x, e = i + (lane >> 1), conflict = twice, before_group = stop;
+        const bool act = run, go1 = live;
+        if (before_group == 16u) fetch(i + 16u);  // independent of this chunk's levels
+        uint32_t lev = 0;
+        if (!conflict) {
+            lev = go1 ? (uint32_t)nlev[node] : 0u;
+            lev = max(lev, __shfl_xor_sync(0xffffffffu, lev, 1)) + 1u;
+            if (go1) nlev[node] = (I)lev;
+            __syncwarp();
+        } else {
+            const uint32_t same = __match_any_sync(0xffffffffu, go1 ? node : 0x80000000u | lane);
+            const uint32_t before = same & ((1u << lane) - 1u);
+            uint32_t pending = __ballot_sync(0xffffffffu, go1);
+            while (pending) {
+                const uint32_t ready = __ballot_sync(0xffffffffu, ((pending >> lane) & 1u) && !(before & pending));
+                const uint32_t both = ready & (((ready & 0x55555555u) << 1) | ((ready >> 1) & 0x55555555u));
+                const bool go = (both >> lane) & 1u;
+                uint32_t l = go ? (uint32_t)nlev[node] : 0u;
+                l = max(l, __shfl_xor_sync(0xffffffffu, l, 1)) + 1u;
+                if (go) {
+                    nlev[node] = (I)l;
+                    lev = l;
+                }
+                __syncwarp();
+                pending &= ~both;
+            }
+        }
+        if (go1) top = max(top, lev);
+        if (act && !side) {
+            A.evl[e] = (I)lev;
+            A.flg[e] = !go1 ? kFlagNoop : directed ? kFlagDir : kFlagIso;
+        }
+        if (before_group < 16u) {
+            end = i + before_group;
+            break;
+        }
+        i += 16u;
+    }
+    __syncwarp();
+    top = __reduce_max_sync(0xffffffffu, top);
+    const uint32_t next = end < E ? end : E;
+    // end of the group at `next`
+    uint32_t g1 = next + 1;
+    if (next < E) {
+        for (;;) {
+            const uint32_t e = g1 + lane;
+            const uint32_t starts = __ballot_sync(0xffffffffu, e >= E || (A.flg[e] & kFlagStart));
+            if (starts) {
+                g1 += __ffs(starts) - 1;
+                break;
+            }
+            g1 += 32u;
+        }
+        if (g1 > E) g1 = E;
+    }
+    if (lane == 0) {
+        sc[kScNext] = next;
+        sc[kScEnd] = g1;
+        if (top > sc[kScMaxlev]) sc[kScMaxlev] = top;
+    }
+}
+
+template <typename I>
+__device__ void schedule_window(const PlanArgs &a, uint32_t w, uint8_t *arena)
 {
     __shared__ uint32_t warp_sums[32];
     __shared__ uint32_t tot;
-    __shared__ uint32_t res[8];  // nops, maxlev, naux, ntemp, nruns, local, nitems
+    __shared__ uint32_t sc[kScCount];
+    __shared__ uint32_t res[2];  // packs, units
 
     const uint64_t s = a.wstart[w];
     const uint32_t E = (uint32_t)(a.wstart[w + 1] - s);
-    uint32_t *cnt = a.wcount + (uint64_t)kWinFields * w;
+    const uint32_t T = blockDim.x, tid = threadIdx.x, lane = tid & 31u;
+    WinDesc *desc = a.desc + w;
     if (E == 0) {
-        if (threadIdx.x < kWinFields) cnt[threadIdx.x] = 0;
+        if (tid == 0) {
+            *desc = WinDesc{};
+            a.naux_w[w] = 0;
+        }
         return;
     }
-    const uint32_t T = blockDim.x, tid = threadIdx.x;
-    const uint32_t H = (uint32_t)hash_slots(E);
-    uint32_t *lu = arena, *lv = lu + E, *grp = lv + E, *evl = grp + E;
-    uint32_t *run_node = evl + E, *run_aux = run_node + E, *run_lev = run_aux + E, *run_temp = run_lev + E;
-    uint32_t *rowsg = run_temp + E;  // [2E] global id of every local row id
-    uint32_t *scratch = rowsg + 2 * E;
-    uint32_t *hkey = scratch, *hval = scratch + H;
+    const Arena<I> A(arena, E);
     const uint32_t *U = a.u + s, *V = a.v + s;
     const int64_t *Tt = a.t + s;
 
-    // 1. compact node ids (local row ids 0..D-1)
-    for (uint32_t i = tid; i < H; i += T) hkey[i] = kEmpty;
-    __syncthreads();
-    for (uint32_t i = tid; i < E; i += T) {
-        hinsert(hkey, H, U[i]);
-        hinsert(hkey, H, V[i]);
-    }
-    __syncthreads();
-    for (uint32_t i = tid; i < H; i += T) hval[i] = hkey[i] != kEmpty ? 1u : 0u;
-    __syncthreads();
-    const uint32_t D = block_excl_scan_array(hval, H, warp_sums, &tot);
-    for (uint32_t i = tid; i < H; i += T)
-        if (hkey[i] != kEmpty) rowsg[hval[i]] = hkey[i];
-    for (uint32_t i = tid; i < E; i += T) {
-        lu[i] = hlookup(hkey, hval, H, U[i]);
-        lv[i] = hlookup(hkey, hval, H, V[i]);
-        grp[i] = (i == 0 || Tt[i] != Tt[i - 1]) ? 1u : 0u;
-    }
-    __syncthreads();
-    block_excl_scan_array(grp, E, warp_sums, &tot);  // grp[i] = starts before i
-    for (uint32_t i = tid; i < E; i += T) grp[i] += (i == 0 || Tt[i] != Tt[i - 1]) ? 1u : 0u;
-    // grp[i] is now 1 + group index, which is all the scan below needs.
-    uint32_t *nlev = scratch, *ncnt = scratch + D, *nrun = scratch + 2 * D;
-    __syncthreads();
-    for (uint32_t i = tid; i < D; i += T) {
-        nlev[i] = 0;
-        ncnt[i] = 0;
-        nrun[i] = kNone;
-    }
-    __syncthreads();
-
-    // 2. level scan in time order: one thread takes the groups one by one and
-    //    hands every large undirected group to the whole CTA.  Rows are named
-    //    by local ids here; PULL source lists hold local ids or temp references.
-    __shared__ uint32_t sc[kScCount];
-    if (tid == 0)
-        for (int q = 0; q < kScCount; ++q) sc[q] = 0;
-    __syncthreads();
-    for (;;) {
-    if (tid == 0) {
-        uint32_t nruns = sc[kScRuns], naux = sc[kScAux], ntemp = sc[kScTemp], maxlev = sc[kScMaxlev];
-        uint32_t *auxw = a.aux_stage + 3 * s;
-        uint32_t i = sc[kScNext];
-        while (i < E && a.directed) {
-            // directed events x -> y: only y is written.  A lone event is one
-            // ONEWAY y |= x; a tie group becomes one PULL per receiver (level
-            // L+1) over its senders' rows, a sender that also receives in the
-            // group being read from a copy saved at level L.
-            const uint32_t g = grp[i];
-            uint32_t g1 = i + 1;
-            while (g1 < E && grp[g1] == g) ++g1;
-            if (g1 == i + 1) {
-                const uint32_t x = lu[i], y = lv[i];
-                if (x == y) {
-                    grp[i] = kFlagNoop;
-                } else {
-                    const uint32_t L = 1 + max(nlev[x], nlev[y]);
-                    nlev[x] = L;
-                    nlev[y] = L;
-                    evl[i] = L;
-                    grp[i] = kFlagDir;
-                    maxlev = max(maxlev, L);
-                }
-                i = g1;
-                continue;
-            }
-            for (uint32_t j = i; j < g1; ++j) {
-                ncnt[lv[j]] = 0;
-                nrun[lu[j]] = kNone;
-                nrun[lv[j]] = kNone;
-            }
-            uint32_t Lc = 0;
-            bool any = false;
-            for (uint32_t j = i; j < g1; ++j) {
-                if (lu[j] == lv[j]) continue;
-                ++ncnt[lv[j]];
-                Lc = max(Lc, max(nlev[lu[j]], nlev[lv[j]]));
-            }
-            const uint32_t run0 = nruns;
-            for (uint32_t j = i; j < g1; ++j) {  // one run per receiver
-                const uint32_t y = lv[j];
-                if (lu[j] == y || nrun[y] != kNone) continue;
-                const uint32_t ry = nruns++;
-                nrun[y] = ry;
-                run_node[ry] = y;
-                run_aux[ry] = naux;
-                run_lev[ry] = 0;  // fill counter until the level is known
-                run_temp[ry] = kNone;
-                auxw[naux] = ncnt[y];
-                naux += 1 + ncnt[y];
-            }
-            for (uint32_t j = i; j < g1; ++j) {
-                const uint32_t x = lu[j], y = lv[j];
-                if (x == y) {
-                    grp[j] = kFlagNoop;
-                    continue;
-                }
-                any = true;
-                grp[j] = kFlagShA | kFlagShB;  // no op of its own: the receiver's PULL covers it
-                uint32_t ref = x;
-                const uint32_t rx = nrun[x];
-                if (rx != kNone) {  // x also receives in this group: read its saved old row
-                    if (run_temp[rx] == kNone) run_temp[rx] = ntemp++;
-                    ref = kTempRef | run_temp[rx];
-                }
-                const uint32_t ry = nrun[y];
-                auxw[run_aux[ry] + 1 + run_lev[ry]++] = ref;
-            }
-            if (any) {
-                const uint32_t L = Lc + 1;
-                for (uint32_t j = i; j < g1; ++j) {
-                    if (grp[j] & kFlagNoop) continue;
-                    nlev[lu[j]] = L + 1;
-                    nlev[lv[j]] = L + 1;
-                }
-                for (uint32_t r = run0; r < nruns; ++r) run_lev[r] = L;
-                maxlev = max(maxlev, L + 1);
-            }
-            i = g1;
+    // 1. local row ids 0..D-1: the node ids themselves in a network of at most
+    //    2E nodes (unless the window may become a record, whose rows are
+    //    gathered), else compacted through a hash table.  The endpoints wait in
+    //    rowsg until it is filled.
+    const bool direct = a.unit8 < 5 && a.n <= 2 * (uint64_t)E;
+    uint32_t D;
+    for (uint32_t i0 = 0; i0 < E; i0 += 4 * T) {
+        uint32_t uu[4], vv[4];
+        int64_t ta[4], tb[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t i = i0 + q * T + tid;
+            const bool in = i < E;
+            uu[q] = in ? U[i] : 0u;
+            vv[q] = in ? V[i] : 0u;
+            ta[q] = in ? Tt[i] : 0;
+            tb[q] = in && i ? Tt[i - 1] : 0;
         }
-        while (i < E) {
-            const uint32_t g = grp[i];
-            if (i + kParGroup <= E && grp[i + kParGroup - 1] == g) break;  // a large group: the whole CTA
-            uint32_t g1 = i + 1;
-            while (g1 < E && grp[g1] == g) ++g1;
-            if (g1 == i + 1) {
-                const uint32_t x = lu[i], y = lv[i];
-                if (x == y) {
-                    grp[i] = kFlagNoop;
-                } else {
-                    const uint32_t L = 1 + max(nlev[x], nlev[y]);
-                    nlev[x] = L;
-                    nlev[y] = L;
-                    evl[i] = L;
-                    grp[i] = kFlagIso;
-                    maxlev = max(maxlev, L);
-                }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t i = i0 + q * T + tid;
+            if (i >= E) continue;
+            A.flg[i] = (i == 0 || ta[q] != tb[q]) ? kFlagStart : 0;
+            if (direct) {
+                A.lu[i] = (I)uu[q];
+                A.lv[i] = (I)vv[q];
             } else {
-                // occurrences of every node inside the group
-                for (uint32_t j = i; j < g1; ++j) {
-                    ncnt[lu[j]] = 0;
-                    ncnt[lv[j]] = 0;
-                    nrun[lu[j]] = kNone;
-                    nrun[lv[j]] = kNone;
-                }
-                for (uint32_t j = i; j < g1; ++j) {
-                    if (lu[j] == lv[j]) continue;
-                    ++ncnt[lu[j]];
-                    ++ncnt[lv[j]];
-                }
-                const uint32_t run0 = nruns;
-                uint32_t Lc = 0;
-                bool any = false;
-                for (uint32_t j = i; j < g1; ++j) {
-                    const uint32_t x = lu[j], y = lv[j];
-                    if (x == y) {
-                        grp[j] = kFlagNoop;
-                        continue;
-                    }
-                    const bool sx = ncnt[x] > 1, sy = ncnt[y] > 1;
-                    if (!sx && !sy) {
-                        const uint32_t L = 1 + max(nlev[x], nlev[y]);
-                        nlev[x] = L;
-                        nlev[y] = L;
-                        evl[j] = L;
-                        grp[j] = kFlagIso;
-                        maxlev = max(maxlev, L);
-                        continue;
-                    }
-                    any = true;
-                    Lc = max(Lc, max(nlev[x], nlev[y]));
-                    grp[j] = (sx ? kFlagShA : 0u) | (sy ? kFlagShB : 0u);
-                    uint32_t rx = kNone, ry = kNone;
-                    if (sx) {
-                        rx = nrun[x];
-                        if (rx == kNone) {
-                            rx = nruns++;
-                            nrun[x] = rx;
-                            run_node[rx] = x;
-                            run_aux[rx] = naux;
-                            run_lev[rx] = 0;  // fill counter until the level is known
-                            run_temp[rx] = kNone;
-                            auxw[naux] = ncnt[x];
-                            naux += 1 + ncnt[x];
-                        }
-                    }
-                    if (sy) {
-                        ry = nrun[y];
-                        if (ry == kNone) {
-                            ry = nruns++;
-                            nrun[y] = ry;
-                            run_node[ry] = y;
-                            run_aux[ry] = naux;
-                            run_lev[ry] = 0;
-                            run_temp[ry] = kNone;
-                            auxw[naux] = ncnt[y];
-                            naux += 1 + ncnt[y];
-                        }
-                    }
-                    if (sx && sy) {
-                        if (run_temp[rx] == kNone) run_temp[rx] = ntemp++;
-                        if (run_temp[ry] == kNone) run_temp[ry] = ntemp++;
-                        auxw[run_aux[rx] + 1 + run_lev[rx]++] = kTempRef | run_temp[ry];
-                        auxw[run_aux[ry] + 1 + run_lev[ry]++] = kTempRef | run_temp[rx];
-                    } else if (sx) {
-                        auxw[run_aux[rx] + 1 + run_lev[rx]++] = y;
-                    } else {
-                        auxw[run_aux[ry] + 1 + run_lev[ry]++] = x;
-                    }
-                }
-                if (any) {
-                    const uint32_t L = Lc + 1;
-                    for (uint32_t j = i; j < g1; ++j) {
-                        const uint32_t f = grp[j];
-                        if (f & (kFlagNoop | kFlagIso)) continue;
-                        evl[j] = L;
-                        nlev[lu[j]] = L + 1;
-                        nlev[lv[j]] = L + 1;
-                    }
-                    for (uint32_t r = run0; r < nruns; ++r) run_lev[r] = L;
-                    maxlev = max(maxlev, L + 1);
-                }
+                A.rowsg[i] = uu[q];
+                A.rowsg[E + i] = vv[q];
             }
-            i = g1;
-        }
-        sc[kScRuns] = nruns;
-        sc[kScAux] = naux;
-        sc[kScTemp] = ntemp;
-        sc[kScMaxlev] = maxlev;
-        sc[kScNext] = i;
-        if (i < E) {  // end of the large group at i: first index past it (grp is non-decreasing there)
-            uint32_t lo = i, hi = E;
-            while (lo < hi) {
-                const uint32_t mid = lo + (hi - lo) / 2;
-                if (grp[mid] > grp[i]) hi = mid;
-                else lo = mid + 1;
-            }
-            sc[kScEnd] = lo;
         }
     }
-    __syncthreads();
-    if (sc[kScNext] >= E) break;
-    schedule_group_parallel(sc[kScNext], sc[kScEnd], lu, lv, grp, evl, run_node, run_aux, run_lev, run_temp, nlev,
-                            ncnt, nrun, a.aux_stage + 3 * s, sc);
-    if (tid == 0) sc[kScNext] = sc[kScEnd];
-    __syncthreads();
+    if (tid < kScCount) sc[tid] = 0;
+    if (direct) {
+        D = a.n;
+        for (uint32_t i = tid; i < D; i += T) A.rowsg[i] = i;
+        __syncthreads();
+    } else {
+        const uint32_t H = (uint32_t)hash_slots(E);
+        uint32_t *hkey = A.scratch;
+        I *hval = reinterpret_cast<I *>(A.scratch + H);
+        for (uint32_t i = tid; i < H; i += T) hkey[i] = kEmpty;
+        __syncthreads();
+        for (uint32_t i = tid; i < 2 * E; i += T) hinsert(hkey, H, A.rowsg[i]);
+        __syncthreads();
+        for (uint32_t i = tid; i < H; i += T) hval[i] = hkey[i] != kEmpty ? 1 : 0;
+        __syncthreads();
+        D = block_excl_scan_array(hval, H, warp_sums, &tot);
+        for (uint32_t i = tid; i < 2 * E; i += T) A.lu[i] = (I)hlookup(hkey, hval, H, A.rowsg[i]);  // lu, then lv
+        __syncthreads();
+        for (uint32_t i = tid; i < H; i += T)
+            if (hkey[i] != kEmpty) A.rowsg[hval[i]] = hkey[i];
+        __syncthreads();
     }
-    if (tid == 0) {
-        res[1] = sc[kScMaxlev];
-        res[2] = sc[kScAux];
-        res[3] = sc[kScTemp];
-        res[4] = sc[kScRuns];
-        res[6] = 0;
-    }
-    __syncthreads();
-    const uint32_t maxlev = res[1], naux = res[2], ntemp = res[3], nruns = res[4];
+    uint32_t *ncnt = A.scratch;
+    I *nlev = reinterpret_cast<I *>(A.scratch + 2 * (uint64_t)E), *nrun = nlev + 2 * (uint64_t)E;
+    for (uint32_t i = tid; i < D; i += T) nlev[i] = 0;
 
-    // 3. counting sort of the updates by level (levels 1..maxlev -> 0..maxlev-1)
-    uint32_t *lh = scratch;  // node state is dead
+    // 2. groups that share nodes (marked on their first event)
+    for (uint32_t i = tid; i < E; i += T) {
+        const uint32_t x = A.lu[i], y = A.lv[i];
+        bool shared = false;
+        uint32_t j = i + 1;
+        for (; j < E && j - i < kPairGroup && !(A.flg[j] & kFlagStart) && !shared; ++j) {
+            const uint32_t p = A.lu[j], q = A.lv[j];
+            shared = x != y && p != q && (x == p || x == q || y == p || y == q);
+        }
+        if (!shared) {
+            if (j - i >= kPairGroup && (A.flg[i] & kFlagStart)) A.flg[i] = kFlagStart | kFlagHard;
+            continue;
+        }
+        uint32_t g = i;
+        while (!(A.flg[g] & kFlagStart) && i - g < kPairGroup) --g;  // (a larger group is marked by its first event)
+        if (A.flg[g] & kFlagStart) A.flg[g] = kFlagStart | kFlagHard;
+    }
+    __syncthreads();
+
+    // 3. levels in time order
+    uint32_t *auxw = a.aux + 3 * s;
+    for (;;) {
+        if (tid < 32) scan_levels(E, a.directed != 0, A, nlev, sc);
+        __syncthreads();
+        const uint32_t next = sc[kScNext], end = sc[kScEnd];
+        if (next >= E) break;
+        schedule_group(next, end, a.directed != 0, A, ncnt, nlev, nrun, auxw, sc);
+        if (tid == 0) sc[kScNext] = end;
+        __syncthreads();
+    }
+    const uint32_t maxlev = sc[kScMaxlev], naux = sc[kScAux], ntemp = sc[kScTemp], nruns = sc[kScRuns];
+    __syncthreads();
+
+    // 4. counting sort of the updates by level (levels 1..maxlev -> 0..maxlev-1)
+    uint32_t *lh = A.scratch;  // node state is dead
     for (uint32_t j = tid; j < maxlev + 1; j += T) lh[j] = 0;
     __syncthreads();
-    for (uint32_t i = tid; i < E; i += T) {
-        const uint32_t f = grp[i];
-        if (f & kFlagNoop) continue;
-        if (f & (kFlagIso | kFlagDir)) {
-            atomicAdd(&lh[evl[i] - 1], 1u);
-        } else {
-            if (!(f & kFlagShA)) atomicAdd(&lh[evl[i] - 1], 1u);
-            if (!(f & kFlagShB)) atomicAdd(&lh[evl[i] - 1], 1u);
-        }
+    // an event is one op: EVENT, a directed ONEWAY, or the ONEWAY of its end that occurs once
+    auto has_op = [&](uint32_t i) {
+        const uint32_t f = i < E ? (uint32_t)A.flg[i] : (uint32_t)kFlagNoop;
+        return !(f & kFlagNoop) && (f & (kFlagShA | kFlagShB)) != (kFlagShA | kFlagShB);
+    };
+    for (uint32_t i0 = 0; i0 < E; i0 += T) {
+        const uint32_t i = i0 + tid;
+        const bool act = has_op(i);
+        level_append(lh, act ? A.evl[i] - 1u : 0u, act);
     }
     for (uint32_t r = tid; r < nruns; r += T) {
-        atomicAdd(&lh[run_lev[r]], 1u);  // PULL at level L+1 -> index L
-        if (run_temp[r] != kNone) atomicAdd(&lh[run_lev[r] - 1], 1u);
+        const uint32_t L = A.run_lev[r];
+        atomicAdd(&lh[L], 1u);  // PULL at level L+1 -> index L
+        if (A.run_temp[r] != (I)~(I)0) atomicAdd(&lh[L - 1], 1u);
     }
     __syncthreads();
     const uint32_t nops = block_excl_scan_array(lh, maxlev + 1, warp_sums, &tot);
 
-    // 4. mode: the window's rows and saved rows fit the streaming kernel's
+    // 5. mode: the window's rows and saved rows fit the streaming kernel's
     //    shared-memory row buffer, and its record fits one staging buffer
     const uint32_t rec_words = 4 + D + (maxlev + 1) + nops + naux;
     const uint32_t rec_words_pad = (rec_words + 3u) & ~3u;
-    const bool local = D + ntemp <= a.dcap && rec_words_pad <= a.max_rec_words;
+    const bool local = E <= kRecordEvents && a.unit8 >= 5 && D + ntemp <= a.dcap && rec_words_pad <= kRecordWords;
+    const uint64_t region = blob_base(s, w, a.unit8);
 
     if (local) {
         // record: header | rows[D] | lvl[maxlev+1] | ops[nops] | aux[naux] | pad
-        uint32_t *rec = a.rec_stage + 10 * s + 8ull * w;
+        uint32_t *pack = reinterpret_cast<uint32_t *>(a.blob + region);
+        uint32_t *rec = pack + 4;
         uint32_t *rrows = rec + 4, *rlvl = rrows + D, *rops = rlvl + maxlev + 1, *raux = rops + nops;
         if (tid == 0) {
+            pack[0] = nops;
+            pack[1] = (kPackLocal | kPackWindow) << 16;
+            pack[2] = pack[3] = 0;
             rec[0] = D;
             rec[1] = ntemp;
             rec[2] = maxlev;
             rec[3] = nops;
         }
-        for (uint32_t d = tid; d < D; d += T) rrows[d] = rowsg[d];
+        for (uint32_t d = tid; d < D; d += T) rrows[d] = A.rowsg[d];
         for (uint32_t j = tid; j < maxlev + 1; j += T) rlvl[j] = lh[j];
         for (uint32_t k = rec_words + tid; k < rec_words_pad; k += T) rec[k] = 0;
-        const uint32_t *auxw = a.aux_stage + 3 * s;
         for (uint32_t r = tid; r < nruns; r += T) {
-            const uint32_t b = run_aux[r], c = auxw[b];
+            const uint32_t b = A.run_aux[r], c = auxw[b];
             raux[b] = c;
             for (uint32_t q = 1; q <= c; ++q) {
                 const uint32_t ref = auxw[b + q];
@@ -640,30 +643,25 @@ __device__ void schedule_window(const PlanArgs &a, uint32_t w, uint32_t *arena)
             }
         }
         __syncthreads();
-        for (uint32_t i = tid; i < E; i += T) {
-            const uint32_t f = grp[i];
-            if (f & kFlagNoop) continue;
-            const uint32_t x = lu[i], y = lv[i];
-            if (f & kFlagDir) {
-                rops[atomicAdd(&lh[evl[i] - 1], 1u)] = local_op(kOneway, y, x);  // y |= x
-                continue;
-            }
-            const uint32_t L = evl[i] - 1;
-            if (f & kFlagIso) {
-                rops[atomicAdd(&lh[L], 1u)] = local_op(kEvent, x, y);
-            } else {
-                if (!(f & kFlagShA)) rops[atomicAdd(&lh[L], 1u)] = local_op(kOneway, x, y);
-                if (!(f & kFlagShB)) rops[atomicAdd(&lh[L], 1u)] = local_op(kOneway, y, x);
-            }
+        for (uint32_t i0 = 0; i0 < E; i0 += T) {
+            const uint32_t i = i0 + tid;
+            const bool act = has_op(i);
+            const uint32_t pos = level_append(lh, act ? A.evl[i] - 1u : 0u, act);
+            if (!act) continue;
+            const uint32_t f = A.flg[i], x = A.lu[i], y = A.lv[i];
+            rops[pos] = (f & kFlagIso) ? local_op(kEvent, x, y)
+                        : ((f & kFlagDir) || (f & kFlagShA)) ? local_op(kOneway, y, x)  // y |= x
+                                                             : local_op(kOneway, x, y);
         }
         for (uint32_t r = tid; r < nruns; r += T) {
-            const uint32_t L = run_lev[r];
-            rops[atomicAdd(&lh[L], 1u)] = local_op(kPull, run_node[r], run_aux[r]);
-            if (run_temp[r] != kNone) rops[atomicAdd(&lh[L - 1], 1u)] = local_op(kCopy, D + run_temp[r], run_node[r]);
+            const uint32_t L = A.run_lev[r];
+            rops[atomicAdd(&lh[L], 1u)] = local_op(kPull, A.run_node[r], A.run_aux[r]);
+            if (A.run_temp[r] != (I)~(I)0)
+                rops[atomicAdd(&lh[L - 1], 1u)] = local_op(kCopy, D + A.run_temp[r], A.run_node[r]);
         }
         // last write of every row: ops are in level order and a level writes a
         // row at most once, so it is the op with the highest index writing it
-        uint32_t *lastw = scratch + maxlev + 2;  // lh holds scratch[0 .. maxlev]
+        uint32_t *lastw = A.scratch + maxlev + 2;  // lh holds scratch[0 .. maxlev]
         for (uint32_t d = tid; d < D; d += T) lastw[d] = 0;
         __syncthreads();
         for (uint32_t i = tid; i < nops; i += T) {
@@ -682,197 +680,198 @@ __device__ void schedule_window(const PlanArgs &a, uint32_t w, uint32_t *arena)
             rops[i] = op;
         }
         if (tid == 0) {
-            cnt[0] = 0;
-            cnt[1] = maxlev;
-            cnt[2] = 0;
-            cnt[3] = 0;
-            cnt[4] = 1;
-            cnt[5] = rec_words_pad / 2;
-            cnt[6] = 1;
-            cnt[7] = nops;
+            res[0] = nops ? 1u : 0u;
+            res[1] = 2 + rec_words_pad / 2;
+            WinDesc d{};
+            d.off = region;
+            d.npacks = res[0];
+            d.pack[0] = res[1];
+            *desc = d;
+            a.naux_w[w] = 0;
         }
-        return;
-    }
-
-    // global mode: ops name rows by node id; PULL lists are converted in place
-    uint32_t *lvl_out = a.lvl_stage + 2 * s + w;
-    for (uint32_t j = tid; j < maxlev + 1; j += T) lvl_out[j] = lh[j];
-    for (uint32_t j = tid; j < maxlev; j += T) {
-        const uint32_t c = lh[j + 1] - lh[j];
-        atomicAdd(&res[6], (c + kTileOps - 1) / kTileOps);
-    }
-    uint32_t *auxw = a.aux_stage + 3 * s;
-    for (uint32_t r = tid; r < nruns; r += T) {
-        const uint32_t b = run_aux[r], c = auxw[b];
-        for (uint32_t q = 1; q <= c; ++q) {
-            const uint32_t ref = auxw[b + q];
-            if (!(ref & kTempRef)) auxw[b + q] = rowsg[ref];
-        }
-    }
-    __syncthreads();
-    uint2 *ops = a.ops_stage + 3 * s;
-    for (uint32_t i = tid; i < E; i += T) {
-        const uint32_t f = grp[i];
-        if (f & kFlagNoop) continue;
-        const uint32_t x = U[i], y = V[i];
-        const uint32_t L = evl[i] - 1;
-        if (f & kFlagDir) {
-            ops[atomicAdd(&lh[L], 1u)] = make_uint2(op_a(kOneway, y), x);  // y |= x
-            continue;
-        }
-        if (f & kFlagIso) {
-            ops[atomicAdd(&lh[L], 1u)] = make_uint2(op_a(kEvent, x), y);
-        } else {
-            if (!(f & kFlagShA)) ops[atomicAdd(&lh[L], 1u)] = make_uint2(op_a(kOneway, x), y);
-            if (!(f & kFlagShB)) ops[atomicAdd(&lh[L], 1u)] = make_uint2(op_a(kOneway, y), x);
-        }
-    }
-    for (uint32_t r = tid; r < nruns; r += T) {
-        const uint32_t L = run_lev[r], xg = rowsg[run_node[r]];
-        ops[atomicAdd(&lh[L], 1u)] = make_uint2(op_a(kPull, xg), (uint32_t)(3 * s) + run_aux[r]);
-        if (run_temp[r] != kNone) ops[atomicAdd(&lh[L - 1], 1u)] = make_uint2(op_a(kCopy, run_temp[r]), xg);
-    }
-    __syncthreads();
-    if (tid == 0) {
-        cnt[0] = nops;
-        cnt[1] = maxlev;
-        cnt[2] = naux;
-        cnt[3] = ntemp;
-        cnt[4] = 0;
-        cnt[5] = (nops + 1u) & ~1u;
-        cnt[6] = res[6];
-        cnt[7] = nops;
-    }
-}
-
-__global__ void __launch_bounds__(kPlanThreads) schedule_smem_kernel(PlanArgs a)
-{
-    extern __shared__ uint32_t smem_arena[];
-    const uint32_t w = blockIdx.x;
-    const uint64_t E = a.wstart[w + 1] - a.wstart[w];
-    if (E > a.smem_max_events) return;  // scheduled by the large-window kernel
-    schedule_window(a, w, smem_arena);
-}
-
-__global__ void __launch_bounds__(kPlanThreads) schedule_big_kernel(PlanArgs a)
-{
-    const uint32_t w = a.big_list[blockIdx.x];
-    schedule_window(a, w, a.big_arena + a.big_off[blockIdx.x]);
-}
-
-// ---------------------------------------------------------------------------
-// concatenation of the windows
-// ---------------------------------------------------------------------------
-struct Totals {
-    unsigned long long items, blob8, naux, tmax, levels, ops, local;
-};
-
-// exclusive scans over windows of nitems / blob8 / naux (one CTA)
-__global__ void window_scan_kernel(const uint32_t *wcount, uint32_t nw, uint64_t *base /* [3*nw] */, Totals *tot)
-{
-    __shared__ uint32_t warp_sums[32];
-    __shared__ uint32_t total;
-    __shared__ unsigned long long carry[3];
-    __shared__ unsigned long long levels, ops, local;
-    __shared__ unsigned int tmax;
-    if (threadIdx.x < 3) carry[threadIdx.x] = 0;
-    if (threadIdx.x == 0) {
-        tmax = 0;
-        levels = ops = local = 0;
-    }
-    __syncthreads();
-    static_assert(kWinFields == 8, "two 16-byte loads per window");
-    for (uint32_t c0 = 0; c0 < nw; c0 += blockDim.x) {
-        const uint32_t w = c0 + threadIdx.x;
-        uint4 lo = make_uint4(0u, 0u, 0u, 0u), hi = make_uint4(0u, 0u, 0u, 0u);
-        if (w < nw) {
-            const uint4 *c = reinterpret_cast<const uint4 *>(wcount + (uint64_t)kWinFields * w);
-            lo = c[0];  // nops, nlev, naux, ntemp
-            hi = c[1];  // local, blob8, nitems, all ops
-        }
-        const uint32_t x[3] = {hi.z, hi.y, lo.z};  // items, blob8, naux
-        for (int k = 0; k < 3; ++k) {
-            uint32_t ex = block_excl_scan_value(x[k], warp_sums, &total);
-            if (w < nw) base[3ull * w + k] = carry[k] + ex;
-            __syncthreads();
-            if (threadIdx.x == 0) carry[k] += total;
-            __syncthreads();
-        }
-        // totals: a warp reduction first, then one shared atomic per warp
-        unsigned long long lv = lo.y, op = hi.w, lc = hi.x;
-        uint32_t tm = lo.w;
-        for (int d = 16; d > 0; d >>= 1) {
-            lv += __shfl_xor_sync(0xffffffffu, lv, d);
-            op += __shfl_xor_sync(0xffffffffu, op, d);
-            lc += __shfl_xor_sync(0xffffffffu, lc, d);
-            tm = max(tm, __shfl_xor_sync(0xffffffffu, tm, d));
-        }
-        if ((threadIdx.x & 31u) == 0) {
-            atomicMax(&tmax, tm);
-            atomicAdd(&levels, lv);
-            atomicAdd(&ops, op);
-            atomicAdd(&local, lc);
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        tot->items = carry[0];
-        tot->blob8 = carry[1];
-        tot->naux = carry[2];
-        tot->tmax = tmax;
-        tot->levels = levels;
-        tot->ops = ops;
-        tot->local = local;
-    }
-}
-
-// concatenation of the windows into the blob, the item list and the aux list
-__global__ void compact_kernel(PlanArgs a, const uint64_t *base, uint2 *blob, uint4 *items, uint32_t *aux)
-{
-    const uint32_t w = blockIdx.x;
-    if (w >= a.nw) return;
-    const uint64_t s = a.wstart[w];
-    const uint32_t *c = a.wcount + (uint64_t)kWinFields * w;
-    const uint64_t ib = base[3ull * w], bb = base[3ull * w + 1], ab = base[3ull * w + 2];
-    if (c[4]) {
-        // local record, copied as 8-byte units
-        const uint2 *src = reinterpret_cast<const uint2 *>(a.rec_stage + 10 * s + 8ull * w);
-        for (uint32_t k = threadIdx.x; k < c[5]; k += blockDim.x) blob[bb + k] = src[k];
-        if (threadIdx.x == 0) items[ib] = make_uint4((uint32_t)bb, c[5], kItemLocal, 0u);
-        return;
-    }
-    const uint32_t nops = c[0], nlev = c[1], naux = c[2];
-    if (nops == 0) return;
-    const uint2 *os = a.ops_stage + 3 * s;
-    for (uint32_t k = threadIdx.x; k < nops; k += blockDim.x) {
-        uint2 op = os[k];
-        if ((op.x >> kKindShift) == kPull) op.y = (uint32_t)(op.y - 3 * s + ab);
-        blob[bb + k] = op;
-    }
-    const uint32_t *as = a.aux_stage + 3 * s;
-    for (uint32_t k = threadIdx.x; k < naux; k += blockDim.x) aux[ab + k] = as[k];
-    if (threadIdx.x == 0) {
-        const uint32_t *ls = a.lvl_stage + 2 * s + w;
-        uint64_t it = ib;
-        for (uint32_t l = 0; l < nlev; ++l) {
-            const uint32_t b = ls[l], e = ls[l + 1];
-            for (uint32_t q = b; q < e; q += kTileOps) {
-                const uint32_t qe = min(e, q + kTileOps);
-                items[it++] = make_uint4((uint32_t)(bb + q), qe - q, qe == e ? kItemLevelEnd : 0u, 0u);
+    } else {
+        // packs: as many whole levels as fit, or a part of a level that does not
+        // fit one pack; warp 0 cuts them and writes their headers
+        uint32_t *pq = A.scratch + maxlev + 2;  // first op of every pack, then its first op's unit
+        if (tid < 32) {
+            uint32_t p = 0, l = 0, q = 0, unit = 0;
+            while (q < nops) {
+                uint32_t fit[2], rel[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const uint32_t j = l + 1 + lane + 32 * h;
+                    rel[h] = j <= maxlev ? lh[j] - q : 0xffffffffu;
+                    fit[h] = __popc(__ballot_sync(0xffffffffu, rel[h] <= kPackOps));
+                }
+                const uint32_t k = fit[0] + (fit[0] == 32u ? fit[1] : 0u);
+                const uint32_t last = k ? lh[l + k] - q : kPackOps;
+                uint32_t *hdr = reinterpret_cast<uint32_t *>(a.blob + region + unit);
+                uint16_t *seg = reinterpret_cast<uint16_t *>(hdr + 4);
+                if (lane == 0) {
+                    hdr[0] = last;
+                    hdr[1] = (k ? k : 1u) | (q == 0 ? kPackWindow << 16 : 0u);
+                    hdr[2] = hdr[3] = 0;
+                    pq[2 * p] = q;
+                    pq[2 * p + 1] = unit + kPackHead;
+                    if (!k) seg[0] = (uint16_t)last;
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    if (lane + 32 * h < k) seg[lane + 32 * h] = (uint16_t)rel[h];
+                unit += (kPackHead + last + 1u) & ~1u;
+                q += last;
+                l += k;
+                ++p;
+            }
+            if (lane == 0) {
+                res[0] = p;
+                res[1] = unit;
             }
         }
+        __syncthreads();
+        const uint32_t np = res[0];
+        // PULL lists name rows by node id
+        for (uint32_t r = tid; r < nruns; r += T) {
+            const uint32_t b = A.run_aux[r], c = auxw[b];
+            for (uint32_t q = 1; q <= c; ++q) {
+                const uint32_t ref = auxw[b + q];
+                if (!(ref & kTempRef)) auxw[b + q] = A.rowsg[ref];
+            }
+        }
+        uint2 *ops = a.blob + region;
+        auto place = [&](uint32_t pos) -> uint2 * {  // unit of op `pos`
+            uint32_t lo = 0, hi = np;
+            while (lo + 1 < hi) {
+                const uint32_t mid = (lo + hi) / 2;
+                if (pq[2 * mid] <= pos) lo = mid;
+                else hi = mid;
+            }
+            return ops + pq[2 * lo + 1] + (pos - pq[2 * lo]);
+        };
+        for (uint32_t i0 = 0; i0 < E; i0 += T) {
+            const uint32_t i = i0 + tid;
+            const bool act = has_op(i);
+            const uint32_t pos = level_append(lh, act ? A.evl[i] - 1u : 0u, act);
+            if (!act) continue;
+            const uint32_t f = A.flg[i], x = A.rowsg[A.lu[i]], y = A.rowsg[A.lv[i]];
+            *place(pos) = (f & kFlagIso) ? make_uint2(op_a(kEvent, x), y)
+                          : ((f & kFlagDir) || (f & kFlagShA)) ? make_uint2(op_a(kOneway, y), x)  // y |= x
+                                                               : make_uint2(op_a(kOneway, x), y);
+        }
+        for (uint32_t r = tid; r < nruns; r += T) {
+            const uint32_t L = A.run_lev[r], xg = A.rowsg[A.run_node[r]];
+            *place(atomicAdd(&lh[L], 1u)) = make_uint2(op_a(kPull, xg), (uint32_t)(3 * s) + A.run_aux[r]);
+            if (A.run_temp[r] != (I)~(I)0)
+                *place(atomicAdd(&lh[L - 1], 1u)) = make_uint2(op_a(kCopy, A.run_temp[r]), xg);
+        }
+        // pack sizes: the first kDescPacks in the descriptor, all of them behind
+        // the packs when there are more
+        for (uint32_t p = tid; p < np; p += T) {
+            const uint32_t b = pq[2 * p + 1] - kPackHead, e = p + 1 < np ? pq[2 * p + 3] - kPackHead : res[1];
+            if (p < kDescPacks) desc->pack[p] = e - b;
+            if (np > kDescPacks) reinterpret_cast<uint32_t *>(ops + res[1])[p] = e - b;
+        }
+        if (tid == 0) {
+            desc->off = region;
+            desc->npacks = np;
+            desc->tab = res[1];
+            a.naux_w[w] = naux;
+        }
+    }
+    if (tid == 0) {
+        PlanCounters *c = a.cnt;
+        const uint32_t units = res[1] + (res[0] > kDescPacks ? (res[0] + 1) / 2 : 0u);
+        atomicAdd(&c->blob8, (unsigned long long)((units + 1) & ~1u));
+        atomicAdd(&c->items, (unsigned long long)res[0]);
+        atomicAdd(&c->ops, (unsigned long long)nops);
+        atomicAdd(&c->levels, (unsigned long long)maxlev);
+        if (local) {
+            atomicAdd(&c->local, 1ull);
+        } else {
+            if (naux) atomicAdd(&c->naux, (unsigned long long)naux);
+            if (ntemp) atomicMax(&c->temps, (unsigned long long)ntemp);
+        }
     }
 }
 
-// the batch's time bounds, known on the host, into the plan (no read of t, so
-// the caller may free the events as soon as tn_plan_create returns)
-__global__ void tbounds_kernel(int64_t t_first, int64_t t_last, int64_t *out)
+// First pass: every window that fits the arena of this launch.  What bounds it
+// is latency: the level walk of one warp per window (about 100 cycles per 16
+// events) between phases of scattered shared-memory accesses.  Small windows
+// leave room for several CTAs per SM; 512 threads shorten the parallel phases of
+// large ones.  tn_plan_create on 10^7 activity-driven events (n = 10^5, windows
+// of 640): 0.78 ms; with one thread walking each window event by event (137 us a
+// window) and three host waits 3.4 ms.  20,000 uniform events: 0.09 ms (0.34).
+__global__ void __launch_bounds__(kPlanThreads) schedule_first_kernel(PlanArgs a)
 {
-    out[0] = t_first;
-    out[1] = t_last;
+    extern __shared__ __align__(16) uint8_t smem_arena[];
+    if (a.cnt->error) return;  // refused input: window bounds may not be ordered
+    const uint32_t w = blockIdx.x;
+    if (a.wstart[w + 1] - a.wstart[w] > a.first_max) return;  // second pass
+    schedule_window<uint16_t>(a, w, smem_arena);
 }
 
-// shared-memory budget of the per-window scheduler
+// Second pass: windows stretched by a large timestamp group, in all of shared
+// memory or, above that, in global memory.
+__global__ void __launch_bounds__(kPlanThreads) schedule_late_kernel(PlanArgs a)
+{
+    extern __shared__ __align__(16) uint8_t smem_arena[];
+    const uint32_t w = a.late_list[blockIdx.x];
+    const uint64_t off = a.late_off[blockIdx.x];
+    if (off == kSmemArena) schedule_window<uint16_t>(a, w, smem_arena);
+    else schedule_window<uint32_t>(a, w, a.late_arena + off);
+}
+
+// Copies every window into buffers of the exact size (in no particular order:
+// descriptors name offsets) and moves PULL lists with it.
+__global__ void compact_kernel(PlanArgs a, uint2 *blob, uint32_t *aux)
+{
+    __shared__ unsigned long long base[2];
+    const uint32_t w = blockIdx.x;
+    WinDesc *desc = a.desc + w;
+    const uint32_t np = desc->npacks;
+    if (np == 0) return;
+    const uint64_t src = desc->off;
+    const uint32_t naux = a.naux_w[w];
+    uint32_t units = 0;
+    if (np > kDescPacks) units = desc->tab + (np + 1) / 2;
+    else
+        for (uint32_t p = 0; p < np; ++p) units += desc->pack[p];
+    units = (units + 1) & ~1u;
+    if (threadIdx.x == 0) {
+        base[0] = atomicAdd(&a.cnt->blob_used, (unsigned long long)units);
+        base[1] = naux ? atomicAdd(&a.cnt->aux_used, (unsigned long long)naux) : 0ull;
+    }
+    __syncthreads();  // every thread has read the descriptor
+    const uint64_t dst = base[0];
+    const uint4 *from = reinterpret_cast<const uint4 *>(a.blob + src);
+    uint4 *to = reinterpret_cast<uint4 *>(blob + dst);
+    for (uint32_t k = threadIdx.x; k < units / 2; k += blockDim.x) to[k] = from[k];
+    if (threadIdx.x == 0) desc->off = dst;
+    if (naux == 0) return;
+    const uint64_t s3 = 3 * a.wstart[w];
+    for (uint32_t k = threadIdx.x; k < naux; k += blockDim.x) aux[base[1] + k] = a.aux[s3 + k];
+    __syncthreads();
+    const uint32_t *table = reinterpret_cast<const uint32_t *>(a.blob + src + desc->tab);
+    uint32_t u0 = 0;
+    for (uint32_t p = 0; p < np; ++p) {
+        const uint32_t n8 = np > kDescPacks ? table[p] : desc->pack[p];
+        const uint32_t nops = a.blob[src + u0].x;
+        uint2 *ops = blob + dst + u0 + kPackHead;
+        for (uint32_t k = threadIdx.x; k < nops; k += blockDim.x)
+            if ((ops[k].x >> kKindShift) == kPull) ops[k].y = (uint32_t)(ops[k].y - s3 + base[1]);
+        u0 += n8;
+    }
+}
+
+template <typename F>
+static uint32_t largest_window(uint64_t budget, F bytes)
+{
+    uint32_t E = 64;
+    while (bytes(E + 64) <= budget) E += 64;
+    return E;
+}
+
+// largest window whose arena fits shared memory
 static uint32_t smem_max_events()
 {
     static uint32_t cached = 0;
@@ -882,10 +881,8 @@ static uint32_t smem_max_events()
     int dev = 0, optin = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    uint64_t budget = (uint64_t)optin - 1024;  // static shared memory of the kernel
-    uint32_t E = 64;
-    while (arena_words(E + 64) * 4 <= budget) E += 64;
-    cached = E;
+    // (static shared memory of the kernels: at most 1 KB)
+    cached = largest_window((uint64_t)optin - 1024, [](uint64_t E) { return arena_bytes<uint16_t>(E); });
     return cached;
 }
 
@@ -897,12 +894,28 @@ static cudaError_t alloc_async(T **p, uint64_t count, cudaStream_t st)
     return cudaMallocAsync((void **)p, count * sizeof(T), st);
 }
 
+// device head of a plan: counters, status word, time bounds
+struct PlanHead {
+    PlanCounters cnt;
+    int64_t tbounds[2];
+    int32_t status;
+    int32_t pad;
+};
+
 }  // namespace tn
 
 using namespace tn;
 
+static void free_plan_buffers(tn_plan *p, cudaStream_t st)
+{
+    if (p->d_blob) cudaFreeAsync(p->d_blob, st);
+    if (p->d_win) cudaFreeAsync(p->d_win, st);
+    if (p->d_aux) cudaFreeAsync(p->d_aux, st);
+    if (p->d_head) cudaFreeAsync(p->d_head, st);
+}
+
 // wait_end: return only once the plan's device buffers are written (else they
-// are written by work enqueued on `stream`, which later users must follow)
+// may be written by work enqueued on `stream`, which later users must follow)
 static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const int64_t *t, uint64_t m, uint32_t n,
                                   const int64_t *t_after, const tn_plan_options *opt, void *stream,
                                   tn_plan **plan_out, bool wait_end)
@@ -925,8 +938,7 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     if (window < 32) window = 32;
     if (resident) {
         // the resident-slab form keeps every row in shared memory: no row
-        // buffer, and every window becomes level-ordered tiles of node-id ops
-        // (a one-slot buffer holds no window that has an op)
+        // buffer, and every window becomes level-ordered packs of node-id ops
         if ((resident != 1 && resident != 2) || opt->slab_words || opt->smem_rows || wave)
             return TN_EINVAL;
         if (n > resident_max_rows(resident)) return TN_EINVAL;
@@ -949,9 +961,12 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     a.window = window;
     a.directed = opt ? opt->directed : 0u;
     a.nw = (uint32_t)((m + window - 1) / window);
-    a.smem_max_events = smem_max_events();
+    a.smem_max = smem_max_events();
+    // room for the rest of a small timestamp group behind the target
+    const uint64_t first_max = (uint64_t)window + 64 < m ? (uint64_t)window + 64 : m;
+    a.first_max = first_max < a.smem_max ? (uint32_t)first_max : a.smem_max;
     a.dcap = rows;
-    a.max_rec_words = kStageBytes / 4;
+    a.unit8 = window <= kRecordEvents && rows > 1 ? 5 : 4;
 
     tn_plan *p = (tn_plan *)calloc(1, sizeof(tn_plan));
     if (!p) return TN_ENOMEM;
@@ -965,13 +980,12 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     p->resident = resident;
 
     tn_status rc = TN_OK;
-    unsigned long long host_counters[4] = {0, 0, 0, 0};
-    Totals host_tot;
-    memset(&host_tot, 0, sizeof(host_tot));
-    uint64_t *base = nullptr;
-    Totals *d_tot = nullptr;
-    const int vblocks = (int)((m + 255) / 256 < 4096 ? (m + 255) / 256 : 4096);
-    const int wblocks = (int)((a.nw + 256) / 256);
+    PlanCounters host;
+    memset(&host, 0, sizeof(host));
+    PlanHead *head = nullptr;
+    uint2 *exact_blob = nullptr;
+    uint32_t *exact_aux = nullptr;
+    const uint64_t blocks = (m + 1023) / 1024;
     cudaError_t err = cudaSuccess;
 
 #define TN_STEP(expr)                  \
@@ -980,105 +994,90 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
         if (err != cudaSuccess) goto fail; \
     } while (0)
 
-    TN_STEP(alloc_async(&a.counters, 4, st));
-    TN_STEP(alloc_async(&a.wstart, (uint64_t)a.nw + 1, st));
-    TN_STEP(alloc_async(&a.wcount, (uint64_t)kWinFields * a.nw, st));
-    TN_STEP(alloc_async(&a.big_list, (uint64_t)a.nw, st));
-    TN_STEP(alloc_async(&a.big_off, (uint64_t)a.nw, st));
-    TN_STEP(cudaMemsetAsync(a.counters, 0, 4 * sizeof(unsigned long long), st));
-    tn_internal_count_launches(3);
-    validate_kernel<<<vblocks, 256, 0, st>>>(a);
-    window_kernel<<<wblocks, 256, 0, st>>>(a);
-    big_window_kernel<<<wblocks, 256, 0, st>>>(a);
+    TN_STEP(alloc_async(&head, 1, st));
+    p->d_head = head;
+    p->d_status = &head->status;
+    p->d_tbounds = head->tbounds;
+    a.cnt = &head->cnt;
+    a.tbounds = head->tbounds;
+    TN_STEP(cudaMemsetAsync(head, 0, sizeof(PlanHead), st));
+    // window bounds, second-pass offsets and list, source-list counts: one buffer
+    TN_STEP(alloc_async(&a.wstart, 3ull * a.nw + 2, st));
+    a.late_off = a.wstart + a.nw + 1;
+    a.late_list = reinterpret_cast<uint32_t *>(a.late_off + a.nw);
+    a.naux_w = a.late_list + a.nw;
+    TN_STEP(alloc_async(&p->d_win, a.nw, st));
+    a.desc = p->d_win;
+    TN_STEP(alloc_async(&p->d_blob, blob_base(m, a.nw, a.unit8) + 64, st));
+    a.blob = p->d_blob;
+    TN_STEP(alloc_async(&p->d_aux, 3 * m, st));
+    a.aux = p->d_aux;
+    TN_STEP(tn_internal_allow_max_dyn_smem((const void *)schedule_first_kernel));
+    tn_internal_count_launches(2);
+    inspect_kernel<<<(unsigned)(blocks < 1216 ? blocks : 1216), 256, 0, st>>>(a);
+    schedule_first_kernel<<<a.nw, a.first_max > 1024 ? kPlanThreads : kPlanThreads / 2, arena_bytes<uint16_t>(a.first_max), st>>>(a);
     TN_STEP(cudaGetLastError());
-    TN_STEP(cudaMemcpyAsync(host_counters, a.counters, sizeof(host_counters), cudaMemcpyDeviceToHost, st));
-    // the batch's time bounds travel with the first synchronisation
-    TN_STEP(cudaMemcpyAsync(&p->t_first, t, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    TN_STEP(cudaMemcpyAsync(&p->t_last, t + (m - 1), sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    TN_STEP(cudaMemcpyAsync(&host, a.cnt, sizeof(host), cudaMemcpyDeviceToHost, st));
     TN_STEP(tn_internal_stream_wait(st));
-    if (host_counters[0] & 1ull) {
+    if (host.error & 1ull) {
         rc = TN_ERANGE;
         goto done;
     }
-    if (host_counters[0] & 2ull) {
+    if (host.error & 2ull) {
         rc = TN_EORDER;
         goto done;
     }
-    p->big_windows = host_counters[1];
-
-    TN_STEP(alloc_async(&a.ops_stage, 3 * m, st));
-    TN_STEP(alloc_async(&a.aux_stage, 3 * m, st));
-    TN_STEP(alloc_async(&a.lvl_stage, 2 * m + a.nw + 1, st));
-    TN_STEP(alloc_async(&a.rec_stage, 10 * m + 8ull * a.nw, st));
-    TN_STEP(alloc_async(&a.big_arena, host_counters[2], st));
-    {
-        const size_t smem = arena_words(host_counters[3] ? host_counters[3] : 1) * 4;
-        TN_STEP(tn_internal_allow_max_dyn_smem((const void *)schedule_smem_kernel));
+    if (host.late) {
+        const uint32_t late = (uint32_t)host.late;
+        TN_STEP(alloc_async(&a.late_arena, host.arena, st));
+        TN_STEP(tn_internal_allow_max_dyn_smem((const void *)schedule_late_kernel));
         tn_internal_count_launches(1);
-        schedule_smem_kernel<<<a.nw, kPlanThreads, smem, st>>>(a);
-        if (host_counters[1]) {
-            tn_internal_count_launches(1);
-            schedule_big_kernel<<<(unsigned)host_counters[1], kPlanThreads, 0, st>>>(a);
-        }
+        schedule_late_kernel<<<late, kPlanThreads, arena_bytes<uint16_t>(a.smem_max), st>>>(a);
         TN_STEP(cudaGetLastError());
+        TN_STEP(cudaMemcpyAsync(&host, a.cnt, sizeof(host), cudaMemcpyDeviceToHost, st));
+        TN_STEP(tn_internal_stream_wait(st));
     }
-    TN_STEP(alloc_async(&base, 3ull * a.nw, st));
-    TN_STEP(alloc_async(&d_tot, 1, st));
-    tn_internal_count_launches(1);
-    // 256 threads: the single scan CTA then fits an SM beside a running streaming
-    // CTA (registers), instead of waiting for a free SM
-    window_scan_kernel<<<1, 256, 0, st>>>(a.wcount, a.nw, base, d_tot);
-    TN_STEP(cudaGetLastError());
-    TN_STEP(cudaMemcpyAsync(&host_tot, d_tot, sizeof(Totals), cudaMemcpyDeviceToHost, st));
-    TN_STEP(tn_internal_stream_wait(st));
-
-    p->items = host_tot.items;
-    p->blob8 = host_tot.blob8;
-    p->aux = host_tot.naux;
-    p->temps = host_tot.tmax;
-    p->levels = host_tot.levels;
-    p->ops = host_tot.ops;
-    p->local_windows = host_tot.local;
+    p->t_first = host.t_first;
+    p->t_last = host.t_last;
+    p->items = host.items;
+    p->blob8 = host.blob8;
+    p->aux = host.naux;
+    p->temps = host.temps;
+    p->levels = host.levels;
+    p->ops = host.ops;
+    p->local_windows = host.local;
+    p->big_windows = host.big;
     if (resident && !resident_fits(n, p->temps, resident)) {  // saved rows of the tie groups do not fit
         rc = TN_EINVAL;
         goto done;
     }
-    TN_STEP(alloc_async(&p->d_blob, p->blob8 + 2, st));  // a global tile may read one op past its end
-    TN_STEP(alloc_async(&p->d_items, p->items > 0 ? p->items : 1, st));
-    TN_STEP(alloc_async(&p->d_aux, p->aux > 0 ? p->aux : 1, st));
-    TN_STEP(alloc_async(&p->d_tbounds, 2, st));
-    TN_STEP(alloc_async(&p->d_status, 1, st));
-    TN_STEP(cudaMemsetAsync(p->d_status, 0, sizeof(int32_t), st));
-    tn_internal_count_launches(2);
-    compact_kernel<<<a.nw, 256, 0, st>>>(a, base, p->d_blob, p->d_items, p->d_aux);
-    tbounds_kernel<<<1, 1, 0, st>>>(p->t_first, p->t_last, p->d_tbounds);
-    TN_STEP(cudaGetLastError());
-    // the plan is complete when this call returns, for use on any stream
-    if (wait_end) TN_STEP(tn_internal_stream_wait(st));
+    if (m >= kCompactEvents) {
+        TN_STEP(alloc_async(&exact_blob, p->blob8 + 2, st));
+        TN_STEP(alloc_async(&exact_aux, p->aux > 0 ? p->aux : 1, st));
+        tn_internal_count_launches(1);
+        compact_kernel<<<a.nw, 256, 0, st>>>(a, exact_blob, exact_aux);
+        TN_STEP(cudaGetLastError());
+        cudaFreeAsync(p->d_blob, st);
+        cudaFreeAsync(p->d_aux, st);
+        p->d_blob = exact_blob;
+        p->d_aux = exact_aux;
+        exact_blob = nullptr;
+        exact_aux = nullptr;
+        // the plan is complete when this call returns, for use on any stream
+        if (wait_end) TN_STEP(tn_internal_stream_wait(st));
+    }
     goto done;
 
 fail:
     tn_internal_set_cuda_error(err);
     rc = err == cudaErrorMemoryAllocation ? TN_ENOMEM : TN_ECUDA;
 done:
-    cudaFreeAsync(a.counters, st);
-    cudaFreeAsync(a.wstart, st);
-    cudaFreeAsync(a.wcount, st);
-    cudaFreeAsync(a.big_list, st);
-    cudaFreeAsync(a.big_off, st);
-    if (a.ops_stage) cudaFreeAsync(a.ops_stage, st);
-    if (a.aux_stage) cudaFreeAsync(a.aux_stage, st);
-    if (a.lvl_stage) cudaFreeAsync(a.lvl_stage, st);
-    if (a.rec_stage) cudaFreeAsync(a.rec_stage, st);
-    if (a.big_arena) cudaFreeAsync(a.big_arena, st);
-    if (base) cudaFreeAsync(base, st);
-    if (d_tot) cudaFreeAsync(d_tot, st);
+    if (a.wstart) cudaFreeAsync(a.wstart, st);
+    if (a.late_arena) cudaFreeAsync(a.late_arena, st);
     if (rc != TN_OK) {
-        if (p->d_blob) cudaFreeAsync(p->d_blob, st);
-        if (p->d_items) cudaFreeAsync(p->d_items, st);
-        if (p->d_aux) cudaFreeAsync(p->d_aux, st);
-        if (p->d_tbounds) cudaFreeAsync(p->d_tbounds, st);
-        if (p->d_status) cudaFreeAsync(p->d_status, st);
+        if (exact_blob) cudaFreeAsync(exact_blob, st);
+        if (exact_aux) cudaFreeAsync(exact_aux, st);
+        free_plan_buffers(p, st);
         free(p);
         return rc;
     }
@@ -1104,11 +1103,7 @@ extern "C" tn_status tn_plan_destroy(tn_plan *p, void *stream)
 {
     if (!p) return TN_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
-    cudaFreeAsync(p->d_blob, st);
-    cudaFreeAsync(p->d_items, st);
-    cudaFreeAsync(p->d_aux, st);
-    cudaFreeAsync(p->d_tbounds, st);
-    if (!p->status_shared) cudaFreeAsync(p->d_status, st);
+    free_plan_buffers(p, st);
     free(p);
     return TN_OK;
 }
@@ -1116,9 +1111,8 @@ extern "C" tn_status tn_plan_destroy(tn_plan *p, void *stream)
 tn_status tn::plan_use_status(tn_plan *p, int32_t *status, cudaStream_t st)
 {
     if (!p || !status) return TN_EINVAL;
-    if (!p->status_shared) TN_CUDA_TRY(cudaFreeAsync(p->d_status, st));
+    (void)st;
     p->d_status = status;
-    p->status_shared = 1;
     return TN_OK;
 }
 
