@@ -182,10 +182,14 @@ tn_status tn_out_sizes(const uint64_t *S, uint32_t n_rows, uint32_t ncols,
 typedef struct tn_plan tn_plan;
 
 typedef struct tn_plan_options {
-    uint32_t window_events; /* target events per scheduling window (0 = default 640) */
+    uint32_t window_events; /* target events per scheduling window (0 = chosen by the
+                               library: 640 for networks or row buffers whose windows
+                               are applied in shared memory, else 1,280 or 2,480) */
     uint32_t slab_words;    /* 64-bit words of every row owned by one CTA when the
                                plan is applied: an even number from 2 to 128
-                               (0 = default 16).  Wide slabs (256-1024 byte row
+                               (0 = 16, or, when no window is applied in shared
+                               memory, the narrowest power of two up to 64 that keeps
+                               the launch within one wave of CTAs).  Wide slabs (256-1024 byte row
                                segments) suit large networks whose windows stream
                                from global memory: fewer, longer DRAM bursts */
     uint32_t smem_rows;     /* row slots of the streaming kernel's shared-memory row

@@ -56,6 +56,14 @@ struct Job {
     uint32_t nwin;  // windows of the schedule
     uint32_t cta_begin;
     uint32_t dcap;  // row slots of the shared-memory row buffer
+    uint32_t track;       // TrackMode of a column slab
+    uint32_t *ids;        // content ids of the rows, then of the saved rows
+    uint32_t pitch;       // ids per row, one per CTA
+    uint32_t mark_words;  // 32-bit words of the marks (0: every op is executed)
+    uint32_t mark_shift;  // 2^mark_shift rows per mark
+    uint32_t mark_init;   // S starts as the identity (1) or the source columns (2); 0: unknown content
+    const uint32_t *src;
+    uint32_t ncols;
     // resident-slab form (rw > 0): each CTA keeps rw words of every row in shared memory
     uint32_t rw;     // words of every row per CTA (1, 2 or 4), 0 = column-slab form
     uint32_t rows;   // rows of the matrix (node count of the plan)
@@ -151,8 +159,13 @@ __device__ void produce_packs(const Job &J, const PackRing &ring, volatile uint3
 struct Lane {
     uint32_t chunk, lane0, stride, cpr;
     uint64_t col;  // first word of this thread's chunk
+    uint8_t *base; // this thread's chunk of row 0
+    uint32_t pitch;  // bytes per row (below 2^28: one multiply-add per row address)
+    const uint32_t *pack;  // the pack being applied (source lists)
     bool active;   // chunk inside the matrix and thread inside the row groups
 };
+
+constexpr uint32_t kRowBufferMax = 192 * 1024;
 
 // consumer threads of this launch (all warps but the producer)
 __device__ inline uint32_t consumers() { return blockDim.x - 32u; }
@@ -165,8 +178,21 @@ __device__ inline Lane make_lane(const Job &J, uint32_t ct, uint64_t w0)
     L.lane0 = ct / L.cpr;
     L.stride = consumers() / L.cpr;
     L.col = w0 + 2ull * L.chunk;
+    L.base = reinterpret_cast<uint8_t *>(J.S + L.col);
+    L.pitch = (uint32_t)(8 * J.ld);
     L.active = L.lane0 < L.stride && L.col < J.ld;
     return L;
+}
+
+__device__ inline uint64_t *row_of(const Lane &L, uint32_t row)
+{
+    return reinterpret_cast<uint64_t *>(L.base + (uint64_t)row * L.pitch);
+}
+
+// Source list of a PULL: its count, then its references.
+__device__ inline const uint32_t *source_list(const uint32_t *aux, const uint32_t *pack, uint32_t b)
+{
+    return b < kOutsideList ? pack + b : aux + (b - kOutsideList);
 }
 
 __device__ inline uint64_t *row_ptr(const Job &J, uint32_t ref, uint64_t col)
@@ -213,12 +239,24 @@ __device__ inline void cp_async16(void *smem_dst, const void *gmem_src)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(smem_dst)), "l"(gmem_src) : "memory");
 }
 
+__device__ inline void cp_async16(uint32_t smem_dst, const void *gmem_src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_dst), "l"(gmem_src) : "memory");
+}
+
 __device__ inline void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 __device__ inline u64x2 lds16(const u64x2 *p)
 {
     u64x2 r;
     asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(r.x), "=l"(r.y) : "r"(smem_addr(p)) : "memory");
+    return r;
+}
+
+__device__ inline u64x2 lds16(uint32_t a)
+{
+    u64x2 r;
+    asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(r.x), "=l"(r.y) : "r"(a) : "memory");
     return r;
 }
 
@@ -232,15 +270,17 @@ __device__ inline void sts16(u64x2 *p, u64x2 v)
 // ---------------------------------------------------------------------------
 // PULL: S[x] |= OR of the listed source rows (aux[b] = count, then refs)
 template <bool kMax>
-__device__ inline void apply_pull(const Job &J, uint32_t x, uint32_t b, uint64_t col)
+__device__ inline void apply_pull(const Job &J, uint32_t x, uint32_t b, const Lane &L)
 {
+    const uint64_t col = L.col;
     uint64_t *pd = J.S + (uint64_t)x * J.ld + col;
     u64x2 acc = ld_row16(pd);
-    const uint32_t c = __ldg(J.aux + b);
+    const uint32_t *list = source_list(J.aux, L.pack, b);
+    const uint32_t c = list[0];
     for (uint32_t i = 0; i < c; i += 8) {
         uint32_t ref[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) ref[k] = (i + k < c) ? __ldg(J.aux + b + 1 + i + k) : kNoRef;
+        for (int k = 0; k < 8; ++k) ref[k] = (i + k < c) ? list[1 + i + k] : kNoRef;
         u64x2 r[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k)
@@ -293,7 +333,7 @@ __device__ inline void apply_tile_direct(const Job &J, const uint2 *ops, uint32_
     // multi-source updates of tie groups (hub rows) in a second pass
     for (uint32_t o = L.lane0; o < count; o += stride) {
         const uint2 op = ops[o];
-        if ((op.x >> kKindShift) == kPull) apply_pull<kMax>(J, op.x & kIdMask, op.y, col);
+        if ((op.x >> kKindShift) == kPull) apply_pull<kMax>(J, op.x & kIdMask, op.y, L);
     }
 }
 
@@ -332,13 +372,14 @@ struct PullCursor {
 };
 
 __device__ inline void pull_cursor_seek(PullCursor &cur, const Job &J, const uint2 *ops, uint32_t count,
-                                        uint32_t stride)
+                                        const Lane &L)
 {
+    const uint32_t stride = L.stride;
     while (cur.o < count && cur.q >= cur.c) {
         cur.o += stride;
         while (cur.o < count && (ops[cur.o].x >> kKindShift) != kPull) cur.o += stride;
         cur.q = 0;
-        cur.c = cur.o < count ? __ldg(J.aux + ops[cur.o].y) : 0u;
+        cur.c = cur.o < count ? source_list(J.aux, L.pack, ops[cur.o].y)[0] : 0u;
     }
 }
 
@@ -349,18 +390,18 @@ __device__ inline void apply_pulls_ring(const Job &J, const uint2 *ops, uint32_t
     PullCursor in{L.lane0, 0u, 0u};
     while (in.o < count && (ops[in.o].x >> kKindShift) != kPull) in.o += stride;
     if (in.o >= count) return;
-    in.c = __ldg(J.aux + ops[in.o].y);
-    pull_cursor_seek(in, J, ops, count, stride);
+    in.c = source_list(J.aux, L.pack, ops[in.o].y)[0];
+    pull_cursor_seek(in, J, ops, count, L);
     PullCursor out = in;
     uint32_t issued = 0, done = 0;
     auto issue = [&]() {
         if (in.o >= count) return;
-        const uint32_t ref = __ldg(J.aux + ops[in.o].y + 1 + in.q);
+        const uint32_t ref = source_list(J.aux, L.pack, ops[in.o].y)[1 + in.q];
         const uint32_t q = L.lane0 + (issued % kRing) * stride;
         cp_async16(mine + (2 * q) * cpr, row_ptr(J, ref, col));
         ++issued;
         ++in.q;
-        pull_cursor_seek(in, J, ops, count, stride);
+        pull_cursor_seek(in, J, ops, count, L);
     };
 #pragma unroll 1
     for (uint32_t k = 0; k < kRing - 1; ++k) {
@@ -376,7 +417,7 @@ __device__ inline void apply_pulls_ring(const Job &J, const uint2 *ops, uint32_t
         red_or16(J.S + (uint64_t)(ops[out.o].x & kIdMask) * J.ld + col, lds16(mine + (2 * q) * cpr));
         ++done;
         ++out.q;
-        pull_cursor_seek(out, J, ops, count, stride);
+        pull_cursor_seek(out, J, ops, count, L);
     }
     cp_async_wait_group<0>();
 }
@@ -433,11 +474,599 @@ __device__ inline void apply_tile(const Job &J, const uint2 *ops, uint32_t count
     if (kMax) {
         for (uint32_t o = L.lane0; o < count; o += stride) {
             const uint2 op = ops[o];
-            if ((op.x >> kKindShift) == kPull) apply_pull<kMax>(J, op.x & kIdMask, op.y, col);
+            if ((op.x >> kKindShift) == kPull) apply_pull<kMax>(J, op.x & kIdMask, op.y, L);
         }
     } else {
         apply_pulls_ring(J, ops, count, mine, L);
     }
+}
+
+// ---------------------------------------------------------------------------
+// tracked rows: updates that cannot change anything are not made
+//
+// Early in a stream most row segments of a slab are still zero; later most
+// events meet rows that already hold the same content.  A CTA keeps what it
+// needs to know about its rows, skips the ops that this shows to change nothing
+// without touching the matrix, and stores only chunks that change.  Every
+// skipped update is one that would write what is there; nothing is carried over
+// between applications.  Two forms:
+//
+// Marks (slabs of up to 16 words): one reference content C (16 bytes per thread)
+// and one bit per row in shared memory, "this row's segment equals C".  An op is
+// skipped when all its rows are marked; marked rows are not loaded; a row is
+// marked when its result equals C.  C starts as zero (all rows but the sources'
+// marked, when the application initialises S).  When most ops are executed all
+// the same, the marks are dropped; when at least half of the executed updates
+// find both rows equal, the largest such content becomes the new C.  When a bit
+// per row does not fit, a bit stands for 2^shift consecutive rows, for C = zero
+// only (rows never return to zero).
+//
+// Ids (wider slabs): a content id per row in global memory; rows with equal ids
+// hold equal segments (the reverse need not be known).  An op is skipped when
+// its rows' ids are equal.  A row that took over the other's content takes its
+// id, rows found equal take the smaller id, new content gets an id no row has had
+// (one per op).  Id 0 is the zero segment, which is never loaded.
+// ids[row][cta]: the CTAs of a matrix run the same ops at about the same time, so
+// the eight ids of a sector are read from DRAM once.
+//
+// Ids find nearly every update that changes nothing, but each level waits for
+// them (an L2 access under load, about 2 us); marks cost two shared-memory reads
+// and find what is zero or in the main component's final state.  Executed share
+// (simulated, n = 10^5, 50 events per node, 64 words): bursty 0.24 by ids, 0.53
+// by marks; activity-driven 0.19 and 0.20.  Measured, stream kernel: bursty n =
+// 5 10^5, m = 2.5 10^7, 64 words 543 ms by ids, 1,037 by marks, 765 with every op
+// executed (1,085 with every chunk stored as well); activity-driven n = 10^5, m =
+// 10^7, 16 words 38.5, 25.0, 90.2 and 119 ms.
+// ---------------------------------------------------------------------------
+constexpr uint32_t kMarkWords = 16;  // widest slab whose rows are marked
+constexpr uint32_t kMarkShift = 2;   // at most 4 rows per bit
+
+extern __shared__ __align__(128) uint8_t dyn_smem[];  // dynamic shared memory of the streaming kernel
+
+// Shared memory behind the row buffer (byte offset `at`): listed ops of all
+// warps (12 x 192 or 4 x 576): uint4 {op.x, row b, a, b}, a and b = 0 for rows
+// whose content is known (C, or zero), else their ids or 1 | their indices |
+// statistics [3][4] (marks: per window, ops, executed, sampled updates, of these
+// equal rows; ids: executed flags of three packs) | key of the largest candidate: size << 10 | row
+// group | (marks) candidates, 16 bytes per consumer | mark bits of the rows, then
+// of the saved rows.
+constexpr uint32_t kListOps = 2304;
+constexpr uint32_t kIdBytes = 18 * kListOps + 64;
+constexpr uint32_t kMarkBytes = kIdBytes + 16 * 32 * kWarpsAlone;
+
+enum TrackMode : int { kNoTrack = 0, kMarks = 1, kIds = 2 };
+
+struct Track {
+    uint32_t at;
+    uint32_t slot;    // this warp's first list entry
+    uint32_t rows;    // first saved row
+    // ids
+    uint32_t *ids;    // this CTA's id of row 0
+    uint32_t pitch;   // ids per row
+    uint32_t fresh;   // the id that op 0 of the current segment may take
+    // marks
+    uint32_t shift;   // 2^shift rows per bit
+    u64x2 c;          // this thread's chunk of C (ids: zero)
+    uint32_t c_size;  // size of C
+    bool on;          // marks are valid
+    bool want;        // this window looks for a candidate
+    bool quiet;       // the last window executed nothing
+    uint32_t best_size;               // of this row group's candidate
+    bool sample;      // this window counts equal rows (every fourth, and those that look for a candidate)
+    uint32_t n_ops, n_live;    // of this window, this warp
+    uint32_t n_seen, n_equal;  // sampled updates, of equal rows, this thread
+    __device__ uint4 *list() const { return reinterpret_cast<uint4 *>(dyn_smem + at) + slot; }
+    __device__ uint16_t *index() const { return reinterpret_cast<uint16_t *>(dyn_smem + at + 16 * kListOps) + slot; }
+    __device__ uint32_t *stat(uint32_t q) const { return reinterpret_cast<uint32_t *>(dyn_smem + at + 18 * kListOps) + 4 * (q % 3u); }
+    __device__ uint32_t *key() const { return reinterpret_cast<uint32_t *>(dyn_smem + at + 18 * kListOps) + 12; }
+    __device__ u64x2 *cand(uint32_t i) const { return reinterpret_cast<u64x2 *>(dyn_smem + at + kIdBytes) + i; }
+    __device__ uint32_t *bits() const { return reinterpret_cast<uint32_t *>(dyn_smem + at + kMarkBytes); }
+    __device__ uint32_t *id_ptr(uint32_t ref) const
+    {
+        return ids + (uint64_t)((ref & kTempRef) ? rows + (ref & ~kTempRef) : ref) * pitch;
+    }
+    __device__ uint32_t id(uint32_t ref) const
+    {
+        uint32_t x;
+        asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(x) : "l"(id_ptr(ref)) : "memory");
+        return x;
+    }
+    // saved rows have a bit each, behind the rows' bits
+    __device__ uint32_t bit_of(uint32_t ref) const
+    {
+        return (ref & kTempRef) ? (rows >> shift) + 1u + (ref & ~kTempRef) : ref >> shift;
+    }
+    __device__ bool marked(uint32_t ref) const
+    {
+        const uint32_t i = bit_of(ref);
+        return (bits()[i >> 5] >> (i & 31u)) & 1u;
+    }
+    __device__ void mark(uint32_t ref) const
+    {
+        const uint32_t i = bit_of(ref);
+        if (shift == 0 || (ref & kTempRef)) atomicOr(bits() + (i >> 5), 1u << (i & 31u));
+    }
+    __device__ void unmark(uint32_t ref) const
+    {
+        const uint32_t i = bit_of(ref);
+        atomicAnd(bits() + (i >> 5), ~(1u << (i & 31u)));
+    }
+};
+
+__device__ inline bool same16(u64x2 a, u64x2 b) { return a.x == b.x && a.y == b.y; }
+
+// Ids: whether an op is to be executed; `e` becomes its list entry.  A PULL whose
+// sources that differ from its row all share one id is the ONEWAY update from
+// any of them.
+__device__ inline bool id_live(const Job &J, const Track &T, uint2 op, const uint32_t *pack, uint4 &e)
+{
+    const uint32_t kind = op.x >> kKindShift, a = op.x & kIdMask;
+    if (kind == kCopy) {
+        e = make_uint4(op.x, op.y, 0u, T.id(op.y));
+        return true;
+    }
+    if (kind != kPull) {
+        const uint32_t ia = T.id(a), ib = T.id(op.y);
+        e = make_uint4(op.x, op.y, ia, ib);
+        return ia != ib && !(kind == kOneway && ib == 0);
+    }
+    const uint32_t ia = T.id(a);
+    const uint32_t *list = source_list(J.aux, pack, op.y);
+    const uint32_t c = list[0];
+    uint32_t found = 0, from = 0, fid = 0;
+    for (uint32_t i = 0; i < c && found < 2; i += 8) {  // eight independent loads at a time
+        uint32_t ref[8], sid[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) ref[k] = list[1 + (i + k < c ? i + k : i)];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) sid[k] = T.id(ref[k]);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (sid[k] == ia || sid[k] == 0 || (found && sid[k] == fid)) continue;
+            ++found;
+            from = ref[k];
+            fid = sid[k];
+        }
+    }
+    if (found == 0) return false;
+    e = found == 1 ? make_uint4(op_a(kOneway, a), from, ia, fid) : make_uint4(op.x, op.y, ia, 0u);
+    return true;
+}
+
+// Marks: likewise.  A COPY of a marked row marks the saved row instead.
+__device__ inline bool mark_live(const Job &J, const Track &T, uint2 op, const uint32_t *pack, uint4 &e)
+{
+    const uint32_t kind = op.x >> kKindShift, a = op.x & kIdMask;
+    e = make_uint4(op.x, op.y, 1u, 1u);
+    if (kind == kCopy) {
+        if (T.marked(op.y)) {
+            T.mark(kTempRef | a);
+            return false;
+        }
+        if (T.marked(kTempRef | a)) T.unmark(kTempRef | a);
+        return true;
+    }
+    const bool ma = T.marked(a);
+    e.z = !ma;
+    if (kind != kPull) {
+        const bool mb = T.marked(op.y);
+        e.w = !mb;
+        return !(ma && mb);
+    }
+    if (!ma) return true;
+    const uint32_t *list = source_list(J.aux, pack, op.y);
+    const uint32_t c = list[0];
+    bool live = false;
+    for (uint32_t i = 0; i < c && !live; i += 8) {  // eight independent loads at a time
+        uint32_t ref[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) ref[k] = list[1 + (i + k < c ? i + k : i)];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) live |= !T.marked(ref[k]);
+    }
+    return live;
+}
+
+// Size of a row group's content (cpr lanes, one chunk each): bits, or the sum of
+// the registers of a sketch; below 2^22.
+template <bool kMax>
+__device__ inline uint32_t content_size(u64x2 r, uint32_t cpr, uint32_t group_mask)
+{
+    uint32_t n;
+    if (kMax) {
+        n = __vsadu4((uint32_t)r.x, 0u) + __vsadu4((uint32_t)(r.x >> 32), 0u) + __vsadu4((uint32_t)r.y, 0u) +
+            __vsadu4((uint32_t)(r.y >> 32), 0u);
+    } else {
+        n = __popcll(r.x) + __popcll(r.y);
+    }
+    for (uint32_t d = 1; d < cpr; d <<= 1) n += __shfl_xor_sync(group_mask, n, d);
+    return n;
+}
+
+// What one executed EVENT, ONEWAY or COPY (entry e, rows' chunks ra, rb) writes:
+// the chunks that change, and what the CTA knows about its rows.  `i` is its list
+// position.  All lanes of the warp call it (lanes without an op with a PULL entry).
+template <bool kMax, int kMode>
+__device__ inline void track_update(const Job &J, Track &T, const Lane &L, uint32_t group_mask, uint4 e, u64x2 ra,
+                                    u64x2 rb, uint32_t i)
+{
+    const bool active = L.active;
+    const uint32_t kind = e.x >> kKindShift, a = e.x & kIdMask, ref = e.y;
+    const bool update = kind == kEvent || kind == kOneway;
+    const u64x2 r = combine16<kMax>(ra, rb);
+    const bool new_a = active && update && !same16(r, ra), new_b = active && update && !same16(r, rb);
+    if (new_a) st_row16(row_of(L, a), r);
+    if (new_b && kind == kEvent) st_row16(row_of(L, ref), r);
+    if (kind == kCopy && active) st_row16(J.tmp + (uint64_t)a * J.ld + L.col, rb);
+    if (kMode == kIds) {
+        const bool any_a = (__ballot_sync(0xffffffffu, new_a) & group_mask) != 0;
+        const bool any_b = (__ballot_sync(0xffffffffu, new_b) & group_mask) != 0;
+        if (L.chunk == 0) {
+            const uint32_t ia = e.z, ib = e.w;
+            if (update) {
+                const uint32_t fresh = T.fresh + T.index()[i];
+                const uint32_t id = any_a && any_b ? fresh : any_a ? ib : any_b ? ia : min(ia, ib);
+                if (id != ia) *T.id_ptr(a) = id;
+                if (kind == kEvent && id != ib) *T.id_ptr(ref) = id;
+            } else if (kind == kCopy) {
+                *T.id_ptr(kTempRef | a) = ib;
+            }
+        }
+        return;
+    }
+    if (kMode == kMarks) {
+        const uint32_t other = __ballot_sync(0xffffffffu, active && !same16(r, T.c));
+        if (update && L.chunk == 0) {
+            const bool all = !(other & group_mask);
+            if (all != (e.z == 0)) {
+                if (all) T.mark(a);
+                else T.unmark(a);
+            }
+            if (kind == kEvent && all != (e.w == 0)) {
+                if (all) T.mark(ref);
+                else T.unmark(ref);
+            }
+        }
+    }
+    if (!T.sample) return;
+    const uint32_t differ = __ballot_sync(0xffffffffu, new_a || new_b);
+    const bool equal = update && !(differ & group_mask);
+    T.n_seen += update;
+    T.n_equal += equal;
+    if (T.want && equal) {
+        const uint32_t size = content_size<kMax>(active ? r : u64x2{0, 0}, L.cpr, group_mask);
+        if (size > T.best_size) {
+            T.best_size = size;
+            *T.cand(L.lane0 * L.cpr + L.chunk) = r;
+        }
+    }
+}
+
+// Entry of this row group's k-th op: this warp's list, or, with kNoTrack, the ops
+// first, first + step, ... themselves; a PULL of no row past the end.
+template <int kMode>
+__device__ inline uint4 track_entry(const Track &T, const uint2 *ops, uint32_t cnt, uint32_t i)
+{
+    if (i >= cnt) return make_uint4(op_a(kPull, kIdMask), 0u, 0u, 0u);
+    if (kMode != kNoTrack) return T.list()[i];
+    const uint2 op = ops[i];
+    return make_uint4(op.x, op.y, 1u, 1u);
+}
+
+template <int kMode>
+__device__ inline uint64_t *track_row_b(const Job &J, const Lane &L, uint32_t ref)
+{
+    if (kMode == kIds) return row_ptr(J, ref, L.col);  // (a PULL run as ONEWAY may read a saved row)
+    return row_of(L, ref);
+}
+
+// Up to two ops per row group, one after the other, loaded straight into
+// registers, a PULL's sources (the first eight) together with its row: one memory
+// latency instead of a copy ring's start and drain.  Levels of tie-heavy streams
+// are that short (hubs chain every timestamp group to the one before).
+template <bool kMax, int kMode>
+__device__ void track_short(const Job &J, Track &T, const uint2 *ops, uint32_t cnt, uint32_t first, uint32_t step,
+                            uint32_t rounds, const Lane &L, uint32_t group_mask)
+{
+    const u64x2 zero{0, 0}, known = kMode == kMarks ? T.c : zero;
+    const bool active = L.active;
+#pragma unroll 1
+    for (uint32_t k = 0; k < rounds; ++k) {
+        const uint32_t i = first + k * step;
+        const uint4 e = track_entry<kMode>(T, ops, cnt, i);
+        const uint32_t kind = e.x >> kKindShift, a = e.x & kIdMask;
+        const bool pull = kind == kPull && a != kIdMask;
+        u64x2 ra = known, rb = known, acc = zero, r[8];
+        if (active && kind != kPull) {
+            if (e.z != 0 && kind != kCopy) ra = ld_row16(row_of(L, a));
+            if (e.w != 0) rb = ld_row16(track_row_b<kMode>(J, L, e.y));
+        }
+        if (pull) {
+            const uint32_t *list = source_list(J.aux, L.pack, e.y);
+            const uint32_t c = list[0];
+            if (active && e.z != 0) ra = ld_row16(row_of(L, a));
+            for (uint32_t q = 0; q < c; q += 8) {
+#pragma unroll
+                for (int h = 0; h < 8; ++h) {
+                    r[h] = zero;
+                    if (q + h >= c) continue;
+                    const uint32_t ref = list[1 + q + h];
+                    if (kMode == kMarks && T.marked(ref)) r[h] = known;
+                    else if (active) r[h] = ld_row16(row_ptr(J, ref, L.col));
+                }
+#pragma unroll
+                for (int h = 0; h < 8; ++h) acc = combine16<kMax>(acc, r[h]);
+            }
+        }
+        track_update<kMax, kMode>(J, T, L, group_mask, e, ra, rb, i);
+        if (!__any_sync(0xffffffffu, pull)) continue;
+        acc = combine16<kMax>(acc, ra);
+        const bool new_a = active && pull && !same16(acc, ra);
+        if (new_a) st_row16(row_of(L, a), acc);
+        if (kMode == kMarks) {
+            const uint32_t other = __ballot_sync(0xffffffffu, active && !same16(acc, T.c));
+            const bool all = !(other & group_mask);
+            if (pull && L.chunk == 0 && all != (e.z == 0)) {
+                if (all) T.mark(a);
+                else T.unmark(a);
+            }
+        } else if (kMode == kIds) {
+            const bool any = (__ballot_sync(0xffffffffu, new_a) & group_mask) != 0;
+            if (any && L.chunk == 0) *T.id_ptr(a) = T.fresh + T.index()[i];
+        }
+    }
+}
+
+// The ops of a segment through the private copy ring of every row group (kRing op
+// slots of two chunks, as apply_tile).  Steps of two ops, the copies of the step
+// kRing / 2 - 1 places ahead issued before the current step's rows are read back;
+// ops are fetched a step before they are needed, so that no copy waits for a
+// shared-memory load.  (One op per step, fetched where it is used, every op
+// executed: 126 ms instead of 90 ms for 10^7 activity-driven events at n = 10^5.)
+template <bool kMax, int kMode>
+__device__ bool track_ring(const Job &J, Track &T, const uint2 *ops, uint32_t cnt, uint32_t first, uint32_t step,
+                           uint32_t rounds, u64x2 *buf, const Lane &L, uint32_t group_mask)
+{
+    const uint32_t cpr = L.cpr;
+    const bool active = L.active;
+    // slot i of this thread: two chunks; cpr * stride = the consumer threads
+    const uint32_t slot0 = smem_addr(buf + L.chunk + 2 * L.lane0 * cpr), slot_step = 32 * consumers(), second = 16 * cpr;
+    bool pulls = false;
+    auto entry = [&](uint32_t k) -> uint4 { return track_entry<kMode>(T, ops, cnt, first + k * step); };
+    uint4 in[2], out[2];  // entries of the next copies and of the next updates
+    auto issue = [&](uint32_t k) {
+#pragma unroll
+        for (uint32_t h = 0; h < 2; ++h) {
+            const uint32_t slot = slot0 + ((k + h) % kRing) * slot_step, kind = in[h].x >> kKindShift;
+            if (active && kind != kPull) {
+                if (in[h].z != 0 && kind != kCopy)
+                    cp_async16(slot, row_of(L, in[h].x & kIdMask));
+                if (in[h].w != 0) cp_async16(slot + second, track_row_b<kMode>(J, L, in[h].y));
+            }
+            in[h] = entry(k + 2 + h);
+        }
+        cp_async_commit();
+    };
+#pragma unroll
+    for (uint32_t h = 0; h < 2; ++h) out[h] = in[h] = entry(h);
+#pragma unroll 1
+    for (uint32_t k = 0; k < kRing - 2; k += 2) issue(k);
+#pragma unroll 1
+    for (uint32_t k = 0; k < rounds; k += 2) {
+        issue(k + kRing - 2);
+        cp_async_wait_group<kRing / 2 - 1>();  // this step's copies have landed
+        u64x2 ra[2], rb[2];
+        const u64x2 known = kMode == kMarks ? T.c : u64x2{0, 0};
+#pragma unroll
+        for (uint32_t h = 0; h < 2; ++h) {
+            const uint32_t slot = slot0 + ((k + h) % kRing) * slot_step;
+            ra[h] = kMode == kNoTrack || out[h].z != 0 ? lds16(slot) : known;
+            rb[h] = kMode == kNoTrack || out[h].w != 0 ? lds16(slot + second) : known;
+        }
+#pragma unroll
+        for (uint32_t h = 0; h < 2; ++h) {
+            track_update<kMax, kMode>(J, T, L, group_mask, out[h], ra[h], rb[h], first + (k + h) * step);
+            pulls |= (out[h].x >> kKindShift) == kPull && (out[h].x & kIdMask) != kIdMask;
+            out[h] = entry(k + 2 + h);
+        }
+    }
+    cp_async_wait_group<0>();
+    return pulls;
+}
+
+// Listed PULLs, x |= every source.  Marks: marked sources stand for C and are not
+// loaded.  Ids: at least two sources differ from x; the result is new content.
+template <bool kMax, int kMode>
+__device__ void track_pulls(const Job &J, Track &T, uint32_t cnt, const Lane &L, uint32_t group_mask)
+{
+    const uint32_t per = 32u / L.cpr, g = (threadIdx.x & 31u) / L.cpr;
+    const u64x2 zero{0, 0};
+    for (uint32_t i = g; i < cnt; i += per) {
+        const uint4 e = T.list()[i];
+        if ((e.x >> kKindShift) != kPull) continue;
+        const uint32_t *list = source_list(J.aux, L.pack, e.y);
+        const uint32_t x = e.x & kIdMask, c = list[0];
+        uint64_t *px = J.S + (uint64_t)x * J.ld + L.col;
+        u64x2 old = zero, acc = zero;
+        if (kMode == kMarks) old = e.z == 0 ? T.c : L.active ? ld_row16(px) : zero;
+        for (uint32_t q = 0; q < c; q += 8) {
+            uint32_t ref[8];
+            u64x2 r[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) ref[k] = list[1 + (q + k < c ? q + k : q)];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                if (kMode == kMarks && T.marked(ref[k])) r[k] = T.c;
+                else r[k] = L.active ? ld_row16(row_ptr(J, ref[k], L.col)) : zero;
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) acc = combine16<kMax>(acc, r[k]);
+        }
+        if (kMode == kMarks) {
+            acc = combine16<kMax>(acc, old);
+            if (L.active && !same16(acc, old)) st_row16(px, acc);
+            const bool all = __all_sync(group_mask, !L.active || same16(acc, T.c));
+            if (L.chunk == 0 && all != (e.z == 0)) {
+                if (all) T.mark(x);
+                else T.unmark(x);
+            }
+        } else {
+            if (L.active) {
+                if (kMax) st_row16(px, combine16<kMax>(ld_row16(px), acc));
+                else red_or16(px, acc);
+            }
+            if (L.chunk == 0) *T.id_ptr(x) = T.fresh + T.index()[i];
+        }
+    }
+}
+
+// One segment with marks or ids (cpr a power of two up to 32: a row group is part
+// of a warp): every warp lists the ops of its share that are to be executed,
+// then its row groups run them.  Whether there were any.
+template <bool kMax, int kMode>
+__device__ bool track_tile(const Job &J, Track &T, const uint2 *ops, uint32_t count, u64x2 *buf, const Lane &L,
+                           uint32_t group_mask)
+{
+    const uint32_t lane = threadIdx.x & 31u, warp = (threadIdx.x >> 5) - 1u, warps = consumers() >> 5, per = 32u / L.cpr;
+    uint32_t cnt = 0;
+    // op i belongs to warp i mod warps: short levels spread over all warps
+    for (uint32_t b = 0; b + warp < count; b += warps * 32u) {
+        const uint32_t i = b + lane * warps + warp;
+        uint4 e;
+        const bool live = i < count && (kMode == kIds ? id_live(J, T, ops[i], L.pack, e) : mark_live(J, T, ops[i], L.pack, e));
+        const uint32_t m = __ballot_sync(0xffffffffu, live);
+        if (live) {
+            const uint32_t to = cnt + __popc(m & ((1u << lane) - 1u));
+            T.list()[to] = e;
+            if (kMode == kIds) T.index()[to] = (uint16_t)i;
+        }
+        cnt += __popc(m);
+    }
+    __syncwarp();
+    if (kMode == kMarks) {
+        T.n_ops += (count - min(count, warp) + warps - 1) / warps;
+        T.n_live += cnt;
+    }
+    if (cnt == 0) return false;
+    const uint32_t rounds = (cnt + per - 1) / per;
+    if (rounds <= 2)
+        track_short<kMax, kMode>(J, T, ops, cnt, lane / L.cpr, per, rounds, L, group_mask);
+    else if (__any_sync(0xffffffffu, track_ring<kMax, kMode>(J, T, ops, cnt, lane / L.cpr, per, rounds, buf, L, group_mask)))
+        track_pulls<kMax, kMode>(J, T, cnt, L, group_mask);
+    return true;
+}
+
+// One segment with every op executed.
+template <bool kMax>
+__device__ void whole_tile(const Job &J, Track &T, const uint2 *ops, uint32_t count, u64x2 *buf, const Lane &L,
+                           uint32_t group_mask)
+{
+    const uint32_t before = ((threadIdx.x >> 5) - 1u) * (32u / L.cpr);  // row groups of the warps before this one
+    if (count <= before) return;
+    const uint32_t rounds = (count - before + L.stride - 1) / L.stride;
+    if (rounds <= 2) {
+        track_short<kMax, kNoTrack>(J, T, ops, count, L.lane0, L.stride, rounds, L, group_mask);
+        return;
+    }
+    const bool pulls = track_ring<kMax, kNoTrack>(J, T, ops, count, L.lane0, L.stride, rounds, buf, L, group_mask);
+    if (!pulls || !L.active) return;
+    // multi-source updates of tie groups (hub rows) in a second pass
+    if (kMax) {
+        for (uint32_t o = L.lane0; o < count; o += L.stride) {
+            const uint2 op = ops[o];
+            if ((op.x >> kKindShift) == kPull) apply_pull<kMax>(J, op.x & kIdMask, op.y, L);
+        }
+    } else {
+        apply_pulls_ring(J, ops, count, buf + L.chunk, L);
+    }
+}
+
+// Marks of a freshly initialised S: every row whose segment is zero.
+__device__ void mark_init(const Job &J, Track &T, uint64_t w0, uint32_t ct)
+{
+    const uint32_t nbits = (T.rows >> T.shift) + 1u, full = nbits / 32u;
+    for (uint32_t i = ct; i < J.mark_words; i += consumers())
+        T.bits()[i] = J.mark_init == 0 || i > full ? 0u : i < full ? 0xffffffffu : (1u << (nbits & 31u)) - 1u;
+    if (ct < 13) T.stat(0)[ct] = 0;  // and the key
+    consumers_sync();
+    if (J.mark_init == 0 || J.mark_words == 0) return;
+    const uint64_t c0 = 64 * w0, c1 = 64 * (w0 + J.sw) < J.ncols ? 64 * (w0 + J.sw) : J.ncols;
+    for (uint64_t c = c0 + ct; c < c1; c += consumers()) {
+        const uint32_t x = J.mark_init == 1 ? (uint32_t)c : __ldg(J.src + c);
+        if (x < T.rows) T.unmark(x);
+    }
+    consumers_sync();
+}
+
+// Marks, end of a window (before the next one's first barrier): statistics.
+// Every lane of a row group has counted its sampled updates.
+__device__ inline void mark_count(Track &T, uint32_t win)
+{
+    uint32_t seen = 0, equal = 0;
+    if (T.sample) {
+        seen = __reduce_add_sync(0xffffffffu, T.n_seen);
+        equal = __reduce_add_sync(0xffffffffu, T.n_equal);
+    }
+    uint32_t *stat = T.stat(win);
+    if ((threadIdx.x & 31u) == 0) {
+        if (T.n_ops) atomicAdd(&stat[0], T.n_ops);
+        if (T.n_live) atomicAdd(&stat[1], T.n_live);
+        if (seen) atomicAdd(&stat[2], seen);
+        if (equal) atomicAdd(&stat[3], equal);
+    }
+    T.n_ops = T.n_live = T.n_seen = T.n_equal = 0;
+}
+
+// Marks, at a window's first pack, all consumers: read the last window's
+// statistics and choose how the next one is run.  `win` counts windows.
+__device__ inline void mark_window(const Job &J, Track &T, uint32_t win, const Lane &L, uint32_t ct)
+{
+    uint32_t *prev = T.stat(win + 2u), *next = T.stat(win + 1u);
+    const uint32_t ops = *(volatile uint32_t *)&prev[0], live = *(volatile uint32_t *)&prev[1],
+                   seen = *(volatile uint32_t *)&prev[2], equal = *(volatile uint32_t *)&prev[3];
+    if (ct < 4) next[ct] = 0;  // read last two windows ago
+    T.quiet = T.on && live == 0;
+    T.sample = (win & 3u) == 0;
+    if (T.want) {
+        if (L.chunk == 0 && T.best_size) atomicMax(T.key(), T.best_size << 10 | L.lane0);
+        consumers_sync();
+        const uint32_t key = *(volatile uint32_t *)T.key();
+        T.want = false;
+        T.best_size = 0;
+        if (key != 0 && (!T.on || (key >> 10) > T.c_size)) {
+            T.c = *T.cand((key & 1023u) * L.cpr + L.chunk);
+            T.c_size = key >> 10;
+            T.on = true;
+            T.quiet = false;
+            for (uint32_t i = ct; i < J.mark_words; i += consumers()) T.bits()[i] = 0;
+        }
+        consumers_sync();
+        if (ct == 0) *T.key() = 0;
+        return;
+    }
+    if (T.shift == 0 && seen && 2 * equal >= seen && (!T.on || 8 * live >= ops)) T.want = T.sample = true;
+    else if (T.on && seen && 2 * live > ops) T.on = false;  // too few rows are marked: the checks do not pay
+}
+
+// Ids at the start: every row its own, or, in a matrix initialised by this
+// application, 0 but for the rows whose source column lies in the CTA's slab.
+__global__ void init_ids_kernel(uint32_t *ids, uint64_t rows, uint32_t pitch, uint32_t sw, bool zero, bool identity)
+{
+    const uint64_t total = rows * pitch / 4;  // pitch is a multiple of 8
+    for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < total; p += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t row = 4 * p / pitch;
+        const uint32_t cta = (uint32_t)(4 * p - row * pitch), own = (uint32_t)(row / 64 / sw);
+        const uint32_t other = zero ? 0u : (uint32_t)row + 1u, mine = identity ? (uint32_t)row + 1u : other;
+        reinterpret_cast<uint4 *>(ids)[p] = make_uint4(own == cta ? mine : other, own == cta + 1 ? mine : other,
+                                                       own == cta + 2 ? mine : other, own == cta + 3 ? mine : other);
+    }
+}
+
+__global__ void init_source_ids_kernel(uint32_t *ids, uint32_t pitch, uint32_t sw, const uint32_t *src, uint32_t nsrc,
+                                       uint32_t rows)
+{
+    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < nsrc; c += gridDim.x * blockDim.x)
+        if (src[c] < rows) ids[(uint64_t)src[c] * pitch + c / 64 / sw] = src[c] + 1u;
 }
 
 // ---------------------------------------------------------------------------
@@ -619,7 +1248,7 @@ __device__ inline uint2 lds_op(uint32_t a)
 // One op of a global tile on the resident rows (shared address rb, node ids)
 // and the saved rows (shared address tb, temp ids).
 template <bool kMax, int RW>
-__device__ inline void resident_op(uint2 op, uint32_t rb, uint32_t tb, const uint32_t *aux)
+__device__ inline void resident_op(uint2 op, uint32_t rb, uint32_t tb, const uint32_t *aux, const uint32_t *pack)
 {
     constexpr uint32_t kRowB = 8u * RW;
     const uint32_t kind = op.x >> kKindShift, a = op.x & kIdMask;
@@ -635,9 +1264,10 @@ __device__ inline void resident_op(uint2 op, uint32_t rb, uint32_t tb, const uin
         sts_rrow<RW>(tb + a * kRowB, lds_rrow<RW>(rb + op.y * kRowB));
     } else {
         RRow<RW> acc = lds_rrow<RW>(pa);
-        const uint32_t c = __ldg(aux + op.y);
+        const uint32_t *list = source_list(aux, pack, op.y);
+        const uint32_t c = list[0];
         for (uint32_t q = 1; q <= c; ++q) {
-            const uint32_t ref = __ldg(aux + op.y + q);
+            const uint32_t ref = list[q];
             acc = rcombine<kMax, RW>(acc, lds_rrow<RW>((ref & kTempRef) ? tb + (ref & ~kTempRef) * kRowB
                                                                      : rb + ref * kRowB));
         }
@@ -720,8 +1350,8 @@ __device__ void resident_slab(const Job &J, uint32_t smem_bytes, uint8_t *smem, 
         uint2 op = lds_op(opa + ct * 8u);  // always inside the stage; used only if ct < e
         for (uint32_t k = 0;;) {
             if (b + ct < e) {
-                resident_op<kMax, RW>(op, rb, tb, aux);
-                for (uint32_t o = b + ct + C; o < e; o += C) resident_op<kMax, RW>(lds_op(opa + o * 8u), rb, tb, aux);
+                resident_op<kMax, RW>(op, rb, tb, aux, head);
+                for (uint32_t o = b + ct + C; o < e; o += C) resident_op<kMax, RW>(lds_op(opa + o * 8u), rb, tb, aux, head);
             }
             if (++k >= nseg) break;
             b = e;
@@ -736,10 +1366,121 @@ __device__ void resident_slab(const Job &J, uint32_t smem_bytes, uint8_t *smem, 
     for (uint32_t i = ct; i < rows; i += C) st_rrow<RW>(S + (uint64_t)i * ld + w0, R[i]);
 }
 
+// The next pack of the ring, once every consumer is done with the one before
+// (level barrier: its stores are ordered before this pack's loads).  All
+// consumers agree on stopping; false = stop.
+__device__ inline bool next_pack(const Job &J, const PackRing &ring, uint32_t q, const uint32_t *abort_flag, bool ready)
+{
+    if (!ready && threadIdx.x == 32) record_status(J.status, TN_ETIMEOUT);
+    const uint32_t meta = reinterpret_cast<const uint32_t *>(ring.at(q))[1];
+    const bool stop = !ready || *(volatile const uint32_t *)abort_flag != 0 || ((meta >> 16) & kPackEnd);
+    return !consumers_sync_or(stop);
+}
+
+// Consumers of a column slab in a plan with records, or whose slab width does not
+// divide a warp into row groups, or whose row buffer is too small for copy rings.
+template <bool kMax>
+__device__ void consume_plain(const Job &J, const PackRing &ring, const uint32_t *abort_flag, u64x2 *rowbuf, Lane L,
+                              uint32_t ct)
+{
+    for (uint32_t q = 0;; ++q) {
+        if (!next_pack(J, ring, q, abort_flag, ring.wait_full(q))) return;
+        const uint32_t *head = reinterpret_cast<const uint32_t *>(ring.at(q));
+        const uint32_t nseg = head[1] & 0xFFFFu;
+        L.pack = head;
+        if ((head[1] >> 16) & kPackLocal) {
+            apply_record<kMax>(J, head + 4, rowbuf, L);
+        } else {
+            const uint16_t *seg = reinterpret_cast<const uint16_t *>(head + 4);
+            const uint2 *ops = reinterpret_cast<const uint2 *>(head) + kPackHead;
+            for (uint32_t k = 0, b = 0; k < nseg; ++k) {
+                const uint32_t e = seg[k];
+                if (e == b) continue;
+                if (b) consumers_sync();
+                apply_tile<kMax>(J, ops + b, e - b, rowbuf, J.dcap, L);
+                b = e;
+            }
+        }
+        __syncwarp();
+        if ((ct & 31u) == 0) mbar_arrive(&ring.empty[q & ring.mask]);
+    }
+}
+
+// Consumers of a column slab with tracked rows (tiles only).  While nothing is
+// executed, the next pack is looked at as a whole, without its level barriers:
+// if none of its ops is to be executed, no row changes between its levels either.
+template <bool kMax, int kMode>
+__device__ void consume_tracked(const Job &J, const PackRing &ring, const uint32_t *abort_flag, u64x2 *rowbuf,
+                                uint64_t w0, uint32_t cta, Lane L, uint32_t ct)
+{
+    Track T;
+    T.at = (uint32_t)(kSlabHead + (size_t)J.dcap * J.sw * 8);
+    T.slot = (ct >> 5) * (kListOps / (consumers() >> 5));
+    T.rows = J.rows;
+    T.c = u64x2{0, 0};
+    T.want = T.quiet = T.on = false;
+    T.best_size = T.n_ops = T.n_live = T.n_seen = T.n_equal = T.c_size = T.shift = T.fresh = 0;
+    T.sample = kMode == kMarks;
+    if (kMode == kIds) {
+        T.ids = J.ids + cta;
+        T.pitch = J.pitch;
+        if (ct < 3) *T.stat(ct) = 1;
+    } else {
+        T.on = J.mark_words != 0;
+        T.shift = J.mark_shift;
+        mark_init(J, T, w0, ct);
+        if (!T.on) T.shift = 1;  // no marks at all: no candidates either
+    }
+    const uint32_t g = (ct & 31u) / L.cpr;
+    const uint32_t group_mask = L.cpr == 32 ? 0xffffffffu : ((1u << L.cpr) - 1u) << (g * L.cpr);
+    uint32_t win = 0, first = J.rows + 1u;  // ids 1..rows are the rows' own
+    for (uint32_t q = 0;; ++q) {
+        const bool ready = __all_sync(0xffffffffu, ring.wait_full(q));
+        const uint32_t *head = reinterpret_cast<const uint32_t *>(ring.at(q));
+        const bool starts = kMode == kMarks && q && ready && ((head[1] >> 16) & kPackWindow);
+        if (starts) mark_count(T, win);  // of the window that ends here, read behind the barrier
+        if (!next_pack(J, ring, q, abort_flag, ready)) return;
+        if (starts) mark_window(J, T, ++win, L, ct);
+        const uint16_t *seg = reinterpret_cast<const uint16_t *>(head + 4);
+        const uint2 *ops = reinterpret_cast<const uint2 *>(head) + kPackHead;
+        const uint32_t nops = head[0];
+        uint32_t nseg = head[1] & 0xFFFFu;
+        L.pack = head;
+        if (kMode == kIds) {
+            T.quiet = *(volatile uint32_t *)T.stat(q + 2) == 0;  // the last pack executed nothing
+            if (ct == 0) *T.stat(q + 1) = 0;                     // read one pack ago, set in the next one
+        }
+        if (T.quiet) {
+            bool live = false;
+            uint4 e;
+            for (uint32_t i = ct; i < nops && !live; i += consumers())
+                live = kMode == kIds ? id_live(J, T, ops[i], L.pack, e) : mark_live(J, T, ops[i], L.pack, e);
+            if (!consumers_sync_or(live)) {
+                nseg = 0;
+                if (kMode == kMarks && ct == 0) T.n_ops += nops;
+            }
+        }
+        bool ran = false;
+        for (uint32_t k = 0, b = 0; k < nseg; ++k) {
+            const uint32_t e = seg[k];
+            if (e == b) continue;
+            if (b) consumers_sync();
+            T.fresh = first + b;
+            if (kMode == kIds || T.on) ran |= track_tile<kMax, kMode>(J, T, ops + b, e - b, rowbuf, L, group_mask);
+            else whole_tile<kMax>(J, T, ops + b, e - b, rowbuf, L, group_mask);
+            b = e;
+        }
+        if (kMode == kIds && ran && (ct & 31u) == 0) *T.stat(q) = 1;
+        first += nops;
+        __syncwarp();
+        if ((ct & 31u) == 0) mbar_arrive(&ring.empty[q & ring.mask]);
+    }
+}
+
 template <bool kMax>
 __global__ void __launch_bounds__(kMaxThreads) stream_kernel(const __grid_constant__ JobList jl)
 {
-    extern __shared__ __align__(128) uint8_t smem[];
+    uint8_t *const smem = dyn_smem;
     __shared__ uint32_t producer_abort;
     __shared__ int32_t gate;
 
@@ -758,7 +1499,7 @@ __global__ void __launch_bounds__(kMaxThreads) stream_kernel(const __grid_consta
     ring.shift = kStageShift;
     u64x2 *rowbuf = reinterpret_cast<u64x2 *>(smem + kSlabHead);
     const uint64_t w0 = J.w_begin + (uint64_t)(blockIdx.x - J.cta_begin) * J.sw;
-    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
+    const uint32_t warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
         gate = *(volatile int32_t *)J.status;  // an earlier error gates this job
         for (int s = 0; s < kStages; ++s) {
@@ -774,35 +1515,12 @@ __global__ void __launch_bounds__(kMaxThreads) stream_kernel(const __grid_consta
         produce_packs(J, ring, &producer_abort);
         return;
     }
-    // ---------------- consumers ----------------
     const uint32_t ct = threadIdx.x - 32;
     const Lane L = make_lane(J, ct, w0);
-    for (uint32_t q = 0;; ++q) {
-        const bool ready = ring.wait_full(q);
-        if (!ready && ct == 0) record_status(J.status, TN_ETIMEOUT);
-        const uint32_t *head = reinterpret_cast<const uint32_t *>(ring.at(q));
-        const bool stop = !ready || *(volatile uint32_t *)&producer_abort != 0 || ((head[1] >> 16) & kPackEnd);
-        // level barrier: the previous pack's stores are ordered before this
-        // pack's loads, and all consumers agree on stopping
-        if (consumers_sync_or(stop)) break;
-        const uint32_t meta = head[1];
-        if ((meta >> 16) & kPackLocal) {
-            apply_record<kMax>(J, head + 4, rowbuf, L);
-        } else {
-            const uint16_t *seg = reinterpret_cast<const uint16_t *>(head + 4);
-            const uint2 *ops = reinterpret_cast<const uint2 *>(head) + kPackHead;
-            const uint32_t nseg = meta & 0xFFFFu;
-            for (uint32_t k = 0, b = 0; k < nseg; ++k) {
-                const uint32_t e = seg[k];
-                if (e == b) continue;
-                if (b) consumers_sync();
-                apply_tile<kMax>(J, ops + b, e - b, rowbuf, J.dcap, L);
-                b = e;
-            }
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&ring.empty[q & ring.mask]);
-    }
+    const uint32_t cta = blockIdx.x - J.cta_begin;
+    if (J.track == kIds) consume_tracked<kMax, kIds>(J, ring, &producer_abort, rowbuf, w0, cta, L, ct);
+    else if (J.track == kMarks) consume_tracked<kMax, kMarks>(J, ring, &producer_abort, rowbuf, w0, cta, L, ct);
+    else consume_plain<kMax>(J, ring, &producer_abort, rowbuf, L, ct);
 }
 
 // Self-test of the bounded waits: one thread waits on an mbarrier that nothing
@@ -977,6 +1695,28 @@ static int grid_for(uint64_t work)
 }
 
 
+// Slab width of the plans of a launch that leave it open: the narrowest that
+// keeps the launch's slabs within one wave (a CTA fills an SM, and every CTA
+// walks the whole schedule), at most 64 words.  One matrix, stream kernel:
+// 5,000 directed columns (79 words), m = 3 10^6: 24.1 ms at 16 words (5 CTAs),
+// 13.4 ms at 2 (40); ER n = 4 10^4, m = 5 10^6: 27.8 ms at 16 words (40), 21.2 ms at
+// 8 (79), 34.7 ms at 4 (157, two waves); bursty n = 2 10^5, m = 5 10^6: 136 ms at 16
+// (196, two waves), 91 ms at 32 (98), 144 ms at 64 (49).
+static uint32_t open_slab_words(const tn_plan *const *plans, const uint32_t *ncols, uint32_t count)
+{
+    uint32_t sw = 2;
+    for (; sw < 64; sw *= 2) {
+        uint64_t ctas = 0;
+        for (uint32_t i = 0; i < count; ++i) {
+            if (plans[i]->resident) continue;
+            const uint32_t w = plans[i]->auto_slab && !plans[i]->local_windows ? sw : plans[i]->slab_words;
+            ctas += ((ncols[i] + 63ull) / 64 + w - 1) / w;
+        }
+        if (ctas <= (uint64_t)multiprocessors()) break;
+    }
+    return sw;
+}
+
 tn_status apply_jobs(const tn_plan *const *plans, uint64_t *const *S, const uint32_t *ncols,
                      const uint32_t *const *src, int64_t *const *t_last, uint32_t count, uint32_t flags,
                      cudaStream_t st)
@@ -994,6 +1734,7 @@ tn_status apply_jobs(const tn_plan *const *plans, uint64_t *const *S, const uint
         for (uint32_t i = 0; i < count; ++i)
             if (plans[i]->resident) return TN_EINVAL;
     uint64_t *tmps[kMaxPlans];
+    uint32_t *idbuf[kMaxPlans];
     for (uint32_t base = 0; base < count; base += kMaxPlans) {
         const uint32_t nj = count - base < (uint32_t)kMaxPlans ? count - base : (uint32_t)kMaxPlans;
         JobList jl;
@@ -1001,11 +1742,13 @@ tn_status apply_jobs(const tn_plan *const *plans, uint64_t *const *S, const uint
         jl.count = 0;
         uint32_t ctas = 0;
         size_t smem = smem_base;
+        const uint32_t open_sw = open_slab_words(plans + base, ncols + base, nj);
         for (uint32_t j = 0; j < nj; ++j) {
             const uint32_t i = base + j;
             const tn_plan *p = plans[i];
             const uint64_t ld = tn_row_words(ncols[i]);
             tmps[j] = nullptr;
+            idbuf[j] = nullptr;
             if (p->resident) continue;  // second pass below
             if (t_last && t_last[i]) {
                 tn_internal_count_launches(1);
@@ -1024,10 +1767,58 @@ tn_status apply_jobs(const tn_plan *const *plans, uint64_t *const *S, const uint
                 }
             }
             if (p->temps) TN_CUDA_TRY(cudaMallocAsync((void **)&tmps[j], p->temps * ld * sizeof(uint64_t), st));
-            const size_t need = smem_base + (size_t)p->dcap * p->slab_words * 8;
+            // Row buffer of the launch: records use all of the plan's; tiles only
+            // the copy rings of 12 consumer warps.
+            const bool open = p->auto_slab && !p->local_windows;
+            const uint32_t sw = open ? open_sw : p->slab_words;
+            // words that hold columns (the rest of the row is zero padding and stays so)
+            const uint64_t wide = open ? (((uint64_t)ncols[i] + 63) / 64 + 1) & ~1ull : ld;
+            uint32_t dcap = open ? kRowBufferMax / (8 * sw) : p->dcap;
+            const uint32_t ring_rows = 2u * kRing * (32u * kWarpsAlone / (sw / 2));
+            if (p->local_windows == 0 && dcap > ring_rows) dcap = ring_rows;
+            size_t need = smem_base + (size_t)dcap * sw * 8;
+            // Tracked rows: tile windows only (records do not keep track), row groups
+            // that are whole parts of a warp, and copy rings that fit.  Wide slabs
+            // by ids, if the ops pay for setting the ids up (4 bytes per row and
+            // CTA against 512 to 2,048 bytes per op and CTA); others by marks, a
+            // row or, where that does not fit, up to 4 rows per mark.
+            const uint32_t cpr = sw / 2, nct = (uint32_t)((wide + sw - 1) / sw);
+            const uint64_t rows = (uint64_t)p->n + p->temps;
+            const bool zero = (flags & TN_INIT_IDENTITY) != 0;
+            uint32_t track = kNoTrack, mark_words = 0, mark_shift = 0, *ids = nullptr;
+            const uint32_t pitch = (nct + 7u) & ~7u;
+            if (!p->local_windows && !(cpr & (cpr - 1)) && cpr <= 32 && dcap >= ring_rows && !p->wave_ctas &&
+                need + kMarkBytes <= smem_limit) {
+                track = kMarks;
+                if (sw > kMarkWords && 16 * p->ops >= p->n && rows + p->ops < 0xFFFFFFF0ull) {
+                    if (cudaMallocAsync((void **)&ids, rows * pitch * 4, st) == cudaSuccess) {
+                        track = kIds;
+                        tn_internal_count_launches(1);
+                        init_ids_kernel<<<grid_for(rows * pitch / 4), 256, 0, st>>>(ids, rows, pitch, sw,
+                                                                                   zero, zero && !src[i]);
+                        if (zero && src[i]) {
+                            tn_internal_count_launches(1);
+                            init_source_ids_kernel<<<grid_for(ncols[i]), 256, 0, st>>>(ids, pitch, sw,
+                                                                                      src[i], ncols[i], p->n);
+                        }
+                    } else {
+                        cudaGetLastError();  // no room for ids: marks
+                        ids = nullptr;
+                    }
+                }
+                if (track == kMarks) {
+                    for (;; ++mark_shift) {
+                        mark_words = (uint32_t)((((uint64_t)p->n >> mark_shift) + 1 + p->temps + 31) / 32);
+                        if (need + kMarkBytes + 4ull * mark_words <= smem_limit || mark_shift == kMarkShift) break;
+                    }
+                    if (need + kMarkBytes + 4ull * mark_words > smem_limit || (mark_shift && !zero)) mark_words = 0;
+                }
+                need += (track == kIds ? kIdBytes : kMarkBytes) + 4ull * mark_words;
+            }
+            idbuf[j] = ids;
             if (need > smem) smem = need;
             SlabSplit sp[2];
-            const int parts = split_slabs(ld, p->slab_words, p->wave_ctas, sp);
+            const int parts = split_slabs(wide, sw, p->wave_ctas, sp);
             for (int k = 0; k < parts; ++k) {
                 Job &J = jl.job[jl.count++];
                 J.blob = p->d_blob;
@@ -1041,7 +1832,16 @@ tn_status apply_jobs(const tn_plan *const *plans, uint64_t *const *S, const uint
                 J.w_begin = sp[k].w_begin;
                 J.sw = sp[k].sw;
                 J.cpr = sp[k].sw / 2;
-                J.dcap = p->dcap;
+                J.dcap = dcap;
+                J.track = track;
+                J.ids = ids;
+                J.pitch = pitch;
+                J.mark_words = mark_words;
+                J.mark_shift = mark_shift;
+                J.mark_init = !zero ? 0u : src[i] ? 2u : 1u;
+                J.src = src[i];
+                J.ncols = ncols[i];
+                J.rows = p->n;
                 J.cta_begin = ctas;
                 ctas += sp[k].ctas;
             }
@@ -1138,6 +1938,7 @@ tn_status apply_jobs(const tn_plan *const *plans, uint64_t *const *S, const uint
                 set_t_last_kernel<<<1, 1, 0, st>>>(plans[i]->d_tbounds, t_last[i], plans[i]->d_status);
             }
             if (tmps[j]) TN_CUDA_TRY(cudaFreeAsync(tmps[j], st));
+            if (idbuf[j]) TN_CUDA_TRY(cudaFreeAsync(idbuf[j], st));
         }
         TN_CUDA_TRY(cudaGetLastError());
     }

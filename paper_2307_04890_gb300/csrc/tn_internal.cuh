@@ -39,14 +39,16 @@ constexpr uint32_t kWaitPolls = 1u << 22;
 
 // Op encoding of the row-update schedule (see tn_plan.cu).
 //   a: bits 31..30 = kind, bits 29..0 = destination node / temp id
-//   b: EVENT / ONEWAY / COPY: source node id;  PULL: index into the aux list
-// aux list of a PULL at index b: aux[b] = count c, aux[b+1 .. b+c] = source
-// references (bit 31 set = temp slot, else node id).
+//   b: EVENT / ONEWAY / COPY: source node id;  PULL: its source list: count c, then
+// c source references (bit 31 set = temp slot, else node id), at word b of the
+// pack, or, from kOutsideList on, at word b - kOutsideList of the plan's list
+// buffer (the lists of one level did not fit a pack).
 enum OpKind : uint32_t { kEvent = 0u, kOneway = 1u, kCopy = 2u, kPull = 3u };
 constexpr uint32_t kKindShift = 30;
 constexpr uint32_t kIdMask = (1u << 30) - 1u;
 constexpr uint32_t kTempRef = 1u << 31;
 constexpr uint32_t kNoRef = 0xFFFFFFFFu;  // empty slot in a batch of source references
+constexpr uint32_t kOutsideList = 8192;
 
 __host__ __device__ inline uint32_t op_a(uint32_t kind, uint32_t id) { return (kind << kKindShift) | id; }
 
@@ -55,7 +57,7 @@ __host__ __device__ inline uint32_t op_a(uint32_t kind, uint32_t id) { return (k
 // (16-byte aligned, sizes in 8-byte units).
 //   tile pack: uint32 ops, uint32 segments | flags << 16, 8 spare bytes,
 //     uint16 end[64] (op offsets where its segments end), then the ops as uint2
-//     (node ids, absolute aux indices).  A segment is a level, or a part of one
+//     (node ids), then the source lists of its PULLs.  A segment is a level, or a part of one
 //     when the level does not fit a pack; ops of one segment never conflict.
 //   record pack (kPackLocal; a window whose rows fit the kernel's shared-memory
 //     row buffer): 16 bytes like the above, then uint32 words D, T, nlev, nops |
@@ -270,12 +272,13 @@ struct tn_plan {
     uint64_t windows, levels, ops, aux, temps, big_windows, local_windows, items, blob8;
     int64_t t_first, t_last;
     uint32_t slab_words;  // 64-bit words of every row owned by one CTA (the widest, with wave_ctas)
+    uint32_t auto_slab;   // slab_words was left open: chosen when the plan is applied, if it has no records
     uint32_t wave_ctas;   // 0, or the number of CTAs one matrix is spread over
     uint32_t dcap;        // row slots of the kernel's shared-memory row buffer
     uint32_t resident;    // 0, or 64-bit words of every row one CTA keeps in shared memory
     uint2 *d_blob;        // packs (8-byte units)
     tn::WinDesc *d_win;   // [windows]    their windows in time order
-    uint32_t *d_aux;      // source lists of PULL ops
+    uint32_t *d_aux;      // source lists outside the packs
     tn::PlanHead *d_head; // owned: counters, time bounds, status word
     int64_t *d_tbounds;   // [2]          t_first, t_last (in d_head)
     int32_t *d_status;    // first asynchronous error (in d_head, or the owner's: tn::plan_use_status)

@@ -47,7 +47,8 @@
 namespace tn {
 
 constexpr int kPlanThreads = 512;
-constexpr uint32_t kDefaultWindow = 640;
+// Default window of plans that name a row buffer: its rows fit a record.
+constexpr uint32_t kRecordWindow = 640;
 constexpr uint32_t kDefaultSlab = 16;
 constexpr uint32_t kRowBufferBytes = 160 * 1024;  // default shared-memory row buffer, slabs of up to 16 words
 constexpr uint32_t kRowBufferWide = 192 * 1024;   // default (and largest) row buffer for wider slabs
@@ -57,6 +58,17 @@ constexpr uint32_t kRecordEvents = 2048;
 // Groups of at least this many events go to the whole CTA unchecked: comparing
 // their events pair by pair would cost more than the group's own phases.
 constexpr uint32_t kPairGroup = 128;
+// Networks below this size keep record windows by default: their levels are short
+// and deep (bursty n = 20,011, 500,009 events: 7.4 ms, 19.6 ms in tiles).
+constexpr uint32_t kTileRows = 24928;
+// Default window otherwise.  Larger windows have fewer levels per event, each of
+// which costs every CTA a barrier and a memory latency, but are scheduled by one
+// CTA each and are stretched by large timestamp groups.  n = 10^5, 10^7
+// activity-driven events: schedule and apply 1.2 + 25.9 ms at 2,480, 1.8 + 23.4 ms
+// at 5,000; bursty n = 5 10^5, groups of 2,786 events: schedule 8.3 ms at 640, 17.5
+// ms at 5,000 (windows of two groups leave shared memory); n = 1,000, 20,000
+// uniform events: 0.10 + 0.08 ms at 1,280, 0.14 + 0.08 ms at 2,480.
+static uint32_t default_window(uint64_t m) { return m < (1u << 16) ? 1280u : 2480u; }
 // Batches of at least this many events are copied into buffers of their exact
 // size; below it the staging buffers (a few times larger, bounded) are kept.
 constexpr uint64_t kCompactEvents = 1ull << 20;
@@ -123,7 +135,7 @@ struct PlanCounters {
     unsigned long long late;        // windows left to the second pass
     unsigned long long arena;       // arena bytes of those scheduled in global memory
     unsigned long long big;         // how many of them are
-    unsigned long long blob8, naux, items, ops, levels, local, temps;
+    unsigned long long blob8, naux, list_words, items, ops, levels, local, temps;
     unsigned long long blob_used, aux_used;  // allocation of the exact buffers
     long long t_first, t_last;
 };
@@ -480,7 +492,7 @@ __device__ void schedule_window(const PlanArgs &a, uint32_t w, uint8_t *arena)
     __shared__ uint32_t warp_sums[32];
     __shared__ uint32_t tot;
     __shared__ uint32_t sc[kScCount];
-    __shared__ uint32_t res[2];  // packs, units
+    __shared__ uint32_t res[3];  // packs, units, lists outside the packs
 
     const uint64_t s = a.wstart[w];
     const uint32_t E = (uint32_t)(a.wstart[w + 1] - s);
@@ -690,35 +702,50 @@ __device__ void schedule_window(const PlanArgs &a, uint32_t w, uint8_t *arena)
             a.naux_w[w] = 0;
         }
     } else {
-        // packs: as many whole levels as fit, or a part of a level that does not
-        // fit one pack; warp 0 cuts them and writes their headers
-        uint32_t *pq = A.scratch + maxlev + 2;  // first op of every pack, then its first op's unit
+        // packs: as many whole levels as fit with the source lists of their PULLs;
+        // a level whose lists do not fit keeps them in the plan's list buffer, and
+        // one with more ops than a pack holds is cut.  Warp 0 cuts the packs and
+        // writes their headers.
+        uint32_t *la = A.scratch + maxlev + 2;  // list words of the levels before
+        uint32_t *pq = la + maxlev + 2;         // per pack: first op, its unit, next free list word (0: none), spare
+        for (uint32_t j = tid; j < maxlev + 1; j += T) la[j] = 0;
+        __syncthreads();
+        for (uint32_t r = tid; r < nruns; r += T) atomicAdd(&la[A.run_lev[r]], 1u + auxw[A.run_aux[r]]);
+        __syncthreads();
+        block_excl_scan_array(la, maxlev + 1, warp_sums, &tot);
         if (tid < 32) {
-            uint32_t p = 0, l = 0, q = 0, unit = 0;
+            uint32_t p = 0, l = 0, q = 0, unit = 0, outside = 0;
             while (q < nops) {
-                uint32_t fit[2], rel[2];
+                uint32_t rel[2], list[2], with[2], fit[2];
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const uint32_t j = l + 1 + lane + 32 * h;
-                    rel[h] = j <= maxlev ? lh[j] - q : 0xffffffffu;
+                    rel[h] = j <= maxlev ? lh[j] - q : 0x10000000u;
+                    list[h] = j <= maxlev ? la[j] - la[l] : 0u;
+                    with[h] = __popc(__ballot_sync(0xffffffffu, rel[h] + (list[h] + 1) / 2 <= kPackOps));
                     fit[h] = __popc(__ballot_sync(0xffffffffu, rel[h] <= kPackOps));
                 }
-                const uint32_t k = fit[0] + (fit[0] == 32u ? fit[1] : 0u);
+                const uint32_t kw = with[0] + (with[0] == 32u ? with[1] : 0u);
+                // levels whose lists stay outside: one at a time, or a part of one
+                const uint32_t k = kw ? kw : fit[0] ? 1u : 0u;
                 const uint32_t last = k ? lh[l + k] - q : kPackOps;
+                const uint32_t words = kw ? la[l + k] - la[l] : 0u;
                 uint32_t *hdr = reinterpret_cast<uint32_t *>(a.blob + region + unit);
                 uint16_t *seg = reinterpret_cast<uint16_t *>(hdr + 4);
                 if (lane == 0) {
                     hdr[0] = last;
                     hdr[1] = (k ? k : 1u) | (q == 0 ? kPackWindow << 16 : 0u);
                     hdr[2] = hdr[3] = 0;
-                    pq[2 * p] = q;
-                    pq[2 * p + 1] = unit + kPackHead;
+                    pq[4 * p] = q;
+                    pq[4 * p + 1] = unit + kPackHead;
+                    pq[4 * p + 2] = kw ? 2 * (kPackHead + last) : 0u;
                     if (!k) seg[0] = (uint16_t)last;
                 }
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
                     if (lane + 32 * h < k) seg[lane + 32 * h] = (uint16_t)rel[h];
-                unit += (kPackHead + last + 1u) & ~1u;
+                if (!kw) outside = 1;
+                unit += (kPackHead + last + (words + 1) / 2 + 1u) & ~1u;
                 q += last;
                 l += k;
                 ++p;
@@ -726,27 +753,24 @@ __device__ void schedule_window(const PlanArgs &a, uint32_t w, uint8_t *arena)
             if (lane == 0) {
                 res[0] = p;
                 res[1] = unit;
+                res[2] = outside;
             }
         }
         __syncthreads();
         const uint32_t np = res[0];
-        // PULL lists name rows by node id
-        for (uint32_t r = tid; r < nruns; r += T) {
-            const uint32_t b = A.run_aux[r], c = auxw[b];
-            for (uint32_t q = 1; q <= c; ++q) {
-                const uint32_t ref = auxw[b + q];
-                if (!(ref & kTempRef)) auxw[b + q] = A.rowsg[ref];
-            }
-        }
         uint2 *ops = a.blob + region;
-        auto place = [&](uint32_t pos) -> uint2 * {  // unit of op `pos`
+        auto pack_of = [&](uint32_t pos) -> uint32_t {
             uint32_t lo = 0, hi = np;
             while (lo + 1 < hi) {
                 const uint32_t mid = (lo + hi) / 2;
-                if (pq[2 * mid] <= pos) lo = mid;
+                if (pq[4 * mid] <= pos) lo = mid;
                 else hi = mid;
             }
-            return ops + pq[2 * lo + 1] + (pos - pq[2 * lo]);
+            return lo;
+        };
+        auto place = [&](uint32_t pos) -> uint2 * {
+            const uint32_t p = pack_of(pos);
+            return ops + pq[4 * p + 1] + (pos - pq[4 * p]);
         };
         for (uint32_t i0 = 0; i0 < E; i0 += T) {
             const uint32_t i = i0 + tid;
@@ -759,15 +783,27 @@ __device__ void schedule_window(const PlanArgs &a, uint32_t w, uint8_t *arena)
                                                                : make_uint2(op_a(kOneway, x), y);
         }
         for (uint32_t r = tid; r < nruns; r += T) {
-            const uint32_t L = A.run_lev[r], xg = A.rowsg[A.run_node[r]];
-            *place(atomicAdd(&lh[L], 1u)) = make_uint2(op_a(kPull, xg), (uint32_t)(3 * s) + A.run_aux[r]);
+            const uint32_t L = A.run_lev[r], xg = A.rowsg[A.run_node[r]], b = A.run_aux[r], c = auxw[b];
+            const uint32_t pos = atomicAdd(&lh[L], 1u), p = pack_of(pos);
+            uint32_t *list = auxw + b;
+            uint32_t where = kOutsideList + (uint32_t)(3 * s) + b;
+            if (pq[4 * p + 2]) {
+                where = atomicAdd(&pq[4 * p + 2], 1u + c);
+                list = reinterpret_cast<uint32_t *>(ops + pq[4 * p + 1] - kPackHead) + where;
+                list[0] = c;
+            }
+            for (uint32_t q = 1; q <= c; ++q) {  // lists name rows by node id
+                const uint32_t ref = auxw[b + q];
+                list[q] = (ref & kTempRef) ? ref : A.rowsg[ref];
+            }
+            ops[pq[4 * p + 1] + (pos - pq[4 * p])] = make_uint2(op_a(kPull, xg), where);
             if (A.run_temp[r] != (I)~(I)0)
                 *place(atomicAdd(&lh[L - 1], 1u)) = make_uint2(op_a(kCopy, A.run_temp[r]), xg);
         }
         // pack sizes: the first kDescPacks in the descriptor, all of them behind
         // the packs when there are more
         for (uint32_t p = tid; p < np; p += T) {
-            const uint32_t b = pq[2 * p + 1] - kPackHead, e = p + 1 < np ? pq[2 * p + 3] - kPackHead : res[1];
+            const uint32_t b = pq[4 * p + 1] - kPackHead, e = p + 1 < np ? pq[4 * p + 5] - kPackHead : res[1];
             if (p < kDescPacks) desc->pack[p] = e - b;
             if (np > kDescPacks) reinterpret_cast<uint32_t *>(ops + res[1])[p] = e - b;
         }
@@ -775,7 +811,8 @@ __device__ void schedule_window(const PlanArgs &a, uint32_t w, uint8_t *arena)
             desc->off = region;
             desc->npacks = np;
             desc->tab = res[1];
-            a.naux_w[w] = naux;
+            a.naux_w[w] = res[2] ? naux : 0u;
+            if (res[2]) atomicAdd(&a.cnt->list_words, (unsigned long long)naux);
         }
     }
     if (tid == 0) {
@@ -858,7 +895,7 @@ __global__ void compact_kernel(PlanArgs a, uint2 *blob, uint32_t *aux)
         const uint32_t nops = a.blob[src + u0].x;
         uint2 *ops = blob + dst + u0 + kPackHead;
         for (uint32_t k = threadIdx.x; k < nops; k += blockDim.x)
-            if ((ops[k].x >> kKindShift) == kPull) ops[k].y = (uint32_t)(ops[k].y - s3 + base[1]);
+            if ((ops[k].x >> kKindShift) == kPull && ops[k].y >= kOutsideList) ops[k].y = (uint32_t)(ops[k].y - s3 + base[1]);
         u0 += n8;
     }
 }
@@ -923,7 +960,7 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     if (!plan_out) return TN_EINVAL;
     *plan_out = nullptr;
     if (!u || !v || !t || m == 0 || n == 0 || n >= (1u << 30) || m >= (1ull << 30)) return TN_EINVAL;
-    uint32_t sw = kDefaultSlab, window = kDefaultWindow, rows = 0, wave = 0, resident = 0;
+    uint32_t sw = kDefaultSlab, window = 0, rows = 0, wave = 0, resident = 0;
     if (opt) {
         for (int i = 0; i < 2; ++i)
             if (opt->reserved[i]) return TN_EINVAL;
@@ -935,6 +972,8 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
         resident = opt->resident_words;
     }
     if (sw < 2 || sw > kMaxSlabWords || (sw & 1u)) return TN_EINVAL;  // even: whole 16-byte chunks
+    const bool auto_window = window == 0 && !resident;
+    if (!window) window = rows || n < kTileRows ? kRecordWindow : default_window(m);
     if (window < 32) window = 32;
     if (resident) {
         // the resident-slab form keeps every row in shared memory: no row
@@ -978,6 +1017,7 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     p->wave_ctas = wave;
     p->dcap = rows;
     p->resident = resident;
+    p->auto_slab = !resident && !wave && (!opt || !opt->slab_words);
 
     tn_status rc = TN_OK;
     PlanCounters host;
@@ -1047,19 +1087,35 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     p->ops = host.ops;
     p->local_windows = host.local;
     p->big_windows = host.big;
+    if (auto_window && window != kRecordWindow && sw <= 16 && 16 * p->aux > p->ops && p->ops < 256 * p->levels && m < 64ull * n) {
+        // Deep schedules of short levels (hubs that chain large timestamp groups)
+        // over rows that mostly do not settle: records walk their levels in shared
+        // memory.  Bursty n = 8 10^4, m = 2 10^6 (240 ops a level, 25 events a
+        // node): 25.9 ms as records, 32 to 36 ms as tiles; n = 2 10^5, m = 5 10^6
+        // (600 ops a level): 146 ms with windows of 640, 136 ms as tiles.
+        free_plan_buffers(p, st);
+        cudaFreeAsync(a.wstart, st);
+        if (a.late_arena) cudaFreeAsync(a.late_arena, st);
+        free(p);
+        tn_plan_options again;
+        memset(&again, 0, sizeof(again));
+        if (opt) again = *opt;
+        again.window_events = kRecordWindow;
+        return plan_create_impl(u, v, t, m, n, t_after, &again, stream, plan_out, wait_end);
+    }
     if (resident && !resident_fits(n, p->temps, resident)) {  // saved rows of the tie groups do not fit
         rc = TN_EINVAL;
         goto done;
     }
     if (m >= kCompactEvents) {
         TN_STEP(alloc_async(&exact_blob, p->blob8 + 2, st));
-        TN_STEP(alloc_async(&exact_aux, p->aux > 0 ? p->aux : 1, st));
+        TN_STEP(alloc_async(&exact_aux, host.list_words, st));
         tn_internal_count_launches(1);
         compact_kernel<<<a.nw, 256, 0, st>>>(a, exact_blob, exact_aux);
         TN_STEP(cudaGetLastError());
         cudaFreeAsync(p->d_blob, st);
         cudaFreeAsync(p->d_aux, st);
-        p->d_blob = exact_blob;
+        p->d_blob = exact_blob;  // (no list outside the packs: no list buffer)
         p->d_aux = exact_aux;
         exact_blob = nullptr;
         exact_aux = nullptr;
