@@ -212,7 +212,8 @@ typedef struct tn_plan_options {
                                2 words), e.g. one full wave of the GPU's SMs.  N
                                below ceil(row words / slab_words) is raised to it */
     uint32_t resident_words;/* 0: the column-slab form above (rows move between HBM and
-                               shared memory).  1 or 2: the resident-slab form for
+                               shared memory), or, with slab_words, smem_rows and
+                               wave_ctas 0 as well, whichever form suits the launch.  1 or 2: the resident-slab form for
                                small networks, the same update of Algorithm 1
                                (Section 3.1) in another launch shape: each CTA keeps
                                resident_words 64-bit
@@ -227,7 +228,8 @@ typedef struct tn_plan_options {
                                smem_rows and wave_ctas must then be 0.  The plan
                                applies like any other (identity, source columns,
                                t_last, batches and graphs, mixed with column-slab
-                               plans in one launch); tn_online_create rejects it */
+                               plans in one launch); tn_online_create rejects it as
+                               an option */
     uint32_t reserved[2];   /* must be zero */
 } tn_plan_options;
 

@@ -117,13 +117,9 @@ extern "C" tn_status tn_hll_sketches(const uint32_t *u, const uint32_t *v, const
         ev = rv;
         et = rt;
     }
-    // register slabs: at least 2 words, about two CTAs per SM for wide sketches
-    const uint64_t ld = row_bytes / 8;
-    uint64_t sw = (ld + 2 * 152 - 1) / (2 * 152);
-    sw = sw < 2 ? 2 : (sw > 16 ? 16 : (sw + 1) & ~1ull);
+    // the form and the slab width are left to the launch (2^p register bytes a row)
     tn_plan_options opt;
     memset(&opt, 0, sizeof(opt));
-    opt.slab_words = (uint32_t)sw;
     opt.directed = (flags & TN_DIRECTED) ? 1u : 0u;
     tn_plan *plan = nullptr;
     tn_status rc = tn_plan_create(eu, ev, et, m, n, nullptr, &opt, stream, &plan);

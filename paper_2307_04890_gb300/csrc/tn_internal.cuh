@@ -77,6 +77,7 @@ constexpr uint32_t kRecordWords = kStageBytes / 4 - 4;
 constexpr uint32_t kPackLocal = 1u;   // a record
 constexpr uint32_t kPackWindow = 2u;  // first pack of its window
 constexpr uint32_t kPackEnd = 4u;     // no pack: the schedule ends here
+constexpr uint32_t kPackTies = 8u;    // holds PULLs or COPYs
 // One window of the schedule: `npacks` packs from unit `off` on; their sizes
 // are pack[] while there are at most kDescPacks, else a uint32 table `tab`
 // units behind `off`.
@@ -273,12 +274,14 @@ struct tn_plan {
     int64_t t_first, t_last;
     uint32_t slab_words;  // 64-bit words of every row owned by one CTA (the widest, with wave_ctas)
     uint32_t auto_slab;   // slab_words was left open: chosen when the plan is applied, if it has no records
+    uint32_t auto_form;   // the form (resident or column slabs) was left open: chosen when the plan is applied
     uint32_t wave_ctas;   // 0, or the number of CTAs one matrix is spread over
     uint32_t dcap;        // row slots of the kernel's shared-memory row buffer
     uint32_t resident;    // 0, or 64-bit words of every row one CTA keeps in shared memory
     uint2 *d_blob;        // packs (8-byte units)
     tn::WinDesc *d_win;   // [windows]    their windows in time order
     uint32_t *d_aux;      // source lists outside the packs
+    uint32_t *d_label;    // [n] component of every node, a node id (NULL: not computed)
     tn::PlanHead *d_head; // owned: counters, time bounds, status word
     int64_t *d_tbounds;   // [2]          t_first, t_last (in d_head)
     int32_t *d_status;    // first asynchronous error (in d_head, or the owner's: tn::plan_use_status)

@@ -58,20 +58,24 @@ constexpr uint32_t kRecordEvents = 2048;
 // Groups of at least this many events go to the whole CTA unchecked: comparing
 // their events pair by pair would cost more than the group's own phases.
 constexpr uint32_t kPairGroup = 128;
-// Networks below this size keep record windows by default: their levels are short
-// and deep (bursty n = 20,011, 500,009 events: 7.4 ms, 19.6 ms in tiles).
+// Networks below this size whose slab width is given keep record windows unless
+// the batch is long enough for rows to settle: their levels are short and deep
+// (bursty n = 20,011, 500,009 events, 16 words: 6.6 ms, 11.4 ms in tiles).
 constexpr uint32_t kTileRows = 24928;
 // Default window otherwise.  Larger windows have fewer levels per event, each of
 // which costs every CTA a barrier and a memory latency, but are scheduled by one
-// CTA each and are stretched by large timestamp groups.  n = 10^5, 10^7
+// CTA each and are stretched by large timestamp groups; 2,000 ops are one pack.  n = 10^5, 10^7
 // activity-driven events: schedule and apply 1.2 + 25.9 ms at 2,480, 1.8 + 23.4 ms
 // at 5,000; bursty n = 5 10^5, groups of 2,786 events: schedule 8.3 ms at 640, 17.5
 // ms at 5,000 (windows of two groups leave shared memory); n = 1,000, 20,000
 // uniform events: 0.10 + 0.08 ms at 1,280, 0.14 + 0.08 ms at 2,480.
-static uint32_t default_window(uint64_t m) { return m < (1u << 16) ? 1280u : 2480u; }
+static uint32_t default_window(uint64_t m) { return m < (1u << 16) ? 1280u : 2000u; }
 // Batches of at least this many events are copied into buffers of their exact
 // size; below it the staging buffers (a few times larger, bounded) are kept.
 constexpr uint64_t kCompactEvents = 1ull << 20;
+// Batches whose rows may all settle well before the end: component labels (three
+// launches), for the forms that use them.
+constexpr uint64_t kLabelEvents = 1ull << 17, kLabelFactor = 40;
 
 // event flags of a window
 constexpr uint8_t kFlagStart = 1;   // first event of its timestamp group
@@ -734,7 +738,7 @@ __device__ void schedule_window(const PlanArgs &a, uint32_t w, uint8_t *arena)
                 uint16_t *seg = reinterpret_cast<uint16_t *>(hdr + 4);
                 if (lane == 0) {
                     hdr[0] = last;
-                    hdr[1] = (k ? k : 1u) | (q == 0 ? kPackWindow << 16 : 0u);
+                    hdr[1] = (k ? k : 1u) | (q == 0 ? kPackWindow << 16 : 0u) | (nruns ? kPackTies << 16 : 0u);
                     hdr[2] = hdr[3] = 0;
                     pq[4 * p] = q;
                     pq[4 * p + 1] = unit + kPackHead;
@@ -900,6 +904,54 @@ __global__ void compact_kernel(PlanArgs a, uint2 *blob, uint32_t *aux)
     }
 }
 
+// ---------------------------------------------------------------------------
+// connected components of the batch's events (long batches): once every row equals
+// its component's root row, no event can change anything any more, and a CTA stops
+// reading the schedule.  Lock-free union by smaller
+// id; a parent read from a stale cache line is still an ancestor, and a failed
+// compare-and-swap returns the true one.  10^7 events on 10^4 nodes: 0.03 ms.
+// ---------------------------------------------------------------------------
+__global__ void label_init_kernel(uint32_t *parent, uint32_t n)
+{
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) parent[i] = i;
+}
+
+__device__ inline uint32_t label_root(const uint32_t *parent, uint32_t x)
+{
+    for (uint32_t p = parent[x]; p != x; p = parent[x]) x = p;  // ids fall along a path
+    return x;
+}
+
+__global__ void label_union_kernel(const uint32_t *u, const uint32_t *v, uint64_t m, uint32_t *parent)
+{
+    for (uint64_t e = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; e < m; e += (uint64_t)gridDim.x * blockDim.x) {
+        uint32_t x = label_root(parent, u[e]), y = label_root(parent, v[e]);
+        while (x != y) {
+            if (x < y) {
+                const uint32_t z = x;
+                x = y;
+                y = z;
+            }
+            const uint32_t was = atomicCAS(&parent[x], x, y);  // x > y: paths keep falling
+            if (was == x) break;
+            x = label_root(parent, was);
+            y = label_root(parent, y);
+        }
+        // short paths for the events that follow
+        if (parent[u[e]] != y) atomicMin(&parent[u[e]], y);
+        if (parent[v[e]] != y) atomicMin(&parent[v[e]], y);
+    }
+}
+
+__global__ void label_flatten_kernel(uint32_t *parent, uint32_t n)
+{
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        uint32_t x = i;
+        for (uint32_t p = *(volatile uint32_t *)&parent[x]; p != x; p = *(volatile uint32_t *)&parent[x]) x = p;
+        parent[i] = x;
+    }
+}
+
 template <typename F>
 static uint32_t largest_window(uint64_t budget, F bytes)
 {
@@ -949,6 +1001,7 @@ static void free_plan_buffers(tn_plan *p, cudaStream_t st)
     if (p->d_win) cudaFreeAsync(p->d_win, st);
     if (p->d_aux) cudaFreeAsync(p->d_aux, st);
     if (p->d_head) cudaFreeAsync(p->d_head, st);
+    if (p->d_label) cudaFreeAsync(p->d_label, st);
 }
 
 // wait_end: return only once the plan's device buffers are written (else they
@@ -972,8 +1025,12 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
         resident = opt->resident_words;
     }
     if (sw < 2 || sw > kMaxSlabWords || (sw & 1u)) return TN_EINVAL;  // even: whole 16-byte chunks
+    // everything but the window left open: no records, and the form is chosen when
+    // the plan is applied
+    const bool auto_form = (!opt || (!opt->slab_words && !rows && !wave && !resident)) && n <= resident_max_rows(1);
     const bool auto_window = window == 0 && !resident;
-    if (!window) window = rows || n < kTileRows ? kRecordWindow : default_window(m);
+    if (!window) window = rows || (n < kTileRows && !auto_form && m < 64ull * n) ? kRecordWindow : default_window(m);
+    const bool records = !auto_form && !(auto_window && window != kRecordWindow);
     if (window < 32) window = 32;
     if (resident) {
         // the resident-slab form keeps every row in shared memory: no row
@@ -1005,7 +1062,7 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     const uint64_t first_max = (uint64_t)window + 64 < m ? (uint64_t)window + 64 : m;
     a.first_max = first_max < a.smem_max ? (uint32_t)first_max : a.smem_max;
     a.dcap = rows;
-    a.unit8 = window <= kRecordEvents && rows > 1 ? 5 : 4;
+    a.unit8 = window <= kRecordEvents && rows > 1 && records ? 5 : 4;
 
     tn_plan *p = (tn_plan *)calloc(1, sizeof(tn_plan));
     if (!p) return TN_ENOMEM;
@@ -1017,6 +1074,7 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     p->wave_ctas = wave;
     p->dcap = rows;
     p->resident = resident;
+    p->auto_form = auto_form;
     p->auto_slab = !resident && !wave && (!opt || !opt->slab_words);
 
     tn_status rc = TN_OK;
@@ -1025,6 +1083,7 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     PlanHead *head = nullptr;
     uint2 *exact_blob = nullptr;
     uint32_t *exact_aux = nullptr;
+    bool must_wait = false;
     const uint64_t blocks = (m + 1023) / 1024;
     cudaError_t err = cudaSuccess;
 
@@ -1087,7 +1146,7 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     p->ops = host.ops;
     p->local_windows = host.local;
     p->big_windows = host.big;
-    if (auto_window && window != kRecordWindow && sw <= 16 && 16 * p->aux > p->ops && p->ops < 256 * p->levels && m < 64ull * n) {
+    if (auto_window && !auto_form && window != kRecordWindow && sw <= 16 && 16 * p->aux > p->ops && p->ops < 256 * p->levels && m < 64ull * n) {
         // Deep schedules of short levels (hubs that chain large timestamp groups)
         // over rows that mostly do not settle: records walk their levels in shared
         // memory.  Bursty n = 8 10^4, m = 2 10^6 (240 ops a level, 25 events a
@@ -1107,7 +1166,18 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
         rc = TN_EINVAL;
         goto done;
     }
+    if ((resident || p->auto_slab || sw <= 16) && !wave && !p->local_windows && m >= kLabelEvents && m >= kLabelFactor * n) {
+        TN_STEP(alloc_async(&p->d_label, n, st));
+        const unsigned nb = (n + 255) / 256;
+        tn_internal_count_launches(3);
+        label_init_kernel<<<nb, 256, 0, st>>>(p->d_label, n);
+        label_union_kernel<<<(unsigned)(blocks < 1216 ? blocks : 1216), 256, 0, st>>>(u, v, m, p->d_label);
+        label_flatten_kernel<<<nb, 256, 0, st>>>(p->d_label, n);
+        TN_STEP(cudaGetLastError());
+        must_wait = true;
+    }
     if (m >= kCompactEvents) {
+        must_wait = true;
         TN_STEP(alloc_async(&exact_blob, p->blob8 + 2, st));
         TN_STEP(alloc_async(&exact_aux, host.list_words, st));
         tn_internal_count_launches(1);
@@ -1119,9 +1189,9 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
         p->d_aux = exact_aux;
         exact_blob = nullptr;
         exact_aux = nullptr;
-        // the plan is complete when this call returns, for use on any stream
-        if (wait_end) TN_STEP(tn_internal_stream_wait(st));
     }
+    // the plan is complete, and its events are read, when this call returns
+    if (must_wait && wait_end) TN_STEP(tn_internal_stream_wait(st));
     goto done;
 
 fail:

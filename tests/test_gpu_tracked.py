@@ -103,3 +103,33 @@ def test_sketches(p, reverse):
     n, u, v, t = STREAMS["late-ties"]()
     R = tn.tn_hll_sketches(*dev(u, v, t), n, p, 11, reverse=reverse)
     assert np.array_equal(R.cpu().numpy()[:, : 1 << p], oracle.hll_sketches(u, v, t, n, p, 11, reverse=reverse))
+
+
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("shape", [dict(), dict(resident_words=1), dict(resident_words=2, window_events=700)])
+@pytest.mark.parametrize("stream", ["late", "late-ties", "er", "bridge"])
+def test_settled_networks(stream, shape, directed):
+    """Long batches of small networks: resident CTAs skip packs that change nothing and
+    stop once every row equals its component's.  `bridge`: two halves settle, one late
+    event joins them, and another one at the very end adds a node."""
+    n = 900
+    if stream == "er":
+        u, v, t = synth.er_poisson(n, 200_000, seed=8)
+    elif stream == "bridge":
+        rng = np.random.default_rng(9)
+        m, half = 200_000, n // 2
+        side = rng.integers(0, 2, m) * half
+        u, v = side + rng.integers(0, half - 1, m), side + rng.integers(0, half - 1, m)
+        u[m // 2], v[m // 2] = 3, half + 5
+        u[-1], v[-1] = n - 1, 0
+        t = np.arange(m)
+    else:
+        u, v, t = late_nodes(n, 200_000, 10, 1 if stream == "late" else 30)
+    plan = tn.Plan(*dev(u, v, t), n, directed=directed, **shape)
+    S = torch.full((n, tn.tn_row_words(n)), -1, dtype=torch.int64, device="cuda")
+    ref = (oracle.component_matrix_directed if directed else oracle.component_matrix)(u, v, t, n)
+    for _ in range(2):
+        plan.apply(S, init=True)
+        assert plan.status() == 0
+        got = S.cpu().numpy().view(np.uint64)
+        assert np.array_equal(got[:, : ref.shape[1]], ref) and not got[:, ref.shape[1]:].any()
