@@ -161,104 +161,218 @@ __global__ void __launch_bounds__(kEstThreads)
 }
 
 // ---------------- fusion, bit-sliced over sources ----------------
-// For many sources the fusion is reorganised around a transposed table:
+// For many sources the fusion is reorganised around a transposed table, built for
+// one chunk of sources at a time:
 //   T[j][b] = bitset over the chunk's sources, bit s = bit h_j(x_s) of row b of P_j
 // (Section 4.2: super-node b reaches h_j(x_s) in proxy j).  Then
 //   est(x_s) = #{w : bit s of AND_j T[j][h_j(w)]},
-// i.e. a column count of the n x nsrc boolean matrix whose row w is the AND
-// of R rows of T -- the same vertical-counter column count as the exact
-// out-sizes.  T rows are padded like component-matrix rows (tn_row_words).
+// i.e. a column count of the n x chunk boolean matrix whose row w is the AND of R
+// rows of T.  A chunk is 4,096 sources (512-byte rows of T, four words a lane) or,
+// for few sources, 1,024: small enough that T stays in L2 (R = 8, k = 16,384: 64
+// MB) while every node reads R of its rows.
 constexpr int kTabThreads = 256;
-constexpr uint32_t kTabRows = 64;       // proxy rows per CTA
-constexpr uint32_t kTabSources = 8192;  // sources per CTA (their columns cached in shared memory)
+constexpr int kTabRows = 32;            // proxy rows per CTA, in shared memory
+constexpr uint32_t kTabSmem = 200 * 1024;  // largest such block of rows (k <= 51,200)
 
+// Bits of 32 rows of P_j at 256 sources' columns per warp step: lane i holds
+// source 32 s + i, reads the 32-bit word of its column in four rows at a time
+// (rows are stored in groups of four, rotated by the 16-byte piece against bank
+// conflicts), and a ballot per row gathers the 32 sources' bits; lane r keeps row
+// r's words and stores a whole 32-byte sector.  Bound by the shared-memory reads
+// of random columns.  R = 8, k = 16,384, 65,536 sources: about 4 ms in all (36 ms
+// with one thread gathering 32 bits through L1 per word).
 __global__ void __launch_bounds__(kTabThreads)
     bitslice_table_kernel(const uint64_t *P, uint32_t k, uint64_t ldk, const uint32_t *H, uint32_t n,
-                          const uint32_t *src, uint32_t s0, uint32_t ns, uint64_t ldT32, uint32_t *T)
+                          const uint32_t *src, uint32_t s0, uint32_t ns, uint32_t words, uint32_t *T)
 {
-    __shared__ uint32_t col[kTabSources];
-    const uint32_t j = blockIdx.z;
-    const uint32_t c0 = blockIdx.y * kTabSources;  // first source of this CTA, relative to the chunk
-    const uint32_t cn = min(kTabSources, ns - c0);
-    for (uint32_t q = threadIdx.x; q < cn; q += blockDim.x) {
-        const uint32_t x = src ? src[s0 + c0 + q] : s0 + c0 + q;
-        col[q] = H[(uint64_t)j * n + x];
+    extern __shared__ uint4 rows4[];  // [ldk32][8]
+    const uint32_t j = blockIdx.z, b0 = blockIdx.x * kTabRows;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint32_t w4 = (k + 127) / 128;  // 16-byte pieces of a row that hold columns
+    uint32_t *flat = reinterpret_cast<uint32_t *>(rows4);
+    for (uint32_t i0 = threadIdx.x; i0 < w4 * kTabRows; i0 += 4 * blockDim.x) {
+        uint4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {  // four loads in flight; consecutive threads read along a row
+            const uint32_t i = i0 + u * blockDim.x, r = i / w4, c = i - r * w4;
+            v[u] = make_uint4(0u, 0u, 0u, 0u);
+            if (i < w4 * kTabRows && b0 + r < k)
+                v[u] = __ldg(reinterpret_cast<const uint4 *>(P + ((uint64_t)j * k + b0 + r) * ldk) + c);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t i = i0 + u * blockDim.x, r = i / w4, c = i - r * w4;
+            if (i >= w4 * kTabRows) continue;
+            const uint32_t word[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+            for (uint32_t h = 0; h < 4; ++h) {
+                const uint32_t w = 4 * c + h;
+                flat[w * kTabRows + (((r >> 2) + c) & 7u) * 4 + (r & 3u)] = word[h];
+            }
+        }
     }
     __syncthreads();
-    const uint32_t b0 = blockIdx.x * kTabRows;
-    const uint32_t b1 = min(k, b0 + kTabRows);
-    // thread t builds 32-bit words (32 sources) of each row
-    const uint32_t words = (cn + 31) / 32;
-    for (uint32_t b = b0; b < b1; ++b) {
+    const uint32_t groups = (ns + 255) / 256;
+    for (uint32_t g = blockIdx.y * (kTabThreads / 32) + warp; g < groups; g += gridDim.y * (kTabThreads / 32)) {
+        uint32_t col[8], mine[8];
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+            const uint32_t q = g * 256 + s * 32 + lane;
+            col[s] = 0xFFFFFFFFu;
+            mine[s] = 0;
+            if (q < ns) col[s] = __ldg(H + (uint64_t)j * n + (src ? __ldg(src + s0 + q) : s0 + q));
+        }
+#pragma unroll 1
+        for (uint32_t q = 0; q < 8; ++q) {  // rows 4q .. 4q + 3
+#pragma unroll
+            for (int s = 0; s < 8; ++s) {
+                const bool in = col[s] != 0xFFFFFFFFu;
+                const uint32_t w = in ? col[s] >> 5 : 0u, bit = in ? 1u << (col[s] & 31u) : 0u;
+                const uint4 v = rows4[w * 8 + ((q + (w >> 2)) & 7u)];
+                const uint32_t x0 = __ballot_sync(0xffffffffu, v.x & bit), x1 = __ballot_sync(0xffffffffu, v.y & bit);
+                const uint32_t x2 = __ballot_sync(0xffffffffu, v.z & bit), x3 = __ballot_sync(0xffffffffu, v.w & bit);
+                if ((lane >> 2) == q) mine[s] = (lane & 2u) ? ((lane & 1u) ? x3 : x2) : ((lane & 1u) ? x1 : x0);
+            }
+        }
+        if (b0 + lane < k) {
+            uint4 *out = reinterpret_cast<uint4 *>(T + ((uint64_t)j * k + b0 + lane) * words + g * 8);
+            out[0] = make_uint4(mine[0], mine[1], mine[2], mine[3]);
+            out[1] = make_uint4(mine[4], mine[5], mine[6], mine[7]);
+        }
+    }
+}
+
+// The same table for proxies whose rows do not fit shared memory 32 at a time:
+// one thread per 32-bit word of T, columns read through L1.
+__global__ void __launch_bounds__(kTabThreads)
+    bitslice_table_wide_kernel(const uint64_t *P, uint32_t k, uint64_t ldk, const uint32_t *H, uint32_t n,
+                               const uint32_t *src, uint32_t s0, uint32_t ns, uint32_t words, uint32_t *T)
+{
+    __shared__ uint32_t col[4096];
+    const uint32_t j = blockIdx.z;
+    for (uint32_t q = threadIdx.x; q < ns; q += blockDim.x)
+        col[q] = H[(uint64_t)j * n + (src ? src[s0 + q] : s0 + q)];
+    __syncthreads();
+    const uint32_t b1 = min(k, (blockIdx.x + 1u) * 64u);
+    for (uint32_t b = blockIdx.x * 64u; b < b1; ++b) {
         const uint64_t *row = P + ((uint64_t)j * k + b) * ldk;
         for (uint32_t wd = threadIdx.x; wd < words; wd += blockDim.x) {
             uint32_t bits = 0;
-            const uint32_t base = wd * 32;
 #pragma unroll 8
             for (uint32_t i = 0; i < 32; ++i) {
-                const uint32_t q = base + i;
-                if (q < cn) {
-                    const uint32_t c = col[q];
-                    bits |= (uint32_t)((__ldg(row + (c >> 6)) >> (c & 63)) & 1ull) << i;
-                }
+                const uint32_t q = wd * 32 + i;
+                if (q < ns) bits |= (uint32_t)((__ldg(row + (col[q] >> 6)) >> (col[q] & 63)) & 1ull) << i;
             }
-            T[((uint64_t)j * k + b) * ldT32 + c0 / 32 + wd] = bits;
+            T[((uint64_t)j * k + b) * words + wd] = bits;
         }
     }
 }
 
 constexpr int kCountWarps = 8;
-constexpr uint32_t kCountNodes = 4096;  // nodes w per CTA
+constexpr int kCountBits = 10;                            // vertical counters hold up to 1,023 rows
+constexpr uint32_t kCountMax = kCountWarps * 1016;        // nodes per CTA at most (1,016 = 127 x 8 per warp)
 
-__global__ void __launch_bounds__(32 * kCountWarps)
-    bitslice_count_kernel(const uint32_t *T, uint64_t ldT32, uint32_t R, uint32_t k, const uint32_t *H, uint32_t n,
-                          uint32_t ns, uint32_t *est)
+// full adder of bit columns: (c, a, b) -> sum in c, carry returned
+__device__ inline uint32_t add_bits(uint32_t &c, uint32_t a, uint32_t b)
 {
-    __shared__ uint32_t part[kCountWarps][32][33];
+    const uint32_t carry = (c & a) | (b & (c | a));
+    c = c ^ a ^ b;
+    return carry;
+}
+
+// Column counts of the chunk: a warp takes every eighth node of the CTA's range,
+// lane l the WPL words at 32 WPL sources.  Eight nodes at a time are added with
+// full adders into 10-bit vertical counters (three operations a word and node,
+// against sixteen for one node at a time), two nodes' R rows in flight; buckets of
+// the range are staged in shared memory.  Bound by the L2 reads of T (R rows a
+// node): n = 10^6, R = 8, 65,536 sources 5.6 ms at 12.8 TB/s (56 ms with the whole
+// table in DRAM, one word a lane and 4-bit counters); counts leave the registers
+// once.
+template <int WPL>
+__global__ void __launch_bounds__(32 * kCountWarps)
+    bitslice_count_kernel(const uint32_t *T, uint32_t words, uint32_t R, uint32_t k, const uint32_t *H, uint32_t n,
+                          uint32_t per_cta, uint32_t ns, uint32_t *est)
+{
+    extern __shared__ uint32_t sh[];
+    uint32_t *counts = sh;                       // [32 bits][32 WPL words]
+    uint32_t *rows = sh + 32 * 32 * WPL;         // [R][256] T rows of a batch of nodes
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const uint64_t word = (uint64_t)blockIdx.x * 32 + lane;  // 32-bit word of a T row (32 sources)
-    const bool live = word < (ns + 31) / 32;                  // words the table kernel wrote
-    const uint32_t w0 = blockIdx.y * kCountNodes;
-    const uint32_t w1 = min(n, w0 + kCountNodes);
-    uint32_t cnt[32];
+    for (uint32_t i = threadIdx.x; i < 32 * 32 * WPL; i += blockDim.x) counts[i] = 0;
+    const uint32_t w0 = blockIdx.x * per_cta, w1 = min(n, w0 + per_cta);
+    uint32_t c[kCountBits][WPL];
 #pragma unroll
-    for (int b = 0; b < 32; ++b) cnt[b] = 0;
-    uint32_t c0 = 0, c1 = 0, c2 = 0, c3 = 0, pending = 0;
-    for (uint32_t w = w0 + warp; w < w1; w += kCountWarps) {
-        uint32_t x = live ? 0xFFFFFFFFu : 0u;
-        for (uint32_t j = 0; j < R && x; ++j) {
-            const uint32_t b = __ldg(H + (uint64_t)j * n + w);
-            x &= __ldg(T + ((uint64_t)j * k + b) * ldT32 + word);
-        }
-        // add x to the 4-bit vertical counters
-        const uint32_t carry = c0 & x;
-        c0 ^= x;
-        const uint32_t carry2 = c1 & carry;
-        c1 ^= carry;
-        const uint32_t carry3 = c2 & carry2;
-        c2 ^= carry2;
-        c3 ^= carry3;
-        if (++pending == 15) {
+    for (int i = 0; i < kCountBits; ++i)
 #pragma unroll
-            for (int b = 0; b < 32; ++b)
-                cnt[b] += ((c0 >> b) & 1u) + (((c1 >> b) & 1u) << 1) + (((c2 >> b) & 1u) << 2) + (((c3 >> b) & 1u) << 3);
-            c0 = c1 = c2 = c3 = 0;
-            pending = 0;
+        for (int q = 0; q < WPL; ++q) c[i][q] = 0;
+    for (uint32_t base = w0; base < w1; base += 256) {
+        __syncthreads();
+        const uint32_t cnt = min(256u, w1 - base);
+        for (uint32_t j = warp; j < R; j += kCountWarps)
+            for (uint32_t i = lane; i < 256; i += 32)
+                rows[j * 256 + i] = i < cnt ? j * k + __ldg(H + (uint64_t)j * n + base + i) : 0xFFFFFFFFu;
+        __syncthreads();
+        // warp's nodes of the batch: 32 consecutive, eight at a time
+#pragma unroll 1
+        for (uint32_t e = 0; e < 4; ++e) {
+            const uint32_t at = warp * 32 + e * 8;
+            if (at >= cnt) break;
+            uint32_t two[4][WPL], four[2][WPL];
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {  // pairs of nodes
+                uint32_t x[2][WPL];
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int q = 0; q < WPL; ++q) x[h][q] = at + 2 * p + h < cnt ? 0xFFFFFFFFu : 0u;
+#pragma unroll 4
+                for (uint32_t j = 0; j < R; ++j) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const uint32_t r = rows[j * 256 + at + 2 * p + h];
+                        const uint32_t *t = T + (uint64_t)(r == 0xFFFFFFFFu ? 0u : r) * words + lane * WPL;
+                        if (WPL == 4) {
+                            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(t));
+                            x[h][0] &= v.x;
+                            x[h][1 % WPL] &= v.y;
+                            x[h][2 % WPL] &= v.z;
+                            x[h][3 % WPL] &= v.w;
+                        } else {
+                            x[h][0] &= __ldg(t);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < WPL; ++q) two[p][q] = add_bits(c[0][q], x[0][q], x[1][q]);
+            }
+#pragma unroll
+            for (int q = 0; q < WPL; ++q) {
+                four[0][q] = add_bits(c[1][q], two[0][q], two[1][q]);
+                four[1][q] = add_bits(c[1][q], two[2][q], two[3][q]);
+                uint32_t carry = add_bits(c[2][q], four[0][q], four[1][q]);
+#pragma unroll
+                for (int i = 3; i < kCountBits; ++i) {
+                    const uint32_t next = c[i][q] & carry;
+                    c[i][q] ^= carry;
+                    carry = next;
+                }
+            }
         }
     }
-#pragma unroll
-    for (int b = 0; b < 32; ++b)
-        cnt[b] += ((c0 >> b) & 1u) + (((c1 >> b) & 1u) << 1) + (((c2 >> b) & 1u) << 2) + (((c3 >> b) & 1u) << 3);
-#pragma unroll
-    for (int b = 0; b < 32; ++b) part[warp][lane][b] = cnt[b];
     __syncthreads();
-    for (uint32_t c = threadIdx.x; c < 1024; c += blockDim.x) {
-        const uint32_t l = c >> 5, bit = c & 31u;
-        uint32_t s = 0;
 #pragma unroll
-        for (int w = 0; w < kCountWarps; ++w) s += part[w][l][bit];
-        const uint64_t q = ((uint64_t)blockIdx.x * 32 + l) * 32 + bit;
-        if (s && q < ns) atomicAdd(&est[q], s);
+    for (int q = 0; q < WPL; ++q)
+#pragma unroll 1
+        for (int b = 0; b < 32; ++b) {
+            uint32_t v = 0;
+#pragma unroll
+            for (int i = 0; i < kCountBits; ++i) v |= ((c[i][q] >> b) & 1u) << i;
+            if (v) atomicAdd(&counts[b * 32 * WPL + q * 32 + lane], v);
+        }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < 32 * 32 * WPL; i += blockDim.x) {
+        const uint32_t b = i / (32 * WPL), q = (i / 32) % WPL, l = i % 32;
+        const uint32_t s = (l * WPL + q) * 32 + b;
+        if (s < ns && counts[i]) atomicAdd(&est[s], counts[i]);
     }
 }
 
@@ -302,21 +416,35 @@ extern "C" tn_status tn_hash_proxy(const uint32_t *u, const uint32_t *v, uint64_
 static tn_status estimate_bitsliced(const uint64_t *P, uint32_t R, uint32_t k, uint64_t ldk, const uint32_t *H,
                                     uint32_t n, const uint32_t *src, uint32_t nsrc, uint32_t *est, cudaStream_t st)
 {
-    // sources in chunks whose table stays within 2 GiB
-    uint32_t chunk = nsrc < 65536u ? nsrc : 65536u;
-    while (chunk > 1024 && (uint64_t)R * k * tn_row_words(chunk) * 8 > (2ull << 30)) chunk /= 2;
-    const uint64_t ldT32 = 2 * tn_row_words(chunk);
+    // four words a lane once that leaves no large part of a chunk empty
+    const uint32_t chunk = nsrc > 3072 && (uint64_t)R * k * 512 <= (2ull << 30) ? 4096u : 1024u;
+    const uint32_t words = chunk / 32;
+    const size_t tab_smem = (size_t)((k + 127) / 128) * 4 * kTabRows * 4;
+    const bool wide = tab_smem > kTabSmem;
+    const size_t cnt_smem = (32ull * words + 256ull * R) * 4;
     uint32_t *T = nullptr;
-    TN_CUDA_TRY(cudaMallocAsync((void **)&T, (uint64_t)R * k * ldT32 * 4, st));
+    TN_CUDA_TRY(cudaMallocAsync((void **)&T, (uint64_t)R * k * words * 4, st));
+    if (!wide) TN_CUDA_TRY(tn_internal_allow_max_dyn_smem((const void *)bitslice_table_kernel));
+    const void *count = chunk == 4096 ? (const void *)bitslice_count_kernel<4> : (const void *)bitslice_count_kernel<1>;
+    TN_CUDA_TRY(tn_internal_allow_max_dyn_smem(count));
+    // nodes per CTA: a multiple of the 256-node batch, about four CTAs per SM
+    uint32_t per_cta = (uint32_t)(((uint64_t)n / (152 * 4) + 255) / 256 * 256);
+    if (per_cta < 256) per_cta = 256;
+    if (per_cta > kCountMax / 256 * 256) per_cta = kCountMax / 256 * 256;
+    const unsigned blocks = (n + per_cta - 1) / per_cta;
     for (uint32_t s0 = 0; s0 < nsrc; s0 += chunk) {
         const uint32_t ns = nsrc - s0 < chunk ? nsrc - s0 : chunk;
-        const uint64_t ld32 = 2 * tn_row_words(ns);
-        // the count kernel reads only the ceil(ns / 32) words the table kernel writes
         tn_internal_count_launches(2);
-        bitslice_table_kernel<<<dim3((k + kTabRows - 1) / kTabRows, (ns + kTabSources - 1) / kTabSources, R),
-                                kTabThreads, 0, st>>>(P, k, ldk, H, n, src, s0, ns, ld32, T);
-        bitslice_count_kernel<<<dim3((unsigned)((ld32 + 31) / 32), (n + kCountNodes - 1) / kCountNodes),
-                                32 * kCountWarps, 0, st>>>(T, ld32, R, k, H, n, ns, est + s0);
+        if (wide)
+            bitslice_table_wide_kernel<<<dim3((k + 63) / 64, 1, R), kTabThreads, 0, st>>>(P, k, ldk, H, n, src, s0, ns,
+                                                                                         words, T);
+        else
+            bitslice_table_kernel<<<dim3((k + kTabRows - 1) / kTabRows, 1, R), kTabThreads, tab_smem, st>>>(
+                P, k, ldk, H, n, src, s0, ns, words, T);
+        if (chunk == 4096)
+            bitslice_count_kernel<4><<<blocks, 32 * kCountWarps, cnt_smem, st>>>(T, words, R, k, H, n, per_cta, ns, est + s0);
+        else
+            bitslice_count_kernel<1><<<blocks, 32 * kCountWarps, cnt_smem, st>>>(T, words, R, k, H, n, per_cta, ns, est + s0);
         TN_CUDA_TRY(cudaGetLastError());
     }
     TN_CUDA_TRY(cudaFreeAsync(T, st));
