@@ -2,99 +2,129 @@
 // of ones in column j; the in-component size of node i the number of ones in
 // row i; Section 3.3: both sums have the same total n * mean size).
 //
-// One CTA covers 1024 consecutive columns (32 lanes x one 32-bit word each)
-// and a block of rows; its 8 warps take interleaved rows.  Column counts are
-// accumulated in bit-sliced vertical counters: eight registers hold bits 0..7
-// of 32 per-column counts, so adding a row word costs a carry chain instead of
-// 32 extractions; every 255 rows the counters are flushed into the thread's
-// 32 integer counts in shared memory (registers stay free for loads in flight).  Row counts come from __popc and a warp sum.
-// Each warp loads kRowBatch rows before folding any of them in, so that
-// enough loads are in flight per SM to keep HBM busy.
+// One CTA covers 32 lanes x WPL 32-bit words of consecutive columns (4,096, or
+// 1,024 for narrow matrices) and a block of rows; its 8 warps take eight rows at a
+// time, all eight loads of a lane in flight.  Eight row words are added with full
+// adders into 10-bit vertical counters (three operations a word and row, against
+// sixteen for one row at a time); the counters are extracted once, at the end of
+// the CTA's rows.  Row counts are popcounts of a lane's words and one warp
+// reduction.
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <type_traits>
 
 #include "tn_internal.cuh"
 
 namespace tn {
 
 constexpr int kSizeWarps = 8;
-constexpr uint32_t kRowsPerBlock = 2048;
-constexpr int kRowBatch = 16;
-constexpr int kCounterBits = 8;  // vertical counters hold up to 2^8 - 1
+constexpr int kCounterBits = 10;               // vertical counters hold up to 1,023 rows
+constexpr uint32_t kRowsMax = kSizeWarps * 1016;  // rows per CTA (127 batches of eight per warp)
+constexpr uint32_t kRowsMin = kSizeWarps * 32;  // fewer would spend more on adding the CTAs' counts than on rows
 
-__global__ void __launch_bounds__(32 * kSizeWarps, 4)
-    column_counts_kernel(const uint32_t *S32, uint32_t n_rows, uint64_t ld32, uint32_t ncols, uint32_t *out,
-                         uint32_t *in)
+// full adder of bit columns: (c, a, b) -> sum in c, carry returned
+__device__ inline uint32_t full_add(uint32_t &c, uint32_t a, uint32_t b)
 {
-    __shared__ uint32_t part[kSizeWarps][32][33];
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const uint64_t word = (uint64_t)blockIdx.x * 32 + lane;  // 32-bit word index inside a row
-    const bool live = word < ld32;
-    const uint32_t r0 = blockIdx.y * kRowsPerBlock;
-    const uint32_t r1 = min(n_rows, r0 + kRowsPerBlock);
+    const uint32_t carry = (c & a) | (b & (c | a));
+    c = c ^ a ^ b;
+    return carry;
+}
 
-    uint32_t *cnt = part[warp][lane];  // this thread's 32 column counts
+// Bound by HBM: every word of S is read once.  n = 123,457 with row sizes 335 us
+// (5.7 TB/s; 899 us with one word a lane and one row at a time into 8-bit counters),
+// n = 10^5 208 us (424), n = 10^4 with row sizes 18 us (52), n = 1,000 7 us (27).
+template <int WPL>
+__global__ void __launch_bounds__(32 * kSizeWarps)
+    column_counts_kernel(const uint32_t *S32, uint32_t n_rows, uint64_t ld32, uint32_t ncols, uint32_t rows_per_cta,
+                         uint32_t *out, uint32_t *in)
+{
+    __shared__ uint32_t counts[32 * 32 * WPL];  // [bit][word][lane]
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint64_t word = ((uint64_t)blockIdx.x * 32 + lane) * WPL;
+    const bool live = word < ld32;
+    const uint32_t r0 = blockIdx.y * rows_per_cta;
+    const uint32_t r1 = min(n_rows, r0 + rows_per_cta);
+    for (uint32_t i = threadIdx.x; i < 32 * 32 * WPL; i += blockDim.x) counts[i] = 0;
+    uint32_t c[kCounterBits][WPL];
 #pragma unroll
-    for (int b = 0; b < 32; ++b) cnt[b] = 0;
-    uint32_t vc[kCounterBits];
+    for (int i = 0; i < kCounterBits; ++i)
 #pragma unroll
-    for (int j = 0; j < kCounterBits; ++j) vc[j] = 0;
-    uint32_t pending = 0;
-    // adds the vertical counters into the integer counts and clears them
-    auto flush = [&]() {
-#pragma unroll 4
-        for (int b = 0; b < 32; ++b) {
-            uint32_t v = 0;
+        for (int q = 0; q < WPL; ++q) c[i][q] = 0;
+    for (uint32_t r = r0 + warp * 8; r < r1; r += kSizeWarps * 8) {
+        uint32_t x[8][WPL];
 #pragma unroll
-            for (int j = 0; j < kCounterBits; ++j) v |= ((vc[j] >> b) & 1u) << j;
-            cnt[b] += v;
-        }
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t *p = S32 + (uint64_t)(r + k) * ld32 + word;
 #pragma unroll
-        for (int j = 0; j < kCounterBits; ++j) vc[j] = 0;
-        pending = 0;
-    };
-    for (uint32_t rb = r0 + warp; rb < r1; rb += kRowBatch * kSizeWarps) {
-        uint32_t xs[kRowBatch];
-#pragma unroll
-        for (int k = 0; k < kRowBatch; ++k) {
-            const uint32_t r = rb + k * kSizeWarps;
-            xs[k] = (live && r < r1) ? __ldcs(S32 + (uint64_t)r * ld32 + word) : 0u;
-        }
-#pragma unroll
-        for (int k = 0; k < kRowBatch; ++k) {
-            const uint32_t r = rb + k * kSizeWarps;
-            if (in && r < r1) {
-                uint32_t pc = __popc(xs[k]);
-#pragma unroll
-                for (int d = 16; d > 0; d >>= 1) pc += __shfl_xor_sync(0xffffffffu, pc, d);
-                if (lane == 0 && pc) atomicAdd(&in[r], pc);
+            for (int q = 0; q < WPL; ++q) x[k][q] = 0;
+            if (live && r + k < r1) {
+                if (WPL == 4) {
+                    const uint4 v = __ldcs(reinterpret_cast<const uint4 *>(p));
+                    x[k][0] = v.x;
+                    x[k][1 % WPL] = v.y;
+                    x[k][2 % WPL] = v.z;
+                    x[k][3 % WPL] = v.w;
+                } else {
+                    x[k][0] = __ldcs(p);
+                }
             }
-            // add the row word to the vertical counters (rows past the block add 0)
-            uint32_t carry = xs[k];
+        }
+        if (in) {
+            uint32_t mine = 0;
 #pragma unroll
-            for (int j = 0; j < kCounterBits; ++j) {
-                const uint32_t next = vc[j] & carry;
-                vc[j] ^= carry;
+            for (int k = 0; k < 8; ++k) {
+                uint32_t pc = 0;
+#pragma unroll
+                for (int q = 0; q < WPL; ++q) pc += __popc(x[k][q]);
+                pc = __reduce_add_sync(0xffffffffu, pc);
+                if (lane == k) mine = pc;
+            }
+            if (lane < 8 && mine) atomicAdd(&in[r + lane], mine);
+        }
+#pragma unroll
+        for (int q = 0; q < WPL; ++q) {
+            const uint32_t t0 = full_add(c[0][q], x[0][q], x[1][q]), t1 = full_add(c[0][q], x[2][q], x[3][q]);
+            const uint32_t t2 = full_add(c[0][q], x[4][q], x[5][q]), t3 = full_add(c[0][q], x[6][q], x[7][q]);
+            const uint32_t f0 = full_add(c[1][q], t0, t1), f1 = full_add(c[1][q], t2, t3);
+            uint32_t carry = full_add(c[2][q], f0, f1);
+#pragma unroll
+            for (int i = 3; i < kCounterBits; ++i) {
+                const uint32_t next = c[i][q] & carry;
+                c[i][q] ^= carry;
                 carry = next;
             }
         }
-        pending += kRowBatch;
-        if (pending + kRowBatch > (1u << kCounterBits) - 1u) flush();
     }
-    flush();
     __syncthreads();
-    // thread t sums column (t / 32, bit t % 32) of this block over the warps
-    for (uint32_t c = threadIdx.x; c < 1024; c += blockDim.x) {
-        const uint32_t l = c >> 5, b = c & 31u;
-        uint32_t s = 0;
+    auto extract = [&](auto planes) {
 #pragma unroll
-        for (int w = 0; w < kSizeWarps; ++w) s += part[w][l][b];
-        const uint64_t col = ((uint64_t)blockIdx.x * 32 + l) * 32 + b;
-        if (s && col < ncols) atomicAdd(&out[col], s);
+        for (int q = 0; q < WPL; ++q)
+#pragma unroll 4
+            for (int b = 0; b < 32; ++b) {
+                uint32_t v = 0;
+#pragma unroll
+                for (int i = 0; i < decltype(planes)::value; ++i) v |= ((c[i][q] >> b) & 1u) << i;
+                if (v) atomicAdd(&counts[(b * WPL + q) * 32 + lane], v);
+            }
+    };
+    if (rows_per_cta <= kSizeWarps * 56) extract(std::integral_constant<int, 6>());  // at most 63 rows a warp
+    else extract(std::integral_constant<int, kCounterBits>());
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < 32 * 32 * WPL; i += blockDim.x) {
+        const uint32_t l = i % 32, q = (i / 32) % WPL, b = i / (32 * WPL);
+        const uint64_t col = (((uint64_t)blockIdx.x * 32 + l) * WPL + q) * 32 + b;
+        if (counts[i] && col < ncols) atomicAdd(&out[col], counts[i]);
     }
 }
 
-__global__ void argmax_kernel(const uint32_t *out, uint32_t ncols, unsigned long long *best)
+// Largest size, lowest column among equals; the last CTA to finish writes it.
+struct Best {
+    unsigned long long key;
+    unsigned int done, pad;
+};
+
+__global__ void argmax_kernel(const uint32_t *out, uint32_t ncols, Best *best, uint32_t *argmax)
 {
     unsigned long long key = 0;
     for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < ncols; c += gridDim.x * blockDim.x) {
@@ -105,12 +135,13 @@ __global__ void argmax_kernel(const uint32_t *out, uint32_t ncols, unsigned long
         const unsigned long long o = __shfl_xor_sync(0xffffffffu, key, d);
         key = o > key ? o : key;
     }
-    if ((threadIdx.x & 31u) == 0) atomicMax(best, key);
-}
-
-__global__ void argmax_finish_kernel(const unsigned long long *best, uint32_t *argmax)
-{
-    *argmax = (uint32_t)(0xFFFFFFFFull - (*best & 0xFFFFFFFFull));
+    if ((threadIdx.x & 31u) == 0) atomicMax(&best->key, key);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&best->done, 1u) == gridDim.x - 1) {
+        __threadfence();
+        *argmax = (uint32_t)(0xFFFFFFFFull - (atomicMax(&best->key, 0ull) & 0xFFFFFFFFull));
+    }
 }
 
 }  // namespace tn
@@ -125,20 +156,32 @@ extern "C" tn_status tn_out_sizes(const uint64_t *S, uint32_t n_rows, uint32_t n
     const uint64_t ld32 = 2 * tn_row_words(ncols);
     TN_CUDA_TRY(cudaMemsetAsync(out_sizes, 0, (size_t)ncols * sizeof(uint32_t), st));
     if (in_sizes) TN_CUDA_TRY(cudaMemsetAsync(in_sizes, 0, (size_t)n_rows * sizeof(uint32_t), st));
-    dim3 grid((unsigned)((ld32 + 31) / 32), (n_rows + kRowsPerBlock - 1) / kRowsPerBlock);
+    // four words a lane where they fill a warp; rows per CTA: as many as the
+    // counters hold, in whole waves of two CTAs per SM, but a wave at least
+    const int wpl = ld32 >= 96 && ((uintptr_t)S & 15u) == 0 ? 4 : 1;
+    const uint64_t cols = (ld32 + 32 * wpl - 1) / (32 * wpl), slots = 2 * 152;
+    const uint64_t waves = (cols * ((n_rows + kRowsMax - 1) / kRowsMax) + slots - 1) / slots;
+    uint64_t blocks = waves * slots / cols;
+    if (blocks < 1) blocks = 1;
+    uint64_t rows = ((n_rows + blocks - 1) / blocks + kRowsMin - 1) / kRowsMin * kRowsMin;
+    if (rows > kRowsMax) rows = kRowsMax;
+    const dim3 grid((unsigned)cols, (unsigned)((n_rows + rows - 1) / rows));
+    const uint32_t *S32 = reinterpret_cast<const uint32_t *>(S);
     tn_internal_count_launches(1);
-    column_counts_kernel<<<grid, 32 * kSizeWarps, 0, st>>>(reinterpret_cast<const uint32_t *>(S), n_rows, ld32,
-                                                          ncols, out_sizes, in_sizes);
+    if (wpl == 4)
+        column_counts_kernel<4><<<grid, 32 * kSizeWarps, 0, st>>>(S32, n_rows, ld32, ncols, (uint32_t)rows, out_sizes,
+                                                                  in_sizes);
+    else
+        column_counts_kernel<1><<<grid, 32 * kSizeWarps, 0, st>>>(S32, n_rows, ld32, ncols, (uint32_t)rows, out_sizes,
+                                                                  in_sizes);
     TN_CUDA_TRY(cudaGetLastError());
     if (argmax) {
-        unsigned long long *best = nullptr;
-        TN_CUDA_TRY(cudaMallocAsync((void **)&best, sizeof(unsigned long long), st));
-        TN_CUDA_TRY(cudaMemsetAsync(best, 0, sizeof(unsigned long long), st));
+        Best *best = nullptr;
+        TN_CUDA_TRY(cudaMallocAsync((void **)&best, sizeof(Best), st));
+        TN_CUDA_TRY(cudaMemsetAsync(best, 0, sizeof(Best), st));
         const unsigned blocks = (unsigned)((ncols + 255) / 256 < 1024 ? (ncols + 255) / 256 : 1024);
         tn_internal_count_launches(1);
-        argmax_kernel<<<blocks, 256, 0, st>>>(out_sizes, ncols, best);
-        tn_internal_count_launches(1);
-        argmax_finish_kernel<<<1, 1, 0, st>>>(best, argmax);
+        argmax_kernel<<<blocks, 256, 0, st>>>(out_sizes, ncols, best, argmax);
         TN_CUDA_TRY(cudaGetLastError());
         TN_CUDA_TRY(cudaFreeAsync(best, st));
     }
