@@ -5,8 +5,8 @@
 // One pass over the pairs accumulates the absolute and relative errors and two
 // histograms of the values.  For integer samples of equal size the
 // Wasserstein-1 distance is the area between the two empirical CDFs, i.e.
-// sum over integers x of |#{est <= x} - #{exact <= x}| / count; a single CTA
-// scans the histogram difference to get that sum exactly, with no sort.
+// sum over integers x of |#{est <= x} - #{exact <= x}| / count; a scan
+// of the histogram difference gives that sum exactly, with no sort.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
@@ -23,7 +23,6 @@ struct ErrAccum {
 };
 
 constexpr int kErrThreads = 256;
-constexpr int kScanThreads = 1024;
 
 __global__ void __launch_bounds__(kErrThreads)
     error_pairs_kernel(const uint32_t *est, const uint32_t *exact, uint32_t count, uint32_t max_value,
@@ -67,41 +66,91 @@ __global__ void __launch_bounds__(kErrThreads)
     }
 }
 
-// One CTA: w1_num = sum over x in [0, max_value] of |C(x)|, C(x) = prefix sum of
-// hist_est - hist_exact up to x.  Thread t owns a contiguous chunk of x.
-__global__ void __launch_bounds__(kScanThreads)
-    error_w1_kernel(const uint32_t *hist_est, const uint32_t *hist_exact, uint32_t max_value, ErrAccum *acc)
+// w1_num = sum over x in [0, max_value] of |C(x)|, C(x) = prefix sum of
+// hist_est - hist_exact up to x.  Every CTA takes `tiles` consecutive tiles of
+// kW1Bins bins (four a thread), at most kW1Ctas CTAs: the first kernel sums the
+// differences of a CTA's bins, the second adds the sums of the CTAs before it and
+// scans its own.  max_value = 10^6: 9 us for both (863 us in one CTA).
+constexpr int kW1Threads = 256;
+constexpr uint32_t kW1Bins = 4 * kW1Threads;
+constexpr uint64_t kW1Ctas = 2048;
+
+// Differences of this thread's four bins of tile `tile`.
+__device__ inline void w1_load(const uint32_t *hist_est, const uint32_t *hist_exact, uint64_t len, uint64_t tile,
+                               long long d[4])
 {
-    __shared__ long long part[kScanThreads];
-    __shared__ unsigned long long tot[kScanThreads / 32];
-    const uint64_t len = (uint64_t)max_value + 1;
-    const uint64_t chunk = (len + kScanThreads - 1) / kScanThreads;
-    const uint64_t x0 = threadIdx.x * chunk, x1 = x0 + chunk < len ? x0 + chunk : len;
-    long long local = 0;
-    for (uint64_t x = x0; x < x1; ++x) local += (long long)hist_est[x] - (long long)hist_exact[x];
-    part[threadIdx.x] = local;
-    __syncthreads();
-    // inclusive Hillis-Steele scan of the chunk sums
-    for (int o = 1; o < kScanThreads; o <<= 1) {
-        const long long v = threadIdx.x >= (unsigned)o ? part[threadIdx.x - o] : 0;
-        __syncthreads();
-        part[threadIdx.x] += v;
-        __syncthreads();
+    const uint64_t x = tile * kW1Bins + 4 * threadIdx.x;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        d[k] = x + k < len ? (long long)hist_est[x + k] - (long long)hist_exact[x + k] : 0;
+}
+
+__device__ inline long long w1_warp_sum(long long s)
+{
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+__global__ void __launch_bounds__(kW1Threads)
+    error_w1_sums_kernel(const uint32_t *hist_est, const uint32_t *hist_exact, uint64_t len, uint64_t tiles,
+                         long long *part)
+{
+    __shared__ long long warp_sum[kW1Threads / 32];
+    long long s = 0, d[4];
+    for (uint64_t i = 0; i < tiles; ++i) {
+        w1_load(hist_est, hist_exact, len, blockIdx.x * tiles + i, d);
+        s += d[0] + d[1] + d[2] + d[3];
     }
-    long long c = threadIdx.x ? part[threadIdx.x - 1] : 0;
-    unsigned long long w = 0;
-    for (uint64_t x = x0; x < x1; ++x) {
-        c += (long long)hist_est[x] - (long long)hist_exact[x];
-        w += (unsigned long long)(c < 0 ? -c : c);
-    }
-    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-    if ((threadIdx.x & 31u) == 0) tot[threadIdx.x >> 5] = w;
+    s = w1_warp_sum(s);
+    if ((threadIdx.x & 31u) == 0) warp_sum[threadIdx.x >> 5] = s;
     __syncthreads();
     if (threadIdx.x == 0) {
-        unsigned long long t = 0;
-        for (int i = 0; i < kScanThreads / 32; ++i) t += tot[i];
-        acc->w1_num = t;
+        long long t = 0;
+        for (int w = 0; w < kW1Threads / 32; ++w) t += warp_sum[w];
+        part[blockIdx.x] = t;
     }
+}
+
+__global__ void __launch_bounds__(kW1Threads)
+    error_w1_kernel(const uint32_t *hist_est, const uint32_t *hist_exact, uint64_t len, uint64_t tiles,
+                    const long long *part, ErrAccum *acc)
+{
+    __shared__ long long warp_sum[kW1Threads / 32], before[kW1Threads / 32];
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    long long b = 0;  // the CTAs before this one
+    for (uint32_t i = threadIdx.x; i < blockIdx.x; i += blockDim.x) b += part[i];
+    b = w1_warp_sum(b);
+    if (lane == 0) before[warp] = b;
+    __syncthreads();
+    long long carry = 0;
+    for (int w = 0; w < kW1Threads / 32; ++w) carry += before[w];
+    unsigned long long w1 = 0;
+    for (uint64_t i = 0; i < tiles; ++i) {
+        const uint64_t tile = blockIdx.x * tiles + i, x = tile * kW1Bins + 4 * threadIdx.x;
+        long long d[4];
+        w1_load(hist_est, hist_exact, len, tile, d);
+        const long long mine = d[0] + d[1] + d[2] + d[3];
+        long long incl = mine;
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= (uint32_t)o) incl += y;
+        }
+        __syncthreads();  // the last tile's sums are read
+        if (lane == 31) warp_sum[warp] = incl;
+        __syncthreads();
+        long long c = carry + incl - mine;
+        for (uint32_t w = 0; w < kW1Threads / 32; ++w) {
+            if (w < warp) c += warp_sum[w];
+            carry += warp_sum[w];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            c += d[k];
+            if (x + k < len) w1 += (unsigned long long)(c < 0 ? -c : c);
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) w1 += __shfl_xor_sync(0xffffffffu, w1, o);
+    if (lane == 0 && w1) atomicAdd(&acc->w1_num, w1);
 }
 
 }  // namespace tn
@@ -117,17 +166,23 @@ extern "C" tn_status tn_error_stats_compute(const uint32_t *est, const uint32_t 
     uint32_t *hist = nullptr;
     ErrAccum *acc = nullptr;
     ErrAccum h;
+    const uint64_t w1_tiles = (len + kW1Bins - 1) / kW1Bins, per_cta = (w1_tiles + kW1Ctas - 1) / kW1Ctas;
+    const unsigned w1_blocks = (unsigned)((w1_tiles + per_cta - 1) / per_cta);
+    long long *part = nullptr;
     TN_CUDA_TRY(cudaMallocAsync((void **)&hist, 2 * len * sizeof(uint32_t), st));
+    TN_CUDA_TRY(cudaMallocAsync((void **)&part, w1_blocks * sizeof(long long), st));
     TN_CUDA_TRY(cudaMallocAsync((void **)&acc, sizeof(ErrAccum), st));
     TN_CUDA_TRY(cudaMemsetAsync(hist, 0, 2 * len * sizeof(uint32_t), st));
     TN_CUDA_TRY(cudaMemsetAsync(acc, 0, sizeof(ErrAccum), st));
     const unsigned blocks = (count + kErrThreads - 1) / kErrThreads < 2048 ? (count + kErrThreads - 1) / kErrThreads : 2048;
-    tn_internal_count_launches(2);
+    tn_internal_count_launches(3);
     error_pairs_kernel<<<blocks, kErrThreads, 0, st>>>(est, exact, count, max_value, hist, hist + len, acc);
-    error_w1_kernel<<<1, kScanThreads, 0, st>>>(hist, hist + len, max_value, acc);
+    error_w1_sums_kernel<<<w1_blocks, kW1Threads, 0, st>>>(hist, hist + len, len, per_cta, part);
+    error_w1_kernel<<<w1_blocks, kW1Threads, 0, st>>>(hist, hist + len, len, per_cta, part, acc);
     TN_CUDA_TRY(cudaGetLastError());
     TN_CUDA_TRY(cudaMemcpyAsync(&h, acc, sizeof(h), cudaMemcpyDeviceToHost, st));
     TN_CUDA_TRY(cudaFreeAsync(hist, st));
+    TN_CUDA_TRY(cudaFreeAsync(part, st));
     TN_CUDA_TRY(cudaFreeAsync(acc, st));
     TN_CUDA_TRY(cudaStreamSynchronize(st));
     if (h.bad) return TN_ERANGE;

@@ -36,3 +36,14 @@ def test_estimates(n, k, R, nsrc):
     est = tn.tn_hash_estimate(dP, R, k, dH, n, src=None if src is None else torch.from_numpy(src.view(np.int32)).cuda())
     ref = oracle.hash_estimate(P[:, :, :full], H, n, src)
     assert np.array_equal(est.cpu().numpy().view(np.uint32), ref)
+
+
+@pytest.mark.parametrize("max_value", [1, 1022, 1023, 1024, 5000, 2_097_151, 2_097_152, 5_000_000])
+def test_error_scan(max_value):
+    """Histogram scans of one tile, of several CTAs, and of several tiles per CTA."""
+    rng = np.random.default_rng(max_value)
+    exact = rng.integers(1, max_value + 1, 4001).astype(np.uint32)
+    est = rng.integers(0, max_value + 1, 4001).astype(np.uint32)
+    got = tn.tn_error_stats(torch.from_numpy(est.view(np.int32)).cuda(), torch.from_numpy(exact.view(np.int32)).cuda(), max_value)
+    assert got["w1_num"] == int(np.abs(np.sort(est).astype(np.int64) - np.sort(exact).astype(np.int64)).sum())
+    assert got["sum_abs"] == int(np.abs(est.astype(np.int64) - exact.astype(np.int64)).sum())
