@@ -31,8 +31,8 @@
 //      pair, by all threads;
 //   3. one warp walks the window in time order, 16 events (32 endpoints) at a
 //      time, and assigns levels (level of an update = 1 + last level at which
-//      any of its rows was touched); every group that shares nodes is handed
-//      to the whole CTA;
+//      any of its rows was touched); a group that shares nodes is scheduled on
+//      the way, a large one by the whole CTA;
 //   4. the window's updates are counting-sorted by level into packs that the
 //      streaming kernel copies whole (tn_internal.cuh describes the layout).
 #include <cuda_runtime.h>
@@ -58,6 +58,9 @@ constexpr uint32_t kRecordEvents = 2048;
 // Groups of at least this many events go to the whole CTA unchecked: comparing
 // their events pair by pair would cost more than the group's own phases.
 constexpr uint32_t kPairGroup = 128;
+// Groups that share nodes and are no longer than this stay with the warp that walks
+// the window: the CTA's barriers would take longer than the group (2.5 us each).
+constexpr uint32_t kWarpGroup = 128;
 // Networks below this size whose slab width is given keep record windows unless
 // the batch is long enough for rows to settle: their levels are short and deep
 // (bursty n = 20,011, 500,009 events, 16 words: 6.6 ms, 11.4 ms in tiles).
@@ -281,21 +284,25 @@ __device__ inline uint32_t level_append(uint32_t *lh, uint32_t level, bool act)
 // saved rows, largest level, next event, end of the group handed over.
 enum { kScRuns = 0, kScAux, kScTemp, kScMaxlev, kScNext, kScEnd, kScCount };
 
-// The snapshot rule for one timestamp group [i, g1) with every thread of the
-// CTA.  The numbering of runs and slots, the order of ops inside a level and
+// The snapshot rule for one timestamp group [i, g1), with every thread of the CTA
+// or (kWarp) with one warp.  The numbering of runs and slots, the order of ops inside a level and
 // of sources inside a PULL list are unspecified; none of them changes the
 // result.  In an undirected group, nodes that occur once take part in exactly
 // one event, so a lone event (both ends once) touches no other event's rows and
 // gets its level at once; the other events share one level L = 1 + the latest
 // level of their nodes, with the PULLs at L + 1.  Phases are separated by
 // barriers, so a run's and a slot's number are final before anyone reads them.
-template <typename I>
+template <typename I, bool kWarp>
 __device__ void schedule_group(uint32_t i, uint32_t g1, bool directed, const Arena<I> &A, uint32_t *ncnt, I *nlev,
                                I *nrun, uint32_t *auxw, uint32_t *sc)
 {
     constexpr I kNone = (I)~(I)0, kClaim = (I)(kNone - 1);
     __shared__ uint32_t Lc, any, run0;
-    const uint32_t T = blockDim.x, tid = threadIdx.x;
+    const uint32_t T = kWarp ? 32u : blockDim.x, tid = kWarp ? threadIdx.x & 31u : threadIdx.x;
+    auto phase_end = [] {
+        if (kWarp) __syncwarp();
+        else __syncthreads();
+    };
     for (uint32_t j = i + tid; j < g1; j += T) {
         const uint32_t x = A.lu[j], y = A.lv[j];
         ncnt[x] = 0;
@@ -308,14 +315,14 @@ __device__ void schedule_group(uint32_t i, uint32_t g1, bool directed, const Are
         any = 0;
         run0 = sc[kScRuns];
     }
-    __syncthreads();
+    phase_end();
     for (uint32_t j = i + tid; j < g1; j += T) {
         const uint32_t x = A.lu[j], y = A.lv[j];
         if (x == y) continue;
         if (!directed) atomicAdd(&ncnt[x], 1u);
         atomicAdd(&ncnt[y], 1u);
     }
-    __syncthreads();
+    phase_end();
     // roles; lone events' levels; one run (PULL) per node occurring several
     // times (directed: per receiver)
     auto claim_run = [&](uint32_t x) {
@@ -351,7 +358,7 @@ __device__ void schedule_group(uint32_t i, uint32_t g1, bool directed, const Are
         if (sx && !directed) claim_run(x);
         if (sy) claim_run(y);
     }
-    __syncthreads();
+    phase_end();
     // saved rows: a node with a run that another run reads is read from a copy
     // of its old row
     auto claim_temp = [&](uint32_t r) {
@@ -362,7 +369,7 @@ __device__ void schedule_group(uint32_t i, uint32_t g1, bool directed, const Are
             if (nrun[A.lu[j]] != kNone) claim_temp(nrun[A.lu[j]]);
             if (!directed) claim_temp(nrun[A.lv[j]]);
         }
-    __syncthreads();
+    phase_end();
     // source lists (entries: local row ids, or temp references)
     auto add_source = [&](uint32_t node, uint32_t from) {
         const uint32_t r = nrun[node];
@@ -377,7 +384,7 @@ __device__ void schedule_group(uint32_t i, uint32_t g1, bool directed, const Are
         if ((f & kFlagShA) && !directed) add_source(x, y);
         if (f & kFlagShB) add_source(y, x);
     }
-    __syncthreads();
+    phase_end();
     // levels of the shared part: ONEWAY / COPY at L, PULL at L + 1
     if (any) {
         const uint32_t L = Lc + 1;
@@ -390,7 +397,7 @@ __device__ void schedule_group(uint32_t i, uint32_t g1, bool directed, const Are
         for (uint32_t r = run0 + tid; r < sc[kScRuns]; r += T) A.run_lev[r] = L;
         if (tid == 0) atomicMax(&sc[kScMaxlev], L + 1);
     }
-    __syncthreads();
+    phase_end();
 }
 
 // Levels of the events from sc[kScNext] up to the next group that shares
@@ -593,11 +600,21 @@ __device__ void schedule_window(const PlanArgs &a, uint32_t w, uint8_t *arena)
     // 3. levels in time order
     uint32_t *auxw = a.aux + 3 * s;
     for (;;) {
-        if (tid < 32) scan_levels(E, a.directed != 0, A, nlev, sc);
+        if (tid < 32) {
+            for (;;) {
+                scan_levels(E, a.directed != 0, A, nlev, sc);
+                __syncwarp();
+                const uint32_t i = sc[kScNext], g1 = sc[kScEnd];
+                if (i >= E || g1 - i > kWarpGroup) break;
+                schedule_group<I, true>(i, g1, a.directed != 0, A, ncnt, nlev, nrun, auxw, sc);
+                if (lane == 0) sc[kScNext] = g1;
+                __syncwarp();
+            }
+        }
         __syncthreads();
         const uint32_t next = sc[kScNext], end = sc[kScEnd];
         if (next >= E) break;
-        schedule_group(next, end, a.directed != 0, A, ncnt, nlev, nrun, auxw, sc);
+        schedule_group<I, false>(next, end, a.directed != 0, A, ncnt, nlev, nrun, auxw, sc);
         if (tid == 0) sc[kScNext] = end;
         __syncthreads();
     }
