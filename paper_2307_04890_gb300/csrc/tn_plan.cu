@@ -56,11 +56,13 @@ constexpr uint32_t kEmpty = 0xFFFFFFFFu;
 // Windows of up to this many events may become shared-memory records.
 constexpr uint32_t kRecordEvents = 2048;
 // Groups of at least this many events go to the whole CTA unchecked: comparing
-// their events pair by pair would cost more than the group's own phases.
-constexpr uint32_t kPairGroup = 128;
+// their events pair by pair would cost more than the group's own phases (bursty
+// n = 20,011, 500,009 events, groups of 107: plan 0.21 ms at 128, 0.18 ms at 48;
+// uniform and activity-driven batches take the same time with both).
+constexpr uint32_t kPairGroup = 48;
 // Groups that share nodes and are no longer than this stay with the warp that walks
 // the window: the CTA's barriers would take longer than the group (2.5 us each).
-constexpr uint32_t kWarpGroup = 128;
+constexpr uint32_t kWarpGroup = 48;
 // Networks below this size whose slab width is given keep record windows unless
 // the batch is long enough for rows to settle: their levels are short and deep
 // (bursty n = 20,011, 500,009 events, 16 words: 6.6 ms, 11.4 ms in tiles).
@@ -73,6 +75,9 @@ constexpr uint32_t kTileRows = 24928;
 // ms at 5,000 (windows of two groups leave shared memory); n = 1,000, 20,000
 // uniform events: 0.10 + 0.08 ms at 1,280, 0.14 + 0.08 ms at 2,480.
 static uint32_t default_window(uint64_t m) { return m < (1u << 16) ? 1280u : 2000u; }
+// Room of the first pass's arena behind the target: a window is stretched by the
+// rest of its last timestamp group (2,400 events: two CTAs per SM).
+constexpr uint32_t kWindowSlack = 400;
 // Batches of at least this many events are copied into buffers of their exact
 // size; below it the staging buffers (a few times larger, bounded) are kept.
 constexpr uint64_t kCompactEvents = 1ull << 20;
@@ -109,7 +114,7 @@ __host__ __device__ inline uint64_t scratch_words(uint64_t E)
 template <typename I>
 __host__ __device__ inline uint64_t arena_bytes(uint64_t E)
 {
-    return (4 * (scratch_words<I>(E) + 3 * E) + sizeof(I) * 6 * E + 3 * E + 15) & ~15ull;
+    return (8 * ((E + 15) / 16) + 4 * (scratch_words<I>(E) + 3 * E) + sizeof(I) * 6 * E + E + 15) & ~15ull;
 }
 
 template <typename I>
@@ -119,10 +124,11 @@ struct Arena {
     uint32_t *scratch;
     I *lu, *lv, *evl, *run_node, *run_aux, *run_temp;  // [E] each
     uint8_t *flg;       // [E]
-    uint8_t *claim;     // [2E] a lane of the chunk being checked, per row
+    uint2 *chunk;       // [ceil(E / 16)] chunks of the level walk
     __device__ Arena(uint8_t *p, uint32_t E)
     {
-        rowsg = reinterpret_cast<uint32_t *>(p);
+        chunk = reinterpret_cast<uint2 *>(p);
+        rowsg = reinterpret_cast<uint32_t *>(chunk + (E + 15) / 16);
         run_lev = rowsg + 2 * (uint64_t)E;
         scratch = run_lev + E;
         lu = reinterpret_cast<I *>(scratch + scratch_words<I>(E));
@@ -132,7 +138,6 @@ struct Arena {
         run_aux = run_node + E;
         run_temp = run_aux + E;
         flg = reinterpret_cast<uint8_t *>(run_temp + E);
-        claim = flg + E;
     }
 };
 
@@ -293,7 +298,7 @@ enum { kScRuns = 0, kScAux, kScTemp, kScMaxlev, kScNext, kScEnd, kScCount };
 // level of their nodes, with the PULLs at L + 1.  Phases are separated by
 // barriers, so a run's and a slot's number are final before anyone reads them.
 template <typename I, bool kWarp>
-__device__ void schedule_group(uint32_t i, uint32_t g1, bool directed, const Arena<I> &A, uint32_t *ncnt, I *nlev,
+__device__ __forceinline__ void schedule_group(uint32_t i, uint32_t g1, bool directed, const Arena<I> &A, uint32_t *ncnt, I *nlev,
                                I *nrun, uint32_t *auxw, uint32_t *sc)
 {
     constexpr I kNone = (I)~(I)0, kClaim = (I)(kNone - 1);
@@ -400,54 +405,76 @@ __device__ void schedule_group(uint32_t i, uint32_t g1, bool directed, const Are
     phase_end();
 }
 
-// Levels of the events from sc[kScNext] up to the next group that shares
-// nodes, by warp 0: lane 2k + side holds one endpoint of the chunk's event k.
-// Each event's level needs only its two nodes' last levels, so a chunk without
-// repeated nodes takes one round: a shared-memory read, a shuffle, a write.
-// Repeated nodes are found one chunk ahead (every lane writes its number to its
-// node's claim and reads it back), off the chain from level to level; in such a
-// chunk an event waits until the earlier events on its nodes are done.  (The
-// warp's match instruction in every chunk made the walk 7 times as long: 770
-// cycles a chunk.)
+// Chunks of 16 events (32 endpoints: lane 2k + side holds one endpoint of event
+// k), prepared by all warps: their events' flags, and per chunk the lanes that take
+// part (no self-loops), whether a node occurs twice, whether a group that shares
+// nodes begins in it.
+constexpr uint32_t kChunkTwice = 1u, kChunkHard = 2u;
+
 template <typename I>
-__device__ void scan_levels(uint32_t E, bool directed, const Arena<I> &A, I *nlev, uint32_t *sc)
+__device__ __forceinline__ void prepare_chunks(uint32_t E, bool directed, const Arena<I> &A)
 {
     const uint32_t lane = threadIdx.x & 31u, side = lane & 1u;
     const I *mine = side ? A.lv : A.lu;
-    uint32_t i = sc[kScNext], top = 0, end = E;
-    uint32_t x = 0, f = 0, twice = 0;
-    bool run = false, live = false;  // before the group; not a self-loop
-    uint32_t stop = 16u;             // events of the chunk before the group
-    auto fetch = [&](uint32_t at) {
-        const uint32_t e = at + (lane >> 1);
-        x = e < E ? (uint32_t)mine[e] : 0u;
-        f = e < E ? (uint32_t)A.flg[e] : 0u;
-        const uint32_t hard = __ballot_sync(0xffffffffu, f & kFlagHard);
-        stop = hard ? (__ffs(hard) - 1) >> 1 : 16u;
-        run = e < E && (lane >> 1) < stop;
+    for (uint32_t c = threadIdx.x >> 5; 16 * c < E; c += blockDim.x >> 5) {
+        const uint32_t e = 16 * c + (lane >> 1);
+        const uint32_t x = e < E ? (uint32_t)mine[e] : 0u, f = e < E ? (uint32_t)A.flg[e] : 0u;
         const uint32_t other = __shfl_xor_sync(0xffffffffu, x, 1);
-        live = run && x != other;
-        if (live) A.claim[x] = (uint8_t)lane;
-        __syncwarp();
-        const bool lost = live && A.claim[x] != (uint8_t)lane;
-        twice = __ballot_sync(0xffffffffu, lost);
-        __syncwarp();
+        const bool live = e < E && x != other;
+        const uint32_t same = __match_any_sync(0xffffffffu, live ? x : 0x80000000u | lane);
+        const bool twice = __any_sync(0xffffffffu, same & (same - 1u)), hard = __any_sync(0xffffffffu, f & kFlagHard);
+        const uint32_t lanes = __ballot_sync(0xffffffffu, live);
+        if (e < E && !side) A.flg[e] = (uint8_t)(f | (!live ? kFlagNoop : directed ? kFlagDir : kFlagIso));
+        if (lane == 0) A.chunk[c] = make_uint2(lanes, (twice ? kChunkTwice : 0u) | (hard ? kChunkHard : 0u));
+    }
+}
+
+// Levels of the events from sc[kScNext] up to the next group that shares nodes,
+// by warp 0.  Each event's level needs only its two nodes' last levels, so a chunk
+// without repeated nodes takes one round: a shared-memory read, a shuffle, a write.
+// In a chunk with repeated nodes an event waits until the earlier events on its
+// nodes are done.  One warp's walk is bound by the number of dependent
+// instructions, so everything else about a chunk is prepared by all warps (550
+// cycles a chunk before, 770 with a match in every chunk).
+template <typename I>
+__device__ __forceinline__ void scan_levels(uint32_t E, const Arena<I> &A, I *nlev, uint32_t *sc)
+{
+    const uint32_t lane = threadIdx.x & 31u, side = lane & 1u;
+    const I *mine = side ? A.lv : A.lu;
+    const uint32_t first = sc[kScNext];
+    uint32_t c = first >> 4, top = 0, end = E;
+    const uint32_t chunks = (E + 15u) >> 4;
+    // events before `first` are done
+    uint32_t keep = 0xffffffffu << (2u * (first & 15u));
+    auto load = [&](uint32_t k) {
+        const uint32_t e = 16 * k + (lane >> 1);
+        return e < E ? (uint32_t)mine[e] : 0u;
     };
-    fetch(i);
-    while (i < E) {
-        const uint32_t node = x, e = i + (lane >> 1), conflict = twice, before_group = stop;
-        const bool act = run, go1 = live;
-        if (before_group == 16u) fetch(i + 16u);  // independent of this chunk's levels
+    uint32_t x = load(c);
+    uint2 info = c < chunks ? A.chunk[c] : make_uint2(0u, 0u);
+    for (; c < chunks; ++c) {
+        const uint32_t node = x, e = 16 * c + (lane >> 1), what = info.y;
+        uint32_t lanes = info.x & keep, stop = 16u;
+        keep = 0xffffffffu;
+        x = load(c + 1);
+        if (c + 1 < chunks) info = A.chunk[c + 1];
+        if (what & kChunkHard) {  // the first such group at or behind `first` ends the walk
+            const uint32_t hard = __ballot_sync(0xffffffffu, e >= first && e < E && (A.flg[e] & kFlagHard));
+            if (hard) {
+                stop = (__ffs(hard) - 1) >> 1;
+                lanes &= (1u << (2u * stop)) - 1u;
+            }
+        }
+        const bool live = (lanes >> lane) & 1u;
         uint32_t lev = 0;
-        if (!conflict) {
-            lev = go1 ? (uint32_t)nlev[node] : 0u;
+        if (!(what & kChunkTwice)) {
+            lev = live ? (uint32_t)nlev[node] : 0u;
             lev = max(lev, __shfl_xor_sync(0xffffffffu, lev, 1)) + 1u;
-            if (go1) nlev[node] = (I)lev;
-            __syncwarp();
+            if (live) nlev[node] = (I)lev;
         } else {
-            const uint32_t same = __match_any_sync(0xffffffffu, go1 ? node : 0x80000000u | lane);
+            const uint32_t same = __match_any_sync(0xffffffffu, live ? node : 0x80000000u | lane);
             const uint32_t before = same & ((1u << lane) - 1u);
-            uint32_t pending = __ballot_sync(0xffffffffu, go1);
+            uint32_t pending = lanes;
             while (pending) {
                 const uint32_t ready = __ballot_sync(0xffffffffu, ((pending >> lane) & 1u) && !(before & pending));
                 const uint32_t both = ready & (((ready & 0x55555555u) << 1) | ((ready >> 1) & 0x55555555u));
@@ -462,16 +489,15 @@ __device__ void scan_levels(uint32_t E, bool directed, const Arena<I> &A, I *nle
                 pending &= ~both;
             }
         }
-        if (go1) top = max(top, lev);
-        if (act && !side) {
-            A.evl[e] = (I)lev;
-            A.flg[e] = !go1 ? kFlagNoop : directed ? kFlagDir : kFlagIso;
+        __syncwarp();
+        if (live) {
+            A.evl[e] = (I)lev;  // (both endpoints' lanes write the same level)
+            top = max(top, lev);
         }
-        if (before_group < 16u) {
-            end = i + before_group;
+        if (stop < 16u) {
+            end = 16 * c + stop;
             break;
         }
-        i += 16u;
     }
     __syncwarp();
     top = __reduce_max_sync(0xffffffffu, top);
@@ -498,7 +524,7 @@ __device__ void scan_levels(uint32_t E, bool directed, const Arena<I> &A, I *nle
 }
 
 template <typename I>
-__device__ void schedule_window(const PlanArgs &a, uint32_t w, uint8_t *arena)
+__device__ __forceinline__ void schedule_window(const PlanArgs &a, uint32_t w, uint8_t *arena)
 {
     __shared__ uint32_t warp_sums[32];
     __shared__ uint32_t tot;
@@ -598,11 +624,13 @@ __device__ void schedule_window(const PlanArgs &a, uint32_t w, uint8_t *arena)
     __syncthreads();
 
     // 3. levels in time order
+    prepare_chunks(E, a.directed != 0, A);
+    __syncthreads();
     uint32_t *auxw = a.aux + 3 * s;
     for (;;) {
         if (tid < 32) {
             for (;;) {
-                scan_levels(E, a.directed != 0, A, nlev, sc);
+                scan_levels(E, A, nlev, sc);
                 __syncwarp();
                 const uint32_t i = sc[kScNext], g1 = sc[kScEnd];
                 if (i >= E || g1 - i > kWarpGroup) break;
@@ -1075,8 +1103,7 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     a.directed = opt ? opt->directed : 0u;
     a.nw = (uint32_t)((m + window - 1) / window);
     a.smem_max = smem_max_events();
-    // room for the rest of a small timestamp group behind the target
-    const uint64_t first_max = (uint64_t)window + 64 < m ? (uint64_t)window + 64 : m;
+    const uint64_t first_max = (uint64_t)window + kWindowSlack < m ? (uint64_t)window + kWindowSlack : m;
     a.first_max = first_max < a.smem_max ? (uint32_t)first_max : a.smem_max;
     a.dcap = rows;
     a.unit8 = window <= kRecordEvents && rows > 1 && records ? 5 : 4;
