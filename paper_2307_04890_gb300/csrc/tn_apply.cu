@@ -1166,8 +1166,8 @@ __device__ inline void apply_record(const Job &J, const uint32_t *rec, u64x2 *bu
 // The plan holds tile packs only (node-id ops).  Consumers take one op each of
 // the current segment (its ops are independent), fetch their op of the next
 // segment beside it, and meet at a named barrier; a level costs its barrier and
-// the latency of two dependent shared-memory accesses (0.17 us for 55 ops, 0.33
-// us for 225: bank conflicts of random rows).
+// about 60 instructions (resident_levels; larger ones also the bank conflicts of
+// random rows: 0.12 us for 93 ops, 0.18 us for 319).
 // Once a pack changes nothing, the next one is checked as a whole without its
 // level barriers (if no op changes a row as the rows stand, none does), and after
 // a run of such packs the rows are compared with their component's root rows: when
@@ -1271,6 +1271,13 @@ __device__ inline uint32_t lds_u16(uint32_t a)
     return r;
 }
 
+__device__ inline uint32_t lds_u32(uint32_t a)
+{
+    uint32_t r;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(r) : "r"(a) : "memory");
+    return r;
+}
+
 template <int RW>
 __device__ inline bool same_row(const RRow<RW> &a, const RRow<RW> &b)
 {
@@ -1280,43 +1287,8 @@ __device__ inline bool same_row(const RRow<RW> &a, const RRow<RW> &b)
     return same;
 }
 
-// One op of a tile pack on the resident rows (shared address rb, node ids) and
-// the saved rows (shared address tb, temp ids); whether a row changed.
-template <bool kMax, int RW>
-__device__ inline bool resident_op(uint2 op, uint32_t rb, uint32_t tb, const uint32_t *aux, const uint32_t *pack)
-{
-    constexpr uint32_t kRowB = 8u * RW;
-    const uint32_t kind = op.x >> kKindShift, a = op.x & kIdMask;
-    if (kind != kPull) {  // one path for EVENT, ONEWAY and COPY: they share warps
-        const uint32_t pa = (kind == kCopy ? tb : rb) + a * kRowB, pb = rb + op.y * kRowB;
-        const RRow<RW> x = lds_rrow<RW>(pa), y = lds_rrow<RW>(pb);
-        const RRow<RW> r = kind == kCopy ? y : rcombine<kMax, RW>(x, y);
-        const bool new_a = !same_row<RW>(r, x), new_b = kind == kEvent && !same_row<RW>(r, y);
-        if (new_a) sts_rrow<RW>(pa, r);
-        if (new_b) sts_rrow<RW>(pb, r);
-        return (new_a && kind != kCopy) || new_b;
-    }
-    const uint32_t pa = rb + a * kRowB;
-    const RRow<RW> x = lds_rrow<RW>(pa);
-    RRow<RW> r = x;
-    const uint32_t *list = source_list(aux, pack, op.y);
-    const uint32_t c = list[0];
-    for (uint32_t q = 0; q < c; q += 4) {  // four independent loads at a time
-        RRow<RW> y[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const uint32_t ref = list[1 + (q + k < c ? q + k : q)];
-            y[k] = lds_rrow<RW>((ref & kTempRef) ? tb + (ref & ~kTempRef) * kRowB : rb + ref * kRowB);
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) r = rcombine<kMax, RW>(r, y[k]);
-    }
-    if (same_row<RW>(x, r)) return false;
-    sts_rrow<RW>(pa, r);
-    return true;
-}
-
-// Whether an op would change a row as the rows stand.
+// Whether an op on rows (shared address rb, node ids; saved rows: tb, temp ids)
+// would change a row as the rows stand.
 template <bool kMax, int RW>
 __device__ inline bool resident_live(uint2 op, uint32_t rb, uint32_t tb, const uint32_t *aux, const uint32_t *pack)
 {
@@ -1334,6 +1306,177 @@ __device__ inline bool resident_live(uint2 op, uint32_t rb, uint32_t tb, const u
         if (!same_row<RW>(rcombine<kMax, RW>(x, y), x)) return true;
     }
     return false;
+}
+
+// One thread's op of a level, with everything worked out before the level's barrier:
+// r = [la] | [lb] (PULL: and its sources) goes to sa and, for an EVENT, to lb.
+// EVENT and ONEWAY: la = sa; PULL: la = lb = sa; COPY: la = lb; no op: row 0.
+struct ResOp {
+    uint32_t la, lb, sa;
+    bool store, both;
+    uint32_t list, c, ref[4];  // PULL: source list, number of sources (else 0), the first ones
+};
+
+// Word b of a source list, in the pack at shared address packa or outside it.
+__device__ inline uint32_t list_word(const uint32_t *aux, uint32_t packa, uint32_t b)
+{
+    return b < kOutsideList ? lds_u32(packa + 4u * b) : __ldg(aux + (b - kOutsideList));
+}
+
+template <int RW, bool kTies, bool kAhead>
+__device__ __forceinline__ ResOp res_decode(uint2 op, bool act, uint32_t rb, uint32_t tb, const uint32_t *aux,
+                                            uint32_t packa)
+{
+    constexpr uint32_t kRowB = 8u * RW;
+    const uint32_t kind = op.x >> kKindShift;
+    ResOp o;
+    o.store = act;
+    o.both = act && kind == kEvent;
+    if (!kTies) {
+        o.sa = o.la = act ? rb + (op.x & kIdMask) * kRowB : rb;
+        o.lb = act ? rb + op.y * kRowB : rb;
+        return o;
+    }
+    const bool pull = act && kind == kPull, copy = act && kind == kCopy;
+    o.sa = (copy ? tb : rb) + (act ? op.x & kIdMask : 0u) * kRowB;
+    o.lb = pull ? o.sa : act ? rb + op.y * kRowB : rb;
+    o.la = copy ? o.lb : o.sa;
+    o.list = op.y;
+    o.c = 0;
+    if (pull) {
+        o.c = list_word(aux, packa, op.y);
+        if (!kAhead) return o;
+        if (op.y < kOutsideList) {  // (words behind the list's end stay unused)
+#pragma unroll
+            for (uint32_t k = 0; k < 4; ++k)
+                o.ref[k] = lds_u32(packa + 4u * (op.y + 1 + k < kStageBytes / 4 ? op.y + 1 + k : op.y));
+        } else {
+#pragma unroll
+            for (uint32_t k = 0; k < 4; ++k) o.ref[k] = k < o.c ? list_word(aux, packa, op.y + 1 + k) : 0u;
+        }
+    }
+    return o;
+}
+
+// Stores the result of an op; whether a row changed.
+template <int RW>
+__device__ __forceinline__ uint64_t res_store(const ResOp &o, const RRow<RW> &x, const RRow<RW> &y, const RRow<RW> &r)
+{
+    if (o.store) sts_rrow<RW>(o.sa, r);
+    if (o.both) sts_rrow<RW>(o.lb, r);
+    uint64_t diff = 0;
+#pragma unroll
+    for (int w = 0; w < RW; ++w) diff |= (r.w[w] ^ x.w[w]) | (o.both ? r.w[w] ^ y.w[w] : 0ull);
+    return o.store ? diff : 0ull;
+}
+
+// r combined with the `c` sources at word b of a list.
+template <bool kMax, int RW>
+__device__ __noinline__ RRow<RW> resident_sources(RRow<RW> r, uint32_t b, uint32_t c, uint32_t rb, uint32_t tb,
+                                                  const uint32_t *aux, uint32_t packa)
+{
+    constexpr uint32_t kRowB = 8u * RW;
+    for (uint32_t q = 0; q < c; q += 4) {  // four independent loads at a time
+        RRow<RW> z[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t ref = list_word(aux, packa, b + (q + j < c ? q + j : q));
+            z[j] = lds_rrow<RW>((ref & kTempRef ? tb : rb) + (ref & ~kTempRef) * kRowB);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) r = rcombine<kMax, RW>(r, z[j]);
+    }
+    return r;
+}
+
+// Ops i, i + C, ..., K of them, of a level that ends at e.
+template <int K, bool kMax, int RW, bool kTies>
+__device__ __forceinline__ uint64_t resident_round(uint32_t opa, uint32_t i, uint32_t e, uint32_t C, uint32_t rb,
+                                                   uint32_t tb, const uint32_t *aux, uint32_t packa)
+{
+    uint2 op[K];
+    ResOp o[K];
+    RRow<RW> x[K], y[K];
+    uint64_t diff = 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) op[k] = lds_op(opa + (i + k * C < e ? i + k * C : i) * 8u);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        o[k] = res_decode<RW, kTies, false>(op[k], i + k * C < e, rb, tb, aux, packa);
+        x[k] = lds_rrow<RW>(o[k].la);
+        y[k] = lds_rrow<RW>(o[k].lb);
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        RRow<RW> r = rcombine<kMax, RW>(x[k], y[k]);
+        if (kTies && o[k].c) r = resident_sources<kMax, RW>(r, o[k].list + 1, o[k].c, rb, tb, aux, packa);
+        diff |= res_store<RW>(o[k], x[k], y[k], r);
+    }
+    return diff;
+}
+
+// The ops of a level behind the consumers' first ones, from op `first` on.  Out of
+// line, as the sources above: rare, and the level loop stays short.
+template <bool kMax, int RW, bool kTies>
+__device__ __noinline__ uint64_t resident_more(uint32_t opa, uint32_t first, uint32_t e, uint32_t ct, uint32_t C,
+                                               uint32_t rb, uint32_t tb, const uint32_t *aux, uint32_t packa)
+{
+    uint64_t diff = 0;
+    for (; first + C < e; first += 2 * C)
+        if (first + ct < e) diff |= resident_round<2, kMax, RW, kTies>(opa, first + ct, e, C, rb, tb, aux, packa);
+    for (; first < e; first += C)
+        if (first + ct < e) diff |= resident_round<1, kMax, RW, kTies>(opa, first + ct, e, C, rb, tb, aux, packa);
+    return diff;
+}
+
+// The levels of one pack; whether a row changed.  The chain of a level runs from
+// barrier to barrier through the rows' load, one combine and the store, all without
+// a branch; the next level's op is decoded while the rows load, and the one after
+// it fetched.  Bound by the instructions of one warp's chain and, with 8 warps, by
+// issue slots.  A level of 93 ops, 256 threads: 307 cycles with ops decoded behind
+// the barrier and conditional stores, 219 now (449 and 317 with the code for ties);
+// warps that skip what they have no op for take 270 (the branch is longer than the
+// skipped part).  Bursty n = 20,011, 500,009 events: 6.46 ms, 5.30 ms now.
+template <bool kMax, int RW, bool kTies>
+__device__ __forceinline__ bool resident_levels(uint32_t opa, uint32_t sega, uint32_t nseg, uint32_t rb, uint32_t tb,
+                                                const uint32_t *aux, uint32_t ct, uint32_t C)
+{
+    constexpr uint32_t kRowB = 8u * RW;
+    const uint32_t packa = opa - kPackHead * 8u;
+    // (ops and ends behind the pack's last are inside the stage and unused)
+    auto fetch = [&](uint32_t i) { return lds_op(opa + (i + ct < kPackOps ? i + ct : 0u) * 8u); };
+    uint64_t diff = 0;
+    uint32_t b = 0, e = lds_u16(sega), e1 = lds_u16(sega + 2u);
+    uint2 next = fetch(e);
+    ResOp o = res_decode<RW, kTies, true>(fetch(0), ct < e, rb, tb, aux, packa);
+    for (uint32_t k = 1;; ++k) {
+        const RRow<RW> x = lds_rrow<RW>(o.la), y = lds_rrow<RW>(o.lb);
+        const uint32_t e2 = lds_u16(sega + 2u * (k + 1));
+        const uint2 after = fetch(e1);
+        const ResOp on = res_decode<RW, kTies, true>(next, e + ct < e1 && k < nseg, rb, tb, aux, packa);
+        RRow<RW> r = rcombine<kMax, RW>(x, y);
+        if (kTies && o.c) {
+            RRow<RW> z[4];  // four independent loads
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t ref = (uint32_t)j < o.c ? o.ref[j] : o.ref[0];
+                z[j] = lds_rrow<RW>((ref & kTempRef ? tb : rb) + (ref & ~kTempRef) * kRowB);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) r = rcombine<kMax, RW>(r, z[j]);
+            if (o.c > 4) r = resident_sources<kMax, RW>(r, o.list + 5, o.c - 4, rb, tb, aux, packa);
+        }
+        diff |= res_store<RW>(o, x, y, r);
+        if (e - b > C) diff |= resident_more<kMax, RW, kTies>(opa, b + C, e, ct, C, rb, tb, aux, packa);
+        if (k >= nseg) break;
+        consumers_sync(C);
+        b = e;
+        e = e1;
+        e1 = e2;
+        next = after;
+        o = on;
+    }
+    return diff != 0;
 }
 
 template <bool kMax, int RW>
@@ -1431,7 +1574,8 @@ __device__ void resident_slab(const Job &J, uint32_t smem_bytes, uint8_t *smem, 
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const uint32_t kind = op[k].x >> kKindShift;
-                        if (kind == kCopy) resident_op<kMax, RW>(op[k], rb, tb, aux, head);
+                        if (kind == kCopy)
+                            sts_rrow<RW>(tb + (op[k].x & kIdMask) * (8u * RW), lds_rrow<RW>(rb + op[k].y * (8u * RW)));
                         else if (kind != kPull) live |= resident_live<kMax, RW>(op[k], rb, tb, aux, head);
                     }
                     continue;
@@ -1474,23 +1618,11 @@ __device__ void resident_slab(const Job &J, uint32_t smem_bytes, uint8_t *smem, 
         if (ct == 0) r_ran[(q + 1u) % 3u] = 0;  // read one pack ago, set in the next one
         bool changed = false;
         const uint32_t sega = smem_addr(seg);
-        uint32_t b = 0, e = nseg ? lds_u16(sega) : 0u;
-        uint2 op = lds_op(opa + ct * 8u);  // always inside the stage; used only if ct < e
-        for (uint32_t k = 0; k < nseg;) {
-            // the next segment's end and this thread's op of it load beside this
-            // segment's rows, off the chain from barrier to barrier
-            const uint32_t next_e = lds_u16(sega + 2u * (k + 1 < kPackSegs ? k + 1 : k));
-            const uint2 next = lds_op(opa + (e + ct < kPackOps ? e + ct : 0u) * 8u);
-            if (b + ct < e) {
-                changed |= resident_op<kMax, RW>(op, rb, tb, aux, head);
-                for (uint32_t o = b + ct + C; o < e; o += C)
-                    changed |= resident_op<kMax, RW>(lds_op(opa + o * 8u), rb, tb, aux, head);
-            }
-            if (++k >= nseg) break;
-            b = e;
-            e = next_e;
-            op = next;
-            consumers_sync(C);
+        if (nseg == 0) {
+        } else if ((head[1] >> 16) & kPackTies) {
+            changed = resident_levels<kMax, RW, true>(opa, sega, nseg, rb, tb, aux, ct, C);
+        } else {
+            changed = resident_levels<kMax, RW, false>(opa, sega, nseg, rb, tb, aux, ct, C);
         }
         changed = __any_sync(0xffffffffu, changed);
         if (lane == 0) {

@@ -133,3 +133,33 @@ def test_settled_networks(stream, shape, directed):
         assert plan.status() == 0
         got = S.cpu().numpy().view(np.uint64)
         assert np.array_equal(got[:, : ref.shape[1]], ref) and not got[:, ref.shape[1]:].any()
+
+
+@pytest.mark.parametrize("words", [1, 2])
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("sources", [1, 3, 4, 5, 8, 9, 2500])
+def test_resident_levels_of_many_ops_and_sources(sources, directed, words):
+    """Star groups of `sources` edges, so many at once that a level has more ops than
+    the CTA has threads, between groups of disjoint pairs; a 2,500-edge star keeps its
+    source list outside the packs."""
+    n = 6000
+    rng = np.random.default_rng(sources)
+    us, vs, ts = [], [], []
+    for step in range(6):
+        nodes = rng.permutation(n)
+        if step % 2:
+            u, v = nodes[: n // 2], nodes[n // 2 :]
+        else:
+            stars = min(1200, n // (sources + 1))
+            hub, leaf = nodes[:stars], nodes[stars : stars * (sources + 1)]
+            u, v = leaf, np.repeat(hub, sources)
+        us.append(u)
+        vs.append(v)
+        ts.append(np.full(len(u), step))
+    u, v, t = np.concatenate(us), np.concatenate(vs), np.concatenate(ts)
+    plan = tn.Plan(*dev(u, v, t), n, resident_words=words, window_events=2480, directed=directed)
+    S = torch.empty((n, tn.tn_row_words(n)), dtype=torch.int64, device="cuda")
+    plan.apply(S, init=True)
+    assert plan.status() == 0
+    ref = (oracle.component_matrix_directed if directed else oracle.component_matrix)(u, v, t, n)
+    assert np.array_equal(S.cpu().numpy().view(np.uint64)[:, : ref.shape[1]], ref)
