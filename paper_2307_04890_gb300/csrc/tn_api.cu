@@ -1,6 +1,10 @@
 // Status strings, layout helper and the host-buffer end-to-end entry point.
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
+
+#include <chrono>
+#include <thread>
 
 #include "tn_internal.cuh"
 
@@ -29,6 +33,10 @@ void tn_internal_keep_pool(void)
     }
     done[dev] = true;
 }
+// How long a thread polls its mailbox before it blocks (the largest schedules take 8
+// ms; a blocked thread wakes up 0.05 to 0.1 ms late).  After kMailYield it lets others run.
+constexpr int kMailSpin = 5000, kMailYield = 300;  // us
+
 cudaError_t tn_internal_stream_wait(cudaStream_t st)
 {
     struct Cached {
@@ -53,6 +61,60 @@ cudaError_t tn_internal_stream_wait(cudaStream_t st)
     err = cudaEventRecord(c.ev, st);
     if (err != cudaSuccess) return err;
     return cudaEventSynchronize(c.ev);
+}
+
+tn::Mail *tn::mail_open(cudaStream_t st, uint32_t *seq)
+{
+    struct Box {
+        Mail *at = nullptr;
+        uint32_t seq = 0;
+        bool tried = false;
+        ~Box()
+        {
+            if (at) cudaFreeHost(at);
+        }
+    };
+    thread_local Box box;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (capture != cudaStreamCaptureStatusNone) return nullptr;
+    if (!box.tried) {
+        box.tried = true;
+        // once per thread; allowed also while some other thread captures
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        void *mem = nullptr;
+        if (cudaHostAlloc(&mem, sizeof(Mail), cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess) {
+            box.at = static_cast<Mail *>(mem);
+            memset(mem, 0, sizeof(Mail));
+        } else {
+            cudaGetLastError();
+        }
+        cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    if (!box.at) return nullptr;
+    if (++box.seq == 0) box.seq = 1;
+    *seq = box.seq;
+    return box.at;
+}
+
+cudaError_t tn::mail_wait(const Mail *mail, uint32_t seq, cudaStream_t st)
+{
+    const auto arrived = [&] { return __atomic_load_n(&mail->seq, __ATOMIC_ACQUIRE) == seq; };
+    const auto begin = std::chrono::steady_clock::now();
+    for (;;) {
+        for (int i = 0; i < 64; ++i)
+            if (arrived()) return cudaSuccess;
+        const auto waited = std::chrono::steady_clock::now() - begin;
+        if (waited > std::chrono::microseconds(kMailSpin)) break;
+        if (waited > std::chrono::microseconds(kMailYield)) std::this_thread::yield();
+    }
+    const cudaError_t err = tn_internal_stream_wait(st);
+    if (err != cudaSuccess) return err;
+    return arrived() ? cudaSuccess : cudaErrorUnknown;
 }
 
 cudaError_t tn_internal_allow_max_dyn_smem(const void *kernel)

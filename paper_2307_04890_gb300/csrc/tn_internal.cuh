@@ -32,6 +32,39 @@ void tn_internal_count_launches(uint64_t count);
 cudaError_t tn_internal_stream_wait(cudaStream_t stream);
 
 namespace tn {
+// A few counters from a kernel's last CTA to the host thread that waits for them, in
+// pinned host memory of that thread: the words, then the call's number in `seq`.  A
+// copy back and an event cost two driver calls (which threads of one process take in
+// turn) and the wake-up of a blocked thread instead.
+constexpr uint32_t kMailWords = 24;
+struct Mail {
+    uint64_t word[kMailWords];
+    uint32_t seq, pad;
+};
+// This thread's mailbox and a new number for a launch on `stream`; nullptr if there is
+// none (no pinned memory, or the stream is being captured: copy back and wait then).
+Mail *mail_open(cudaStream_t stream, uint32_t *seq);
+// Waits until the kernel has written `seq`: polls for a while, then blocks until the
+// stream's work is done.  Every opened mailbox is waited for before its thread goes on.
+cudaError_t mail_wait(const Mail *mail, uint32_t seq, cudaStream_t stream);
+
+// By one thread of the last CTA, behind a fence for what it has read.
+template <typename T>
+__device__ inline void mail_send(Mail *mail, uint32_t seq, const T *from)
+{
+    static_assert(sizeof(T) % 8 == 0 && sizeof(T) / 8 <= kMailWords, "mailbox too small");
+    const volatile uint64_t *w = reinterpret_cast<const volatile uint64_t *>(from);
+    uint64_t x[sizeof(T) / 8];
+#pragma unroll
+    for (uint32_t k = 0; k < sizeof(T) / 8; ++k) x[k] = w[k];
+#pragma unroll
+    for (uint32_t k = 0; k < sizeof(T) / 8; ++k) *(volatile uint64_t *)&mail->word[k] = x[k];
+    __threadfence_system();
+    *(volatile uint32_t *)&mail->seq = seq;
+}
+}  // namespace tn
+
+namespace tn {
 
 // Bounded device-side waits: a wait that has not completed after this many
 // polls (each poll suspends for up to ~1 us) records TN_ETIMEOUT and gives up.
@@ -281,6 +314,7 @@ struct tn_plan {
     uint2 *d_blob;        // packs (8-byte units)
     tn::WinDesc *d_win;   // [windows]    their windows in time order
     uint32_t *d_aux;      // source lists outside the packs
+    void *d_mem;          // owned: head, window bounds, windows, and packs and lists unless they are compacted
     uint32_t *d_label;    // [n] component of every node, a node id (NULL: not computed)
     tn::PlanHead *d_head; // owned: counters, time bounds, status word
     int64_t *d_tbounds;   // [2]          t_first, t_last (in d_head)

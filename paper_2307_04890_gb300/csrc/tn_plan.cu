@@ -47,6 +47,7 @@
 namespace tn {
 
 constexpr int kPlanThreads = 512;
+constexpr int kPlanThreadsSmall = 256;  // windows of up to 1,024 events
 // Default window of plans that name a row buffer: its rows fit a record.
 constexpr uint32_t kRecordWindow = 640;
 constexpr uint32_t kDefaultSlab = 16;
@@ -76,8 +77,9 @@ constexpr uint32_t kTileRows = 24928;
 // uniform events: 0.10 + 0.08 ms at 1,280, 0.14 + 0.08 ms at 2,480.
 static uint32_t default_window(uint64_t m) { return m < (1u << 16) ? 1280u : 2000u; }
 // Room of the first pass's arena behind the target: a window is stretched by the
-// rest of its last timestamp group (2,400 events: two CTAs per SM).
-constexpr uint32_t kWindowSlack = 400;
+// rest of its last timestamp group (2,400 events at the largest default window: two
+// CTAs per SM).
+static uint64_t window_slack(uint32_t window) { return window < 320 ? 64 : window / 5; }
 // Batches of at least this many events are copied into buffers of their exact
 // size; below it the staging buffers (a few times larger, bounded) are kept.
 constexpr uint64_t kCompactEvents = 1ull << 20;
@@ -150,9 +152,12 @@ struct PlanCounters {
     unsigned long long blob8, naux, list_words, items, ops, levels, local, temps;
     unsigned long long blob_used, aux_used;  // allocation of the exact buffers
     long long t_first, t_last;
+    unsigned long long done;  // CTAs of the first pass
 };
 
 struct PlanArgs {
+    Mail *mail;  // of the waiting thread, or nullptr
+    uint32_t mail_seq;
     const uint32_t *u, *v;
     const int64_t *t;
     uint64_t m;
@@ -890,10 +895,18 @@ __device__ __forceinline__ void schedule_window(const PlanArgs &a, uint32_t w, u
 __global__ void __launch_bounds__(kPlanThreads) schedule_first_kernel(PlanArgs a)
 {
     extern __shared__ __align__(16) uint8_t smem_arena[];
-    if (a.cnt->error) return;  // refused input: window bounds may not be ordered
     const uint32_t w = blockIdx.x;
-    if (a.wstart[w + 1] - a.wstart[w] > a.first_max) return;  // second pass
-    schedule_window<uint16_t>(a, w, smem_arena);
+    // refused input: window bounds may not be ordered; too large: second pass
+    if (!a.cnt->error && a.wstart[w + 1] - a.wstart[w] <= a.first_max) schedule_window<uint16_t>(a, w, smem_arena);
+    if (!a.mail) return;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&a.cnt->done, 1ull) == gridDim.x - 1) {
+            __threadfence();
+            mail_send(a.mail, a.mail_seq, a.cnt);
+        }
+    }
 }
 
 // Second pass: windows stretched by a large timestamp group, in all of shared
@@ -1042,10 +1055,11 @@ using namespace tn;
 
 static void free_plan_buffers(tn_plan *p, cudaStream_t st)
 {
-    if (p->d_blob) cudaFreeAsync(p->d_blob, st);
-    if (p->d_win) cudaFreeAsync(p->d_win, st);
-    if (p->d_aux) cudaFreeAsync(p->d_aux, st);
-    if (p->d_head) cudaFreeAsync(p->d_head, st);
+    if (p->m >= kCompactEvents) {  // (else in d_mem)
+        if (p->d_blob) cudaFreeAsync(p->d_blob, st);
+        if (p->d_aux) cudaFreeAsync(p->d_aux, st);
+    }
+    if (p->d_mem) cudaFreeAsync(p->d_mem, st);
     if (p->d_label) cudaFreeAsync(p->d_label, st);
 }
 
@@ -1103,7 +1117,7 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     a.directed = opt ? opt->directed : 0u;
     a.nw = (uint32_t)((m + window - 1) / window);
     a.smem_max = smem_max_events();
-    const uint64_t first_max = (uint64_t)window + kWindowSlack < m ? (uint64_t)window + kWindowSlack : m;
+    const uint64_t first_max = window + window_slack(window) < m ? window + window_slack(window) : m;
     a.first_max = first_max < a.smem_max ? (uint32_t)first_max : a.smem_max;
     a.dcap = rows;
     a.unit8 = window <= kRecordEvents && rows > 1 && records ? 5 : 4;
@@ -1124,7 +1138,6 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     tn_status rc = TN_OK;
     PlanCounters host;
     memset(&host, 0, sizeof(host));
-    PlanHead *head = nullptr;
     uint2 *exact_blob = nullptr;
     uint32_t *exact_aux = nullptr;
     bool must_wait = false;
@@ -1137,31 +1150,56 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
         if (err != cudaSuccess) goto fail; \
     } while (0)
 
-    TN_STEP(alloc_async(&head, 1, st));
-    p->d_head = head;
-    p->d_status = &head->status;
-    p->d_tbounds = head->tbounds;
-    a.cnt = &head->cnt;
-    a.tbounds = head->tbounds;
-    TN_STEP(cudaMemsetAsync(head, 0, sizeof(PlanHead), st));
-    // window bounds, second-pass offsets and list, source-list counts: one buffer
-    TN_STEP(alloc_async(&a.wstart, 3ull * a.nw + 2, st));
+    {
+        // head, window bounds, second-pass offsets and list, source-list counts,
+        // windows and, unless they are compacted below, packs and lists: one buffer
+        const auto part = [](uint64_t bytes) { return (bytes + 255) & ~255ull; };
+        const uint64_t at_bounds = part(sizeof(PlanHead)), at_win = at_bounds + part(8 * (3ull * a.nw + 2));
+        const uint64_t at_blob = at_win + part(sizeof(WinDesc) * (uint64_t)a.nw);
+        const uint64_t blob_bytes = part(8 * (blob_base(m, a.nw, a.unit8) + 64)), aux_bytes = 12 * m;
+        const bool apart = m >= kCompactEvents;
+        uint8_t *mem = nullptr;
+        TN_STEP(alloc_async(&mem, apart ? at_blob : at_blob + blob_bytes + aux_bytes, st));
+        p->d_mem = mem;
+        p->d_head = reinterpret_cast<PlanHead *>(mem);
+        a.wstart = reinterpret_cast<uint64_t *>(mem + at_bounds);
+        p->d_win = reinterpret_cast<WinDesc *>(mem + at_win);
+        if (apart) {
+            TN_STEP(alloc_async(&p->d_blob, blob_bytes / 8, st));
+            TN_STEP(alloc_async(&p->d_aux, 3 * m, st));
+        } else {
+            p->d_blob = reinterpret_cast<uint2 *>(mem + at_blob);
+            p->d_aux = reinterpret_cast<uint32_t *>(mem + at_blob + blob_bytes);
+        }
+    }
+    p->d_status = &p->d_head->status;
+    p->d_tbounds = p->d_head->tbounds;
+    a.cnt = &p->d_head->cnt;
+    a.tbounds = p->d_head->tbounds;
+    TN_STEP(cudaMemsetAsync(p->d_head, 0, sizeof(PlanHead), st));
     a.late_off = a.wstart + a.nw + 1;
     a.late_list = reinterpret_cast<uint32_t *>(a.late_off + a.nw);
     a.naux_w = a.late_list + a.nw;
-    TN_STEP(alloc_async(&p->d_win, a.nw, st));
     a.desc = p->d_win;
-    TN_STEP(alloc_async(&p->d_blob, blob_base(m, a.nw, a.unit8) + 64, st));
     a.blob = p->d_blob;
-    TN_STEP(alloc_async(&p->d_aux, 3 * m, st));
     a.aux = p->d_aux;
     TN_STEP(tn_internal_allow_max_dyn_smem((const void *)schedule_first_kernel));
+    // Counters by mailbox where a call's latency counts (20,000 events: 146 us with
+    // sizes, 133 us with the mailbox; 32 serving jobs on 16 threads: 15.0 and 11.8 ms);
+    // batches that are compacted wait for their copies anyway (ER, 10^7 events: 16 us
+    // more for the 5,000 CTAs' count).
+    if (m < kCompactEvents) a.mail = mail_open(st, &a.mail_seq);
     tn_internal_count_launches(2);
     inspect_kernel<<<(unsigned)(blocks < 1216 ? blocks : 1216), 256, 0, st>>>(a);
-    schedule_first_kernel<<<a.nw, a.first_max > 1024 ? kPlanThreads : kPlanThreads / 2, arena_bytes<uint16_t>(a.first_max), st>>>(a);
+    schedule_first_kernel<<<a.nw, a.first_max > 1024 ? kPlanThreads : kPlanThreadsSmall, arena_bytes<uint16_t>(a.first_max), st>>>(a);
     TN_STEP(cudaGetLastError());
-    TN_STEP(cudaMemcpyAsync(&host, a.cnt, sizeof(host), cudaMemcpyDeviceToHost, st));
-    TN_STEP(tn_internal_stream_wait(st));
+    if (a.mail) {
+        TN_STEP(mail_wait(a.mail, a.mail_seq, st));
+        memcpy(&host, a.mail->word, sizeof(host));
+    } else {
+        TN_STEP(cudaMemcpyAsync(&host, a.cnt, sizeof(host), cudaMemcpyDeviceToHost, st));
+        TN_STEP(tn_internal_stream_wait(st));
+    }
     if (host.error & 1ull) {
         rc = TN_ERANGE;
         goto done;
@@ -1197,7 +1235,6 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
         // node): 25.9 ms as records, 32 to 36 ms as tiles; n = 2 10^5, m = 5 10^6
         // (600 ops a level): 146 ms with windows of 640, 136 ms as tiles.
         free_plan_buffers(p, st);
-        cudaFreeAsync(a.wstart, st);
         if (a.late_arena) cudaFreeAsync(a.late_arena, st);
         free(p);
         tn_plan_options again;
@@ -1242,7 +1279,6 @@ fail:
     tn_internal_set_cuda_error(err);
     rc = err == cudaErrorMemoryAllocation ? TN_ENOMEM : TN_ECUDA;
 done:
-    if (a.wstart) cudaFreeAsync(a.wstart, st);
     if (a.late_arena) cudaFreeAsync(a.late_arena, st);
     if (rc != TN_OK) {
         if (exact_blob) cudaFreeAsync(exact_blob, st);

@@ -1,5 +1,5 @@
 """Schedules at the edges of the planner's units (needs a GPU: -m gpu): chunks of
-16 events, packs of 64 levels and 2,030 ops, timestamp groups around the 128
+16 events, packs of 64 levels and 2,030 ops, timestamp groups around the 48
 events above which the whole CTA takes them unchecked, local ids that are the
 node ids (networks of at most two nodes per window event), windows stretched by a
 group into the second pass, and batches large enough to be copied into buffers of
@@ -8,6 +8,7 @@ import numpy as np
 import pytest
 
 import oracle
+from paper_2307_04890_gb300 import synth
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -51,7 +52,7 @@ def test_one_level_per_event_and_one_level_for_all(m, shape):
 
 
 @pytest.mark.parametrize("directed", [False, True])
-@pytest.mark.parametrize("group", [2, 16, 17, 127, 128, 129, 400])
+@pytest.mark.parametrize("group", [2, 16, 17, 47, 48, 49, 127, 128, 129, 400])
 def test_groups_with_and_without_shared_nodes(group, directed):
     """Groups of one size whose events share no node, with one pair that shares one
     at either end of the group, self-loops and duplicates among them."""
@@ -97,3 +98,36 @@ def test_exact_buffers(shape, extra):
     u, v = rng.integers(0, n, m), rng.integers(0, n, m)
     t = np.sort(rng.integers(0, m // 3, m))
     check(u, v, t, n, **shape)
+
+
+def test_plans_of_many_threads():
+    """Threads that schedule at the same time, each on its own stream, with refused
+    batches in between: every thread gets the counters of its own plan."""
+    from concurrent.futures import ThreadPoolExecutor
+
+    n = 600
+    batches = [synth.uniform_events(n, 700 + 911 * k, t_range=300, seed=k) for k in range(8)]
+    refs = [oracle.component_matrix(u, v, t, n) for u, v, t in batches]
+
+    def work(k):
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            u, v = (torch.from_numpy(np.ascontiguousarray(x, dtype=np.uint32).view(np.int32)).cuda() for x in batches[k][:2])
+            t = torch.from_numpy(np.ascontiguousarray(batches[k][2], dtype=np.int64)).cuda()
+            back = t.flip(0).contiguous()
+            for _ in range(6):
+                with pytest.raises(tn.TnError):
+                    tn.Plan(u, v, back, n, stream=stream)
+                plan = tn.Plan(u, v, t, n, stream=stream)
+                S = torch.empty((n, tn.tn_row_words(n)), dtype=torch.int64, device="cuda")
+                plan.apply(S, init=True, stream=stream)
+                stats = plan.stats()
+                assert stats["windows"] == -(-len(batches[k][0]) // 1280)
+                stream.synchronize()
+                assert plan.status() == 0
+                assert np.array_equal(S.cpu().numpy().view(np.uint64)[:, : refs[k].shape[1]], refs[k])
+                plan.destroy(stream=stream)
+        return True
+
+    with ThreadPoolExecutor(8) as pool:
+        assert all(pool.map(work, range(8)))
