@@ -184,7 +184,7 @@ typedef struct tn_plan tn_plan;
 typedef struct tn_plan_options {
     uint32_t window_events; /* target events per scheduling window (0 = chosen by the
                                library: 640 for networks or row buffers whose windows
-                               are applied in shared memory, else 1,280 or 2,480) */
+                               are applied in shared memory, else 1,280 or 2,000) */
     uint32_t slab_words;    /* 64-bit words of every row owned by one CTA when the
                                plan is applied: an even number from 2 to 128
                                (0 = 16, or, when no window is applied in shared
