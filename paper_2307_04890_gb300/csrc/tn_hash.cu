@@ -242,8 +242,9 @@ __global__ void __launch_bounds__(kTabThreads)
     }
 }
 
-// The same table for proxies whose rows do not fit shared memory 32 at a time:
-// one thread per 32-bit word of T, columns read through L1.
+// The same table for proxies whose rows do not fit shared memory 32 at a time, and
+// for a P that is not 16-byte aligned: one thread per 32-bit word of T, columns read
+// through L1 in 8-byte loads.
 __global__ void __launch_bounds__(kTabThreads)
     bitslice_table_wide_kernel(const uint64_t *P, uint32_t k, uint64_t ldk, const uint32_t *H, uint32_t n,
                                const uint32_t *src, uint32_t s0, uint32_t ns, uint32_t words, uint32_t *T)
@@ -420,7 +421,7 @@ static tn_status estimate_bitsliced(const uint64_t *P, uint32_t R, uint32_t k, u
     const uint32_t chunk = nsrc > 3072 && (uint64_t)R * k * 512 <= (2ull << 30) ? 4096u : 1024u;
     const uint32_t words = chunk / 32;
     const size_t tab_smem = (size_t)((k + 127) / 128) * 4 * kTabRows * 4;
-    const bool wide = tab_smem > kTabSmem;
+    const bool wide = tab_smem > kTabSmem || ((uintptr_t)P & 15u);  // (rows are whole 128-byte units)
     const size_t cnt_smem = (32ull * words + 256ull * R) * 4;
     uint32_t *T = nullptr;
     TN_CUDA_TRY(cudaMallocAsync((void **)&T, (uint64_t)R * k * words * 4, st));

@@ -52,8 +52,10 @@ __global__ void hll_init_kernel(uint8_t *R, uint32_t n, uint64_t row_bytes, uint
 // One warp per row: sum of 2^-M over the registers and the number of zeros.  The
 // sum is exact, in fixed point: ranks up to 30 in units of 2^-30, larger ones (at
 // most 61) in units of 2^-61; a lane's share of 2^16 registers stays below 2^42.
-// Sixteen registers a lane and load.  n = 20,000, p = 10: 17 us (227 us with a byte
-// a lane and double-precision powers).
+// Sixteen registers a lane and load (kWide; byte by byte where R is not 16-byte
+// aligned).  n = 20,000, p = 10: 17 us (227 us with a byte a lane and
+// double-precision powers).
+template <bool kWide>
 __global__ void hll_estimate_kernel(const uint8_t *R, uint32_t n, uint64_t row_bytes, uint32_t p, double alpha,
                                     double *est)
 {
@@ -65,8 +67,17 @@ __global__ void hll_estimate_kernel(const uint8_t *R, uint32_t n, uint64_t row_b
         uint64_t small = 0, large = 0;
         uint32_t zeros = 0;
         for (uint32_t j = 16 * lane; j < s; j += 512) {
-            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(M + j));
-            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+            uint32_t w[4] = {0u, 0u, 0u, 0u};
+            if (kWide) {
+                const uint4 v = __ldg(reinterpret_cast<const uint4 *>(M + j));
+                w[0] = v.x;
+                w[1] = v.y;
+                w[2] = v.z;
+                w[3] = v.w;
+            } else {
+#pragma unroll
+                for (int b = 0; b < 16; ++b) w[b >> 2] |= (uint32_t)__ldg(M + j + b) << (8 * (b & 3));
+            }
 #pragma unroll
             for (int q = 0; q < 4; ++q)
 #pragma unroll
@@ -158,7 +169,8 @@ extern "C" tn_status tn_hll_estimate(const uint8_t *R, uint32_t n, uint32_t p, d
     const uint32_t s = 1u << p;
     const double alpha = s == 16 ? 0.673 : s == 32 ? 0.697 : s == 64 ? 0.709 : 0.7213 / (1.0 + 1.079 / (double)s);
     tn_internal_count_launches(1);
-    hll_estimate_kernel<<<grid_rows(n), 256, 0, (cudaStream_t)stream>>>(R, n, tn_hll_row_bytes(p), p, alpha, est);
+    const auto kernel = ((uintptr_t)R & 15u) == 0 ? hll_estimate_kernel<true> : hll_estimate_kernel<false>;
+    kernel<<<grid_rows(n), 256, 0, (cudaStream_t)stream>>>(R, n, tn_hll_row_bytes(p), p, alpha, est);
     TN_CUDA_TRY(cudaGetLastError());
     return TN_OK;
 }
