@@ -71,7 +71,12 @@ tn::Mail *tn::mail_open(cudaStream_t st, uint32_t *seq)
         bool tried = false;
         ~Box()
         {
-            if (at) cudaFreeHost(at);
+            if (!at) return;
+            // as for the allocation: some other thread may be capturing (and the
+            // free would otherwise break its capture)
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            cudaFreeHost(at);
         }
     };
     thread_local Box box;
