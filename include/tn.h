@@ -306,7 +306,10 @@ tn_status tn_plan_destroy(tn_plan *plan, void *stream);
  * tn_graph_launch replays it on `stream` (one launch), recomputing the same
  * matrices from the same plans.  The plans and matrices must stay alive and
  * unchanged in size while the graph exists.  The first plan status error
- * still gates the replay as it gates a direct call.
+ * still gates the replay as it gates a direct call.  A replay allocates what the
+ * direct call does: the saved rows of tie groups and, for slabs wider than 16 words,
+ * 4 bytes per row and CTA (left out, at a lower speed, when that is more than half of
+ * the device memory that is free at capture).
  */
 typedef struct tn_graph tn_graph;
 

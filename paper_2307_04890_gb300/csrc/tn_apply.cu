@@ -2075,6 +2075,26 @@ static void choose_forms(const tn_plan *const *plans, const uint32_t *ncols, uin
         if (!rw[i] && fits(plans[i], 1)) rw[i] = w;
 }
 
+// Whether content ids of `bytes` may be allocated on `st`.  A call learns from the
+// allocation itself that there is no room; a capture only records it, and the graph's
+// launch would fail instead.  `held`: bytes of the launch's earlier ids; half of the
+// free memory is left for what the caller allocates before the graph runs.
+static bool ids_allowed(cudaStream_t st, uint64_t bytes, uint64_t held)
+{
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (capture == cudaStreamCaptureStatusNone) return true;
+    size_t free_b = 0, total_b = 0;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const cudaError_t err = cudaMemGetInfo(&free_b, &total_b);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return err == cudaSuccess && bytes + held <= free_b / 2;
+}
+
 tn_status apply_jobs(const tn_plan *const *plans, uint64_t *const *S, const uint32_t *ncols,
                      const uint32_t *const *src, int64_t *const *t_last, uint32_t count, uint32_t flags,
                      cudaStream_t st)
@@ -2093,6 +2113,7 @@ tn_status apply_jobs(const tn_plan *const *plans, uint64_t *const *S, const uint
             if (plans[i]->resident) return TN_EINVAL;
     uint64_t *tmps[kMaxPlans];
     uint32_t *idbuf[kMaxPlans];
+    uint64_t ids_held = 0;
     for (uint32_t base = 0; base < count; base += kMaxPlans) {
         const uint32_t nj = count - base < (uint32_t)kMaxPlans ? count - base : (uint32_t)kMaxPlans;
         JobList jl;
@@ -2151,9 +2172,11 @@ tn_status apply_jobs(const tn_plan *const *plans, uint64_t *const *S, const uint
             if (!p->local_windows && !(cpr & (cpr - 1)) && cpr <= 32 && dcap >= ring_rows && !p->wave_ctas &&
                 need + kMarkBytes <= smem_limit) {
                 track = kMarks;
-                if (sw > kMarkWords && 16 * p->ops >= p->n && rows + p->ops < 0xFFFFFFF0ull) {
+                if (sw > kMarkWords && 16 * p->ops >= p->n && rows + p->ops < 0xFFFFFFF0ull &&
+                    ids_allowed(st, rows * pitch * 4, ids_held)) {
                     if (cudaMallocAsync((void **)&ids, rows * pitch * 4, st) == cudaSuccess) {
                         track = kIds;
+                        ids_held += rows * pitch * 4;
                         tn_internal_count_launches(1);
                         init_ids_kernel<<<grid_for(rows * pitch / 4), 256, 0, st>>>(ids, rows, pitch, sw,
                                                                                    zero, zero && !src[i]);
