@@ -193,7 +193,9 @@ typedef struct tn_plan_options {
                                segments) suit large networks whose windows stream
                                from global memory: fewer, longer DRAM bursts */
     uint32_t smem_rows;     /* row slots of the streaming kernel's shared-memory row
-                               buffer (at most 192 KB / (8 slab_words)); windows with
+                               buffer (at most 192 KB / (8 slab_words); with
+                               slab_words 0, slots of 16 words, and a slab of another
+                               width gets a buffer of as many bytes); windows with
                                more rows (plus saved copies) stream from global
                                memory (0 = 160 KB / (8 slab_words) for slabs of up to
                                16 words, 192 KB / (8 slab_words) above).  A buffer small

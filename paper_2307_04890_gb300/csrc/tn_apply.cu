@@ -172,8 +172,6 @@ struct Lane {
     bool active;   // chunk inside the matrix and thread inside the row groups
 };
 
-constexpr uint32_t kRowBufferMax = 192 * 1024;
-
 // consumer threads of this launch (all warps but the producer)
 __device__ inline uint32_t consumers() { return blockDim.x - 32u; }
 
@@ -2155,7 +2153,7 @@ tn_status apply_jobs(const tn_plan *const *plans, uint64_t *const *S, const uint
             const uint32_t sw = sws[j];
             // words that hold columns (the rest of the row is zero padding and stays so)
             const uint64_t wide = open ? (((uint64_t)ncols[i] + 63) / 64 + 1) & ~1ull : ld;
-            uint32_t dcap = open ? kRowBufferMax / (8 * sw) : p->dcap;
+            uint32_t dcap = open ? p->buffer_bytes / (8 * sw) : p->dcap;
             const uint32_t ring_rows = 2u * kRing * (32u * kWarpsAlone / (sw / 2));
             if (p->local_windows == 0 && dcap > ring_rows) dcap = ring_rows;
             size_t need = smem_base + (size_t)dcap * sw * 8;

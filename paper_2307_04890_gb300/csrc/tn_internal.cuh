@@ -310,6 +310,7 @@ struct tn_plan {
     uint32_t auto_form;   // the form (resident or column slabs) was left open: chosen when the plan is applied
     uint32_t wave_ctas;   // 0, or the number of CTAs one matrix is spread over
     uint32_t dcap;        // row slots of the kernel's shared-memory row buffer
+    uint32_t buffer_bytes;  // largest row buffer of a width chosen when the plan is applied (smem_rows was given: its bytes)
     uint32_t resident;    // 0, or 64-bit words of every row one CTA keeps in shared memory
     uint2 *d_blob;        // packs (8-byte units)
     tn::WinDesc *d_win;   // [windows]    their windows in time order

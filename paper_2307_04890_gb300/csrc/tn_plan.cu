@@ -1099,6 +1099,7 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
         if (n > resident_max_rows(resident)) return TN_EINVAL;
         rows = 1;
     }
+    const bool rows_given = rows != 0;
     if (rows == 0) rows = (sw <= 16 ? kRowBufferBytes : kRowBufferWide) / (sw * 8);
     if (rows > kLocalSlotLimit) rows = kLocalSlotLimit;
     if ((uint64_t)rows * sw * 8 > kRowBufferWide) return TN_EINVAL;  // row buffer must fit the kernel's shared memory
@@ -1131,6 +1132,7 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     p->slab_words = sw;
     p->wave_ctas = wave;
     p->dcap = rows;
+    p->buffer_bytes = rows_given ? rows * sw * 8 : kRowBufferWide;
     p->resident = resident;
     p->auto_form = auto_form;
     p->auto_slab = !resident && !wave && (!opt || !opt->slab_words);

@@ -1,0 +1,56 @@
+"""Which form a plan takes (needs a GPU: -m gpu): row buffers that the options name,
+windows kept as shared-memory records or run as tiles.  Results bit for bit against the
+oracle in every form."""
+import json
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2307_04890_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if torch.cuda.is_available():
+    import paper_2307_04890_gb300 as tn
+    from paper_2307_04890_gb300.build import build_library
+
+    build_library()
+    oracle.build_oracle()
+
+
+def dev(u, v, t):
+    f = lambda x, d: torch.from_numpy(np.ascontiguousarray(x, dtype=d).view(np.int32 if d == np.uint32 else d)).cuda()  # noqa: E731
+    return f(u, np.uint32), f(v, np.uint32), f(t, np.int64)
+
+
+def applied(events, n, directed=False, **options):
+    plan = tn.Plan(*dev(*events), n, directed=directed, **options)
+    S = torch.full((n, tn.tn_row_words(n)), -1, dtype=torch.int64, device="cuda")
+    plan.apply(S, init=True)
+    assert plan.status() == 0
+    ref = (oracle.component_matrix_directed if directed else oracle.component_matrix)(*events, n)
+    assert np.array_equal(S.cpu().numpy().view(np.uint64)[:, : ref.shape[1]], ref)
+    return plan
+
+
+@pytest.mark.parametrize("rows,threads", [(640, 160), (0, 416)])
+def test_row_buffer_of_an_open_width(rows, threads, tmp_path):
+    """An 80 KB row buffer gives two CTAs of 4 consumer warps per SM also where the slab
+    width is left open and no window fits the buffer."""
+    n, m = 3000, 20_000
+    u, v, _ = synth.uniform_events(n, m, t_range=m, seed=3)
+    options = dict(smem_rows=rows) if rows else dict(window_events=2100)
+    plan = applied((u, v, np.arange(m) // 1000), n, slab_words=0, **options)
+    assert plan.stats()["local_windows"] == 0
+    S = torch.empty((n, tn.tn_row_words(n)), dtype=torch.int64, device="cuda")
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        plan.apply(S, init=True)
+        torch.cuda.synchronize()
+    prof.export_chrome_trace(str(tmp_path / "trace.json"))
+    trace = json.loads((tmp_path / "trace.json").read_text())["traceEvents"]
+    blocks = [e["args"]["block"][0] for e in trace if "stream_kernel" in e.get("name", "") and "block" in e.get("args", {})]
+    if not blocks:
+        pytest.skip("no kernel records from the profiler")
+    assert blocks == [threads]
