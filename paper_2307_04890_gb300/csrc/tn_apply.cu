@@ -1981,6 +1981,15 @@ static int multiprocessors()
 // dynamic shared memory of a CTA that leaves room for a second one on its SM
 constexpr uint64_t kHalfSmSmem = 112 * 1024;
 
+// Row slots of the copy rings of 12 consumer warps.
+static uint32_t ring_slots(uint32_t words) { return 2u * kRing * (32u * kWarpsAlone / (words / 2)); }
+
+bool tracked_slab(uint32_t words, uint64_t bytes)
+{
+    const uint32_t cpr = words / 2;
+    return !(cpr & (cpr - 1)) && cpr <= 32 && bytes / (8 * words) >= ring_slots(words);
+}
+
 bool resident_fits(uint64_t rows, uint64_t temps, uint32_t words)
 {
     if (words != 1 && words != 2) return false;
@@ -2154,7 +2163,7 @@ tn_status apply_jobs(const tn_plan *const *plans, uint64_t *const *S, const uint
             // words that hold columns (the rest of the row is zero padding and stays so)
             const uint64_t wide = open ? (((uint64_t)ncols[i] + 63) / 64 + 1) & ~1ull : ld;
             uint32_t dcap = open ? p->buffer_bytes / (8 * sw) : p->dcap;
-            const uint32_t ring_rows = 2u * kRing * (32u * kWarpsAlone / (sw / 2));
+            const uint32_t ring_rows = ring_slots(sw);
             if (p->local_windows == 0 && dcap > ring_rows) dcap = ring_rows;
             size_t need = smem_base + (size_t)dcap * sw * 8;
             // Tracked rows: tile windows only (records do not keep track), row groups
@@ -2162,12 +2171,12 @@ tn_status apply_jobs(const tn_plan *const *plans, uint64_t *const *S, const uint
             // by ids, if the ops pay for setting the ids up (4 bytes per row and
             // CTA against 512 to 2,048 bytes per op and CTA); others by marks, a
             // row or, where that does not fit, up to 4 rows per mark.
-            const uint32_t cpr = sw / 2, nct = (uint32_t)((wide + sw - 1) / sw);
+            const uint32_t nct = (uint32_t)((wide + sw - 1) / sw);
             const uint64_t rows = (uint64_t)p->n + p->temps;
             const bool zero = (flags & TN_INIT_IDENTITY) != 0;
             uint32_t track = kNoTrack, mark_words = 0, mark_shift = 0, *ids = nullptr;
             const uint32_t pitch = (nct + 7u) & ~7u;
-            if (!p->local_windows && !(cpr & (cpr - 1)) && cpr <= 32 && dcap >= ring_rows && !p->wave_ctas &&
+            if (!p->local_windows && tracked_slab(sw, (uint64_t)dcap * sw * 8) && !p->wave_ctas &&
                 need + kMarkBytes <= smem_limit) {
                 track = kMarks;
                 if (sw > kMarkWords && 16 * p->ops >= p->n && rows + p->ops < 0xFFFFFFF0ull &&

@@ -56,6 +56,8 @@ constexpr uint32_t kRowBufferWide = 192 * 1024;   // default (and largest) row b
 constexpr uint32_t kEmpty = 0xFFFFFFFFu;
 // Windows of up to this many events may become shared-memory records.
 constexpr uint32_t kRecordEvents = 2048;
+// Records are kept if more than one window in this many is one.
+constexpr uint64_t kTileShare = 64;
 // Groups of at least this many events go to the whole CTA unchecked: comparing
 // their events pair by pair would cost more than the group's own phases (bursty
 // n = 20,011, 500,009 events, groups of 107: plan 0.21 ms at 128, 0.18 ms at 48;
@@ -170,6 +172,7 @@ struct PlanArgs {
     uint32_t smem_max;   // largest window scheduled in shared memory
     uint32_t dcap;       // row slots of a local window
     uint32_t unit8;      // staging units (8 bytes) per event
+    uint32_t redo;       // 1: the windows scheduled as records become tiles
     uint64_t *wstart;    // [nw + 1]
     uint32_t *naux_w;    // [nw] source-list entries of every window
     WinDesc *desc;       // [nw]
@@ -540,6 +543,7 @@ __device__ __forceinline__ void schedule_window(const PlanArgs &a, uint32_t w, u
     const uint32_t E = (uint32_t)(a.wstart[w + 1] - s);
     const uint32_t T = blockDim.x, tid = threadIdx.x, lane = tid & 31u;
     WinDesc *desc = a.desc + w;
+    const uint32_t record_units = a.redo ? desc->pack[0] : 0u;  // (overwritten below, by thread 0 at the earliest)
     if (E == 0) {
         if (tid == 0) {
             *desc = WinDesc{};
@@ -680,7 +684,7 @@ __device__ __forceinline__ void schedule_window(const PlanArgs &a, uint32_t w, u
     //    shared-memory row buffer, and its record fits one staging buffer
     const uint32_t rec_words = 4 + D + (maxlev + 1) + nops + naux;
     const uint32_t rec_words_pad = (rec_words + 3u) & ~3u;
-    const bool local = E <= kRecordEvents && a.unit8 >= 5 && D + ntemp <= a.dcap && rec_words_pad <= kRecordWords;
+    const bool local = !a.redo && E <= kRecordEvents && a.unit8 >= 5 && D + ntemp <= a.dcap && rec_words_pad <= kRecordWords;
     const uint64_t region = blob_base(s, w, a.unit8);
 
     if (local) {
@@ -872,10 +876,14 @@ __device__ __forceinline__ void schedule_window(const PlanArgs &a, uint32_t w, u
     if (tid == 0) {
         PlanCounters *c = a.cnt;
         const uint32_t units = res[1] + (res[0] > kDescPacks ? (res[0] + 1) / 2 : 0u);
-        atomicAdd(&c->blob8, (unsigned long long)((units + 1) & ~1u));
-        atomicAdd(&c->items, (unsigned long long)res[0]);
-        atomicAdd(&c->ops, (unsigned long long)nops);
-        atomicAdd(&c->levels, (unsigned long long)maxlev);
+        atomicAdd(&c->blob8, (unsigned long long)((units + 1) & ~1u) - record_units);
+        atomicAdd(&c->items, (unsigned long long)res[0] - a.redo);
+        if (a.redo) {  // (a record, counted once already)
+            atomicAdd(&c->local, ~0ull);
+        } else {
+            atomicAdd(&c->ops, (unsigned long long)nops);
+            atomicAdd(&c->levels, (unsigned long long)maxlev);
+        }
         if (local) {
             atomicAdd(&c->local, 1ull);
         } else {
@@ -918,6 +926,17 @@ __global__ void __launch_bounds__(kPlanThreads) schedule_late_kernel(PlanArgs a)
     const uint64_t off = a.late_off[blockIdx.x];
     if (off == kSmemArena) schedule_window<uint16_t>(a, w, smem_arena);
     else schedule_window<uint32_t>(a, w, a.late_arena + off);
+}
+
+// The few records of a plan of tiles, as tiles: records keep no track of rows, so one
+// of them would have every update of the plan executed.  A tile's descriptor has
+// tab > 0.
+__global__ void __launch_bounds__(kPlanThreads) schedule_tiles_kernel(PlanArgs a)
+{
+    extern __shared__ __align__(16) uint8_t smem_arena[];
+    const WinDesc *desc = a.desc + blockIdx.x;
+    if (desc->npacks == 0 || desc->tab != 0) return;
+    schedule_window<uint16_t>(a, blockIdx.x, smem_arena);
 }
 
 // Copies every window into buffers of the exact size (in no particular order:
@@ -1216,6 +1235,19 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
         TN_STEP(tn_internal_allow_max_dyn_smem((const void *)schedule_late_kernel));
         tn_internal_count_launches(1);
         schedule_late_kernel<<<late, kPlanThreads, arena_bytes<uint16_t>(a.smem_max), st>>>(a);
+        TN_STEP(cudaGetLastError());
+        TN_STEP(cudaMemcpyAsync(&host, a.cnt, sizeof(host), cudaMemcpyDeviceToHost, st));
+        TN_STEP(tn_internal_stream_wait(st));
+    }
+    // Records among many more tiles: 1 of 1,001 windows (2,000 events, the last one short)
+    // takes 25.3 ms to apply, all as tiles 19.9 ms (activity-driven, n = 10^5, m = 2 10^6,
+    // 16 words).  With a tenth of the windows as records, every update executed, some
+    // streams are faster than as tiles (bursty n = 1.2 10^5, m = 3 10^6: 42.7 ms, 51.3).
+    if (host.local && kTileShare * host.local <= a.nw && !wave && tracked_slab(sw, (uint64_t)rows * sw * 8)) {
+        a.redo = 1;
+        TN_STEP(tn_internal_allow_max_dyn_smem((const void *)schedule_tiles_kernel));
+        tn_internal_count_launches(1);
+        schedule_tiles_kernel<<<a.nw, kPlanThreads, arena_bytes<uint16_t>(kRecordEvents), st>>>(a);
         TN_STEP(cudaGetLastError());
         TN_STEP(cudaMemcpyAsync(&host, a.cnt, sizeof(host), cudaMemcpyDeviceToHost, st));
         TN_STEP(tn_internal_stream_wait(st));

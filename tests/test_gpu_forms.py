@@ -54,3 +54,23 @@ def test_row_buffer_of_an_open_width(rows, threads, tmp_path):
     if not blocks:
         pytest.skip("no kernel records from the profiler")
     assert blocks == [threads]
+
+
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("windows,ties", [(10, 1), (70, 1), (70, 3), (1050, 3)])
+def test_a_short_last_window(windows, ties, directed):
+    """Windows of 1,000 events whose rows do not fit the row buffer, and a last one of 9
+    events (at most one window in 64: as a tile, so that the plan's rows are tracked),
+    below and above the batch size from which schedules are copied."""
+    n, m = 20_000, 1000 * windows + 9
+    u, v, _ = synth.uniform_events(n, m, t_range=m, seed=windows)
+    t = np.arange(m) // ties
+    t[-9:] = t[-10] + 1 + np.arange(9) // 3  # 1,000 is no multiple of 3: the last window starts with the first of these
+    v[-2] = u[-3]
+    plan = applied((u, v, t), n, directed=directed, slab_words=16, window_events=1000)
+    stats = plan.stats()
+    assert stats["windows"] == windows + 1 and stats["local_windows"] == (1 if windows < 64 else 0)
+    whole = tn.Plan(*dev(u, v, t), n, directed=directed, slab_words=16, window_events=1000, smem_rows=1).stats()
+    assert (stats["ops"], stats["levels"]) == (whole["ops"], whole["levels"])
+    if windows > 64:  # the counters are those of a plan that never had a record
+        assert all(stats[k] == whole[k] for k in ("items", "aux", "temps"))
