@@ -2082,6 +2082,13 @@ static void choose_forms(const tn_plan *const *plans, const uint32_t *ncols, uin
         if (!rw[i] && fits(plans[i], 1)) rw[i] = w;
 }
 
+uint32_t resident_form(const tn_plan *p, uint32_t ncols)
+{
+    uint32_t rw = 0;
+    choose_forms(&p, &ncols, 1, &rw);
+    return rw;
+}
+
 // Whether content ids of `bytes` may be allocated on `st`.  A call learns from the
 // allocation itself that there is no room; a capture only records it, and the graph's
 // launch would fail instead.  `held`: bytes of the launch's earlier ids; half of the

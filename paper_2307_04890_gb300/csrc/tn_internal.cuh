@@ -329,6 +329,9 @@ namespace tn {
 // largest row count that fits with no saved rows (0 for an unsupported width).
 bool resident_fits(uint64_t rows, uint64_t temps, uint32_t words);
 uint32_t resident_max_rows(uint32_t words);
+// Words of a row per resident CTA that an open plan takes when it alone is applied to
+// `ncols` columns; 0: column slabs.
+uint32_t resident_form(const tn_plan *p, uint32_t ncols);
 // Whether the rows of a slab of `words` words can be tracked beside a row buffer of
 // `bytes`: row groups that are whole parts of a warp, and copy rings that fit.
 bool tracked_slab(uint32_t words, uint64_t bytes);

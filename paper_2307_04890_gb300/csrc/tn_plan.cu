@@ -66,11 +66,7 @@ constexpr uint32_t kPairGroup = 48;
 // Groups that share nodes and are no longer than this stay with the warp that walks
 // the window: the CTA's barriers would take longer than the group (2.5 us each).
 constexpr uint32_t kWarpGroup = 48;
-// Networks below this size whose slab width is given keep record windows unless
-// the batch is long enough for rows to settle: their levels are short and deep
-// (bursty n = 20,011, 500,009 events, 16 words: 6.6 ms, 11.4 ms in tiles).
-constexpr uint32_t kTileRows = 24928;
-// Default window otherwise.  Larger windows have fewer levels per event, each of
+// Default window of tiles.  Larger windows have fewer levels per event, each of
 // which costs every CTA a barrier and a memory latency, but are scheduled by one
 // CTA each and are stretched by large timestamp groups; 2,000 ops are one pack.  n = 10^5, 10^7
 // activity-driven events: schedule and apply 1.2 + 25.9 ms at 2,480, 1.8 + 23.4 ms
@@ -1082,11 +1078,33 @@ static void free_plan_buffers(tn_plan *p, cudaStream_t st)
     if (p->d_label) cudaFreeAsync(p->d_label, st);
 }
 
+// Whether a schedule made for tiles is walked faster as records, in shared memory:
+// one of short levels, over rows that mostly do not settle.  A level costs a CTA 0.27 us
+// there, 0.85 us (8 words) to 1.5 us (32 words) in tiles, which win by the rows that they
+// need not move.  Apply, tiles and records:
+//  - without ties.  Streams around 96 hubs (60 ops a level), n = 6 10^4: 6 events a node
+//    7.6 and 4.5 ms, 24 events a node 28.2 and 17.4, 50 events a node (every row settles)
+//    28.8 and 35.3; 256 hubs (119), n = 2 10^5: 11.7 and 7.2; activity-driven, n =
+//    2.6 10^4 (122): 2.1 and 2.1, n = 6 10^4 (202): 9.4 and 11.3.
+//  - large timestamp groups that share nodes.  Bursty n = 2.6 10^4, m = 10^6 (81): 21.0
+//    and 15.5 ms; n = 10^5, m = 5 10^6 (306): 90.1 and 62.2; n = 1.2 10^5, m = 10^6
+//    (424): 14.5 and 14.6; n = 2 10^5, m = 5 10^6 (645): 92 and 137.
+// From kRecordLevels levels on: below, the second schedule takes as long as it saves.
+constexpr uint64_t kRecordLevels = 256;
+static bool records_faster(const tn_plan *p)
+{
+    if (p->levels < kRecordLevels) return false;
+    if (16 * p->aux > p->ops) return p->ops < 400 * p->levels && p->m < 64ull * p->n;
+    const uint64_t limit = 72 + p->n / 1024;
+    return p->ops < (limit < 256 ? limit : 256) * p->levels && p->m < 32ull * p->n;
+}
+
 // wait_end: return only once the plan's device buffers are written (else they
-// may be written by work enqueued on `stream`, which later users must follow)
+// may be written by work enqueued on `stream`, which later users must follow).
+// as_records: a plan of open options whose windows are to be records.
 static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const int64_t *t, uint64_t m, uint32_t n,
                                   const int64_t *t_after, const tn_plan_options *opt, void *stream,
-                                  tn_plan **plan_out, bool wait_end)
+                                  tn_plan **plan_out, bool wait_end, bool as_records = false)
 {
     if (!plan_out) return TN_EINVAL;
     *plan_out = nullptr;
@@ -1104,10 +1122,13 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     }
     if (sw < 2 || sw > kMaxSlabWords || (sw & 1u)) return TN_EINVAL;  // even: whole 16-byte chunks
     // everything but the window left open: no records, and the form is chosen when
-    // the plan is applied
-    const bool auto_form = (!opt || (!opt->slab_words && !rows && !wave && !resident)) && n <= resident_max_rows(1);
+    // the plan is applied.  Networks of the same size whose slab width is given keep
+    // record windows unless the batch is long enough for rows to settle: their levels
+    // are short and deep (bursty n = 20,011, 500,009 events, 16 words: 6.6 ms, 11.4 ms
+    // in tiles).
+    const bool auto_form = !as_records && (!opt || (!opt->slab_words && !rows && !wave && !resident)) && n <= resident_max_rows(1);
     const bool auto_window = window == 0 && !resident;
-    if (!window) window = rows || (n < kTileRows && !auto_form && m < 64ull * n) ? kRecordWindow : default_window(m);
+    if (!window) window = rows || as_records || (n <= resident_max_rows(1) && !auto_form && m < 64ull * n) ? kRecordWindow : default_window(m);
     const bool records = !auto_form && !(auto_window && window != kRecordWindow);
     if (window < 32) window = 32;
     if (resident) {
@@ -1262,20 +1283,11 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     p->ops = host.ops;
     p->local_windows = host.local;
     p->big_windows = host.big;
-    if (auto_window && !auto_form && window != kRecordWindow && sw <= 16 && 16 * p->aux > p->ops && p->ops < 256 * p->levels && m < 64ull * n) {
-        // Deep schedules of short levels (hubs that chain large timestamp groups)
-        // over rows that mostly do not settle: records walk their levels in shared
-        // memory.  Bursty n = 8 10^4, m = 2 10^6 (240 ops a level, 25 events a
-        // node): 25.9 ms as records, 32 to 36 ms as tiles; n = 2 10^5, m = 5 10^6
-        // (600 ops a level): 146 ms with windows of 640, 136 ms as tiles.
+    if (auto_window && window != kRecordWindow && sw <= 16 && !(p->auto_form && resident_form(p, n)) && records_faster(p)) {
         free_plan_buffers(p, st);
         if (a.late_arena) cudaFreeAsync(a.late_arena, st);
         free(p);
-        tn_plan_options again;
-        memset(&again, 0, sizeof(again));
-        if (opt) again = *opt;
-        again.window_events = kRecordWindow;
-        return plan_create_impl(u, v, t, m, n, t_after, &again, stream, plan_out, wait_end);
+        return plan_create_impl(u, v, t, m, n, t_after, opt, stream, plan_out, wait_end, true);
     }
     if (resident && !resident_fits(n, p->temps, resident)) {  // saved rows of the tie groups do not fit
         rc = TN_EINVAL;

@@ -74,3 +74,31 @@ def test_a_short_last_window(windows, ties, directed):
     assert (stats["ops"], stats["levels"]) == (whole["ops"], whole["levels"])
     if windows > 64:  # the counters are those of a plan that never had a record
         assert all(stats[k] == whole[k] for k in ("items", "aux", "temps"))
+
+
+def hubs(n, m, h, ties, seed):
+    """Every event joins one of h hubs and any other node; `ties` events a timestamp."""
+    rng = np.random.default_rng(seed)
+    return rng.integers(0, h, m), rng.integers(h, n, m), np.arange(m) // ties
+
+
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("stream", ["hubs", "bursty", "open"])
+def test_short_levels_become_records(stream, directed):
+    """Open options: streams of short levels, without ties, with large timestamp groups,
+    and of a network whose rows would fit a resident CTA but for its saved rows."""
+    if stream == "hubs":
+        n, events = 26_000, hubs(26_000, 60_000, 32, 1, 1)
+    elif stream == "bursty":
+        n = 26_000
+        events = synth.powerlaw_bursty(n, 100_000, seed=3)
+    else:
+        n, events = 24_920, hubs(24_920, 60_000, 1, 64, 2)
+    stats = applied(events, n, directed=directed).stats()
+    assert stats["levels"] >= 256 and 0 < stats["local_windows"] <= stats["windows"] == -(-len(events[0]) // 640)
+
+
+def test_long_levels_stay_tiles():
+    n = 26_000
+    stats = applied(synth.er_poisson(n, 200_000, seed=3), n).stats()
+    assert stats["levels"] >= 256 and stats["local_windows"] == 0
