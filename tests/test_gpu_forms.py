@@ -45,9 +45,10 @@ def test_row_buffer_of_an_open_width(rows, threads, tmp_path):
     plan = applied((u, v, np.arange(m) // 1000), n, slab_words=0, **options)
     assert plan.stats()["local_windows"] == 0
     S = torch.empty((n, tn.tn_row_words(n)), dtype=torch.int64, device="cuda")
-    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
-        plan.apply(S, init=True)
-        torch.cuda.synchronize()
+    for _ in range(2):  # (a process's first session may start too late for its kernels)
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+            plan.apply(S, init=True)
+            torch.cuda.synchronize()
     prof.export_chrome_trace(str(tmp_path / "trace.json"))
     trace = json.loads((tmp_path / "trace.json").read_text())["traceEvents"]
     blocks = [e["args"]["block"][0] for e in trace if "stream_kernel" in e.get("name", "") and "block" in e.get("args", {})]
@@ -79,7 +80,9 @@ def test_a_short_last_window(windows, ties, directed):
 def hubs(n, m, h, ties, seed):
     """Every event joins one of h hubs and any other node; `ties` events a timestamp."""
     rng = np.random.default_rng(seed)
-    return rng.integers(0, h, m), rng.integers(h, n, m), np.arange(m) // ties
+    ends = np.stack([rng.integers(0, h, m), rng.integers(h, n, m)])
+    u, v = np.where(rng.random(m) < 0.5, ends, ends[::-1])
+    return u, v, np.arange(m) // ties
 
 
 @pytest.mark.parametrize("directed", [False, True])
@@ -93,7 +96,8 @@ def test_short_levels_become_records(stream, directed):
         n = 26_000
         events = synth.powerlaw_bursty(n, 100_000, seed=3)
     else:
-        n, events = 24_920, hubs(24_920, 60_000, 1, 64, 2)
+        n = tn.tn_resident_max_rows(1)
+        events = hubs(n, 60_000, 1, 64, 2)
     stats = applied(events, n, directed=directed).stats()
     assert stats["levels"] >= 256 and 0 < stats["local_windows"] <= stats["windows"] == -(-len(events[0]) // 640)
 
