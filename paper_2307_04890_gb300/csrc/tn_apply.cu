@@ -2089,6 +2089,12 @@ uint32_t resident_form(const tn_plan *p, uint32_t ncols)
     return rw;
 }
 
+uint64_t resident_waves(uint32_t ncols, uint32_t words)
+{
+    const uint64_t ctas = ((ncols + 63ull) / 64 + words - 1) / words, sms = (uint64_t)multiprocessors();
+    return (ctas + sms - 1) / sms;
+}
+
 // Whether content ids of `bytes` may be allocated on `st`.  A call learns from the
 // allocation itself that there is no room; a capture only records it, and the graph's
 // launch would fail instead.  `held`: bytes of the launch's earlier ids; half of the
@@ -2465,7 +2471,7 @@ static tn_status one_shot(const uint32_t *u, const uint32_t *v, const int64_t *t
     memset(&opt, 0, sizeof(opt));
     opt.directed = (flags & TN_DIRECTED) ? 1u : 0u;
     tn_plan *plan = nullptr;
-    tn_status rc = tn_plan_create(u, v, t, m, n, t_last, &opt, stream, &plan);
+    tn_status rc = plan_create_for(u, v, t, m, n, t_last, &opt, ncols, stream, &plan);
     if (rc != TN_OK) return rc;
     flags &= ~TN_DIRECTED;
     rc = apply_jobs((const tn_plan *const *)&plan, &S, &ncols, &src, &t_last, 1, flags, st);

@@ -332,6 +332,7 @@ uint32_t resident_max_rows(uint32_t words);
 // Words of a row per resident CTA that an open plan takes when it alone is applied to
 // `ncols` columns; 0: column slabs.
 uint32_t resident_form(const tn_plan *p, uint32_t ncols);
+uint64_t resident_waves(uint32_t ncols, uint32_t words);
 // Whether the rows of a slab of `words` words can be tracked beside a row buffer of
 // `bytes`: row groups that are whole parts of a warp, and copy rings that fit.
 bool tracked_slab(uint32_t words, uint64_t bytes);
@@ -355,6 +356,10 @@ tn_status online_use_apply_stream(tn_online *online, cudaStream_t apply_stream);
 // Two-stream mode: the device status word every batch's plan records errors
 // in (0 = none), for a caller that copies it out behind the updates.
 const int32_t *online_status_word(const tn_online *online);
+// tn_plan_create for a plan that will be applied to `ncols` columns.
+tn_status plan_create_for(const uint32_t *u, const uint32_t *v, const int64_t *t, uint64_t m, uint32_t n,
+                          const int64_t *t_after, const tn_plan_options *opt, uint32_t ncols, void *stream,
+                          tn_plan **plan_out);
 // tn_plan_create without its last host wait: the plan's device buffers are
 // written by work enqueued on `stream`, so a use on another stream must first
 // wait for an event recorded on `stream` after this call.

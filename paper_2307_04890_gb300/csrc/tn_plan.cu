@@ -150,6 +150,7 @@ struct PlanCounters {
     unsigned long long blob8, naux, list_words, items, ops, levels, local, temps;
     unsigned long long blob_used, aux_used;  // allocation of the exact buffers
     long long t_first, t_last;
+    unsigned long long chain; // sum over the levels of tiles of their longest source list
     unsigned long long done;  // CTAs of the first pass
 };
 
@@ -168,6 +169,7 @@ struct PlanArgs {
     uint32_t smem_max;   // largest window scheduled in shared memory
     uint32_t dcap;       // row slots of a local window
     uint32_t unit8;      // staging units (8 bytes) per event
+    uint32_t chain;      // 1: count the longest source lists
     uint32_t redo;       // 1: the windows scheduled as records become tiles
     uint64_t *wstart;    // [nw + 1]
     uint32_t *naux_w;    // [nw] source-list entries of every window
@@ -761,11 +763,22 @@ __device__ __forceinline__ void schedule_window(const PlanArgs &a, uint32_t w, u
         // one with more ops than a pack holds is cut.  Warp 0 cuts the packs and
         // writes their headers.
         uint32_t *la = A.scratch + maxlev + 2;  // list words of the levels before
-        uint32_t *pq = la + maxlev + 2;         // per pack: first op, its unit, next free list word (0: none), spare
-        for (uint32_t j = tid; j < maxlev + 1; j += T) la[j] = 0;
+        uint32_t *lm = la + maxlev + 2;         // longest list of the level (a.chain)
+        uint32_t *pq = lm + maxlev + 2;         // per pack: first op, its unit, next free list word (0: none), spare
+        for (uint32_t j = tid; j < maxlev + 1; j += T) la[j] = lm[j] = 0;
         __syncthreads();
-        for (uint32_t r = tid; r < nruns; r += T) atomicAdd(&la[A.run_lev[r]], 1u + auxw[A.run_aux[r]]);
+        for (uint32_t r = tid; r < nruns; r += T) {
+            const uint32_t c = auxw[A.run_aux[r]];
+            atomicAdd(&la[A.run_lev[r]], 1u + c);
+            if (a.chain) atomicMax(&lm[A.run_lev[r]], c);
+        }
         __syncthreads();
+        if (a.chain && nruns) {
+            uint32_t sum = 0;
+            for (uint32_t j = tid; j < maxlev + 1; j += T) sum += lm[j];
+            sum = __reduce_add_sync(0xffffffffu, sum);
+            if (lane == 0 && sum) atomicAdd(&a.cnt->chain, (unsigned long long)sum);
+        }
         block_excl_scan_array(la, maxlev + 1, warp_sums, &tot);
         if (tid < 32) {
             uint32_t p = 0, l = 0, q = 0, unit = 0, outside = 0;
@@ -1089,11 +1102,28 @@ static void free_plan_buffers(tn_plan *p, cudaStream_t st)
 //  - large timestamp groups that share nodes.  Bursty n = 2.6 10^4, m = 10^6 (81): 21.0
 //    and 15.5 ms; n = 10^5, m = 5 10^6 (306): 90.1 and 62.2; n = 1.2 10^5, m = 10^6
 //    (424): 14.5 and 14.6; n = 2 10^5, m = 5 10^6 (645): 92 and 137.
+// Resident CTAs walk a level in 0.1 us (rows of two words 0.12, in packs with ties 0.17
+// and 0.2), but one thread combines a PULL's sources (27 or 36 ns each, all others wait
+// at the level's barrier), every wave of CTAs walks all levels, and 16-word records of
+// such a network take one wave.  Settled rows are not walked, from about 20 events a node
+// on.  The estimates of both, apply (estimate), n = 24,000, 200,000 events around one hub:
+//   groups of 3, 8, 64 events: resident 75.3 (78.9), 41.3 (41.8), 19.0 (19.5) ms, records
+//   45.5 (40.5), 15.4 (16.5), 4.3 (4.3); no groups 59.9 (60.3), 54.3 (55.6); n = 12,000,
+//   groups of 8, 64: 16.1 (17.2), 7.3 (8.5), records 15.3 (16.5), 4.3 (4.3); bursty n =
+//   20,011, m = 500,009: 6.1, records 7.1 (6.3).  The margin covers the error.
 // From kRecordLevels levels on: below, the second schedule takes as long as it saves.
 constexpr uint64_t kRecordLevels = 256;
-static bool records_faster(const tn_plan *p)
+static bool records_faster(const tn_plan *p, uint64_t chain, uint32_t ncols)
 {
     if (p->levels < kRecordLevels) return false;
+    const uint32_t rw = p->auto_form ? resident_form(p, ncols) : 0u;
+    if (rw) {
+        const double L = (double)p->levels, ops = (double)p->ops, waves = (double)resident_waves(ncols, rw);
+        const double level = rw == 1 ? (p->aux ? 170.0 : 100.0) : (p->aux ? 200.0 : 120.0);
+        const double moving = 20.0 * p->n < (double)p->m ? 20.0 * p->n / (double)p->m : 1.0;
+        const double resident = moving * waves * (level * L + 0.5 * ops + (rw == 1 ? 27.0 : 36.0) * (double)chain);
+        return resident > 1.25 * (270.0 * L + 7.8 * ops + 5.0 * (double)chain);
+    }
     if (16 * p->aux > p->ops) return p->ops < 400 * p->levels && p->m < 64ull * p->n;
     const uint64_t limit = 72 + p->n / 1024;
     return p->ops < (limit < 256 ? limit : 256) * p->levels && p->m < 32ull * p->n;
@@ -1101,10 +1131,11 @@ static bool records_faster(const tn_plan *p)
 
 // wait_end: return only once the plan's device buffers are written (else they
 // may be written by work enqueued on `stream`, which later users must follow).
-// as_records: a plan of open options whose windows are to be records.
+// ncols: columns that the plan is made for (0: one per node).  as_records: a plan of
+// open options whose windows are to be records.
 static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const int64_t *t, uint64_t m, uint32_t n,
                                   const int64_t *t_after, const tn_plan_options *opt, void *stream,
-                                  tn_plan **plan_out, bool wait_end, bool as_records = false)
+                                  tn_plan **plan_out, bool wait_end, uint32_t ncols, bool as_records = false)
 {
     if (!plan_out) return TN_EINVAL;
     *plan_out = nullptr;
@@ -1161,6 +1192,7 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     const uint64_t first_max = window + window_slack(window) < m ? window + window_slack(window) : m;
     a.first_max = first_max < a.smem_max ? (uint32_t)first_max : a.smem_max;
     a.dcap = rows;
+    a.chain = auto_form;
     a.unit8 = window <= kRecordEvents && rows > 1 && records ? 5 : 4;
 
     tn_plan *p = (tn_plan *)calloc(1, sizeof(tn_plan));
@@ -1283,11 +1315,11 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     p->ops = host.ops;
     p->local_windows = host.local;
     p->big_windows = host.big;
-    if (auto_window && window != kRecordWindow && sw <= 16 && !(p->auto_form && resident_form(p, n)) && records_faster(p)) {
+    if (auto_window && window != kRecordWindow && sw <= 16 && records_faster(p, host.chain, ncols ? ncols : n)) {
         free_plan_buffers(p, st);
         if (a.late_arena) cudaFreeAsync(a.late_arena, st);
         free(p);
-        return plan_create_impl(u, v, t, m, n, t_after, opt, stream, plan_out, wait_end, true);
+        return plan_create_impl(u, v, t, m, n, t_after, opt, stream, plan_out, wait_end, ncols, true);
     }
     if (resident && !resident_fits(n, p->temps, resident)) {  // saved rows of the tie groups do not fit
         rc = TN_EINVAL;
@@ -1342,13 +1374,20 @@ extern "C" tn_status tn_plan_create(const uint32_t *u, const uint32_t *v, const 
                                     uint32_t n, const int64_t *t_after, const tn_plan_options *opt,
                                     void *stream, tn_plan **plan_out)
 {
-    return plan_create_impl(u, v, t, m, n, t_after, opt, stream, plan_out, true);
+    return plan_create_impl(u, v, t, m, n, t_after, opt, stream, plan_out, true, 0);
+}
+
+tn_status tn::plan_create_for(const uint32_t *u, const uint32_t *v, const int64_t *t, uint64_t m, uint32_t n,
+                              const int64_t *t_after, const tn_plan_options *opt, uint32_t ncols, void *stream,
+                              tn_plan **plan_out)
+{
+    return plan_create_impl(u, v, t, m, n, t_after, opt, stream, plan_out, true, ncols);
 }
 
 tn_status tn::plan_create_ordered(const uint32_t *u, const uint32_t *v, const int64_t *t, uint64_t m, uint32_t n,
                                   const tn_plan_options *opt, cudaStream_t stream, tn_plan **plan_out)
 {
-    return plan_create_impl(u, v, t, m, n, nullptr, opt, stream, plan_out, false);
+    return plan_create_impl(u, v, t, m, n, nullptr, opt, stream, plan_out, false, 0);
 }
 
 extern "C" tn_status tn_plan_destroy(tn_plan *p, void *stream)

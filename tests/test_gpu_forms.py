@@ -106,3 +106,11 @@ def test_long_levels_stay_tiles():
     n = 26_000
     stats = applied(synth.er_poisson(n, 200_000, seed=3), n).stats()
     assert stats["levels"] >= 256 and stats["local_windows"] == 0
+
+
+@pytest.mark.parametrize("n,h,ties,records", [(24_000, 1, 64, True), (24_000, 12, 300, True), (24_000, 500, 1, False)])
+def test_resident_networks_around_hubs(n, h, ties, records):
+    """Open options, rows that fit resident CTAs: long source lists in every level are
+    walked as records, streams without them stay resident."""
+    stats = applied(hubs(n, 100_000, h, ties, n + h), n).stats()
+    assert stats["levels"] >= 256 and (stats["local_windows"] > 0) == records
