@@ -1026,7 +1026,7 @@ def run_sweep(args, w, rank, world, local_rank):
         ex = tn.tn_autotune(dus, dvs, dts, n, sample_events=2_000_000)
         _, pus, pvs = tn.tn_hash_proxy(dus, dvs, n, k, K, w["seed"])
         px = tn.tn_autotune(pus[0].contiguous(), pvs[0].contiguous(), dts, k, replicas=K, sample_events=2_000_000)
-        tuned[n] = ({key: ex[key] for key in keys}, {key: px[key] for key in keys})
+        tuned[n] = tuple({key: r[key] if r["best_ms"] <= r["open_ms"] else 0 for key in keys} for r in (ex, px))
         del dus, dvs, dts, pus, pvs
         m = 10_000
         while m <= mmax:
@@ -1166,8 +1166,8 @@ def main():
     tuned = None
     if args.autotune == "on" or (args.autotune == "auto" and w["kind"] in ("bursty", "er")):
         tuned = tn.tn_autotune(du, dv, dt, n, sample_events=args.tune_sample, ncols=ncols)
-        opts = {key: tuned[key] for key in ("window_events", "slab_words", "smem_rows", "wave_ctas",
-                                             "resident_words")}
+        opts = {key: tuned[key] if tuned["best_ms"] <= tuned["open_ms"] else 0
+                for key in ("window_events", "slab_words", "smem_rows", "wave_ctas", "resident_words")}
 
     def step(record):
         plan = tn.Plan(du, dv, dt, n, **opts)                                            # a1
@@ -1213,13 +1213,14 @@ def main():
     # roofline of the dominant kernel (the column-slab stream of this rank)
     words = (ncols + 63) // 64
     rw = opts.get("resident_words", 0)
+    sw = opts["slab_words"]
     peak, peak_kind = measured_peaks()
     # An update whose rows are already equal moves no row, so the bytes of all
     # updates over the time are no bandwidth (they may exceed the peak); the
     # launch's DRAM bytes (ncu) are, or, without them, what no launch on these
     # sources can do without: the schedule in once and the matrix out once.
     update_bytes = m * 4 * words * 8
-    traffic = profiled_traffic(args.workload, opts["slab_words"] or 16) if world == 1 and not rw else None
+    traffic = profiled_traffic(args.workload, sw) if world == 1 and sw else None
     alg_bytes = 8 * stats["ops"] + n * W * 8
     achieved = (traffic or alg_bytes) / (k1_ms * 1e-3) / 1e9
     roofline = {"bound": "hbm", "kernel": "stream_kernel" + (" (resident slabs)" if rw else ""),
@@ -1242,11 +1243,11 @@ def main():
                          "parallelism": f"source columns split over {world} GPUs, sizes all-gathered"
                                         if world > 1 else "single GPU",
                          "l2": "inputs larger than L2 (S %.2f GB, events %.0f MB)" % (n * W * 8 / 1e9, m * 16 / 1e6),
-                         "window_events": opts["window_events"] or 640,
-                         "slab_words": None if rw else (opts["slab_words"] or 16),
+                         "window_events": opts["window_events"] or "chosen by the library",
+                         "slab_words": None if rw else (sw or "chosen at launch"),
                          "smem_rows": None if rw else (opts["smem_rows"] or "default"),
                          "resident_words": rw or None,
-                         "ctas": -(-words // rw) if rw else -(-tn.tn_row_words(ncols) // (opts["slab_words"] or 16)),
+                         "ctas": -(-words // rw) if rw else -(-tn.tn_row_words(ncols) // sw) if sw else None,
                          "autotuned": tuned is not None,
                          "levels": stats["levels"], "ops": stats["ops"], "windows": stats["windows"],
                          "global_memory_windows": stats["windows"] - stats["local_windows"]},

@@ -322,8 +322,8 @@ tn_status tn_graph_launch(tn_graph *graph, void *stream);
 tn_status tn_graph_destroy(tn_graph *graph);
 
 /* ---------------------------------------------------------------------------
- * tn_autotune -- picks the plan options (slab width = columns per CTA, window
- * depth, shared-memory row buffer = CTAs per SM) for a batch of `replicas`
+ * tn_autotune -- picks the fastest of the plan options below (slab width = columns
+ * per CTA, window depth, shared-memory row buffer = CTAs per SM) for a batch of `replicas`
  * networks shaped like (u, v, t, m, n), each with `ncols` source columns
  * (0 = n; fewer = a column subset as in tn_component_columns).  The full problem runs replicas x
  * ceil(row words / slab) CTAs in waves of (SMs x CTAs per SM); every candidate
@@ -335,7 +335,9 @@ tn_status tn_graph_destroy(tn_graph *graph);
  * most the row width), window 320/640/1024 events, row buffer 160 or 80 KB
  * (192 KB above 16 words).  Candidates of the resident-slab form, when the
  * network's rows fit (tn_resident_max_rows): resident_words 1/2, window
- * 640/2048 events.  Scratch of one timing run is kept under half of the free
+ * 640/2048 events.  A plan with every option 0, whose form is chosen at launch (its
+ * windows are no candidates here), is timed as well, on the whole problem where that
+ * fits the scratch: leave the options out when open_ms is below best_ms.  Scratch of one timing run is kept under half of the free
  * device memory and 64 GiB.  The choice is cached per (device, n, ncols,
  * replicas, floor(log2 m)) for the life of the process.  Synchronous.
  */
@@ -344,7 +346,7 @@ typedef struct tn_tune_result {
     float best_ms;          /* its score: waves x timed sample + replicas x plan time (ms) */
     uint32_t tried;         /* candidates timed */
     uint32_t cached;        /* 1 if the result came from the cache */
-    uint32_t pad;
+    float open_ms;          /* the score of a plan with every option 0 (ms) */
     uint64_t sample_events;
 } tn_tune_result;
 

@@ -88,7 +88,7 @@ class _ServerStats(ctypes.Structure):
 
 class _TuneResult(ctypes.Structure):
     _fields_ = [("best", _Options), ("best_ms", ctypes.c_float), ("tried", ctypes.c_uint32),
-                ("cached", ctypes.c_uint32), ("pad", ctypes.c_uint32), ("sample_events", ctypes.c_uint64)]
+                ("cached", ctypes.c_uint32), ("open_ms", ctypes.c_float), ("sample_events", ctypes.c_uint64)]
 
 
 class _Stats(ctypes.Structure):
@@ -560,7 +560,9 @@ def tn_autotune(u, v, t, n: int, replicas: int = 1, sample_events: int = 200_000
                 stream=None) -> dict:
     """Plan options for a batch of ``replicas`` networks shaped like (u, v, t, n)
     with ``ncols`` source columns each (0 = n), chosen by timing the candidates
-    on the first ``sample_events`` events (scored as waves x one wave's time)."""
+    on the first ``sample_events`` events (scored as waves x one wave's time).
+    ``open_ms`` is the score of a plan without options: where it is below
+    ``best_ms``, leave them out."""
     lib = load_library()
     m = _events(u, v, t)
     res = _TuneResult()
@@ -568,7 +570,7 @@ def tn_autotune(u, v, t, n: int, replicas: int = 1, sample_events: int = 200_000
                            ctypes.byref(res)), "tn_autotune")
     return {"window_events": res.best.window_events, "slab_words": res.best.slab_words,
             "smem_rows": res.best.smem_rows, "wave_ctas": res.best.wave_ctas,
-            "resident_words": res.best.resident_words, "best_ms": res.best_ms, "tried": res.tried,
+            "resident_words": res.best.resident_words, "best_ms": res.best_ms, "open_ms": res.open_ms, "tried": res.tried,
             "cached": bool(res.cached), "sample_events": res.sample_events}
 
 

@@ -11,7 +11,8 @@
 // size of the shared-memory row buffer (hence CTAs per SM), or the
 // resident-slab form for small networks -- by timing the candidates (their
 // schedule and their application) on a prefix of the events, for a batch of
-// `replicas` networks of the same size, and caches the choice per (device, n,
+// `replicas` networks of the same size, times a plan without any options beside
+// them, and caches the choice per (device, n,
 // ncols, replicas, log2 m).
 #include <cuda_runtime.h>
 #include <math.h>
@@ -329,6 +330,57 @@ extern "C" tn_status tn_autotune(const uint32_t *u, const uint32_t *v, const int
                 out->best = opt;
                 out->best_ms = score;
             }
+        }
+        for (uint64_t *p : mats)
+            if (p) cudaFreeAsync(p, st);
+    }
+    // no options at all: the form is the launch's choice, made for the whole problem, so
+    // all of it is timed where it fits the scratch limit (slabs are 64 words wide where
+    // one matrix does not), else its share by columns and replicas
+    if (rc == TN_OK) {
+        uint32_t ncols = ncols_full;
+        const uint64_t slots = (uint64_t)nsm, full_ctas = (used_words + kTuneWidest - 1) / kTuneWidest;
+        double scale = 1.0;
+        if ((uint64_t)n * ld * 8 > kTuneBytesLimit) {
+            uint64_t c = slots < full_ctas ? slots : full_ctas;
+            while (c > 1 && (uint64_t)n * tn_row_words(c * kTuneWidest * 64) * 8 > kTuneBytesLimit) c /= 2;
+            if (c * kTuneWidest * 64 < ncols_full) {
+                ncols = (uint32_t)(c * kTuneWidest * 64);
+                scale = (double)((full_ctas + slots - 1) / slots);
+            }
+        }
+        if (ncols < n && ncols > max_cols) {
+            ncols = max_cols;
+            scale = (double)ncols_full / max_cols;
+        }
+        const uint32_t *src = ncols < n ? ids : nullptr;
+        const uint64_t mbytes = (uint64_t)n * tn_row_words(ncols) * 8;
+        uint32_t reps = replicas;
+        while (reps > 1 && reps * mbytes > kTuneBytesLimit) --reps;
+        scale *= (double)replicas / reps;
+        std::vector<uint64_t *> mats(reps, nullptr);
+        for (uint32_t r = 0; r < reps && rc == TN_OK; ++r) {
+            const cudaError_t e = cudaMallocAsync((void **)&mats[r], mbytes, st);
+            if (e != cudaSuccess) {
+                tn_internal_set_cuda_error(e);
+                rc = e == cudaErrorMemoryAllocation ? TN_ENOMEM : TN_ECUDA;
+            }
+        }
+        tn_plan_options opt;
+        memset(&opt, 0, sizeof(opt));
+        tn_plan *plan = nullptr;
+        float pms = 0.f, tms = INFINITY;
+        if (rc == TN_OK) rc = timed_plan(u, v, t, msample, n, &opt, st, &plan, &pms);
+        if (rc == TN_OK) {
+            rc = time_apply(plan, mats.data(), reps, ncols, src, st, &tms);
+            if (rc == TN_OK) rc = tn_plan_status(plan, st);
+            tn_plan_destroy(plan, st);
+            out->tried++;
+            out->open_ms = (float)(tms * scale) + pms * (float)replicas;
+        }
+        if (rc == TN_ENOMEM) {  // the candidates fitted: their answer stands
+            out->open_ms = INFINITY;
+            rc = TN_OK;
         }
         for (uint64_t *p : mats)
             if (p) cudaFreeAsync(p, st);

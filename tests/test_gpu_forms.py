@@ -114,3 +114,12 @@ def test_resident_networks_around_hubs(n, h, ties, records):
     walked as records, streams without them stay resident."""
     stats = applied(hubs(n, 100_000, h, ties, n + h), n).stats()
     assert stats["levels"] >= 256 and (stats["local_windows"] > 0) == records
+
+
+@pytest.mark.parametrize("n,m,replicas,ncols", [(2000, 40_000, 3, 0), (30_000, 60_000, 1, 0), (30_000, 60_000, 2, 1500)])
+def test_autotune_times_a_plan_without_options(n, m, replicas, ncols):
+    events = dev(*synth.activity_driven(n, m, seed=n))
+    first = tn.tn_autotune(*events, n, replicas=replicas, ncols=ncols)
+    assert 0 < first["open_ms"] < float("inf") and 0 < first["best_ms"] < float("inf")
+    again = tn.tn_autotune(*events, n, replicas=replicas, ncols=ncols)
+    assert again["cached"] and again["open_ms"] == first["open_ms"]
