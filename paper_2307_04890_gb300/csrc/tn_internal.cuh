@@ -316,6 +316,7 @@ struct tn_plan {
     tn::WinDesc *d_win;   // [windows]    their windows in time order
     uint32_t *d_aux;      // source lists outside the packs
     void *d_mem;          // owned: head, window bounds, windows, and packs and lists unless they are compacted
+    void *d_packs;        // owned: packs and lists that are (NULL: in d_mem)
     uint32_t *d_label;    // [n] component of every node, a node id (NULL: not computed)
     tn::PlanHead *d_head; // owned: counters, time bounds, status word
     int64_t *d_tbounds;   // [2]          t_first, t_last (in d_head)

@@ -78,8 +78,10 @@ static uint32_t default_window(uint64_t m) { return m < (1u << 16) ? 1280u : 200
 // rest of its last timestamp group (2,400 events at the largest default window: two
 // CTAs per SM).
 static uint64_t window_slack(uint32_t window) { return window < 320 ? 64 : window / 5; }
-// Batches of at least this many events are copied into buffers of their exact
-// size; below it the staging buffers (a few times larger, bounded) are kept.
+// Batches of at least this many events are copied into buffers of their exact size (8
+// to 12 bytes per event); below it the staging buffers (44 to 53 bytes) are kept, except
+// by plans made without a host wait: an online state with its own update stream keeps up
+// to kOnlineFlight of them, and the serving engine charges a job for exact ones.
 constexpr uint64_t kCompactEvents = 1ull << 20;
 // Batches whose rows may all settle well before the end: component labels (three
 // launches), for the forms that use them.
@@ -1083,10 +1085,7 @@ using namespace tn;
 
 static void free_plan_buffers(tn_plan *p, cudaStream_t st)
 {
-    if (p->m >= kCompactEvents) {  // (else in d_mem)
-        if (p->d_blob) cudaFreeAsync(p->d_blob, st);
-        if (p->d_aux) cudaFreeAsync(p->d_aux, st);
-    }
+    if (p->d_packs) cudaFreeAsync(p->d_packs, st);
     if (p->d_mem) cudaFreeAsync(p->d_mem, st);
     if (p->d_label) cudaFreeAsync(p->d_label, st);
 }
@@ -1212,9 +1211,9 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     tn_status rc = TN_OK;
     PlanCounters host;
     memset(&host, 0, sizeof(host));
-    uint2 *exact_blob = nullptr;
-    uint32_t *exact_aux = nullptr;
+    void *exact = nullptr;
     bool must_wait = false;
+    const bool compact = m >= kCompactEvents || !wait_end;
     const uint64_t blocks = (m + 1023) / 1024;
     cudaError_t err = cudaSuccess;
 
@@ -1231,20 +1230,19 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
         const uint64_t at_bounds = part(sizeof(PlanHead)), at_win = at_bounds + part(8 * (3ull * a.nw + 2));
         const uint64_t at_blob = at_win + part(sizeof(WinDesc) * (uint64_t)a.nw);
         const uint64_t blob_bytes = part(8 * (blob_base(m, a.nw, a.unit8) + 64)), aux_bytes = 12 * m;
-        const bool apart = m >= kCompactEvents;
         uint8_t *mem = nullptr;
-        TN_STEP(alloc_async(&mem, apart ? at_blob : at_blob + blob_bytes + aux_bytes, st));
+        TN_STEP(alloc_async(&mem, compact ? at_blob : at_blob + blob_bytes + aux_bytes, st));
         p->d_mem = mem;
         p->d_head = reinterpret_cast<PlanHead *>(mem);
         a.wstart = reinterpret_cast<uint64_t *>(mem + at_bounds);
         p->d_win = reinterpret_cast<WinDesc *>(mem + at_win);
-        if (apart) {
-            TN_STEP(alloc_async(&p->d_blob, blob_bytes / 8, st));
-            TN_STEP(alloc_async(&p->d_aux, 3 * m, st));
-        } else {
-            p->d_blob = reinterpret_cast<uint2 *>(mem + at_blob);
-            p->d_aux = reinterpret_cast<uint32_t *>(mem + at_blob + blob_bytes);
+        uint8_t *packs = mem + at_blob;
+        if (compact) {
+            TN_STEP(alloc_async(&packs, blob_bytes + aux_bytes, st));
+            p->d_packs = packs;
         }
+        p->d_blob = reinterpret_cast<uint2 *>(packs);
+        p->d_aux = reinterpret_cast<uint32_t *>(packs + blob_bytes);
     }
     p->d_status = &p->d_head->status;
     p->d_tbounds = p->d_head->tbounds;
@@ -1335,19 +1333,20 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
         TN_STEP(cudaGetLastError());
         must_wait = true;
     }
-    if (m >= kCompactEvents) {
+    if (compact) {
         must_wait = true;
-        TN_STEP(alloc_async(&exact_blob, p->blob8 + 2, st));
-        TN_STEP(alloc_async(&exact_aux, host.list_words, st));
+        const uint64_t lists_at = p->blob8 + 2;  // in units; no list outside the packs: no list buffer
+        TN_STEP(cudaMallocAsync(&exact, 8 * lists_at + 4 * host.list_words, st));
+        uint2 *blob = static_cast<uint2 *>(exact);
+        uint32_t *aux = reinterpret_cast<uint32_t *>(blob + lists_at);
         tn_internal_count_launches(1);
-        compact_kernel<<<a.nw, 256, 0, st>>>(a, exact_blob, exact_aux);
+        compact_kernel<<<a.nw, 256, 0, st>>>(a, blob, aux);
         TN_STEP(cudaGetLastError());
-        cudaFreeAsync(p->d_blob, st);
-        cudaFreeAsync(p->d_aux, st);
-        p->d_blob = exact_blob;  // (no list outside the packs: no list buffer)
-        p->d_aux = exact_aux;
-        exact_blob = nullptr;
-        exact_aux = nullptr;
+        cudaFreeAsync(p->d_packs, st);
+        p->d_packs = exact;
+        p->d_blob = blob;
+        p->d_aux = aux;
+        exact = nullptr;
     }
     // the plan is complete, and its events are read, when this call returns
     if (must_wait && wait_end) TN_STEP(tn_internal_stream_wait(st));
@@ -1359,8 +1358,7 @@ fail:
 done:
     if (a.late_arena) cudaFreeAsync(a.late_arena, st);
     if (rc != TN_OK) {
-        if (exact_blob) cudaFreeAsync(exact_blob, st);
-        if (exact_aux) cudaFreeAsync(exact_aux, st);
+        if (exact) cudaFreeAsync(exact, st);
         free_plan_buffers(p, st);
         free(p);
         return rc;
