@@ -1104,12 +1104,14 @@ static void free_plan_buffers(tn_plan *p, cudaStream_t st)
 // Resident CTAs walk a level in 0.1 us (rows of two words 0.12, in packs with ties 0.17
 // and 0.2), but one thread combines a PULL's sources (27 or 36 ns each, all others wait
 // at the level's barrier), every wave of CTAs walks all levels, and 16-word records of
-// such a network take one wave.  Settled rows are not walked, from about 20 events a node
-// on.  The estimates of both, apply (estimate), n = 24,000, 200,000 events around one hub:
+// such a network take one wave.  Levels of settled rows are not walked: from about 11
+// events a node on, with long source lists from about 24.  Apply (estimate) around one
+// hub, n = 24,000, m = 200,000:
 //   groups of 3, 8, 64 events: resident 75.3 (78.9), 41.3 (41.8), 19.0 (19.5) ms, records
-//   45.5 (40.5), 15.4 (16.5), 4.3 (4.3); no groups 59.9 (60.3), 54.3 (55.6); n = 12,000,
-//   groups of 8, 64: 16.1 (17.2), 7.3 (8.5), records 15.3 (16.5), 4.3 (4.3); bursty n =
-//   20,011, m = 500,009: 6.1, records 7.1 (6.3).  The margin covers the error.
+//   45.5 (40.5), 15.4 (16.5), 4.3 (4.3); no groups 59.9 (60.3), 54.3 (55.6); 30 events a
+//   node in groups of 4: 97.8 (114), records 108 (107); n = 12,000, groups of 8, 64: 16.1
+//   (17.2), 7.3 (8.5), records 15.3 (16.5), 4.3 (4.3).  Bursty n = 20,011, m = 500,009:
+//   6.1, records 7.1 (6.3).  The margin covers the error.
 // From kRecordLevels levels on: below, the second schedule takes as long as it saves.
 constexpr uint64_t kRecordLevels = 256;
 static bool records_faster(const tn_plan *p, uint64_t chain, uint32_t ncols)
@@ -1119,8 +1121,9 @@ static bool records_faster(const tn_plan *p, uint64_t chain, uint32_t ncols)
     if (rw) {
         const double L = (double)p->levels, ops = (double)p->ops, waves = (double)resident_waves(ncols, rw);
         const double level = rw == 1 ? (p->aux ? 170.0 : 100.0) : (p->aux ? 200.0 : 120.0);
-        const double moving = 20.0 * p->n < (double)p->m ? 20.0 * p->n / (double)p->m : 1.0;
-        const double resident = moving * waves * (level * L + 0.5 * ops + (rw == 1 ? 27.0 : 36.0) * (double)chain);
+        const double per_event = (double)p->n / (double)p->m;
+        const double walked = 11.0 * per_event < 1.0 ? 11.0 * per_event : 1.0, listed = 24.0 * per_event < 1.0 ? 24.0 * per_event : 1.0;
+        const double resident = waves * (walked * (level * L + 0.5 * ops) + listed * (rw == 1 ? 27.0 : 36.0) * (double)chain);
         return resident > 1.25 * (270.0 * L + 7.8 * ops + 5.0 * (double)chain);
     }
     if (16 * p->aux > p->ops) return p->ops < 400 * p->levels && p->m < 64ull * p->n;
