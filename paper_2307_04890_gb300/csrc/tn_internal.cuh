@@ -315,10 +315,9 @@ struct tn_plan {
     uint2 *d_blob;        // packs (8-byte units)
     tn::WinDesc *d_win;   // [windows]    their windows in time order
     uint32_t *d_aux;      // source lists outside the packs
-    void *d_mem;          // owned: head, window bounds, windows, and packs and lists unless they are compacted
-    void *d_packs;        // owned: packs and lists that are (NULL: in d_mem)
+    void *d_mem;          // owned: all of the below but the labels
     uint32_t *d_label;    // [n] component of every node, a node id (NULL: not computed)
-    tn::PlanHead *d_head; // owned: counters, time bounds, status word
+    tn::PlanHead *d_head; // counters, time bounds, status word
     int64_t *d_tbounds;   // [2]          t_first, t_last (in d_head)
     int32_t *d_status;    // first asynchronous error (in d_head, or the owner's: tn::plan_use_status)
 };

@@ -156,6 +156,14 @@ struct PlanCounters {
     unsigned long long done;  // CTAs of the first pass
 };
 
+// device head of a plan: counters, status word, time bounds
+struct PlanHead {
+    PlanCounters cnt;
+    int64_t tbounds[2];
+    int32_t status;
+    int32_t pad;
+};
+
 struct PlanArgs {
     Mail *mail;  // of the waiting thread, or nullptr
     uint32_t mail_seq;
@@ -950,14 +958,23 @@ __global__ void __launch_bounds__(kPlanThreads) schedule_tiles_kernel(PlanArgs a
     schedule_window<uint16_t>(a, blockIdx.x, smem_arena);
 }
 
-// Copies every window into buffers of the exact size (in no particular order:
-// descriptors name offsets) and moves PULL lists with it.
-__global__ void compact_kernel(PlanArgs a, uint2 *blob, uint32_t *aux)
+// Copies the plan into a buffer of its exact size: what a finished plan needs of the
+// head, and every window (in no particular order: descriptors name offsets) with its
+// PULL lists.
+__global__ void compact_kernel(PlanArgs a, PlanHead *head, WinDesc *to_desc, uint2 *blob, uint32_t *aux)
 {
     __shared__ unsigned long long base[2];
     const uint32_t w = blockIdx.x;
-    WinDesc *desc = a.desc + w;
+    const WinDesc *desc = a.desc + w;
     const uint32_t np = desc->npacks;
+    if (threadIdx.x == 0) {
+        if (w == 0) {
+            head->tbounds[0] = a.tbounds[0];
+            head->tbounds[1] = a.tbounds[1];
+            head->status = 0;
+        }
+        to_desc[w] = *desc;
+    }
     if (np == 0) return;
     const uint64_t src = desc->off;
     const uint32_t naux = a.naux_w[w];
@@ -970,12 +987,12 @@ __global__ void compact_kernel(PlanArgs a, uint2 *blob, uint32_t *aux)
         base[0] = atomicAdd(&a.cnt->blob_used, (unsigned long long)units);
         base[1] = naux ? atomicAdd(&a.cnt->aux_used, (unsigned long long)naux) : 0ull;
     }
-    __syncthreads();  // every thread has read the descriptor
+    __syncthreads();
     const uint64_t dst = base[0];
     const uint4 *from = reinterpret_cast<const uint4 *>(a.blob + src);
     uint4 *to = reinterpret_cast<uint4 *>(blob + dst);
     for (uint32_t k = threadIdx.x; k < units / 2; k += blockDim.x) to[k] = from[k];
-    if (threadIdx.x == 0) desc->off = dst;
+    if (threadIdx.x == 0) to_desc[w].off = dst;
     if (naux == 0) return;
     const uint64_t s3 = 3 * a.wstart[w];
     for (uint32_t k = threadIdx.x; k < naux; k += blockDim.x) aux[base[1] + k] = a.aux[s3 + k];
@@ -1071,21 +1088,12 @@ static cudaError_t alloc_async(T **p, uint64_t count, cudaStream_t st)
     return cudaMallocAsync((void **)p, count * sizeof(T), st);
 }
 
-// device head of a plan: counters, status word, time bounds
-struct PlanHead {
-    PlanCounters cnt;
-    int64_t tbounds[2];
-    int32_t status;
-    int32_t pad;
-};
-
 }  // namespace tn
 
 using namespace tn;
 
 static void free_plan_buffers(tn_plan *p, cudaStream_t st)
 {
-    if (p->d_packs) cudaFreeAsync(p->d_packs, st);
     if (p->d_mem) cudaFreeAsync(p->d_mem, st);
     if (p->d_label) cudaFreeAsync(p->d_label, st);
 }
@@ -1214,7 +1222,7 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     tn_status rc = TN_OK;
     PlanCounters host;
     memset(&host, 0, sizeof(host));
-    void *exact = nullptr;
+    const auto part = [](uint64_t bytes) { return (bytes + 255) & ~255ull; };
     bool must_wait = false;
     const bool compact = m >= kCompactEvents || !wait_end;
     const uint64_t blocks = (m + 1023) / 1024;
@@ -1228,24 +1236,18 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
 
     {
         // head, window bounds, second-pass offsets and list, source-list counts,
-        // windows and, unless they are compacted below, packs and lists: one buffer
-        const auto part = [](uint64_t bytes) { return (bytes + 255) & ~255ull; };
+        // windows, packs and lists: one buffer
         const uint64_t at_bounds = part(sizeof(PlanHead)), at_win = at_bounds + part(8 * (3ull * a.nw + 2));
         const uint64_t at_blob = at_win + part(sizeof(WinDesc) * (uint64_t)a.nw);
         const uint64_t blob_bytes = part(8 * (blob_base(m, a.nw, a.unit8) + 64)), aux_bytes = 12 * m;
         uint8_t *mem = nullptr;
-        TN_STEP(alloc_async(&mem, compact ? at_blob : at_blob + blob_bytes + aux_bytes, st));
+        TN_STEP(alloc_async(&mem, at_blob + blob_bytes + aux_bytes, st));
         p->d_mem = mem;
         p->d_head = reinterpret_cast<PlanHead *>(mem);
         a.wstart = reinterpret_cast<uint64_t *>(mem + at_bounds);
         p->d_win = reinterpret_cast<WinDesc *>(mem + at_win);
-        uint8_t *packs = mem + at_blob;
-        if (compact) {
-            TN_STEP(alloc_async(&packs, blob_bytes + aux_bytes, st));
-            p->d_packs = packs;
-        }
-        p->d_blob = reinterpret_cast<uint2 *>(packs);
-        p->d_aux = reinterpret_cast<uint32_t *>(packs + blob_bytes);
+        p->d_blob = reinterpret_cast<uint2 *>(mem + at_blob);
+        p->d_aux = reinterpret_cast<uint32_t *>(mem + at_blob + blob_bytes);
     }
     p->d_status = &p->d_head->status;
     p->d_tbounds = p->d_head->tbounds;
@@ -1338,18 +1340,25 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     }
     if (compact) {
         must_wait = true;
-        const uint64_t lists_at = p->blob8 + 2;  // in units; no list outside the packs: no list buffer
-        TN_STEP(cudaMallocAsync(&exact, 8 * lists_at + 4 * host.list_words, st));
-        uint2 *blob = static_cast<uint2 *>(exact);
-        uint32_t *aux = reinterpret_cast<uint32_t *>(blob + lists_at);
+        const uint64_t at_win = part(sizeof(PlanHead)), at_blob = at_win + part(sizeof(WinDesc) * (uint64_t)a.nw);
+        const uint64_t at_lists = at_blob + 8 * (p->blob8 + 2);
+        uint8_t *exact = nullptr;
+        TN_STEP(alloc_async(&exact, at_lists + 4 * host.list_words, st));
+        PlanHead *head = reinterpret_cast<PlanHead *>(exact);
+        WinDesc *win = reinterpret_cast<WinDesc *>(exact + at_win);
+        uint2 *blob = reinterpret_cast<uint2 *>(exact + at_blob);
+        uint32_t *aux = reinterpret_cast<uint32_t *>(exact + at_lists);
         tn_internal_count_launches(1);
-        compact_kernel<<<a.nw, 256, 0, st>>>(a, blob, aux);
-        TN_STEP(cudaGetLastError());
-        cudaFreeAsync(p->d_packs, st);
-        p->d_packs = exact;
+        compact_kernel<<<a.nw, 256, 0, st>>>(a, head, win, blob, aux);
+        cudaFreeAsync(p->d_mem, st);
+        p->d_mem = exact;
+        p->d_head = head;
+        p->d_win = win;
         p->d_blob = blob;
         p->d_aux = aux;
-        exact = nullptr;
+        p->d_status = &head->status;
+        p->d_tbounds = head->tbounds;
+        TN_STEP(cudaGetLastError());
     }
     // the plan is complete, and its events are read, when this call returns
     if (must_wait && wait_end) TN_STEP(tn_internal_stream_wait(st));
@@ -1361,7 +1370,6 @@ fail:
 done:
     if (a.late_arena) cudaFreeAsync(a.late_arena, st);
     if (rc != TN_OK) {
-        if (exact) cudaFreeAsync(exact, st);
         free_plan_buffers(p, st);
         free(p);
         return rc;
