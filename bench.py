@@ -656,9 +656,7 @@ def run_hashed(args, w, rank, world, local_rank):
     """Network hashing end to end (Section 4): hash tables and super-events, the
     R proxy schedules and the schedule of the sampled exact columns, the R
     proxy matrices and the exact sampled columns in ONE persistent launch
-    (job list: proxies at 24-word slabs, 11 CTAs each, and the 65,536 sampled
-    columns at 16-word slabs, 64 CTAs: one wave of 152 CTAs of 12 consumer
-    warps), the fused
+    (a job list over slab widths chosen so that the launch is one wave), the fused
     estimate for the sampled sources, their exact out-sizes and the error
     against them.  Beside the step: the same work in separate launches, the
     proxies replayed as a CUDA graph against one launch per proxy (identical
@@ -696,9 +694,8 @@ def run_hashed(args, w, rank, world, local_rank):
     stream = torch.cuda.current_stream(dev)
     seed = 0  # replica j hashes with splitmix64(seed ^ j): seeds 0..R-1
     ev = lambda: torch.cuda.Event(enable_timing=True)
-    # launch shapes of the combined launch, the fastest of the alternatives measured at these sizes
-    popts = dict(slab_words=24, window_events=480, smem_rows=192 * 1024 // (8 * 24))
-    xopts = dict(slab_words=16, window_events=640, smem_rows=0)
+    # no options: slab widths are chosen for the whole launch, and rows are tracked
+    popts, xopts = {}, {}
     timing = {"combined_ms": [], "estimate_ms": []}
 
     def step(record):
@@ -748,13 +745,12 @@ def run_hashed(args, w, rank, world, local_rank):
     # replay against single launches, and the error on unsaturated prefixes
     proxies_alone_ms = exact_alone_ms = graph_ms = single_ms = None
     separate_identical = identical = None
-    sopts = dict(slab_words=8, window_events=640, smem_rows=80 * 1024 // (8 * 8))
+    sopts = {}
     keys = ("mean_abs", "max_abs", "mean_rel", "max_rel", "w1")
     prefixes = []
     if world == 1:
-        # the same work in separate launches, each at its own best shape (the proxies alone:
-        # 8-word slabs in 80 KB row buffers, two 4-warp CTAs per SM; the exact columns:
-        # the defaults), and the proxies as a graph vs one launch each
+        # the same work in separate launches (each with the widths chosen for it alone),
+        # and the proxies as a graph vs one launch each
         P_ref, Sx_ref = P.clone(), Sx.clone()
         plans = [tn.Plan(pu[j].contiguous(), pv[j].contiguous(), dt, k, **sopts) for j in range(R)]
         plan_x = tn.Plan(du, dv, dt, n, **xopts)
