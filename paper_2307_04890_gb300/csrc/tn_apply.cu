@@ -65,7 +65,7 @@ struct Job {
     const uint32_t *src;
     uint32_t ncols;
     // resident-slab form (rw > 0): each CTA keeps rw words of every row in shared memory
-    uint32_t rw;     // words of every row per CTA (1, 2 or 4), 0 = column-slab form
+    uint32_t rw;     // words of every row per CTA (1 or 2), 0 = column-slab form
     uint32_t res_threads;  // consumer threads of a resident CTA
     const uint32_t *label; // component of every node, or NULL
     uint32_t identity;     // resident: S starts as the identity (and is not read)
@@ -225,19 +225,7 @@ __device__ inline bool consumers_sync_or(bool p, uint32_t count)
     return r != 0;
 }
 
-__device__ inline bool consumers_sync_or(bool p)
-{
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred ip, op;\n\t"
-        "setp.ne.u32 ip, %1, 0;\n\t"
-        "bar.red.or.pred op, 1, %2, ip;\n\t"
-        "selp.u32 %0, 1, 0, op;\n\t}"
-        : "=r"(r)
-        : "r"((uint32_t)p), "r"(consumers())
-        : "memory");
-    return r != 0;
-}
+__device__ inline bool consumers_sync_or(bool p) { return consumers_sync_or(p, consumers()); }
 
 __device__ inline void cp_async16(void *smem_dst, const void *gmem_src)
 {

@@ -273,14 +273,6 @@ constexpr int kCountWarps = 8;
 constexpr int kCountBits = 10;                            // vertical counters hold up to 1,023 rows
 constexpr uint32_t kCountMax = kCountWarps * 1016;        // nodes per CTA at most (1,016 = 127 x 8 per warp)
 
-// full adder of bit columns: (c, a, b) -> sum in c, carry returned
-__device__ inline uint32_t add_bits(uint32_t &c, uint32_t a, uint32_t b)
-{
-    const uint32_t carry = (c & a) | (b & (c | a));
-    c = c ^ a ^ b;
-    return carry;
-}
-
 // Column counts of the chunk: a warp takes every eighth node of the CTA's range,
 // lane l the WPL words at 32 WPL sources.  Eight nodes at a time are added with
 // full adders into 10-bit vertical counters (three operations a word and node,
@@ -343,13 +335,13 @@ __global__ void __launch_bounds__(32 * kCountWarps)
                     }
                 }
 #pragma unroll
-                for (int q = 0; q < WPL; ++q) two[p][q] = add_bits(c[0][q], x[0][q], x[1][q]);
+                for (int q = 0; q < WPL; ++q) two[p][q] = full_add(c[0][q], x[0][q], x[1][q]);
             }
 #pragma unroll
             for (int q = 0; q < WPL; ++q) {
-                four[0][q] = add_bits(c[1][q], two[0][q], two[1][q]);
-                four[1][q] = add_bits(c[1][q], two[2][q], two[3][q]);
-                uint32_t carry = add_bits(c[2][q], four[0][q], four[1][q]);
+                four[0][q] = full_add(c[1][q], two[0][q], two[1][q]);
+                four[1][q] = full_add(c[1][q], two[2][q], two[3][q]);
+                uint32_t carry = full_add(c[2][q], four[0][q], four[1][q]);
 #pragma unroll
                 for (int i = 3; i < kCountBits; ++i) {
                     const uint32_t next = c[i][q] & carry;
@@ -493,8 +485,8 @@ extern "C" tn_status tn_hash_estimate(const uint64_t *P, uint32_t R, uint32_t k,
 // For callers that cannot allocate device memory during a call (code inside
 // another framework's memory budget, latency-bound loops).  Same result as
 // tn_hash_estimate, but only its byte-table fusion (one CTA per 8 sources):
-// the bit-sliced path for many sources needs R * k * nsrc / 8 bytes of
-// transposed tables, more than a fixed array should hold, so every call here
+// the bit-sliced path for many sources needs R * k * 128 or 512 bytes of transposed
+// tables, more than a fixed array should hold, so every call here
 // reads H once per 8 sources (about ceil(nsrc / 8) * R * n * 4 bytes).  The
 // source-check flag and the per-CTA tables of the global-table path live in
 // one fixed device array of this module instead of the stream-ordered

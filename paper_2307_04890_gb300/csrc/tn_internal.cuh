@@ -243,6 +243,14 @@ __device__ inline u64x2 combine16(u64x2 a, u64x2 b)
     return or16(a, b);
 }
 
+// Full adder of bit columns: (c, a, b) -> sum in c, carry returned.
+__device__ inline uint32_t full_add(uint32_t &c, uint32_t a, uint32_t b)
+{
+    const uint32_t carry = (c & a) | (b & (c | a));
+    c = c ^ a ^ b;
+    return carry;
+}
+
 // ---------------------------------------------------------------------------
 // Block-wide exclusive scan of an array (generic pointer: shared or global).
 // All threads of the block must call it; returns the total.  `warp_sums` must

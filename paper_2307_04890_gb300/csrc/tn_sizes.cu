@@ -23,14 +23,6 @@ constexpr int kCounterBits = 10;               // vertical counters hold up to 1
 constexpr uint32_t kRowsMax = kSizeWarps * 1016;  // rows per CTA (127 batches of eight per warp)
 constexpr uint32_t kRowsMin = kSizeWarps * 32;  // fewer would spend more on adding the CTAs' counts than on rows
 
-// full adder of bit columns: (c, a, b) -> sum in c, carry returned
-__device__ inline uint32_t full_add(uint32_t &c, uint32_t a, uint32_t b)
-{
-    const uint32_t carry = (c & a) | (b & (c | a));
-    c = c ^ a ^ b;
-    return carry;
-}
-
 // Bound by HBM: every word of S is read once.  n = 123,457 with row sizes 335 us
 // (5.7 TB/s; 899 us with one word a lane and one row at a time into 8-bit counters),
 // n = 10^5 208 us (424), n = 10^4 with row sizes 18 us (52), n = 1,000 7 us (27).
