@@ -67,12 +67,14 @@ constexpr uint32_t kPairGroup = 48;
 // the window: the CTA's barriers would take longer than the group (2.5 us each).
 constexpr uint32_t kWarpGroup = 48;
 // Default window of tiles.  Larger windows have fewer levels per event, each of
-// which costs every CTA a barrier and a memory latency, but are scheduled by one
-// CTA each and are stretched by large timestamp groups; 2,000 ops are one pack.  n = 10^5, 10^7
-// activity-driven events: schedule and apply 1.2 + 25.9 ms at 2,480, 1.8 + 23.4 ms
-// at 5,000; bursty n = 5 10^5, groups of 2,786 events: schedule 8.3 ms at 640, 17.5
-// ms at 5,000 (windows of two groups leave shared memory); n = 1,000, 20,000
-// uniform events: 0.10 + 0.08 ms at 1,280, 0.14 + 0.08 ms at 2,480.
+// which costs every CTA a barrier and a memory latency, but are scheduled by one CTA
+// each and are stretched by large timestamp groups; 2,000 ops are one pack.  Schedule
+// and apply at 1,280, 2,000, 2,480, 5,000 events: activity-driven n = 10^5, m = 10^7, 16
+// words, 1.3 + 25.1, 1.3 + 23.2, 1.9 + 23.2, 1.8 + 20.7 ms; ER n = 10^4, m = 10^7, resident,
+// 1.2 + 0.7, 1.2 + 0.6, 1.7 + 0.6, 1.5 + 0.6; bursty n = 2 10^5, m = 5 10^6, 32 words, 1.0 +
+// 88.0, 1.0 + 91.6, 1.3 + 92.7, 2.1 + 91.0 (windows of two groups leave shared memory).  Short
+// batches gain more from a short schedule: n = 1,000, 20,000 uniform events, resident,
+// 94 + 65 us at 1,280, 114 + 62 at 2,000, 125 + 65 at 2,480.
 static uint32_t default_window(uint64_t m) { return m < (1u << 16) ? 1280u : 2000u; }
 // Room of the first pass's arena behind the target: a window is stretched by the
 // rest of its last timestamp group (2,400 events at the largest default window: two
@@ -916,8 +918,8 @@ __device__ __forceinline__ void schedule_window(const PlanArgs &a, uint32_t w, u
 // is latency: the level walk of one warp per window (about 100 cycles per 16
 // events) between phases of scattered shared-memory accesses.  Small windows
 // leave room for several CTAs per SM; 512 threads shorten the parallel phases of
-// large ones.  tn_plan_create on 10^7 activity-driven events (n = 10^5, windows
-// of 640): 0.78 ms; with one thread walking each window event by event (137 us a
+// large ones.  tn_plan_create on 10^7 activity-driven events (n = 10^5, windows of
+// 2,000): 1.27 ms; windows of 640: 1.16 ms; with one thread walking each window event by event (137 us a
 // window) and three host waits 3.4 ms.  20,000 uniform events: 0.09 ms (0.34).
 __global__ void __launch_bounds__(kPlanThreads) schedule_first_kernel(PlanArgs a)
 {
