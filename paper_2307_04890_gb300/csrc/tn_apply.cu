@@ -1168,7 +1168,11 @@ constexpr uint32_t kResidentMinStages = 2;
 // Consumer threads of a resident CTA (the rest exit): enough for a level of
 // average size, since every level's barrier waits for all of them.
 constexpr uint32_t kResidentConsumers = 256;
-constexpr uint64_t kResidentWaves = 3;  // of open plans in one launch
+// Most waves of open plans in one launch; beyond, column slabs.  Batches of networks,
+// resident and column slabs: ER n = 8,000 (5 waves) 1.09, 1.81 ms, n = 20,000 (9, 13 waves)
+// 2.84, 3.06 and 4.08, 3.17; activity-driven n = 16,384 (11 waves) 4.9, 5.4; bursty n =
+// 20,000 (5, 7, 9 waves) 5.8, 7.8 and 8.65, 8.57 and 11.1, 9.8.
+constexpr uint64_t kResidentWaves = 11, kResidentTieWaves = 7;
 
 template <int RW>
 struct alignas(RW == 1 ? 8 : 16) RRow {
@@ -2043,14 +2047,27 @@ static void open_slab_words(const tn_plan *const *plans, const uint32_t *ncols, 
     }
 }
 
+// Waves of `ctas` resident CTAs of `rows` bytes of rows: two fit an SM beside the
+// smallest ring (the launch then gives them one), at the same speed, since a level's
+// latency bounds each.
+static uint64_t resident_waves_of(uint64_t ctas, uint64_t rows)
+{
+    const uint64_t slots = (uint64_t)multiprocessors() *
+                           (kResidentHead + rows + (uint64_t)kResidentMinStages * kStageBytes <= kHalfSmSmem ? 2 : 1);
+    return (ctas + slots - 1) / slots;
+}
+
 // Form of every plan of a launch: words of a row per resident CTA, or 0 for column
 // slabs.  Plans that leave the form open take the resident one if their rows fit
-// and the batch touches enough of them to pay for loading and storing all rows,
-// while the launch's resident CTAs make at most three waves; of one and two words
-// the one with fewer waves.
+// and the batch touches enough of them to pay for loading and storing all rows (n =
+// 20,000: 2,500 events of distinct nodes 0.15 ms, in tiles 0.05; 5,000 events 0.155,
+// 0.125), while the launch's resident CTAs make at most kResidentWaves waves, or
+// kResidentTieWaves of plans with large groups that share nodes; of one and two words
+// the one with fewer waves (one word where both have as many: 3 networks of n = 8,000,
+// two waves each, 0.68 and 0.91 ms).
 static void choose_forms(const tn_plan *const *plans, const uint32_t *ncols, uint32_t count, uint32_t *rw)
 {
-    uint64_t ctas[3] = {0, 0, 0};
+    uint64_t ctas[3] = {0, 0, 0}, rows[3] = {0, 0, 0};
     bool two = true;
     auto fits = [&](const tn_plan *p, uint32_t w) {
         return p->auto_form && 4 * p->ops >= p->n && resident_fits(p->n, p->temps, w);
@@ -2059,15 +2076,20 @@ static void choose_forms(const tn_plan *const *plans, const uint32_t *ncols, uin
         rw[i] = plans[i]->resident;
         if (rw[i] || !fits(plans[i], 1)) continue;
         two = two && fits(plans[i], 2);
-        for (uint32_t w = 1; w <= 2; ++w) ctas[w] += ((ncols[i] + 63ull) / 64 + w - 1) / w;
+        for (uint32_t w = 1; w <= 2; ++w) {
+            ctas[w] += ((ncols[i] + 63ull) / 64 + w - 1) / w;
+            const uint64_t bytes = resident_rows_bytes(plans[i]->n, plans[i]->temps, w);
+            if (bytes > rows[w]) rows[w] = bytes;
+        }
     }
     if (!ctas[1]) return;
-    const uint64_t sms = (uint64_t)multiprocessors();
     uint32_t w = 1;
-    if (two && (ctas[2] + sms - 1) / sms < (ctas[1] + sms - 1) / sms) w = 2;
-    if (ctas[w] > kResidentWaves * sms) return;
-    for (uint32_t i = 0; i < count; ++i)
-        if (!rw[i] && fits(plans[i], 1)) rw[i] = w;
+    if (two && resident_waves_of(ctas[2], rows[2]) < resident_waves_of(ctas[1], rows[1])) w = 2;
+    const uint64_t waves = resident_waves_of(ctas[w], rows[w]);
+    for (uint32_t i = 0; i < count; ++i) {
+        const uint64_t most = 16 * plans[i]->aux > plans[i]->ops ? kResidentTieWaves : kResidentWaves;
+        if (!rw[i] && fits(plans[i], 1) && waves <= most) rw[i] = w;
+    }
 }
 
 uint32_t resident_form(const tn_plan *p, uint32_t ncols)
@@ -2077,10 +2099,9 @@ uint32_t resident_form(const tn_plan *p, uint32_t ncols)
     return rw;
 }
 
-uint64_t resident_waves(uint32_t ncols, uint32_t words)
+uint64_t resident_waves(const tn_plan *p, uint32_t ncols, uint32_t words)
 {
-    const uint64_t ctas = ((ncols + 63ull) / 64 + words - 1) / words, sms = (uint64_t)multiprocessors();
-    return (ctas + sms - 1) / sms;
+    return resident_waves_of(((ncols + 63ull) / 64 + words - 1) / words, resident_rows_bytes(p->n, p->temps, words));
 }
 
 // Whether content ids of `bytes` may be allocated on `st`.  A call learns from the

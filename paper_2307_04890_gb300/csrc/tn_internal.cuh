@@ -340,7 +340,7 @@ uint32_t resident_max_rows(uint32_t words);
 // Words of a row per resident CTA that an open plan takes when it alone is applied to
 // `ncols` columns; 0: column slabs.
 uint32_t resident_form(const tn_plan *p, uint32_t ncols);
-uint64_t resident_waves(uint32_t ncols, uint32_t words);
+uint64_t resident_waves(const tn_plan *p, uint32_t ncols, uint32_t words);
 // Whether the rows of a slab of `words` words can be tracked beside a row buffer of
 // `bytes`: row groups that are whole parts of a warp, and copy rings that fit.
 bool tracked_slab(uint32_t words, uint64_t bytes);

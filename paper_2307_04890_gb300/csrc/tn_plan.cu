@@ -1129,7 +1129,7 @@ static bool records_faster(const tn_plan *p, uint64_t chain, uint32_t ncols)
     if (p->levels < kRecordLevels) return false;
     const uint32_t rw = p->auto_form ? resident_form(p, ncols) : 0u;
     if (rw) {
-        const double L = (double)p->levels, ops = (double)p->ops, waves = (double)resident_waves(ncols, rw);
+        const double L = (double)p->levels, ops = (double)p->ops, waves = (double)resident_waves(p, ncols, rw);
         const double level = rw == 1 ? (p->aux ? 170.0 : 100.0) : (p->aux ? 200.0 : 120.0);
         const double per_event = (double)p->n / (double)p->m;
         const double walked = 11.0 * per_event < 1.0 ? 11.0 * per_event : 1.0, listed = 24.0 * per_event < 1.0 ? 24.0 * per_event : 1.0;
