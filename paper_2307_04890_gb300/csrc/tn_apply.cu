@@ -1171,7 +1171,9 @@ constexpr uint32_t kResidentConsumers = 256;
 // Most waves of open plans in one launch; beyond, column slabs.  Batches of networks,
 // resident and column slabs: ER n = 8,000 (5 waves) 1.09, 1.81 ms, n = 20,000 (9, 13 waves)
 // 2.84, 3.06 and 4.08, 3.17; activity-driven n = 16,384 (11 waves) 4.9, 5.4; bursty n =
-// 20,000 (5, 7, 9 waves) 5.8, 7.8 and 8.65, 8.57 and 11.1, 9.8.
+// 20,000 (5, 7, 9 waves) 5.8, 7.8 and 8.65, 8.57 and 11.1, 9.8.  With records kept for
+// that launch: bursty n = 8,000 (3, 5 waves) 3.0, 3.0 and 4.6, 3.1; activity-driven n =
+// 8,000 (7 waves) 2.4, 2.3.
 constexpr uint64_t kResidentWaves = 11, kResidentTieWaves = 7;
 
 template <int RW>
@@ -2087,7 +2089,8 @@ static void choose_forms(const tn_plan *const *plans, const uint32_t *ncols, uin
     if (two && resident_waves_of(ctas[2], rows[2]) < resident_waves_of(ctas[1], rows[1])) w = 2;
     const uint64_t waves = resident_waves_of(ctas[w], rows[w]);
     for (uint32_t i = 0; i < count; ++i) {
-        const uint64_t most = 16 * plans[i]->aux > plans[i]->ops ? kResidentTieWaves : kResidentWaves;
+        const bool ties = 16 * plans[i]->aux > plans[i]->ops;
+        const uint64_t most = plans[i]->batch_plan ? (ties ? 3 : 7) : ties ? kResidentTieWaves : kResidentWaves;
         if (!rw[i] && fits(plans[i], 1) && waves <= most) rw[i] = w;
     }
 }
@@ -2152,11 +2155,16 @@ tn_status apply_jobs(const tn_plan *const *plans, uint64_t *const *S, const uint
         size_t smem = smem_base;
         uint32_t rws[kMaxPlans];
         choose_forms(plans + base, ncols + base, nj, rws);
+        const tn_plan *used[kMaxPlans];  // the schedule applied
+        for (uint32_t j = 0; j < nj; ++j) {
+            const tn_plan *p = plans[base + j];
+            used[j] = !rws[j] && p->batch_plan ? p->batch_plan : p;
+        }
         uint32_t sws[kMaxPlans];
-        open_slab_words(plans + base, ncols + base, rws, nj, sws);
+        open_slab_words(used, ncols + base, rws, nj, sws);
         for (uint32_t j = 0; j < nj; ++j) {
             const uint32_t i = base + j;
-            const tn_plan *p = plans[i];
+            const tn_plan *p = used[j];
             const uint64_t ld = tn_row_words(ncols[i]);
             tmps[j] = nullptr;
             idbuf[j] = nullptr;

@@ -316,6 +316,7 @@ struct tn_plan {
     uint32_t slab_words;  // 64-bit words of every row owned by one CTA (the widest, with wave_ctas)
     uint32_t auto_slab;   // slab_words was left open: chosen when the plan is applied, if it has no records
     uint32_t auto_form;   // the form (resident or column slabs) was left open: chosen when the plan is applied
+    tn_plan *batch_plan;  // owned: the schedule as records, for launches where this plan is in column slabs (or NULL)
     uint32_t wave_ctas;   // 0, or the number of CTAs one matrix is spread over
     uint32_t dcap;        // row slots of the kernel's shared-memory row buffer
     uint32_t buffer_bytes;  // largest row buffer of a width chosen when the plan is applied (smem_rows was given: its bytes)

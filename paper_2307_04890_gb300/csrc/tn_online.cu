@@ -310,7 +310,7 @@ tn_status apply_ready(tn_online *o, const uint32_t *u, const uint32_t *v, const 
     // two-stream mode: the update waits for the plan's last kernels through an
     // event on the apply stream instead of a host wait
     tn_status rc = o->ast ? tn::plan_create_ordered(u, v, t, count, o->n, &o->opt, st, &plan)
-                          : tn_plan_create(u, v, t, count, o->n, nullptr, &o->opt, st, &plan);
+                          : tn::plan_create_for(u, v, t, count, o->n, nullptr, &o->opt, o->n, st, &plan);
     if (rc != TN_OK) return rc;
     if (o->ast) {
         rc = tn::plan_use_status(plan, o->dstatus, st);

@@ -35,6 +35,21 @@ def applied(events, n, directed=False, **options):
     return plan
 
 
+def stream_launch(run, tmp_path):
+    """The launch (grid, block) of the one streaming kernel that `run` launches."""
+    for _ in range(2):  # (a process's first session may start too late for its kernels)
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+            run()
+            torch.cuda.synchronize()
+    prof.export_chrome_trace(str(tmp_path / "trace.json"))
+    trace = json.loads((tmp_path / "trace.json").read_text())["traceEvents"]
+    launches = [e["args"] for e in trace if "stream_kernel" in e.get("name", "") and "block" in e.get("args", {})]
+    if not launches:
+        pytest.skip("no kernel records from the profiler")
+    assert len(launches) == 1
+    return launches[0]
+
+
 @pytest.mark.parametrize("rows,threads", [(640, 160), (0, 416)])
 def test_row_buffer_of_an_open_width(rows, threads, tmp_path):
     """An 80 KB row buffer gives two CTAs of 4 consumer warps per SM also where the slab
@@ -45,16 +60,7 @@ def test_row_buffer_of_an_open_width(rows, threads, tmp_path):
     plan = applied((u, v, np.arange(m) // 1000), n, slab_words=0, **options)
     assert plan.stats()["local_windows"] == 0
     S = torch.empty((n, tn.tn_row_words(n)), dtype=torch.int64, device="cuda")
-    for _ in range(2):  # (a process's first session may start too late for its kernels)
-        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
-            plan.apply(S, init=True)
-            torch.cuda.synchronize()
-    prof.export_chrome_trace(str(tmp_path / "trace.json"))
-    trace = json.loads((tmp_path / "trace.json").read_text())["traceEvents"]
-    blocks = [e["args"]["block"][0] for e in trace if "stream_kernel" in e.get("name", "") and "block" in e.get("args", {})]
-    if not blocks:
-        pytest.skip("no kernel records from the profiler")
-    assert blocks == [threads]
+    assert stream_launch(lambda: plan.apply(S, init=True), tmp_path)["block"][0] == threads
 
 
 @pytest.mark.parametrize("directed", [False, True])
@@ -123,3 +129,35 @@ def test_autotune_times_a_plan_without_options(n, m, replicas, ncols):
     assert 0 < first["open_ms"] < float("inf") and 0 < first["best_ms"] < float("inf")
     again = tn.tn_autotune(*events, n, replicas=replicas, ncols=ncols)
     assert again["cached"] and again["open_ms"] == first["open_ms"]
+
+
+@pytest.mark.parametrize("directed", [False, True])
+def test_batches_of_small_networks(directed, tmp_path):
+    """Ten networks of short levels: resident CTAs would make five waves, so the launch
+    takes their record schedules (8 CTAs each).  One network alone is resident."""
+    n, copies = 8000, 5
+    streams = [synth.powerlaw_bursty(n, 170_000, seed=k) for k in range(2)]
+    plans = [tn.Plan(*dev(*s), n, directed=directed) for s in streams]
+    assert all(p.stats()["levels"] >= 4096 and p.stats()["local_windows"] == 0 for p in plans)
+    refs = [(oracle.component_matrix_directed if directed else oracle.component_matrix)(*s, n) for s in streams]
+    mats = [torch.empty((n, tn.tn_row_words(n)), dtype=torch.int64, device="cuda") for _ in range(2 * copies)]
+
+    def check():
+        for k, S in enumerate(mats):
+            got = S.cpu().numpy().view(np.uint64)
+            assert np.array_equal(got[:, : refs[k % 2].shape[1]], refs[k % 2])
+            S.fill_(-1)
+
+    tn.tn_plan_apply_batch(plans * copies, mats)
+    check()
+    graph = tn.BatchGraph(plans * copies, mats)
+    for _ in range(2):
+        graph.launch()
+        check()
+    graph.destroy()
+    assert all(p.status() == 0 for p in plans)
+    for k in range(2):
+        plans[k].apply(mats[k], init=True)
+        assert np.array_equal(mats[k].cpu().numpy().view(np.uint64)[:, : refs[k].shape[1]], refs[k])
+    assert stream_launch(lambda: plans[0].apply(mats[0], init=True), tmp_path)["grid"][0] == 125
+    assert stream_launch(lambda: tn.tn_plan_apply_batch(plans * copies, mats), tmp_path)["grid"][0] == 2 * copies * 8
