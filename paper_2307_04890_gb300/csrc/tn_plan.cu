@@ -1152,9 +1152,10 @@ static bool records_faster(const tn_plan *p, uint64_t chain, uint32_t ncols)
 
 // Resident plans that may be launched with others keep a record schedule beside their
 // own, for launches of so many networks that column slabs are due: from this many
-// levels on, where it costs 5 % of applying the plan once (n = 20,000, m = 300,000, bursty:
-// 0.2 of 4.2 ms) and six such networks in one launch take 4.9 ms instead of 10.1 as tiles.
-constexpr uint64_t kBatchLevels = 4096;
+// levels (times the waves of CTAs that walk them) on, where it costs 5 to 7 % of applying
+// the plan once (n = 20,000, m = 300,000, bursty: 0.2 of 4.2 ms) and six such networks in
+// one launch take 4.9 ms instead of 10.1 as tiles.
+constexpr uint64_t kBatchLevels = 8192;
 
 // wait_end: return only once the plan's device buffers are written (else they
 // may be written by work enqueued on `stream`, which later users must follow).
@@ -1377,13 +1378,16 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
         p->d_tbounds = head->tbounds;
         TN_STEP(cudaGetLastError());
     }
-    if (p->auto_form && !ncols && p->levels >= kBatchLevels && records_over_tiles(p) && resident_form(p, n)) {
-        // (without memory for it, the plan does without)
-        if (plan_create_impl(u, v, t, m, n, nullptr, opt, stream, &p->batch_plan, false, n, true) == TN_OK)
-            p->batch_plan->d_status = p->d_status;
-        else
-            cudaGetLastError();
-        must_wait = true;
+    if (p->auto_form && !ncols && records_over_tiles(p)) {
+        const uint32_t alone = resident_form(p, n);
+        if (alone && p->levels * resident_waves(p, n, alone) >= kBatchLevels) {
+            // (without memory for it, the plan does without)
+            if (plan_create_impl(u, v, t, m, n, nullptr, opt, stream, &p->batch_plan, false, n, true) == TN_OK)
+                p->batch_plan->d_status = p->d_status;
+            else
+                cudaGetLastError();
+            must_wait = true;
+        }
     }
     // the plan is complete, and its events are read, when this call returns
     if (must_wait && wait_end) TN_STEP(tn_internal_stream_wait(st));
