@@ -1216,7 +1216,7 @@ def main():
     # launch's DRAM bytes (ncu) are, or, without them, what no launch on these
     # sources can do without: the schedule in once and the matrix out once.
     update_bytes = m * 4 * words * 8
-    traffic = profiled_traffic(args.workload, sw) if world == 1 and sw else None
+    traffic = profiled_traffic(args.workload, sw or None) if world == 1 and not rw else None
     alg_bytes = 8 * stats["ops"] + n * W * 8
     achieved = (traffic or alg_bytes) / (k1_ms * 1e-3) / 1e9
     roofline = {"bound": "hbm", "kernel": "stream_kernel" + (" (resident slabs)" if rw else ""),

@@ -2049,13 +2049,13 @@ static void open_slab_words(const tn_plan *const *plans, const uint32_t *ncols, 
     }
 }
 
-// Waves of `ctas` resident CTAs of `rows` bytes of rows: two fit an SM beside the
-// smallest ring (the launch then gives them one), at the same speed, since a level's
-// latency bounds each.
-static uint64_t resident_waves_of(uint64_t ctas, uint64_t rows)
+// Waves of `ctas` resident CTAs of `rows` bytes of rows.  In a launch of such CTAs alone
+// two share an SM if they fit beside the smallest ring (the launch then gives them one),
+// at the same speed, since a level's latency bounds each.
+static uint64_t resident_waves_of(uint64_t ctas, uint64_t rows, bool alone)
 {
-    const uint64_t slots = (uint64_t)multiprocessors() *
-                           (kResidentHead + rows + (uint64_t)kResidentMinStages * kStageBytes <= kHalfSmSmem ? 2 : 1);
+    const bool pair = alone && kResidentHead + rows + (uint64_t)kResidentMinStages * kStageBytes <= kHalfSmSmem;
+    const uint64_t slots = (uint64_t)multiprocessors() * (pair ? 2 : 1);
     return (ctas + slots - 1) / slots;
 }
 
@@ -2070,13 +2070,17 @@ static uint64_t resident_waves_of(uint64_t ctas, uint64_t rows)
 static void choose_forms(const tn_plan *const *plans, const uint32_t *ncols, uint32_t count, uint32_t *rw)
 {
     uint64_t ctas[3] = {0, 0, 0}, rows[3] = {0, 0, 0};
-    bool two = true;
+    bool two = true, alone = true;
     auto fits = [&](const tn_plan *p, uint32_t w) {
         return p->auto_form && 4 * p->ops >= p->n && resident_fits(p->n, p->temps, w);
     };
     for (uint32_t i = 0; i < count; ++i) {
         rw[i] = plans[i]->resident;
-        if (rw[i] || !fits(plans[i], 1)) continue;
+        if (rw[i]) continue;
+        if (!fits(plans[i], 1)) {
+            alone = false;
+            continue;
+        }
         two = two && fits(plans[i], 2);
         for (uint32_t w = 1; w <= 2; ++w) {
             ctas[w] += ((ncols[i] + 63ull) / 64 + w - 1) / w;
@@ -2086,8 +2090,8 @@ static void choose_forms(const tn_plan *const *plans, const uint32_t *ncols, uin
     }
     if (!ctas[1]) return;
     uint32_t w = 1;
-    if (two && resident_waves_of(ctas[2], rows[2]) < resident_waves_of(ctas[1], rows[1])) w = 2;
-    const uint64_t waves = resident_waves_of(ctas[w], rows[w]);
+    if (two && resident_waves_of(ctas[2], rows[2], alone) < resident_waves_of(ctas[1], rows[1], alone)) w = 2;
+    const uint64_t waves = resident_waves_of(ctas[w], rows[w], alone);
     for (uint32_t i = 0; i < count; ++i) {
         const bool ties = 16 * plans[i]->aux > plans[i]->ops;
         const uint64_t most = plans[i]->batch_plan ? (ties ? 3 : 7) : ties ? kResidentTieWaves : kResidentWaves;
@@ -2104,7 +2108,7 @@ uint32_t resident_form(const tn_plan *p, uint32_t ncols)
 
 uint64_t resident_waves(const tn_plan *p, uint32_t ncols, uint32_t words)
 {
-    return resident_waves_of(((ncols + 63ull) / 64 + words - 1) / words, resident_rows_bytes(p->n, p->temps, words));
+    return resident_waves_of(((ncols + 63ull) / 64 + words - 1) / words, resident_rows_bytes(p->n, p->temps, words), true);
 }
 
 // Whether content ids of `bytes` may be allocated on `st`.  A call learns from the
