@@ -2065,8 +2065,9 @@ static uint64_t resident_waves_of(uint64_t ctas, uint64_t rows, bool alone)
 // 20,000: 2,500 events of distinct nodes 0.15 ms, in tiles 0.05; 5,000 events 0.155,
 // 0.125), while the launch's resident CTAs make at most kResidentWaves waves, or
 // kResidentTieWaves of plans with large groups that share nodes; of one and two words
-// the one with fewer waves (one word where both have as many: 3 networks of n = 8,000,
-// two waves each, 0.68 and 0.91 ms).
+// the one with fewer waves, and where both have as many, one word (3 activity-driven
+// networks of n = 8,000, two waves each, 0.68 and 0.91 ms), but two where that needs no
+// second CTA on an SM (five ER networks of 1,500 nodes and one of 5,000 0.197 and 0.189).
 static void choose_forms(const tn_plan *const *plans, const uint32_t *ncols, uint32_t count, uint32_t *rw)
 {
     uint64_t ctas[3] = {0, 0, 0}, rows[3] = {0, 0, 0};
@@ -2089,9 +2090,9 @@ static void choose_forms(const tn_plan *const *plans, const uint32_t *ncols, uin
         }
     }
     if (!ctas[1]) return;
-    uint32_t w = 1;
-    if (two && resident_waves_of(ctas[2], rows[2], alone) < resident_waves_of(ctas[1], rows[1], alone)) w = 2;
-    const uint64_t waves = resident_waves_of(ctas[w], rows[w], alone);
+    const uint64_t one = resident_waves_of(ctas[1], rows[1], alone), other = resident_waves_of(ctas[2], rows[2], alone);
+    const uint32_t w = two && (other < one || (other == 1 && ctas[1] > (uint64_t)multiprocessors())) ? 2 : 1;
+    const uint64_t waves = w == 2 ? other : one;
     for (uint32_t i = 0; i < count; ++i) {
         const bool ties = 16 * plans[i]->aux > plans[i]->ops;
         const uint64_t most = plans[i]->batch_plan ? (ties ? 3 : 7) : ties ? kResidentTieWaves : kResidentWaves;
