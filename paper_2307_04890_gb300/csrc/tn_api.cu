@@ -186,7 +186,7 @@ extern "C" tn_status tn_out_component_sizes_host(const uint32_t *u, const uint32
         rc = tn_init_matrix(S, n, n, nullptr, stream);
     } else {
         tn_plan *plan = nullptr;
-        rc = tn::plan_create_for(du, dv, dt, m, n, nullptr, opt, n, stream, &plan);
+        rc = tn::plan_create_for(du, dv, dt, m, n, nullptr, opt, tn::PlanUse{n, false}, stream, &plan);
         if (rc == TN_OK) {
             rc = tn_plan_apply(plan, S, n, nullptr, nullptr, TN_INIT_IDENTITY, stream);
             tn_plan_destroy(plan, stream);

@@ -1960,7 +1960,7 @@ static uint32_t stream_smem_limit()
     return cached[dev];
 }
 
-static int multiprocessors()
+int multiprocessors()
 {
     static std::mutex mu;
     static int cached[64] = {0};
@@ -2493,7 +2493,7 @@ static tn_status one_shot(const uint32_t *u, const uint32_t *v, const int64_t *t
     memset(&opt, 0, sizeof(opt));
     opt.directed = (flags & TN_DIRECTED) ? 1u : 0u;
     tn_plan *plan = nullptr;
-    tn_status rc = plan_create_for(u, v, t, m, n, t_last, &opt, ncols, stream, &plan);
+    tn_status rc = plan_create_for(u, v, t, m, n, t_last, &opt, PlanUse{ncols, false}, stream, &plan);
     if (rc != TN_OK) return rc;
     flags &= ~TN_DIRECTED;
     rc = apply_jobs((const tn_plan *const *)&plan, &S, &ncols, &src, &t_last, 1, flags, st);

@@ -421,7 +421,7 @@ static tn_status estimate_bitsliced(const uint64_t *P, uint32_t R, uint32_t k, u
     const void *count = chunk == 4096 ? (const void *)bitslice_count_kernel<4> : (const void *)bitslice_count_kernel<1>;
     TN_CUDA_TRY(tn_internal_allow_max_dyn_smem(count));
     // nodes per CTA: a multiple of the 256-node batch, about four CTAs per SM
-    uint32_t per_cta = (uint32_t)(((uint64_t)n / (152 * 4) + 255) / 256 * 256);
+    uint32_t per_cta = (uint32_t)(((uint64_t)n / (4 * (uint64_t)multiprocessors()) + 255) / 256 * 256);
     if (per_cta < 256) per_cta = 256;
     if (per_cta > kCountMax / 256 * 256) per_cta = kCountMax / 256 * 256;
     const unsigned blocks = (n + per_cta - 1) / per_cta;

@@ -147,7 +147,7 @@ extern "C" tn_status tn_hll_sketches(const uint32_t *u, const uint32_t *v, const
     memset(&opt, 0, sizeof(opt));
     opt.directed = (flags & TN_DIRECTED) ? 1u : 0u;
     tn_plan *plan = nullptr;
-    tn_status rc = plan_create_for(eu, ev, et, m, n, nullptr, &opt, 8u << p, stream, &plan);
+    tn_status rc = plan_create_for(eu, ev, et, m, n, nullptr, &opt, PlanUse{8u << p, true}, stream, &plan);
     if (rc == TN_OK) {
         uint64_t *S = reinterpret_cast<uint64_t *>(R);
         const uint32_t ncols = 8u << p;

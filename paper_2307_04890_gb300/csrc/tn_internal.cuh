@@ -332,6 +332,8 @@ struct tn_plan {
 };
 
 namespace tn {
+// SMs of the current device (cached per device).
+int multiprocessors();
 // Resident-slab form (tn_plan_options.resident_words): whether a network of
 // `rows` rows and `temps` saved-row slots fits one CTA's shared memory at
 // `words` 64-bit words per row, beside the smallest schedule ring; and the
@@ -365,9 +367,14 @@ tn_status online_use_apply_stream(tn_online *online, cudaStream_t apply_stream);
 // Two-stream mode: the device status word every batch's plan records errors
 // in (0 = none), for a caller that copies it out behind the updates.
 const int32_t *online_status_word(const tn_online *online);
-// tn_plan_create for a plan that will be applied to `ncols` columns.
+// tn_plan_create for a plan whose use is known: applied alone, to `ncols` columns (0: not
+// known), with the byte-wise maximum (kApplyMax).
+struct PlanUse {
+    uint32_t ncols;
+    bool max;
+};
 tn_status plan_create_for(const uint32_t *u, const uint32_t *v, const int64_t *t, uint64_t m, uint32_t n,
-                          const int64_t *t_after, const tn_plan_options *opt, uint32_t ncols, void *stream,
+                          const int64_t *t_after, const tn_plan_options *opt, const PlanUse &use, void *stream,
                           tn_plan **plan_out);
 // tn_plan_create without its last host wait: the plan's device buffers are
 // written by work enqueued on `stream`, so a use on another stream must first

@@ -61,7 +61,7 @@ __global__ void grow_kernel(const uint64_t *S_old, uint64_t W_old, uint32_t n_ol
 int grow_blocks(uint64_t pairs)
 {
     const uint64_t b = (pairs + 255) / 256;
-    const uint64_t cap = 152ull * 8;  // grid-stride over 8 CTAs of 256 threads per SM
+    const uint64_t cap = (uint64_t)tn::multiprocessors() * 8;  // grid-stride over 8 CTAs of 256 threads per SM
     return (int)(b < 1 ? 1 : b < cap ? b : cap);
 }
 
@@ -310,7 +310,7 @@ tn_status apply_ready(tn_online *o, const uint32_t *u, const uint32_t *v, const 
     // two-stream mode: the update waits for the plan's last kernels through an
     // event on the apply stream instead of a host wait
     tn_status rc = o->ast ? tn::plan_create_ordered(u, v, t, count, o->n, &o->opt, st, &plan)
-                          : tn::plan_create_for(u, v, t, count, o->n, nullptr, &o->opt, o->n, st, &plan);
+                          : tn::plan_create_for(u, v, t, count, o->n, nullptr, &o->opt, tn::PlanUse{o->n, false}, st, &plan);
     if (rc != TN_OK) return rc;
     if (o->ast) {
         rc = tn::plan_use_status(plan, o->dstatus, st);

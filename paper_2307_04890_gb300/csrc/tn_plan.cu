@@ -1111,7 +1111,9 @@ static void free_plan_buffers(tn_plan *p, cudaStream_t st)
 //  - without ties.  Streams around 96 hubs (60 ops a level), n = 6 10^4: 6 events a node
 //    7.6 and 4.5 ms, 24 events a node 28.2 and 17.4, 50 events a node (every row settles)
 //    28.8 and 35.3; 256 hubs (119), n = 2 10^5: 11.7 and 7.2; activity-driven, n =
-//    2.6 10^4 (122): 2.1 and 2.1, n = 6 10^4 (202): 9.4 and 11.3.
+//    2.6 10^4 (122): 2.1 and 2.1, n = 6 10^4 (202): 9.4 and 11.3.  In narrow slabs (few
+//    columns) records gain, 5,000 columns, 2 words: activity-driven n = 2.6 10^4 (128) 2.1
+//    and 1.4, n = 6 10^4 (218) 3.5 and 2.9, n = 10^5 (293) 2.7 and 2.8.
 //  - large timestamp groups that share nodes.  Bursty n = 2.6 10^4, m = 10^6 (81): 21.0
 //    and 15.5 ms; n = 10^5, m = 5 10^6 (306): 90.1 and 62.2; n = 1.2 10^5, m = 10^6
 //    (424): 14.5 and 14.6; n = 2 10^5, m = 5 10^6 (645): 92 and 137.
@@ -1125,29 +1127,32 @@ static void free_plan_buffers(tn_plan *p, cudaStream_t st)
 //   45.5 (40.5), 15.4 (16.5), 4.3 (4.3); no groups 59.9 (60.3), 54.3 (55.6); 30 events a
 //   node in groups of 4: 97.8 (114), records 108 (107); n = 12,000, groups of 8, 64: 16.1
 //   (17.2), 7.3 (8.5), records 15.3 (16.5), 4.3 (4.3).  Bursty n = 20,011, m = 500,009:
-//   6.1, records 7.1 (6.3).  The margin covers the error.
+//   6.1, records 7.1 (6.3).  The margin covers the error.  Sketches (byte-wise maximum)
+//   pay 42 ns a source, and 39 in records: one hub, groups of 64, n = 20,000, m = 300,000,
+//   p = 10 14.9, records 16.5; p = 12 (four waves) 28.5 and 17.6.
 // From kRecordLevels levels on: below, the second schedule takes as long as it saves.
 constexpr uint64_t kRecordLevels = 256;
-static bool records_over_tiles(const tn_plan *p)
+static bool records_over_tiles(const tn_plan *p, uint32_t slab)
 {
     if (16 * p->aux > p->ops) return p->ops < 400 * p->levels && p->m < 64ull * p->n;
-    const uint64_t limit = 72 + p->n / 1024;
+    const uint64_t limit = slab < kDefaultSlab ? 256 : 72 + p->n / 1024;
     return p->ops < (limit < 256 ? limit : 256) * p->levels && p->m < 32ull * p->n;
 }
 
-static bool records_faster(const tn_plan *p, uint64_t chain, uint32_t ncols)
+static bool records_faster(const tn_plan *p, uint64_t chain, const PlanUse &use, uint32_t slab)
 {
     if (p->levels < kRecordLevels) return false;
-    const uint32_t rw = p->auto_form ? resident_form(p, ncols) : 0u;
+    const uint32_t ncols = use.ncols ? use.ncols : p->n, rw = p->auto_form ? resident_form(p, ncols) : 0u;
     if (rw) {
         const double L = (double)p->levels, ops = (double)p->ops, waves = (double)resident_waves(p, ncols, rw);
         const double level = rw == 1 ? (p->aux ? 170.0 : 100.0) : (p->aux ? 200.0 : 120.0);
+        const double source = (use.max ? 42.0 : 27.0) * (rw == 1 ? 1.0 : 1.33);
         const double per_event = (double)p->n / (double)p->m;
         const double walked = 11.0 * per_event < 1.0 ? 11.0 * per_event : 1.0, listed = 24.0 * per_event < 1.0 ? 24.0 * per_event : 1.0;
-        const double resident = waves * (walked * (level * L + 0.5 * ops) + listed * (rw == 1 ? 27.0 : 36.0) * (double)chain);
-        return resident > 1.25 * (270.0 * L + 7.8 * ops + 5.0 * (double)chain);
+        const double resident = waves * (walked * (level * L + 0.5 * ops) + listed * source * (double)chain);
+        return resident > 1.25 * (270.0 * L + (3.5 + 0.27 * slab) * ops + (use.max ? 39.0 : 5.0) * (double)chain);
     }
-    return records_over_tiles(p);
+    return records_over_tiles(p, slab);
 }
 
 // Resident plans that may be launched with others keep a record schedule beside their
@@ -1159,11 +1164,10 @@ constexpr uint64_t kBatchLevels = 8192;
 
 // wait_end: return only once the plan's device buffers are written (else they
 // may be written by work enqueued on `stream`, which later users must follow).
-// ncols: columns that the plan is made for, alone (0: not known).  as_records: a plan of
-// open options whose windows are to be records.
+// as_records: a plan of open options whose windows are to be records.
 static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const int64_t *t, uint64_t m, uint32_t n,
                                   const int64_t *t_after, const tn_plan_options *opt, void *stream,
-                                  tn_plan **plan_out, bool wait_end, uint32_t ncols, bool as_records = false)
+                                  tn_plan **plan_out, bool wait_end, const PlanUse &use, bool as_records = false)
 {
     if (!plan_out) return TN_EINVAL;
     *plan_out = nullptr;
@@ -1180,6 +1184,11 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
         resident = opt->resident_words;
     }
     if (sw < 2 || sw > kMaxSlabWords || (sw & 1u)) return TN_EINVAL;  // even: whole 16-byte chunks
+    // records of a column subset or of sketches: as many CTAs as one wave holds
+    uint32_t record_slab = sw;
+    if (use.ncols && use.ncols != n && !wave && (!opt || !opt->slab_words))
+        while (record_slab > 2 && (use.ncols + 63ull) / 64 <= (uint64_t)multiprocessors() * (record_slab / 2)) record_slab /= 2;
+    if (as_records) sw = record_slab;
     // everything but the window left open: no records, and the form is chosen when
     // the plan is applied.  Networks of the same size whose slab width is given keep
     // record windows unless the batch is long enough for rows to settle: their levels
@@ -1336,11 +1345,11 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     p->ops = host.ops;
     p->local_windows = host.local;
     p->big_windows = host.big;
-    if (auto_window && window != kRecordWindow && sw <= 16 && records_faster(p, host.chain, ncols ? ncols : n)) {
+    if (auto_window && window != kRecordWindow && sw <= 16 && records_faster(p, host.chain, use, record_slab)) {
         free_plan_buffers(p, st);
         if (a.late_arena) cudaFreeAsync(a.late_arena, st);
         free(p);
-        return plan_create_impl(u, v, t, m, n, t_after, opt, stream, plan_out, wait_end, ncols, true);
+        return plan_create_impl(u, v, t, m, n, t_after, opt, stream, plan_out, wait_end, use, true);
     }
     if (resident && !resident_fits(n, p->temps, resident)) {  // saved rows of the tie groups do not fit
         rc = TN_EINVAL;
@@ -1378,11 +1387,11 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
         p->d_tbounds = head->tbounds;
         TN_STEP(cudaGetLastError());
     }
-    if (p->auto_form && !ncols && records_over_tiles(p)) {
+    if (p->auto_form && !use.ncols && records_over_tiles(p, kDefaultSlab)) {
         const uint32_t alone = resident_form(p, n);
         if (alone && p->levels * resident_waves(p, n, alone) >= kBatchLevels) {
             // (without memory for it, the plan does without)
-            if (plan_create_impl(u, v, t, m, n, nullptr, opt, stream, &p->batch_plan, false, n, true) == TN_OK)
+            if (plan_create_impl(u, v, t, m, n, nullptr, opt, stream, &p->batch_plan, false, PlanUse{n, false}, true) == TN_OK)
                 p->batch_plan->d_status = p->d_status;
             else
                 cudaGetLastError();
@@ -1412,20 +1421,20 @@ extern "C" tn_status tn_plan_create(const uint32_t *u, const uint32_t *v, const 
                                     uint32_t n, const int64_t *t_after, const tn_plan_options *opt,
                                     void *stream, tn_plan **plan_out)
 {
-    return plan_create_impl(u, v, t, m, n, t_after, opt, stream, plan_out, true, 0);
+    return plan_create_impl(u, v, t, m, n, t_after, opt, stream, plan_out, true, PlanUse{0, false});
 }
 
 tn_status tn::plan_create_for(const uint32_t *u, const uint32_t *v, const int64_t *t, uint64_t m, uint32_t n,
-                              const int64_t *t_after, const tn_plan_options *opt, uint32_t ncols, void *stream,
+                              const int64_t *t_after, const tn_plan_options *opt, const PlanUse &use, void *stream,
                               tn_plan **plan_out)
 {
-    return plan_create_impl(u, v, t, m, n, t_after, opt, stream, plan_out, true, ncols);
+    return plan_create_impl(u, v, t, m, n, t_after, opt, stream, plan_out, true, use);
 }
 
 tn_status tn::plan_create_ordered(const uint32_t *u, const uint32_t *v, const int64_t *t, uint64_t m, uint32_t n,
                                   const tn_plan_options *opt, cudaStream_t stream, tn_plan **plan_out)
 {
-    return plan_create_impl(u, v, t, m, n, nullptr, opt, stream, plan_out, false, n);
+    return plan_create_impl(u, v, t, m, n, nullptr, opt, stream, plan_out, false, PlanUse{n, false});
 }
 
 extern "C" tn_status tn_plan_destroy(tn_plan *p, void *stream)

@@ -151,7 +151,7 @@ extern "C" tn_status tn_out_sizes(const uint64_t *S, uint32_t n_rows, uint32_t n
     // four words a lane where they fill a warp; rows per CTA: as many as the
     // counters hold, in whole waves of two CTAs per SM, but a wave at least
     const int wpl = ld32 >= 96 && ((uintptr_t)S & 15u) == 0 ? 4 : 1;
-    const uint64_t cols = (ld32 + 32 * wpl - 1) / (32 * wpl), slots = 2 * 152;
+    const uint64_t cols = (ld32 + 32 * wpl - 1) / (32 * wpl), slots = 2 * (uint64_t)multiprocessors();
     const uint64_t waves = (cols * ((n_rows + kRowsMax - 1) / kRowsMax) + slots - 1) / slots;
     uint64_t blocks = waves * slots / cols;
     if (blocks < 1) blocks = 1;

@@ -161,3 +161,19 @@ def test_batches_of_small_networks(directed, tmp_path):
         assert np.array_equal(mats[k].cpu().numpy().view(np.uint64)[:, : refs[k].shape[1]], refs[k])
     assert stream_launch(lambda: plans[0].apply(mats[0], init=True), tmp_path)["grid"][0] == 125
     assert stream_launch(lambda: tn.tn_plan_apply_batch(plans * copies, mats), tmp_path)["grid"][0] == 2 * copies * 8
+
+
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("n,h,ties", [(26_000, 32, 1), (26_000, 8, 64), (20_000, 1, 64)])
+def test_columns_and_sketches_around_hubs(n, h, ties, directed):
+    """Few columns and sketches of streams of short levels: narrow records, with the
+    maximum as well."""
+    u, v, t = hubs(n, 60_000, h, ties, h)
+    events = dev(u, v, t)
+    src = np.random.default_rng(h).integers(0, n, 700).astype(np.uint32)
+    S = tn.tn_component_columns(*events, n, torch.from_numpy(src.view(np.int32)).cuda(), directed=directed)
+    ref = oracle.component_matrix_directed(u, v, t, n, src=src) if directed else oracle.component_matrix(u, v, t, n, src=src)
+    assert np.array_equal(S.cpu().numpy().view(np.uint64)[:, : ref.shape[1]], ref)
+    for p in (4, 10, 13):
+        R = tn.tn_hll_sketches(*events, n, p, 5, directed=directed)
+        assert np.array_equal(R.cpu().numpy()[:, : 1 << p], oracle.hll_sketches(u, v, t, n, p, 5, directed=directed))
