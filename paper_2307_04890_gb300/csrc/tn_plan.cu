@@ -182,7 +182,6 @@ struct PlanArgs {
     uint32_t dcap;       // row slots of a local window
     uint32_t unit8;      // staging units (8 bytes) per event
     uint32_t chain;      // 1: count the longest source lists
-    uint32_t redo;       // 1: the windows scheduled as records become tiles
     uint64_t *wstart;    // [nw + 1]
     uint32_t *naux_w;    // [nw] source-list entries of every window
     WinDesc *desc;       // [nw]
@@ -541,7 +540,8 @@ __device__ __forceinline__ void scan_levels(uint32_t E, const Arena<I> &A, I *nl
     }
 }
 
-template <typename I>
+// kTiles: a window that was scheduled as a record, again as tiles.
+template <typename I, bool kTiles = false>
 __device__ __forceinline__ void schedule_window(const PlanArgs &a, uint32_t w, uint8_t *arena)
 {
     __shared__ uint32_t warp_sums[32];
@@ -553,7 +553,7 @@ __device__ __forceinline__ void schedule_window(const PlanArgs &a, uint32_t w, u
     const uint32_t E = (uint32_t)(a.wstart[w + 1] - s);
     const uint32_t T = blockDim.x, tid = threadIdx.x, lane = tid & 31u;
     WinDesc *desc = a.desc + w;
-    const uint32_t record_units = a.redo ? desc->pack[0] : 0u;  // (overwritten below, by thread 0 at the earliest)
+    const uint32_t record_units = kTiles ? desc->pack[0] : 0u;  // (overwritten below, by thread 0 at the earliest)
     if (E == 0) {
         if (tid == 0) {
             *desc = WinDesc{};
@@ -694,7 +694,7 @@ __device__ __forceinline__ void schedule_window(const PlanArgs &a, uint32_t w, u
     //    shared-memory row buffer, and its record fits one staging buffer
     const uint32_t rec_words = 4 + D + (maxlev + 1) + nops + naux;
     const uint32_t rec_words_pad = (rec_words + 3u) & ~3u;
-    const bool local = !a.redo && E <= kRecordEvents && a.unit8 >= 5 && D + ntemp <= a.dcap && rec_words_pad <= kRecordWords;
+    const bool local = !kTiles && E <= kRecordEvents && a.unit8 >= 5 && D + ntemp <= a.dcap && rec_words_pad <= kRecordWords;
     const uint64_t region = blob_base(s, w, a.unit8);
 
     if (local) {
@@ -777,17 +777,21 @@ __device__ __forceinline__ void schedule_window(const PlanArgs &a, uint32_t w, u
         uint32_t *la = A.scratch + maxlev + 2;  // list words of the levels before
         uint32_t *lm = la + maxlev + 2;         // longest list of the level (a.chain)
         uint32_t *pq = lm + maxlev + 2;         // per pack: first op, its unit, next free list word (0: none), spare
-        for (uint32_t j = tid; j < maxlev + 1; j += T) la[j] = lm[j] = 0;
+        const bool chain = a.chain && nruns;
+        for (uint32_t j = tid; j < maxlev + 1; j += T) {
+            la[j] = 0;
+            if (chain) lm[j] = 0;
+        }
         __syncthreads();
         for (uint32_t r = tid; r < nruns; r += T) {
             const uint32_t c = auxw[A.run_aux[r]];
             atomicAdd(&la[A.run_lev[r]], 1u + c);
-            if (a.chain) atomicMax(&lm[A.run_lev[r]], c);
+            if (chain) atomicMax(&lm[A.run_lev[r]], c);
         }
         __syncthreads();
-        if (a.chain && nruns) {
+        if (chain && tid >= T - 32) {  // (the last warp: warp 0 cuts the packs)
             uint32_t sum = 0;
-            for (uint32_t j = tid; j < maxlev + 1; j += T) sum += lm[j];
+            for (uint32_t j = lane; j < maxlev + 1; j += 32) sum += lm[j];
             sum = __reduce_add_sync(0xffffffffu, sum);
             if (lane == 0 && sum) atomicAdd(&a.cnt->chain, (unsigned long long)sum);
         }
@@ -898,8 +902,8 @@ __device__ __forceinline__ void schedule_window(const PlanArgs &a, uint32_t w, u
         PlanCounters *c = a.cnt;
         const uint32_t units = res[1] + (res[0] > kDescPacks ? (res[0] + 1) / 2 : 0u);
         atomicAdd(&c->blob8, (unsigned long long)((units + 1) & ~1u) - record_units);
-        atomicAdd(&c->items, (unsigned long long)res[0] - a.redo);
-        if (a.redo) {  // (a record, counted once already)
+        atomicAdd(&c->items, (unsigned long long)res[0] - (kTiles ? 1u : 0u));
+        if (kTiles) {  // (a record, counted once already)
             atomicAdd(&c->local, ~0ull);
         } else {
             atomicAdd(&c->ops, (unsigned long long)nops);
@@ -957,7 +961,7 @@ __global__ void __launch_bounds__(kPlanThreads) schedule_tiles_kernel(PlanArgs a
     extern __shared__ __align__(16) uint8_t smem_arena[];
     const WinDesc *desc = a.desc + blockIdx.x;
     if (desc->npacks == 0 || desc->tab != 0) return;
-    schedule_window<uint16_t>(a, blockIdx.x, smem_arena);
+    schedule_window<uint16_t, true>(a, blockIdx.x, smem_arena);
 }
 
 // Copies the plan into a buffer of its exact size: what a finished plan needs of the
@@ -1327,7 +1331,6 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     // 16 words).  With a tenth of the windows as records, every update executed, some
     // streams are faster than as tiles (bursty n = 1.2 10^5, m = 3 10^6: 42.7 ms, 51.3).
     if (host.local && kTileShare * host.local <= a.nw && !wave && tracked_slab(sw, (uint64_t)rows * sw * 8)) {
-        a.redo = 1;
         TN_STEP(tn_internal_allow_max_dyn_smem((const void *)schedule_tiles_kernel));
         tn_internal_count_launches(1);
         schedule_tiles_kernel<<<a.nw, kPlanThreads, arena_bytes<uint16_t>(kRecordEvents), st>>>(a);
