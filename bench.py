@@ -40,7 +40,7 @@ ONLINE_METRIC = "events/s through the online state (batches that split timestamp
 STREAM_SOURCES = ["paper_2307_04890_gb300/csrc/tn_apply.cu", "paper_2307_04890_gb300/csrc/tn_internal.cuh",
                   "paper_2307_04890_gb300/csrc/tn_plan.cu"]
 PROFILE_SUMMARIES = {"activity": ("stream_kernel_activity_n1e5_m1e7.txt", STREAM_SOURCES),
-                     "bursty": ("stream_kernel_bursty_n5e5_m1e8_traffic.txt", STREAM_SOURCES),
+                     "bursty-scaled": ("stream_kernel_bursty_scaled_40000x503808_m2e6_traffic.txt", STREAM_SOURCES),
                      "online": ("grow_kernel_online_n1e5_to_102048.txt",
                                 ["paper_2307_04890_gb300/csrc/tn_online.cu",
                                  "paper_2307_04890_gb300/csrc/tn_internal.cuh"])}
@@ -514,6 +514,7 @@ def run_scaled(args, w, rank, world, local_rank):
     assert plan.status() == 0
     ms = statistics.mean(times)
     alg = 8 * plan.stats()["ops"] + n * tn.tn_row_words(ncols) * 8  # schedule in, matrix out
+    traffic = profiled_traffic("bursty-scaled", w["slab"])  # DRAM bytes of the launch (ncu)
     peak, _ = measured_peaks()
     if rank == 0:
         print(json.dumps({"metric": "bit-updates/s of the scaled bursty launch (profiling case)",
@@ -521,9 +522,9 @@ def run_scaled(args, w, rank, world, local_rank):
                           "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True,
                           "scaling": "weak", "vs_baseline": None, "dtype": "u64", "data": "synthetic",
                           "config": {"workload": w["desc"], "plan": plan.stats()},
-                          "roofline": {"bound": "hbm", "achieved": alg / (ms * 1e-3) / 1e9, "peak": peak,
-                                       "unit": "GB/s", "frac": alg / (ms * 1e-3) / 1e9 / peak, "traffic": None,
-                                       "algorithmic_bytes_per_launch": alg}}), flush=True)
+                          "roofline": {"bound": "hbm", "achieved": (traffic or alg) / (ms * 1e-3) / 1e9, "peak": peak,
+                                       "unit": "GB/s", "frac": (traffic or alg) / (ms * 1e-3) / 1e9 / peak,
+                                       "traffic": traffic, "algorithmic_bytes_per_launch": alg}}), flush=True)
 
 
 def run_serving(args, w, rank, world, local_rank):
@@ -1022,7 +1023,7 @@ def run_sweep(args, w, rank, world, local_rank):
         ex = tn.tn_autotune(dus, dvs, dts, n, sample_events=2_000_000)
         _, pus, pvs = tn.tn_hash_proxy(dus, dvs, n, k, K, w["seed"])
         px = tn.tn_autotune(pus[0].contiguous(), pvs[0].contiguous(), dts, k, replicas=K, sample_events=2_000_000)
-        tuned[n] = tuple({key: r[key] if r["best_ms"] <= r["open_ms"] else 0 for key in keys} for r in (ex, px))
+        tuned[n] = tuple({key: r[key] if r["best_ms"] <= 1.05 * r["open_ms"] else 0 for key in keys} for r in (ex, px))
         del dus, dvs, dts, pus, pvs
         m = 10_000
         while m <= mmax:
@@ -1162,7 +1163,7 @@ def main():
     tuned = None
     if args.autotune == "on" or (args.autotune == "auto" and w["kind"] in ("bursty", "er")):
         tuned = tn.tn_autotune(du, dv, dt, n, sample_events=args.tune_sample, ncols=ncols)
-        opts = {key: tuned[key] if tuned["best_ms"] <= tuned["open_ms"] else 0
+        opts = {key: tuned[key] if tuned["best_ms"] <= 1.05 * tuned["open_ms"] else 0  # (5 %: the timings' noise)
                 for key in ("window_events", "slab_words", "smem_rows", "wave_ctas", "resident_words")}
 
     def step(record):
