@@ -1117,7 +1117,8 @@ static void free_plan_buffers(tn_plan *p, cudaStream_t st)
 //    28.8 and 35.3; 256 hubs (119), n = 2 10^5: 11.7 and 7.2; activity-driven, n =
 //    2.6 10^4 (122): 2.1 and 2.1, n = 6 10^4 (202): 9.4 and 11.3.  In narrow slabs (few
 //    columns) records gain, 5,000 columns, 2 words: activity-driven n = 2.6 10^4 (128) 2.1
-//    and 1.4, n = 6 10^4 (218) 3.5 and 2.9, n = 10^5 (293) 2.7 and 2.8.
+//    and 1.4, n = 6 10^4 (218) 3.5 and 2.9, n = 10^5 (293) 2.7 and 2.8.  64 hubs (44), n =
+//    10^5, 32 words 63.3 and 18.7.
 //  - large timestamp groups that share nodes.  Bursty n = 2.6 10^4, m = 10^6 (81): 21.0
 //    and 15.5 ms; n = 10^5, m = 5 10^6 (306): 90.1 and 62.2; n = 1.2 10^5, m = 10^6
 //    (424): 14.5 and 14.6; n = 2 10^5, m = 5 10^6 (645): 92 and 137.
@@ -1348,11 +1349,25 @@ static tn_status plan_create_impl(const uint32_t *u, const uint32_t *v, const in
     p->ops = host.ops;
     p->local_windows = host.local;
     p->big_windows = host.big;
-    if (auto_window && window != kRecordWindow && sw <= 16 && records_faster(p, host.chain, use, record_slab)) {
-        free_plan_buffers(p, st);
-        if (a.late_arena) cudaFreeAsync(a.late_arena, st);
-        free(p);
-        return plan_create_impl(u, v, t, m, n, t_after, opt, stream, plan_out, wait_end, use, true);
+    if (auto_window && window != kRecordWindow && sw <= 32 && records_faster(p, host.chain, use, record_slab)) {
+        tn_plan *q = nullptr;
+        rc = plan_create_impl(u, v, t, m, n, t_after, opt, stream, &q, wait_end, use, true);
+        // in wide slabs the row buffer may hold too few rows for most windows (256 hubs,
+        // n = 6 10^4, 32 words: none, 25.0 ms in windows of 640, 20.6 ms as they were)
+        if (rc == TN_OK && (sw <= 16 || 2 * q->local_windows >= q->windows)) {
+            free_plan_buffers(p, st);
+            if (a.late_arena) cudaFreeAsync(a.late_arena, st);
+            free(p);
+            *plan_out = q;
+            return TN_OK;
+        }
+        if (q) {
+            free_plan_buffers(q, st);
+            free(q);
+        } else if (rc != TN_OK) {
+            cudaGetLastError();  // (no memory for a second schedule: the first one stands)
+            rc = TN_OK;
+        }
     }
     if (resident && !resident_fits(n, p->temps, resident)) {  // saved rows of the tie groups do not fit
         rc = TN_EINVAL;

@@ -108,6 +108,15 @@ def test_short_levels_become_records(stream, directed):
     assert stats["levels"] >= 256 and 0 < stats["local_windows"] <= stats["windows"] == -(-len(events[0]) // 640)
 
 
+@pytest.mark.parametrize("slab,h,records", [(24, 32, True), (32, 32, True), (32, 300, False), (64, 32, False)])
+def test_short_levels_in_wide_slabs(slab, h, records):
+    """Records where most windows fit the row buffer, else the tiles stay as they were."""
+    n = 60_000
+    stats = applied(hubs(n, 60_000, h, 1, h), n, slab_words=slab).stats()
+    assert stats["levels"] >= 256 and (stats["local_windows"] > 0) == records
+    assert stats["windows"] == -(-60_000 // (640 if records else 1280))
+
+
 def test_long_levels_stay_tiles():
     n = 26_000
     stats = applied(synth.er_poisson(n, 200_000, seed=3), n).stats()
